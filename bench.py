@@ -48,17 +48,14 @@ def _measured_peaks():
 
 BF16_PEAK_TFLOPS, BF16_SUSTAINED_TFLOPS = _measured_peaks()
 # BF16 tensor-core work per FP64-equivalent flop in the emulated mode: one modular product per
-# modulus of the Ozaki scheme II (17 moduli <= 256); a complex product is three real products
-# of order n (Gauss's form: Ar Vr, Ai Vi, (Ar + Ai)(Vr + Vi)), 3 x 2 n^2 per column against the
-# 8 n^2 FP64-equivalent flops of a complex column MatVec: 17 x 3/4 = 12.75 (17 for real).
-OZAKI_MODULI = 17
-OZAKI_PAIRS = OZAKI_MODULI * 0.75   # the default workload is complex
+# modulus of the Ozaki scheme II (17 moduli <= 256 for real products); a complex product is two
+# real products of order n for each of 15 moduli <= 509 in which -1 is a square, 2 x 2 n^2 per
+# column against the 8 n^2 FP64-equivalent flops of a complex column MatVec: 15 / 2 = 7.5.
+RING_MODULI = 15
+OZAKI_PAIRS = RING_MODULI * 0.5   # the default workload is complex
 # DRAM bytes (read + write) of one emulated product of the default workload (complex
-# n = 10000, 600 active columns), measured by one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum, 1 pass): the grouped modular products of the three real products
-# 12.12 GB read and 0.456 GB written; the reconstruction 0.404 GB read and 0.076 GB written.
-# Launches with fewer active columns read the same residue planes of A, which are most of it.
-OZ_TRAFFIC_PER_LAUNCH = 12.125e9 + 0.456e9 + 0.404e9 + 0.076e9
+# n = 10000, 600 active columns) by an ncu capture; None until one of these kernels is taken.
+OZ_TRAFFIC_PER_LAUNCH = None
 # Column MatVecs of one complete solve of the default workload as counted by the GPU path
 # (filter MatVecs plus the 2 (ell - k) products of Rayleigh-Ritz and residuals per
 # iteration); used to scale the oracle's timed sample to a whole solve.  Measured on a
@@ -152,12 +149,11 @@ def run_filter(args):
         line["frac_of_fp64_peak"] = flops / t / 1e12 / FP64_PEAK_TFLOPS
     else:
         # BF16 tensor-core work per step: BF16x3 three products of the stacked real operator
-        # (2n x 2n); the Ozaki scheme II 17 modular products of each of Gauss's three real
-        # products of order n
+        # (2n x 2n); the Ozaki scheme II two modular products of order n for each ring modulus
         if args.prec == "bf16x3":
             tc = 3 * 2.0 * (2 * n) * (2 * n) * k * args.degree / t / 1e12
         else:
-            tc = OZAKI_MODULI * 3 * 2.0 * n * n * k * args.degree / t / 1e12
+            tc = RING_MODULI * 2 * 2.0 * n * n * k * args.degree / t / 1e12
         line["bf16_tensor_tflops"] = tc
         line["frac_of_bf16_peak"] = tc / BF16_PEAK_TFLOPS
     print(json.dumps(line), flush=True)
@@ -718,9 +714,8 @@ def main():
         pipe = tc_flops / nl / dur_launch / 1e12 if dur_launch > 0 else None
         traffic = (OZ_TRAFFIC_PER_LAUNCH if (OZ_TRAFFIC_PER_LAUNCH and lp == 0 and args.n == 10000
                                              and args.prec == "fp64_emu") else None)
-        roof = {"kernel": "ozm_group_kernel + crt3_kernel (Ozaki scheme II FP64 product: 17 modular "
-                          "BF16 tcgen05 products of each of Gauss's three real products, CRT "
-                          "reconstruction)" +
+        roof = {"kernel": "ozm_group_kernel + crt_ring_kernel (Ozaki scheme II FP64 product: 15 "
+                          "moduli x 2 modular BF16 tcgen05 products, CRT reconstruction)" +
                           (" + tc_filter_bf16x3_kernel" if lp > 0 else ""),
                 "bound": "tensor", "achieved": achieved, "peak": BF16_SUSTAINED_TFLOPS,
                 "unit": "TFLOP/s", "frac": achieved / BF16_SUSTAINED_TFLOPS if achieved else None,

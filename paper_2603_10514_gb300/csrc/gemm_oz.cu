@@ -27,6 +27,10 @@
 // ((P/p_j)^{-1} mod p_j), in 160-bit integer arithmetic (32-bit limbs), mapped
 // to the symmetric range (-P/2, P/2] and rounded once to FP64.
 //
+// Complex A*V and A*Q products use a second set of moduli in which -1 is a square (every prime
+// factor is 1 mod 4): Z_p[i] then splits into two copies of Z_p, and one complex product takes
+// TWO real modular products per modulus (see "Complex products in split residue rings").
+//
 // Modular product kernel (ozm_kernel): CTA pairs (clusters of two along grid x), one pair
 // per (256-row block, column tile of BN <= 256 columns, modulus[, K split]).  The even CTA
 // issues tcgen05.mma.cta_group::2.kind::f16 (M 256, N BN, K 16) over the pair: each CTA
@@ -180,6 +184,119 @@ static_assert(oz_moduli_above(160), "epilogue reduction: p > 160");
 static_assert((long long)kOzSplitMaxK * 128 * 128 <= (1ll << 30), "epilogue reduction: |sum| <= 2^30");
 static_assert(kOzMaxK <= kOzMaxSplits * kOzSplitMaxK, "every admissible K fits the splits");
 
+// ---------------------------------------------------------------------------
+// Complex products in split residue rings
+// ---------------------------------------------------------------------------
+// For a modulus p whose prime factors are all 1 mod 4 there is an s with s^2 = -1 mod p, and
+//   a + i b  ->  (a + s b, a - s b) mod p
+// turns a complex product into two independent real ones:  with U = sum (Ar + s Ai)(Vr + s Vi)
+// and W = sum (Ar - s Ai)(Vr - s Vi),  Re(A V) = (U + W) / 2  and  Im(A V) = (U - W) / (2 s)
+// mod p.  Two modular products per modulus where the product of order n by Gauss's form takes
+// three and the stacked real operator of order 2n four; the integers of A and V, and so the
+// results, are the same bit for bit.  Moduli up to 509 keep residues |r| <= 254 exact in BF16
+// (8 significant bits) and give ~8.8 bits each: 15 of them (P ~ 2^131.4) cover |Re|, |Im| <=
+// 2 K 2^114 for K <= 2^15, 16 (2^139.8) every admissible K.  Their price: an exact FP32 chunk
+// is 256 wide (256 254^2 < 2^24) instead of 1024, and a residue of the product takes two bytes.
+// Per complex product of order n: 30 BF16 products (17 moduli x 3 by Gauss's form: 51).
+// Bound: the tensor pipe and its L2 feed.  Measured (filter call, degrees 10-36, GB300): n = 10000,
+// 600 columns 136.0 -> 84.0 ms, n = 3000, 180 columns 11.50 -> 7.06 ms against Gauss's form.
+__host__ __device__ constexpr int ring_modulus(int j) {
+  constexpr int tr[kRingModuli] = {509, 505, 493, 481, 461, 457, 449, 433,
+                                   421, 409, 401, 397, 389, 373, 353, 349};
+  return tr[j];
+}
+// s with s^2 = -1 mod p_j
+__host__ __device__ constexpr uint32_t ring_root(int j) {
+  const uint32_t p = (uint32_t)ring_modulus(j);
+  for (uint32_t s = 1; s < p; ++s)
+    if ((s * s + 1) % p == 0) return s;
+  return 0;
+}
+
+// CRT constants of the first NM ring moduli: X_re = sum_j (U_j + W_j) Cre_j mod P and
+// X_im = sum_j (U_j - W_j + p_j) Cim_j mod P, with Cre_j = 1/2 and Cim_j = 1/(2 s_j) mod p_j,
+// both 0 mod every other modulus.
+template <int NM>
+struct RingTable {
+  uint32_t Cre[NM][5], Cim[NM][5];
+  uint32_t P[5], Ph[5];
+  float p96_over_P;
+};
+
+template <int NM>
+constexpr RingTable<NM> make_ring_table() {
+  RingTable<NM> t{};
+  Big P = big_small(1);
+  for (int j = 0; j < NM; ++j) P = big_mul_small(P, (uint32_t)ring_modulus(j));
+  for (int j = 0; j < NM; ++j) {
+    const uint32_t p = (uint32_t)ring_modulus(j);
+    Big Mj = big_small(1);
+    for (int i = 0; i < NM; ++i)
+      if (i != j) Mj = big_mul_small(Mj, (uint32_t)ring_modulus(i));
+    const uint32_t inv = inv_mod(big_mod_small(Mj, p), p);
+    const Big Cre = big_mul_small(Mj, inv * inv_mod(2, p) % p);
+    const Big Cim = big_mul_small(Mj, inv * inv_mod(2 * ring_root(j) % p, p) % p);
+    for (int l = 0; l < 5; ++l) {
+      t.Cre[j][l] = Cre.w[l];
+      t.Cim[j][l] = Cim.w[l];
+    }
+  }
+  const Big Ph = big_shr1(P);
+  double pd = 0.0;
+  for (int l = 4; l >= 0; --l) {
+    t.P[l] = P.w[l];
+    t.Ph[l] = Ph.w[l];
+    pd = pd * 4294967296.0 + (double)P.w[l];
+  }
+  t.p96_over_P = (float)(79228162514264337593543950336.0 / pd);
+  return t;
+}
+constexpr int kRingShort = 15;
+__constant__ RingTable<kRingShort> c_ring15 = make_ring_table<kRingShort>();
+__constant__ RingTable<kRingModuli> c_ring16 = make_ring_table<kRingModuli>();
+template <int NM> __device__ __forceinline__ const RingTable<NM>& ring_table();
+template <> __device__ __forceinline__ const RingTable<kRingShort>& ring_table<kRingShort>() { return c_ring15; }
+template <> __device__ __forceinline__ const RingTable<kRingModuli>& ring_table<kRingModuli>() { return c_ring16; }
+
+constexpr bool ring_moduli_ok() {
+  for (int i = 0; i < kRingModuli; ++i) {
+    const uint32_t p = (uint32_t)ring_modulus(i), s = ring_root(i);
+    if (s == 0 || (s * s + 1) % p != 0) return false;
+    // exact chunks, with the folded sum of the earlier ones (fold2)
+    if (kRingChunk * (long long)(p / 2) * (p / 2) + p >= (1ll << 24)) return false;
+    for (int j = i + 1; j < kRingModuli; ++j)
+      if (oz_gcd((int)p, ring_modulus(j)) != 1) return false;
+  }
+  return true;
+}
+template <int NM>
+constexpr bool ring_crt_ok() {
+  const RingTable<NM> t = make_ring_table<NM>();
+  for (int j = 0; j < NM; ++j) {
+    const Big Cre{{t.Cre[j][0], t.Cre[j][1], t.Cre[j][2], t.Cre[j][3], t.Cre[j][4]}};
+    const Big Cim{{t.Cim[j][0], t.Cim[j][1], t.Cim[j][2], t.Cim[j][3], t.Cim[j][4]}};
+    for (int i = 0; i < NM; ++i) {
+      const uint32_t p = (uint32_t)ring_modulus(i);
+      if (big_mod_small(Cre, p) * 2 % p != (i == j ? 1u : 0u)) return false;
+      if (big_mod_small(Cim, p) * (2 * ring_root(i) % p) % p != (i == j ? 1u : 0u)) return false;
+    }
+  }
+  return true;
+}
+static_assert(ring_moduli_ok(), "ring moduli: -1 a square, exact chunks, pairwise coprime");
+static_assert(ring_crt_ok<kRingShort>() && ring_crt_ok<kRingModuli>(), "ring CRT basis");
+// P > 2 * (2 K 2^114): K <= 2^15 with 15 moduli, K <= 2^17 with 16
+static_assert(make_ring_table<kRingShort>().P[4] >= (1u << (2 * OZ_KBITS + 15 + 2 - 128)), "ring range, 15");
+static_assert(make_ring_table<kRingModuli>().P[4] >= (1u << (2 * OZ_KBITS + 17 + 2 - 128)), "ring range, 16");
+static_assert(kRingShortMaxK == (1 << 15), "ring_moduli()");
+
+__constant__ int c_ring_p[kRingModuli] = {ring_modulus(0),  ring_modulus(1),  ring_modulus(2),
+                                          ring_modulus(3),  ring_modulus(4),  ring_modulus(5),
+                                          ring_modulus(6),  ring_modulus(7),  ring_modulus(8),
+                                          ring_modulus(9),  ring_modulus(10), ring_modulus(11),
+                                          ring_modulus(12), ring_modulus(13), ring_modulus(14),
+                                          ring_modulus(15)};
+
 constexpr int MBM = 128, MBK = 64;
 constexpr int MKS = 2;             // 64-wide K blocks per stage: 8 MMAs per barrier round trip
 constexpr int MNST = 3;            // stages
@@ -187,6 +304,7 @@ constexpr int MBN_MAX = 256;
 constexpr int M_EPI_WARPS = 16;
 constexpr int M_THREADS = 64 + 32 * M_EPI_WARPS;
 constexpr int M_CHUNK_ST = 1024 / (MKS * MBK);  // stages per exact 1024-wide K chunk
+constexpr int M_RING_CHUNK_ST = kRingChunk / (MKS * MBK);          // and of a ring modulus
 constexpr int M_A1 = MBM * MBK * 2;              // 16 KB: 128 rows of A, one K block
 constexpr int M_B1 = (MBN_MAX / 2) * MBK * 2;    // 16 KB: up to 128 rows of V (half a tile)
 constexpr int M_STG = MKS * (M_A1 + M_B1);       // 64 KB
@@ -207,10 +325,42 @@ using namespace tc;
 // residues into Rz (column-major M x N).  kbeg is even; an odd nkb reads one zero-filled
 // block past kp (the K-padded operands end there), or the first block of the next split
 // only when nkb is odd, which the launch never makes for a split other than the last.
+// s mod p in [0, p) by a float quotient that is off by at most one.
+__device__ __forceinline__ int mod_sum(int s, int p, float ip) {
+  const int q = (int)floorf((float)s * ip);
+  int r = s - q * p;
+  if (r < 0) r += p;
+  if (r >= p) r -= p;
+  return r;
+}
+
+__device__ __forceinline__ uint64_t pack2(float x, float y) {
+  return (uint64_t)__float_as_uint(x) | ((uint64_t)__float_as_uint(y) << 32);
+}
+// Two sums mod p advanced by one chunk each: s = acc + v is an exact integer below 2^24
+// (256 254^2 + p/2), q = round(s / p) to within 2^-8, and s - q p, exact, lies within 0.51 p.
+// Four packed FP32 operations per pair: float-to-integer conversions issue at 16 per clock
+// per SM and would take longer than the chunk's MMAs.
+__device__ __forceinline__ uint64_t fold2(uint64_t acc, uint32_t v0, uint32_t v1, uint64_t ip2, uint64_t np2) {
+  const uint64_t magic = 0x4B4000004B400000ull;   // 1.5 * 2^23, twice
+  const uint64_t nmagic = 0xCB400000CB400000ull;
+  uint64_t v, s, q, r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(v0), "r"(v1));
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(acc), "l"(v));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(s), "l"(ip2), "l"(magic));
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(q), "l"(nmagic));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(q), "l"(np2), "l"(s));
+  return r;
+}
+
+// RING: modulus jm of the ring set, 256-wide exact chunks folded mod p as they come (no limit
+// on the length of K), two-byte residues.
+template <bool RING>
 __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUtensorMap* mapV,
                                               int M, int N, int BN, int col0, int m0, int n0,
-                                              int jm, int kbeg, int nkb, uint8_t* __restrict__ Rz,
+                                              int jm, int kbeg, int nkb, void* __restrict__ Rv,
                                               DevStatus* status) {
+  constexpr int CHUNK_ST = RING ? M_RING_CHUNK_ST : M_CHUNK_ST;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + MNST * M_STG);
@@ -226,7 +376,7 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
   const uint32_t rank = cluster_rank();
   const int half = BN >> 1;
   const int nst = (nkb + MKS - 1) / MKS;
-  const int nchunks = (nst + M_CHUNK_ST - 1) / M_CHUNK_ST;
+  const int nchunks = (nst + CHUNK_ST - 1) / CHUNK_ST;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < MNST; ++i) { bar_init(&full[i], 1); bar_init(&empty[i], 1); }
@@ -278,9 +428,9 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
                            ((uint32_t)((2 * MBM) >> 4) << 24);
     bool bad = false;
     for (int kb = 0; kb < nst && !bad; ++kb) {
-      const int chunk = kb / M_CHUNK_ST;
-      const bool cstart = (kb % M_CHUNK_ST) == 0;
-      const bool clast = (kb % M_CHUNK_ST) == M_CHUNK_ST - 1 || kb == nst - 1;
+      const int chunk = kb / CHUNK_ST;
+      const bool cstart = (kb % CHUNK_ST) == 0;
+      const bool clast = (kb % CHUNK_ST) == CHUNK_ST - 1 || kb == nst - 1;
       const uint32_t buf = (uint32_t)(chunk & 1);
       if (cstart && chunk >= 2) {
         // both CTAs' epilogues have read this buffer's previous chunk (chunk - 2)
@@ -310,9 +460,16 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
     const int r = m0 + 32 * q + lane;
     const int cw = BN >> 2;
     const uint32_t cfree0 = peer_addr(cfree, 0);
-    int sum[64];
+    const int pm = RING ? c_ring_p[jm] : c_crt.p[jm];
+    const float ip = 1.0f / (float)pm;
+    // sums of the chunks: 32-bit integers, or (ring) pairs of floats in (-0.51 p, 0.51 p)
+    int sum[RING ? 1 : 64];
+    uint64_t acc[RING ? 32 : 1];
+    const uint64_t ip2 = pack2(ip, ip), np2 = pack2(-(float)pm, -(float)pm);
 #pragma unroll
-    for (int j = 0; j < 64; ++j) sum[j] = 0;
+    for (int j = 0; j < (RING ? 1 : 64); ++j) sum[j] = 0;
+#pragma unroll
+    for (int j = 0; j < (RING ? 32 : 1); ++j) acc[j] = 0;
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       const uint32_t buf = (uint32_t)(c & 1);
@@ -323,38 +480,38 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * MBN_MAX + (uint32_t)(cq * cw);
-      uint32_t v[32];
-      ld32(ta, v);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      // 16 columns at a time: wider reads spill, and a spill in this loop costs more than the reads
 #pragma unroll
-      for (int j = 0; j < 32; ++j) sum[j] += __float2int_rn(__uint_as_float(v[j]));
-      if (cw > 32) {
-        ld32(ta + 32, v);
+      for (int g = 0; g < 4; ++g) {
+        if (16 * g >= cw) break;
+        uint32_t v[16];
+        ld16(ta + 16 * g, v);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if constexpr (RING) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            acc[8 * g + j] = fold2(acc[8 * g + j], v[2 * j], v[2 * j + 1], ip2, np2);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) sum[16 * g + j] += __float2int_rn(__uint_as_float(v[j]));
+        }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0 && c + 2 < nchunks) arrive_remote(cfree0 + 8u * buf);
-      if (cw > 32) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) sum[32 + j] += __float2int_rn(__uint_as_float(v[j]));
-      }
+      if (lane == 0 && c + 2 < nchunks) arrive_remote_relaxed(cfree0 + 8u * buf);
     }
     if (__shfl_sync(0xffffffffu, (int)(ok && !*(volatile int*)s_err), 0) && r < M) {
-      // sum mod p in [0, p): |sum| <= 2^30 (K <= kOzSplitMaxK per split), so the float quotient is
-      // off by at most one
-      const int pm = c_crt.p[jm];
-      const float ip = 1.0f / (float)pm;
+      // the sum mod p in [0, p)
 #pragma unroll
       for (int j = 0; j < 64; ++j) {
         const int col = n0 + cq * cw + j;
         if (j < cw && col - n0 < BN && col < N) {
-          const int sv = sum[j];
-          const int qq = (int)floorf((float)sv * ip);
-          int rr = sv - qq * pm;
-          if (rr < 0) rr += pm;
-          if (rr >= pm) rr -= pm;
-          Rz[(size_t)col * M + r] = (uint8_t)rr;
+          if constexpr (RING) {
+            const int rr = (int)__uint_as_float((uint32_t)(acc[j >> 1] >> (32 * (j & 1))));
+            ((uint16_t*)Rv)[(size_t)col * M + r] = (uint16_t)(rr < 0 ? rr + pm : rr);
+          } else {
+            ((uint8_t*)Rv)[(size_t)col * M + r] = (uint8_t)mod_sum(sum[j], pm, ip);
+          }
         }
       }
     }
@@ -387,8 +544,8 @@ __global__ void __launch_bounds__(M_THREADS, 1)
   const int nkb = max(0, min(kbs, nkb_total - kbeg));
   int m0, n0;
   pair_tile_coords(blockIdx.x, ntile, BN, &m0, &n0);
-  ozm_pair_tile(&mapA, &mapV, M, N, BN, col0, m0, n0, jm, kbeg, nkb,
-                R + (size_t)blockIdx.z * N * M, status);
+  ozm_pair_tile<false>(&mapA, &mapV, M, N, BN, col0, m0, n0, jm, kbeg, nkb,
+                       R + (size_t)blockIdx.z * N * M, status);
 }
 
 // Grouped products: the tiles of up to kOzGroupMax independent problems in one launch
@@ -398,7 +555,8 @@ __global__ void __launch_bounds__(M_THREADS, 1)
 struct OzmGroupParams {
   CUtensorMap mapA[kOzGroupMax];
   CUtensorMap mapV[kOzGroupMax];
-  uint8_t* R[kOzGroupMax];
+  void* R[kOzGroupMax];        // residues: one byte, or two (ring products)
+  int ring[kOzGroupMax];       // 0: the real moduli; else the number of ring moduli
   int tile0[kOzGroupMax + 1];  // first grid-x CTA of each problem (even: pairs never straddle)
   int M[kOzGroupMax], N[kOzGroupMax], BN[kOzGroupMax], col0[kOzGroupMax], ntile[kOzGroupMax],
       nkb[kOzGroupMax];
@@ -411,10 +569,16 @@ __global__ void __launch_bounds__(M_THREADS, 1)
   int p = 0;
   while (p + 1 < P.count && (int)blockIdx.x >= P.tile0[p + 1]) ++p;
   const int jm = blockIdx.z;
+  if (jm >= (P.ring[p] ? P.ring[p] : kOzModuli)) return;  // (the pair leaves together)
   int m0, n0;
   pair_tile_coords((int)blockIdx.x - P.tile0[p], P.ntile[p], P.BN[p], &m0, &n0);
-  ozm_pair_tile(&P.mapA[p], &P.mapV[p], P.M[p], P.N[p], P.BN[p], P.col0[p], m0, n0, jm, 0,
-                P.nkb[p], P.R[p] + (size_t)jm * P.N[p] * P.M[p], status);
+  const size_t slab = (size_t)jm * P.N[p] * P.M[p];
+  if (P.ring[p])
+    ozm_pair_tile<true>(&P.mapA[p], &P.mapV[p], P.M[p], P.N[p], P.BN[p], P.col0[p], m0, n0, jm, 0,
+                        P.nkb[p], (uint16_t*)P.R[p] + slab, status);
+  else
+    ozm_pair_tile<false>(&P.mapA[p], &P.mapV[p], P.M[p], P.N[p], P.BN[p], P.col0[p], m0, n0, jm, 0,
+                         P.nkb[p], (uint8_t*)P.R[p] + slab, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -426,7 +590,8 @@ __global__ void __launch_bounds__(M_THREADS, 1)
 // Returns the FP64 rounding m of |X| and the sign, with X = m 2^{*shift}.
 // X = sum_j r_j C_j mod P from the residues r_j < p_j, rounded once to FP64: returns the
 // signed magnitude and *shift_out with |X| = |value| 2^shift.
-__device__ __forceinline__ double crt_finish(const unsigned long long* acc, int* shift_out);
+template <class Tab>
+__device__ __forceinline__ double crt_finish(const unsigned long long* acc, const Tab& tab, int* shift_out);
 __device__ __forceinline__ double crt_combine(const uint32_t* rj, int* shift_out) {
   unsigned long long acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll
@@ -434,12 +599,13 @@ __device__ __forceinline__ double crt_combine(const uint32_t* rj, int* shift_out
 #pragma unroll
     for (int l = 0; l < 5; ++l) acc[l] += (unsigned long long)rj[j] * c_crt.C[j][l];
   }
-  return crt_finish(acc, shift_out);
+  return crt_finish(acc, c_crt, shift_out);
 }
 
 // X = (sum_j r_j C_j, accumulated in 32-bit limbs with 64-bit headroom) mod P, rounded once to
 // FP64.
-__device__ __forceinline__ double crt_finish(const unsigned long long* acc, int* shift_out) {
+template <class Tab>
+__device__ __forceinline__ double crt_finish(const unsigned long long* acc, const Tab& tab, int* shift_out) {
   uint32_t x[5];
   unsigned long long carry = 0;
 #pragma unroll
@@ -448,16 +614,16 @@ __device__ __forceinline__ double crt_finish(const unsigned long long* acc, int*
     x[l] = (uint32_t)t;
     carry = t >> 32;
   }
-  // X < 17 * 256 * P < 2^146: reduce mod P with q = floor(X / P) from the top limbs.  q is
-  // below 2^13, so the FP32 estimate (relative error ~2^-22) is off by at most one; both
+  // X < 17 * 256 * P < 2^146 (ring: 16 * 1024 * P < 2^154): reduce mod P with q = floor(X / P) from the top limbs.  q is
+  // below 2^15, so the FP32 estimate (relative error ~2^-22) is off by at most one; both
   // corrections follow.
   const float xf = (float)x[4] * 4294967296.0f + (float)x[3];  // X / 2^96, rounded
-  const unsigned int qv = (unsigned int)floorf(xf * c_crt.p96_over_P);
+  const unsigned int qv = (unsigned int)floorf(xf * tab.p96_over_P);
   {
     unsigned long long borrow = 0, cq = 0;
 #pragma unroll
     for (int l = 0; l < 5; ++l) {
-      const unsigned long long prod = (unsigned long long)c_crt.P[l] * qv + cq;
+      const unsigned long long prod = (unsigned long long)tab.P[l] * qv + cq;
       cq = prod >> 32;
       const unsigned long long sub = (unsigned long long)(uint32_t)prod + borrow;
       const long long d = (long long)x[l] - (long long)sub;
@@ -468,7 +634,7 @@ __device__ __forceinline__ double crt_finish(const unsigned long long* acc, int*
       unsigned long long c = 0;
 #pragma unroll
       for (int l = 0; l < 5; ++l) {
-        const unsigned long long t = (unsigned long long)x[l] + c_crt.P[l] + c;
+        const unsigned long long t = (unsigned long long)x[l] + tab.P[l] + c;
         x[l] = (uint32_t)t;
         c = t >> 32;
       }
@@ -480,11 +646,11 @@ __device__ __forceinline__ double crt_finish(const unsigned long long* acc, int*
     }
     return true;
   };
-  if (cmp_ge(c_crt.P)) {  // q was one too small
+  if (cmp_ge(tab.P)) {  // q was one too small
     long long br = 0;
 #pragma unroll
     for (int l = 0; l < 5; ++l) {
-      const long long d = (long long)x[l] - (long long)c_crt.P[l] - br;
+      const long long d = (long long)x[l] - (long long)tab.P[l] - br;
       x[l] = (uint32_t)d;
       br = d < 0 ? 1 : 0;
     }
@@ -493,14 +659,14 @@ __device__ __forceinline__ double crt_finish(const unsigned long long* acc, int*
   bool neg = false;
   bool gt_half = false;
   for (int l = 4; l >= 0; --l) {
-    if (x[l] != c_crt.Ph[l]) { gt_half = x[l] > c_crt.Ph[l]; break; }
+    if (x[l] != tab.Ph[l]) { gt_half = x[l] > tab.Ph[l]; break; }
   }
   if (gt_half) {
     neg = true;
     long long br = 0;
 #pragma unroll
     for (int l = 0; l < 5; ++l) {
-      const long long d = (long long)c_crt.P[l] - (long long)x[l] - br;
+      const long long d = (long long)tab.P[l] - (long long)x[l] - br;
       x[l] = (uint32_t)d;
       br = d < 0 ? 1 : 0;
     }
@@ -608,55 +774,67 @@ __global__ void __launch_bounds__(256) crt4_kernel(int M, int N, int splits, con
   }
 }
 
-// Reconstruction of one problem in the three-product layout (residues of P1 | P2 | P3, n x N
-// each): four consecutive entries per thread, every residue plane read as 4-byte words;
-// Re = P1 - P2 to stacked row r, Im = P3 - P1 - P2 to row n + r (both scaled by row r).
-__global__ void __launch_bounds__(256) crt3_kernel(int n, int N, const uint8_t* __restrict__ R,
-                                                   const int* __restrict__ rowexp,
-                                                   const int* __restrict__ colexp, int col0,
-                                                   double alpha, double beta, const double* X64,
-                                                   double gamma, const double* Z64, double* out64,
-                                                   int ldo) {
+// Re and Im of one entry from its ring residues U_j, W_j (u, w < p_j), each rounded once.
+template <int NM>
+__device__ __forceinline__ void ring_combine(const uint32_t* u, const uint32_t* w, double* re, int* sre,
+                                             double* im, int* sim) {
+  const RingTable<NM>& tab = ring_table<NM>();
+  unsigned long long are[5] = {0, 0, 0, 0, 0}, aim[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    const uint32_t s = u[j] + w[j], d = u[j] + (uint32_t)ring_modulus(j) - w[j];
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+      are[l] += (unsigned long long)s * tab.Cre[j][l];
+      aim[l] += (unsigned long long)d * tab.Cim[j][l];
+    }
+  }
+  *re = crt_finish(are, tab, sre);
+  *im = crt_finish(aim, tab, sim);
+}
+
+// Reconstruction of one ring problem (residues of U | W, n x N each, two bytes): four
+// consecutive entries per thread, every residue plane read as 8-byte words; Re to stacked row
+// r, Im to row n + r (both scaled by row r).
+template <int NM>
+__global__ void __launch_bounds__(256) crt_ring_kernel(int n, int N, const uint16_t* __restrict__ R,
+                                                       const int* __restrict__ rowexp,
+                                                       const int* __restrict__ colexp, int col0,
+                                                       double alpha, double beta, const double* X64,
+                                                       double gamma, const double* Z64, double* out64,
+                                                       int ldo) {
   const size_t total = (size_t)n * N, quads = total / 4;
-  const uint32_t* R4 = (const uint32_t*)R;
-  const size_t stride4 = total / 4, set4 = (size_t)kOzModuli * stride4;
+  const uint2* R4 = (const uint2*)R;
+  const size_t stride4 = total / 4, set4 = (size_t)NM * stride4;
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < quads;
        q += (size_t)gridDim.x * blockDim.x) {
-    uint32_t w1[kOzModuli], w2[kOzModuli], w3[kOzModuli];
+    uint2 wu[NM], ww[NM];
 #pragma unroll
-    for (int j = 0; j < kOzModuli; ++j) {
-      w1[j] = __ldg(R4 + (size_t)j * stride4 + q);
-      w2[j] = __ldg(R4 + set4 + (size_t)j * stride4 + q);
-      w3[j] = __ldg(R4 + 2 * set4 + (size_t)j * stride4 + q);
+    for (int j = 0; j < NM; ++j) {
+      wu[j] = __ldg(R4 + (size_t)j * stride4 + q);
+      ww[j] = __ldg(R4 + set4 + (size_t)j * stride4 + q);
     }
 #pragma unroll 1
     for (int e = 0; e < 4; ++e) {
-      unsigned long long are[5] = {0, 0, 0, 0, 0}, aim[5] = {0, 0, 0, 0, 0};
+      uint32_t u[NM], w[NM];
 #pragma unroll
-      for (int j = 0; j < kOzModuli; ++j) {
-        const uint32_t pj = (uint32_t)oz_modulus(j);
-        const uint32_t r1 = (w1[j] >> (8 * e)) & 0xFFu, r2 = (w2[j] >> (8 * e)) & 0xFFu,
-                       r3 = (w3[j] >> (8 * e)) & 0xFFu;
-        const uint32_t re = (r1 + pj - r2) % pj, im = (r3 + 2 * pj - r1 - r2) % pj;
-#pragma unroll
-        for (int l = 0; l < 5; ++l) {
-          are[l] += (unsigned long long)re * c_crt.C[j][l];
-          aim[l] += (unsigned long long)im * c_crt.C[j][l];
-        }
+      for (int j = 0; j < NM; ++j) {
+        u[j] = ((e & 2 ? wu[j].y : wu[j].x) >> (16 * (e & 1))) & 0xFFFFu;
+        w[j] = ((e & 2 ? ww[j].y : ww[j].x) >> (16 * (e & 1))) & 0xFFFFu;
       }
       const size_t t = 4 * q + e;
       const int r = (int)(t % n), c = (int)(t / n);
-      int sh;
-      double x = crt_finish(are, &sh);
-      crt_store(x, sh, r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo);
-      x = crt_finish(aim, &sh);
-      crt_store(x, sh, n + r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo, r);
+      double re, im;
+      int sre, sim;
+      ring_combine<NM>(u, w, &re, &sre, &im, &sim);
+      crt_store(re, sre, r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo);
+      crt_store(im, sim, n + r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo, r);
     }
   }
 }
 
 struct CrtGroupParams {
-  const uint8_t* R[kOzGroupMax];
+  const void* R[kOzGroupMax];
   const int* rowexp[kOzGroupMax];
   const int* colexp[kOzGroupMax];
   const double* X64[kOzGroupMax];
@@ -665,10 +843,30 @@ struct CrtGroupParams {
   double alpha[kOzGroupMax], beta[kOzGroupMax], gamma[kOzGroupMax];
   long long out0[kOzGroupMax + 1];  // first output index of each problem
   int M[kOzGroupMax], N[kOzGroupMax], col0[kOzGroupMax], ldo[kOzGroupMax];
-  int c3[kOzGroupMax];  // three-product layout: M = n, residues of P1 | P2 | P3, stacked output
+  int ring[kOzGroupMax];  // ring moduli (0: a real problem): M = n, residues of U | W, stacked output
   int count;
 };
 static_assert(sizeof(CrtGroupParams) <= 32000, "kernel parameter space");
+
+template <int NM>
+__device__ __forceinline__ void crt_ring_entry(const CrtGroupParams& P, int p, long long u, int r, int c) {
+  const int M = P.M[p];
+  const size_t stride_z = (size_t)M * P.N[p];
+  const uint16_t* R = (const uint16_t*)P.R[p] + u;
+  uint32_t ru[NM], rw[NM];
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    ru[j] = R[(size_t)j * stride_z];
+    rw[j] = R[(size_t)(NM + j) * stride_z];
+  }
+  double re, im;
+  int sre, sim;
+  ring_combine<NM>(ru, rw, &re, &sre, &im, &sim);
+  crt_store(re, sre, r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
+            P.gamma[p], P.Z64[p], P.out64[p], P.ldo[p]);
+  crt_store(im, sim, M + r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
+            P.gamma[p], P.Z64[p], P.out64[p], P.ldo[p], r);
+}
 
 __global__ void __launch_bounds__(256) crt_group_kernel(const __grid_constant__ CrtGroupParams P) {
   const long long total = P.out0[P.count];
@@ -683,30 +881,13 @@ __global__ void __launch_bounds__(256) crt_group_kernel(const __grid_constant__ 
     const long long u = t - P.out0[p];
     const int M = P.M[p];
     const int r = (int)(u % M), c = (int)(u / M);
-    if (P.c3[p]) {
-      // Re = P1 - P2 (output row r), Im = P3 - P1 - P2 (row n + r), both scaled by row r
-      const size_t stride_z = (size_t)M * P.N[p], set = (size_t)kOzModuli * stride_z;
-      const uint8_t* R = P.R[p];
-      uint32_t re[kOzModuli], im[kOzModuli];
-#pragma unroll
-      for (int j = 0; j < kOzModuli; ++j) {
-        const uint32_t pj = (uint32_t)oz_modulus(j);
-        const size_t at = (size_t)j * stride_z + (size_t)u;
-        const uint32_t r1 = R[at], r2 = R[set + at], r3 = R[2 * set + at];
-        re[j] = (r1 + pj - r2) % pj;
-        im[j] = (r3 + 2 * pj - r1 - r2) % pj;
-      }
-      int sh;
-      double x = crt_combine(re, &sh);
-      crt_store(x, sh, r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
-                P.gamma[p], P.Z64[p], P.out64[p], P.ldo[p]);
-      x = crt_combine(im, &sh);
-      crt_store(x, sh, M + r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
-                P.gamma[p], P.Z64[p], P.out64[p], P.ldo[p], r);
+    if (P.ring[p]) {
+      if (P.ring[p] == kRingShort) crt_ring_entry<kRingShort>(P, p, u, r, c);
+      else crt_ring_entry<kRingModuli>(P, p, u, r, c);
       continue;
     }
     int sh;
-    const double x = crt_value(P.R[p], (size_t)M * P.N[p], (size_t)u, 1, &sh);
+    const double x = crt_value((const uint8_t*)P.R[p], (size_t)M * P.N[p], (size_t)u, 1, &sh);
     const int E = sh + P.rowexp[p][r] + P.colexp[p][P.col0[p] + c] - 2 * OZ_KBITS;
     const double v0 = (E > -1022 && E < 1024) ? x * __longlong_as_double((long long)(E + 1023) << 52)
                                               : ldexp(x, E);
@@ -778,44 +959,49 @@ __device__ __forceinline__ void write_residues_int(long long X, __nv_bfloat16* b
   }
 }
 
-// The symmetric residues of X (|X| < 2^59) mod p_j as small integers (|r| <= 128).
-__device__ __forceinline__ void residues_of(long long X, int* r) {
-  const unsigned long long U = (unsigned long long)(X < 0 ? -X : X);
-  const uint32_t U1 = (uint32_t)(U >> 29), U0 = (uint32_t)(U & ((1u << 29) - 1));
+// Ring residues of four adjacent K entries: u = (xr + s xi) mod p and w = (xr - s xi) mod p in
+// symmetric range (|r| <= 254, exact in BF16), planes u then w, stored as 8-byte words.
+// X + 2^58 >= 0 is cut into 21 | 19 | 19 bits, so X mod p needs one unreduced 31-bit sum of
+// three products by constants and one division by a constant (the shift's class is taken off
+// in the same sum): integer work bounds the slicing, not HBM.
+template <int NM>
+__device__ __forceinline__ void write_ring4(const long long* xr, const long long* xi, __nv_bfloat16* base,
+                                            size_t idx, size_t plane) {
+  uint32_t r0[4], r1[4], r2[4], i0[4], i1[4], i2[4];
 #pragma unroll
-  for (int j = 0; j < kOzModuli; ++j) {
-    const uint32_t p = (uint32_t)oz_modulus(j);
-    const uint32_t k29 = (uint32_t)((1ull << 29) % p);
-    const uint32_t u = ((U1 % p) * k29 + U0 % p) % p;
-    int rr = X < 0 ? -(int)u : (int)u;
-    if (rr > (int)p / 2) rr -= (int)p;
-    else if (rr < -((int)p / 2)) rr += (int)p;
-    r[j] = rr;
+  for (int d = 0; d < 4; ++d) {
+    const unsigned long long R = (unsigned long long)(xr[d] + (1LL << 58));
+    const unsigned long long I = (unsigned long long)(xi[d] + (1LL << 58));
+    r0[d] = (uint32_t)R & 0x7FFFFu;
+    r1[d] = (uint32_t)(R >> 19) & 0x7FFFFu;
+    r2[d] = (uint32_t)(R >> 38);
+    i0[d] = (uint32_t)I & 0x7FFFFu;
+    i1[d] = (uint32_t)(I >> 19) & 0x7FFFFu;
+    i2[d] = (uint32_t)(I >> 38);
   }
-}
-
-// Residues of two adjacent K entries (idx, idx + 1) of three plane sets: the parts' integers
-// Xr, Xi and their sum, whose residue is the sum of the parts' residues brought back into the
-// symmetric range (a representative of the same class: the modular products use only the
-// class, and |r| <= 128 keeps their K chunks exact).  Stored as BF16 pairs.
-__device__ __forceinline__ void write_residues3_pair(long long xr0, long long xi0, long long xr1,
-                                                     long long xi1, __nv_bfloat16* base, size_t idx,
-                                                     size_t plane, size_t set) {
-  int a0[kOzModuli], b0[kOzModuli], a1[kOzModuli], b1[kOzModuli];
-  residues_of(xr0, a0);
-  residues_of(xi0, b0);
-  residues_of(xr1, a1);
-  residues_of(xi1, b1);
 #pragma unroll
-  for (int j = 0; j < kOzModuli; ++j) {
-    const int p = oz_modulus(j);
-    int s0 = a0[j] + b0[j], s1 = a1[j] + b1[j];
-    if (s0 > p / 2) s0 -= p; else if (s0 < -(p / 2)) s0 += p;
-    if (s1 > p / 2) s1 -= p; else if (s1 < -(p / 2)) s1 += p;
+  for (int j = 0; j < NM; ++j) {
+    const uint32_t p = (uint32_t)ring_modulus(j), s = ring_root(j);
+    const uint32_t k19 = (uint32_t)((1ull << 19) % p), k38 = (uint32_t)((1ull << 38) % p);
+    const uint32_t off = p - (uint32_t)((1ull << 58) % p), half = p / 2;
+    float fu[4], fw[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      // < 2^21 2^9 + 2^19 2^9 + 2^19 + 2^9 < 2^31, and + s ti < 2^18
+      const uint32_t tr = r2[d] * k38 + r1[d] * k19 + r0[d] + off;
+      const uint32_t ti = (i2[d] * k38 + i1[d] * k19 + i0[d] + off) % p;
+      const uint32_t u = tr + s * ti + half, w = tr + (p - s) * ti + half;
+      fu[d] = (float)((int)(u % p) - (int)half);
+      fw[d] = (float)((int)(w % p) - (int)half);
+    }
     const size_t at = idx + (size_t)j * plane;
-    *(__nv_bfloat162*)(base + at) = __nv_bfloat162(__int2bfloat16_rn(a0[j]), __int2bfloat16_rn(a1[j]));
-    *(__nv_bfloat162*)(base + set + at) = __nv_bfloat162(__int2bfloat16_rn(b0[j]), __int2bfloat16_rn(b1[j]));
-    *(__nv_bfloat162*)(base + 2 * set + at) = __nv_bfloat162(__int2bfloat16_rn(s0), __int2bfloat16_rn(s1));
+    __nv_bfloat162 pk[2];
+    pk[0] = __floats2bfloat162_rn(fu[0], fu[1]);
+    pk[1] = __floats2bfloat162_rn(fu[2], fu[3]);
+    *(uint2*)(base + at) = *(const uint2*)pk;
+    pk[0] = __floats2bfloat162_rn(fw[0], fw[1]);
+    pk[1] = __floats2bfloat162_rn(fw[2], fw[3]);
+    *(uint2*)(base + (size_t)NM * plane + at) = *(const uint2*)pk;
   }
 }
 
@@ -838,37 +1024,23 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
   return mx;
 }
 
-// Stacked real A (M = n or 2n): residues of row m into planes (row-major, ld kp), row
-// exponent into rowexp[m].  Row m of Ahat = column m of Ahat (symmetric), read from A.
-template <class T>
-__global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const T* __restrict__ A, int lda,
+// Real A (n x n): residues of row m (column m of A: symmetric) into planes (row-major, ld kp),
+// row exponent into rowexp[m].
+__global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __restrict__ A, int lda,
                                                          int kp, __nv_bfloat16* planes,
                                                          size_t plane, int* rowexp) {
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
-  const int mm = m % n;
-  const bool mre = m < n;
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  auto elem = [&](int k) -> double {
-    if constexpr (Sc<T>::cplx) {
-      const z64 a = A[(size_t)(k % n) + (size_t)mm * lda];  // A[k mod n, mm]
-      const bool kre = k < n;
-      return (kre == mre) ? a.x : (kre ? -a.y : a.y);
-    } else {
-      return A[(size_t)k + (size_t)m * lda];
-    }
-  };
+  const double* col = A + (size_t)m * lda;
   unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < M; k += 256) {
-    const unsigned long long b = abs_bits(elem(k));
+  for (int k = threadIdx.x; k < n; k += 256) {
+    const unsigned long long b = abs_bits(col[k]);
     amax = b > amax ? b : amax;
   }
   const int e = exp_bound(block_max(amax, red));
   if (threadIdx.x == 0) rowexp[m] = e;
-  for (int k = threadIdx.x; k < kp; k += 256) {
-    const double x = (k < M) ? elem(k) : 0.0;
-    write_residues(x, e, planes, (size_t)m * kp + k, plane);
-  }
+  for (int k = threadIdx.x; k < kp; k += 256)
+    write_residues(k < n ? col[k] : 0.0, e, planes, (size_t)m * kp + k, plane);
 }
 
 // FP64 stacked block V64 (M x ncols, ld ldi): residues of column c into planes
@@ -892,23 +1064,17 @@ __global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const do
   }
 }
 
-// ---- Gauss's three products for complex operands ----
-// A = Ar + i Ai, V = Vr + i Vi: with the row exponents of A (over Re and Im together) and the
-// column exponents of V as in the stacked form, the integers of Ar, Ai, Vr, Vi are those of
-// the stacked operands, and
-//   P1 = Ar Vr,  P2 = Ai Vi,  P3 = (Ar + Ai)(Vr + Vi)   (exact integer products mod p_j)
-//   Re(A V) = P1 - P2,  Im(A V) = P3 - P1 - P2
-// are the stacked product's two halves as the same integers: three real products of order n
-// instead of one of order 2n (3/4 of the MMA work and of A's residue planes), the same
-// results bit for bit.  The residues of Ar + Ai (|.| <= 2^58) come from the integer sums.
-// Layout: three plane sets (Ar | Ai | Ar + Ai, or Vr | Vi | Vr + Vi), each kOzModuli planes,
-// one after another.
+// ---- operands of the ring products ----
+// The row exponents of A (over Re and Im together) and the column exponents of V are those of
+// the stacked form, and so are the integers of Ar, Ai, Vr, Vi.  Layout: two plane sets (u | w),
+// each NM planes of one row per row of A (column of V), K contiguous.
 
-// Row m of A (complex Hermitian, column-major): its three integer rows from column m of A
+// Row m of A (complex Hermitian, column-major): its integer row from column m of A
 // (A[m, k] = conj(A[k, m])): Ar[m, k] = Re A[k, m], Ai[m, k] = -Im A[k, m].
-__global__ void __launch_bounds__(256) oz_slice_A3_kernel(int n, const z64* __restrict__ A, int lda,
-                                                          int kpn, __nv_bfloat16* planes, size_t plane,
-                                                          size_t set, int* rowexp) {
+template <int NM>
+__global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* __restrict__ A, int lda,
+                                                              int kpn, __nv_bfloat16* planes, size_t plane,
+                                                              int* rowexp) {
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const z64* col = A + (size_t)m * lda;
@@ -919,25 +1085,24 @@ __global__ void __launch_bounds__(256) oz_slice_A3_kernel(int n, const z64* __re
   }
   const int e = exp_bound(block_max(amax, red));
   if (threadIdx.x == 0) rowexp[m] = e;
-  for (int k = 2 * threadIdx.x; k < kpn; k += 512) {  // kpn is even: pairs (k, k + 1)
-    long long xr[2] = {0, 0}, xi[2] = {0, 0};
+  for (int k = 4 * threadIdx.x; k < kpn; k += 1024) {  // kpn is a multiple of 64
+    long long xr[4], xi[4];
 #pragma unroll
-    for (int d = 0; d < 2; ++d) {
-      if (k + d < n) {
-        const z64 a = col[k + d];
-        xr[d] = oz_int(a.x, e);
-        xi[d] = -oz_int(a.y, e);
-      }
+    for (int d = 0; d < 4; ++d) {
+      const z64 a = (k + d < n) ? col[k + d] : z64{0.0, 0.0};
+      xr[d] = oz_int(a.x, e);
+      xi[d] = -oz_int(a.y, e);
     }
-    write_residues3_pair(xr[0], xi[0], xr[1], xi[1], planes, (size_t)m * kpn + k, plane, set);
+    write_ring4<NM>(xr, xi, planes, (size_t)m * kpn + k, plane);
   }
 }
 
 // Column c of the stacked FP64 block V64 ([Re V; Im V], 2n rows, ld ldi): its exponent over
-// both halves, then the three integer columns (Vr | Vi | Vr + Vi), ld kpn.
-__device__ __forceinline__ void slice_V3_column(int n, int c, const double* __restrict__ V64, int ldi,
-                                                int kpn, __nv_bfloat16* planes, size_t plane, size_t set,
-                                                int* colexp, unsigned long long* red) {
+// both halves, then its two plane rows (u | w), ld kpn.
+template <int NM>
+__device__ __forceinline__ void slice_V_ring_column(int n, int c, const double* __restrict__ V64, int ldi,
+                                                    int kpn, __nv_bfloat16* planes, size_t plane,
+                                                    int* colexp, unsigned long long* red) {
   const double* col = V64 + (size_t)c * ldi;
   unsigned long long amax = 0;
   for (int k = threadIdx.x; k < 2 * n; k += 256) {
@@ -946,16 +1111,15 @@ __device__ __forceinline__ void slice_V3_column(int n, int c, const double* __re
   }
   const int e = exp_bound(block_max(amax, red));
   if (threadIdx.x == 0) colexp[c] = e;
-  for (int k = 2 * threadIdx.x; k < kpn; k += 512) {  // kpn is even: pairs (k, k + 1)
-    long long xr[2] = {0, 0}, xi[2] = {0, 0};
+  for (int k = 4 * threadIdx.x; k < kpn; k += 1024) {
+    long long xr[4], xi[4];
 #pragma unroll
-    for (int d = 0; d < 2; ++d) {
-      if (k + d < n) {
-        xr[d] = oz_int(col[k + d], e);
-        xi[d] = oz_int(col[n + k + d], e);
-      }
+    for (int d = 0; d < 4; ++d) {
+      const bool in = k + d < n;
+      xr[d] = oz_int(in ? col[k + d] : 0.0, e);
+      xi[d] = oz_int(in ? col[n + k + d] : 0.0, e);
     }
-    write_residues3_pair(xr[0], xi[0], xr[1], xi[1], planes, (size_t)c * kpn + k, plane, set);
+    write_ring4<NM>(xr, xi, planes, (size_t)c * kpn + k, plane);
   }
 }
 
@@ -967,7 +1131,7 @@ struct SliceGroupParams {
   long long plane[kOzGroupMax];
   int blk0[kOzGroupMax + 1];  // first block of each problem
   int M[kOzGroupMax], c0[kOzGroupMax], ldi[kOzGroupMax], kp[kOzGroupMax];
-  int c3[kOzGroupMax];  // complex problem in the three-product layout (M = n)
+  int ring[kOzGroupMax];  // ring moduli of a complex problem (M = n); 0: real
   int count;
 };
 static_assert(sizeof(SliceGroupParams) <= 32000, "kernel parameter space");
@@ -978,9 +1142,13 @@ __global__ void __launch_bounds__(256) oz_slice_V_group_kernel(const __grid_cons
   while (p + 1 < P.count && (int)blockIdx.x >= P.blk0[p + 1]) ++p;
   const int c = P.c0[p] + (blockIdx.x - P.blk0[p]);
   const int M = P.M[p], kp = P.kp[p];
-  if (P.c3[p]) {
-    slice_V3_column(M, c, P.V64[p], P.ldi[p], kp, P.planes[p], (size_t)P.plane[p],
-                    (size_t)kOzModuli * P.plane[p], P.colexp[p], red);
+  if (P.ring[p]) {
+    if (P.ring[p] == kRingShort)
+      slice_V_ring_column<kRingShort>(M, c, P.V64[p], P.ldi[p], kp, P.planes[p], (size_t)P.plane[p],
+                                      P.colexp[p], red);
+    else
+      slice_V_ring_column<kRingModuli>(M, c, P.V64[p], P.ldi[p], kp, P.planes[p], (size_t)P.plane[p],
+                                       P.colexp[p], red);
     return;
   }
   const double* col = P.V64[p] + (size_t)c * P.ldi[p];
@@ -1144,12 +1312,13 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
   return fn;
 }
 
-// 3-D BF16 map over the residue planes: {kp (contiguous), rows, S}, box {64, box_rows, 1},
+// 3-D BF16 map over the residue planes: {kp (contiguous), rows, planes}, box {64, box_rows, 1},
 // 128-byte swizzle; consecutive planes are plane_rows * kp elements apart.
-int make_map3(CUtensorMap* map, const void* base, int kp, int rows, int plane_rows, int box_rows) {
+int make_map3(CUtensorMap* map, const void* base, int kp, int rows, int plane_rows, int box_rows,
+              int planes = kOzModuli) {
   auto enc = encoder();
   if (!enc) return CHASE_ERR_CUDA;
-  cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)kOzModuli};
+  cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)rows, (cuuint64_t)planes};
   cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)kp * 2 * (cuuint64_t)plane_rows};
   cuuint32_t box[3] = {MBK, (cuuint32_t)box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
@@ -1161,26 +1330,29 @@ int make_map3(CUtensorMap* map, const void* base, int kp, int rows, int plane_ro
 
 }  // namespace
 
+size_t ring_residue_bytes(int n, int kpn, int N) {
+  return (size_t)2 * ring_moduli(kpn) * sizeof(uint16_t) * (size_t)n * (size_t)N;
+}
+
 size_t oz_residue_bytes(int M, int N) {
   return (size_t)kOzMaxSplits * kOzModuli * (size_t)M * (size_t)N;
 }
 
-template <class T>
-int oz_slice_A(cudaStream_t st, int n, const T* A, int lda, int kp, void* planes, int* rowexp,
+int oz_slice_A(cudaStream_t st, int n, const double* A, int lda, int kp, void* planes, int* rowexp,
                int* launches) {
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  oz_slice_A_kernel<T><<<M, 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)planes,
-                                          (size_t)M * kp, rowexp);
+  oz_slice_A_kernel<<<n, 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
 }
 
-int oz_slice_A3(cudaStream_t st, int n, const z64* A, int lda, int kpn, void* planes, int* rowexp,
-                int* launches) {
+int oz_slice_A_ring(cudaStream_t st, int n, const z64* A, int lda, int kpn, void* planes, int* rowexp,
+                    int* launches) {
   const size_t plane = (size_t)n * kpn;
-  oz_slice_A3_kernel<<<n, 256, 0, st>>>(n, A, lda, kpn, (__nv_bfloat16*)planes, plane,
-                                        (size_t)kOzModuli * plane, rowexp);
+  if (ring_moduli(kpn) == kRingShort)
+    oz_slice_A_ring_kernel<kRingShort><<<n, 256, 0, st>>>(n, A, lda, kpn, (__nv_bfloat16*)planes, plane, rowexp);
+  else
+    oz_slice_A_ring_kernel<kRingModuli><<<n, 256, 0, st>>>(n, A, lda, kpn, (__nv_bfloat16*)planes, plane, rowexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1340,7 +1512,7 @@ int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* 
       P.c0[p] = it.col0;
       P.ldi[p] = it.ldi;
       P.kp[p] = it.kp;
-      P.c3[p] = it.c3;
+      P.ring[p] = it.ring ? ring_moduli(it.kp) : 0;
       blocks += it.N;
     }
     if (P.count == 0) continue;
@@ -1363,13 +1535,16 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     if (P.count == 0) return 0;
     P.tile0[P.count] = tiles;
     C.out0[C.count] = outs;
-    TRY_OZ(launch_pairs(ozm_group_kernel, dim3(tiles, 1, kOzModuli), st, P, dst));
+    int planes = 0;  // moduli of the longest set in the launch
+    for (int p = 0; p < P.count; ++p) planes = std::max(planes, P.ring[p] ? P.ring[p] : kOzModuli);
+    TRY_OZ(launch_pairs(ozm_group_kernel, dim3(tiles, 1, planes), st, P, dst));
     if (launches) ++*launches;
-    if (C.count == 1 && C.c3[0] && outs % 4 == 0) {  // one complex problem: the vector form
+    if (C.count == 1 && C.ring[0] && outs % 4 == 0) {  // one complex problem: the vector form
       const int b4 = (int)std::max<long long>(1, std::min<long long>((outs / 4 + 255) / 256, (long long)kNumSMs * 16));
-      crt3_kernel<<<b4, 256, 0, st>>>(C.M[0], C.N[0], C.R[0], C.rowexp[0], C.colexp[0], C.col0[0],
-                                      C.alpha[0], C.beta[0], C.X64[0], C.gamma[0], C.Z64[0],
-                                      C.out64[0], C.ldo[0]);
+      auto kern = C.ring[0] == kRingShort ? crt_ring_kernel<kRingShort> : crt_ring_kernel<kRingModuli>;
+      kern<<<b4, 256, 0, st>>>(C.M[0], C.N[0], (const uint16_t*)C.R[0], C.rowexp[0], C.colexp[0],
+                               C.col0[0], C.alpha[0], C.beta[0], C.X64[0], C.gamma[0], C.Z64[0],
+                               C.out64[0], C.ldo[0]);
     } else {
       const int blocks = (int)std::max<long long>(1, std::min<long long>((outs + 255) / 256, (long long)kNumSMs * 16));
       crt_group_kernel<<<blocks, 256, 0, st>>>(C);
@@ -1386,23 +1561,26 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     const OzGroupItem& it = items[i];
     if (it.N <= 0 || it.M <= 0) continue;
     if (it.kp % MBK != 0 || it.kp > kOzSplitMaxK) return CHASE_ERR_UNSUPPORTED;  // K is not split here
-    const int sets = it.c3 ? 3 : 1;  // three-product layout: P1, P2, P3
-    if ((size_t)sets * kOzModuli * it.M * it.N > it.resbuf.bytes) return CHASE_ERR_OOM;
+    const int sets = it.ring ? 2 : 1;  // ring products: U, W
+    const int nm = it.ring ? ring_moduli(it.kp) : kOzModuli;
+    const size_t rset = (size_t)nm * (it.ring ? 2 : 1) * it.M * it.N;  // residue bytes of one set
+    if (sets * rset > it.resbuf.bytes) return CHASE_ERR_OOM;
     if (P.count + sets > kOzGroupMax || C.count + 1 > kOzGroupMax) TRY_OZ(flush());
     OzPlan plan;  // the autotuner's tile width for this shape, if it measured one
     oz_plan_lookup(it.M, it.N, it.kp, &plan);
     const int ntile = ceil_div(it.N, std::min(plan.bn_max, MBN_MAX));
     const int BN = ceil_div(ceil_div(it.N, ntile), 16) * 16;
     const int rows = std::max(it.a_plane_rows, it.M);
-    const size_t aset = (size_t)kOzModuli * rows * it.kp * 2;             // bytes of one A plane set
-    const size_t vset = (size_t)kOzModuli * it.ncols_total * it.kp * 2;   // of one V plane set
+    const size_t aset = (size_t)nm * rows * it.kp * 2;             // bytes of one A plane set
+    const size_t vset = (size_t)nm * it.ncols_total * it.kp * 2;   // of one V plane set
     for (int sidx = 0; sidx < sets; ++sidx) {
       const int p = P.count++;
-      if (make_map3(&P.mapA[p], (const char*)it.Aplanes + sidx * aset, it.kp, it.M, rows, MBM) ||
+      if (make_map3(&P.mapA[p], (const char*)it.Aplanes + sidx * aset, it.kp, it.M, rows, MBM, nm) ||
           make_map3(&P.mapV[p], (const char*)it.Vplanes + sidx * vset, it.kp, it.ncols_total,
-                    it.ncols_total, BN / 2))
+                    it.ncols_total, BN / 2, nm))
         return CHASE_ERR_CUDA;
-      P.R[p] = (uint8_t*)it.resbuf.ptr + (size_t)sidx * kOzModuli * it.M * it.N;
+      P.R[p] = (char*)it.resbuf.ptr + sidx * rset;
+      P.ring[p] = it.ring ? nm : 0;
       P.tile0[p] = tiles;
       P.M[p] = it.M;
       P.N[p] = it.N;
@@ -1413,7 +1591,7 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
       tiles += ntile * ceil_div(it.M, 2 * MBM) * 2;  // CTA pairs over 256-row blocks
     }
     const int c = C.count++;
-    C.R[c] = (const uint8_t*)it.resbuf.ptr;
+    C.R[c] = it.resbuf.ptr;
     C.rowexp[c] = it.rowexp;
     C.colexp[c] = it.colexp;
     C.X64[c] = it.X64;
@@ -1427,7 +1605,7 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     C.N[c] = it.N;
     C.col0[c] = it.col0;
     C.ldo[c] = it.ldo;
-    C.c3[c] = it.c3;
+    C.ring[c] = it.ring ? nm : 0;
     outs += (long long)it.M * it.N;
   }
   return flush();
@@ -1503,7 +1681,5 @@ OZ_INST(z64)
 
 template int oz_stack_V<double>(cudaStream_t, int, int, const double*, int, double*, int, int*);
 template int oz_stack_V<z64>(cudaStream_t, int, int, const z64*, int, double*, int, int*);
-template int oz_slice_A<double>(cudaStream_t, int, const double*, int, int, void*, int*, int*);
-template int oz_slice_A<z64>(cudaStream_t, int, const z64*, int, int, void*, int*, int*);
 
 }  // namespace chase

@@ -123,16 +123,25 @@ constexpr int kOzMaxSplits = 2;                 // K splits of one product (resi
 constexpr int kOzMaxK = 1 << 17;                // longest K the moduli's product covers
 constexpr int kOzSplitMaxK = 1 << 16;           // longest K of one split: |sum| <= 2^16 * 128^2 = 2^30,
                                                 // the range of the modular epilogue's reduction
+// Complex A V products run in split residue rings: moduli <= 509 with s^2 = -1 mod p, two plane
+// sets (a + s b | a - s b), 15 moduli for K <= 2^15 and 16 above.
+constexpr int kRingModuli = 16;
+constexpr int kRingChunk = 256;                 // exact FP32 chunk: 256 * 254^2 < 2^24
+constexpr int kRingShortMaxK = 1 << 15;
+constexpr int ring_moduli(int kp) { return kp <= kRingShortMaxK ? 15 : kRingModuli; }
+// bytes of residue planes per (complex) operand element, and of the product's residues
+constexpr size_t ring_plane_bytes(int kp) { return (size_t)2 * 2 * ring_moduli(kp); }
+size_t ring_residue_bytes(int n, int kpn, int N);
 // Device bytes of the residue buffer oz_gemm needs for an M x N product.
 size_t oz_residue_bytes(int M, int N);
-template <class T>
-int oz_slice_A(cudaStream_t st, int n, const T* A, int lda, int kp, void* planes, int* rowexp,
+// Real A (n x n, symmetric, column-major): kOzModuli planes of n x kp, row exponents.
+int oz_slice_A(cudaStream_t st, int n, const double* A, int lda, int kp, void* planes, int* rowexp,
                int* launches);
-// Complex A (n x n, Hermitian, column-major) into the three-product layout: plane sets
-// Re A | Im A | Re A + Im A, each kOzModuli planes of n x kpn (row-major, K contiguous),
-// row exponents over Re and Im together (those of the stacked form).
-int oz_slice_A3(cudaStream_t st, int n, const z64* A, int lda, int kpn, void* planes, int* rowexp,
-                int* launches);
+// Complex A (n x n, Hermitian, column-major) into ring residues: plane sets u | w, each
+// ring_moduli(kpn) planes of n x kpn (row-major, K contiguous), row exponents over Re and Im
+// together (those of the stacked form).
+int oz_slice_A_ring(cudaStream_t st, int n, const z64* A, int lda, int kpn, void* planes, int* rowexp,
+                    int* launches);
 int oz_slice_V(cudaStream_t st, int M, int c0, int c1, const double* V64, int ldi, int kp,
                int ncols_total, void* planes, int* colexp, int* launches);
 template <class T>
@@ -195,9 +204,9 @@ struct OzGroupItem {
   Scratch resbuf{nullptr, 0};
   const double* V64_in = nullptr;
   int ldi = 0;
-  // complex problem in the three-product layout: M = n, Aplanes / Vplanes hold three plane
-  // sets (Re | Im | Re + Im), V64_in / X64 / Z64 / out64 are the stacked [Re; Im] blocks
-  int c3 = 0;
+  // complex problem in ring residues: M = n, Aplanes / Vplanes hold two plane sets (u | w),
+  // V64_in / X64 / Z64 / out64 are the stacked [Re; Im] blocks
+  int ring = 0;
 };
 int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* launches);
 int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatus* dst, int* launches);

@@ -321,27 +321,38 @@ int filter_mixed(chase_ctx* h, int n, const T* A, int lda, bool split_A, int nco
 // ---------------------------------------------------------------------------
 struct OzBufs {
   int M = 0, kp = 0, ncols = 0;  // stacked FP64 blocks: M rows, ld kp
-  // complex problems: the three-product layout (Gauss): A and V planes as Re | Im | Re + Im
-  // sets of n rows (K padded to kpn); the FP64 blocks stay stacked
-  int c3 = 0, n = 0, kpn = 0;
+  // complex problems: ring residues, A and V planes as u | w sets of n rows (K padded to kpn);
+  // the FP64 blocks stay stacked
+  int ring = 0, n = 0, kpn = 0;
   void* Ap = nullptr;
   int* rowexp = nullptr;
   void* Vp = nullptr;
   int* colexp = nullptr;
   double* V64[2] = {nullptr, nullptr};
-  Scratch res{nullptr, 0};  // residues of the modular products (oz_residue_bytes(kp, ncols))
+  Scratch res{nullptr, 0};  // residues of the modular products
 };
+
+// Bytes of the residue planes of A and V and of the modular products' residues: stacked real
+// operands, or ring residues of order n (complex).
+struct OzSizes { size_t a, v, res; };
+template <class T>
+OzSizes oz_sizes(int n, int ncols) {
+  const int kpn = tc_kpad(n);
+  if (Sc<T>::cplx) {
+    const size_t pb = ring_plane_bytes(kpn);
+    return OzSizes{align256(pb * n * (size_t)kpn), align256(pb * kpn * (size_t)ncols),
+                   align256(ring_residue_bytes(n, kpn, ncols))};
+  }
+  return OzSizes{align256(kOzPlaneBytes * n * (size_t)kpn), align256(kOzPlaneBytes * kpn * (size_t)ncols),
+                 align256(oz_residue_bytes(kpn, ncols))};
+}
 
 template <class T>
 size_t oz_bytes(int n, int ncols) {
   const int M = Sc<T>::cplx ? 2 * n : n;
   const size_t kp = (size_t)tc_kpad(M);
-  // plane rows x K of A and K x columns of V: stacked (real) or three sets of order n (complex)
-  const size_t arows = Sc<T>::cplx ? 3 * (size_t)n : (size_t)M;
-  const size_t ak = Sc<T>::cplx ? (size_t)tc_kpad(n) : kp;
-  const size_t vk = Sc<T>::cplx ? 3 * (size_t)tc_kpad(n) : kp;
-  return align256(kOzPlaneBytes * arows * ak) + align256(4 * (size_t)M) + align256(kOzPlaneBytes * vk * ncols) +
-         align256(4 * (size_t)ncols) + 2 * align256(8 * kp * ncols) + align256(oz_residue_bytes((int)kp, ncols));
+  const OzSizes s = oz_sizes<T>(n, ncols);
+  return s.a + align256(4 * (size_t)M) + s.v + align256(4 * (size_t)ncols) + 2 * align256(8 * kp * ncols) + s.res;
 }
 
 template <class T>
@@ -350,30 +361,27 @@ OzBufs oz_carve(char* base, int n, int ncols) {
   B.M = Sc<T>::cplx ? 2 * n : n;
   B.kp = tc_kpad(B.M);
   B.ncols = ncols;
-  B.c3 = Sc<T>::cplx ? 1 : 0;
+  B.ring = Sc<T>::cplx ? 1 : 0;
   B.n = n;
   B.kpn = tc_kpad(n);
-  const size_t arows = B.c3 ? 3 * (size_t)n : (size_t)B.M;
-  const size_t ak = B.c3 ? (size_t)B.kpn : (size_t)B.kp;
-  const size_t vk = B.c3 ? 3 * (size_t)B.kpn : (size_t)B.kp;
+  const OzSizes s = oz_sizes<T>(n, ncols);
   size_t off = 0;
-  B.Ap = base + off; off += align256(kOzPlaneBytes * arows * ak);
+  B.Ap = base + off; off += s.a;
   B.rowexp = (int*)(base + off); off += align256(4 * (size_t)B.M);
-  B.Vp = base + off; off += align256(kOzPlaneBytes * vk * ncols);
+  B.Vp = base + off; off += s.v;
   B.colexp = (int*)(base + off); off += align256(4 * (size_t)ncols);
   for (int i = 0; i < 2; ++i) { B.V64[i] = (double*)(base + off); off += align256(8 * (size_t)B.kp * ncols); }
-  B.res = Scratch{base + off, oz_residue_bytes(B.kp, ncols)};
-  off += align256(oz_residue_bytes(B.kp, ncols));
+  B.res = Scratch{base + off, s.res};
   return B;
 }
 
-// A's planes in the layout of B (three-product sets for complex problems, stacked otherwise).
+// A's planes in the layout of B (ring residues for complex problems).
 template <class T>
 int oz_slice_A_bufs(chase_ctx* h, int n, const T* A, int lda, OzBufs& B) {
-  if constexpr (Sc<T>::cplx) {
-    if (B.c3) return oz_slice_A3(h->stream, n, A, lda, B.kpn, B.Ap, B.rowexp, &h->launches);
-  }
-  return oz_slice_A<T>(h->stream, n, A, lda, B.kp, B.Ap, B.rowexp, &h->launches);
+  if constexpr (Sc<T>::cplx)
+    return oz_slice_A_ring(h->stream, n, A, lda, B.kpn, B.Ap, B.rowexp, &h->launches);
+  else
+    return oz_slice_A(h->stream, n, A, lda, B.kp, B.Ap, B.rowexp, &h->launches);
 }
 
 // A grouped-product item of B's operands: out64 = alpha A V64_in[:, col0 .. col0 + N) +
@@ -382,9 +390,9 @@ inline OzGroupItem oz_item(const OzBufs& B, int ncols_total, int col0, int N, do
                            const double* X64, double gamma, const double* Z64, double* out64,
                            const double* V64_in) {
   OzGroupItem it;
-  it.c3 = B.c3;
-  it.M = B.c3 ? B.n : B.M;
-  it.kp = B.c3 ? B.kpn : B.kp;
+  it.ring = B.ring;
+  it.M = B.ring ? B.n : B.M;
+  it.kp = B.ring ? B.kpn : B.kp;
   it.a_plane_rows = it.M;
   it.Aplanes = B.Ap;
   it.rowexp = B.rowexp;
@@ -438,7 +446,7 @@ int filter_oz_enqueue(chase_ctx* h, int n, const T* A, int lda, bool split_A, in
       gamma = -sigma * sn;
       sigma = sn;
     }
-    if (B.c3) {
+    if (B.ring) {
       const OzGroupItem it = oz_item(B, ncols, first, act, alpha, beta, B.V64[in], gamma, B.V64[out],
                                      B.V64[out], B.V64[in]);
       TRY(oz_slice_V_group(st, 1, &it, &h->launches));
@@ -535,7 +543,7 @@ int aq_oz(chase_ctx* h, int n, const T* Q, int nu, T* AQ, OzBufs& B, Scratch scr
   cudaStream_t st = h->stream;
   if (nu <= 0) return 0;
   TRY(oz_stack_V<T>(st, n, nu, Q, n, B.V64[0], B.kp, &h->launches));
-  if (B.c3) {
+  if (B.ring) {
     const OzGroupItem it = oz_item(B, B.ncols, 0, nu, 1.0, 0.0, nullptr, 0.0, nullptr, B.V64[1], B.V64[0]);
     TRY(oz_slice_V_group(st, 1, &it, &h->launches));
     TRY(oz_gemm_group(st, 1, &it, h->dstat, &h->launches));
