@@ -74,7 +74,7 @@ typedef enum { CHASE_R64 = 0, CHASE_C128 = 1 } chase_dtype;
  *   CHASE_BF16X3    mixed: BF16x3 filter products (three BF16 tensor-core
  *                   products of hi/lo splits, FP32 accumulation) while the
  *                   residuals are large, then as CHASE_FP64_EMU.
- * The Cholesky factor, its inverse, Householder QR, the Jacobi eigensolver and the
+ * The Cholesky factor, its inverse, Householder QR, the reduced eigensolver and the
  * residual norms are FP64 in every mode. */
 typedef enum { CHASE_FP64 = 0, CHASE_TF32 = 1, CHASE_BF16X3 = 2, CHASE_FP64_EMU = 3 } chase_precision;
 
@@ -155,8 +155,8 @@ typedef struct {
   int n_lowprec_iters;     /* iterations whose filter ran in BF16x3 */
   double t_filter_lowprec; /* seconds of those filters */
   double filter_flops_lowprec; /* their algorithmic flops (counted as for FP64) */
-  double t_rr_eig;         /* part of t_rr spent in the Jacobi eigensolver */
-  int jacobi_sweeps;       /* Jacobi sweeps summed over iterations */
+  double t_rr_eig;         /* part of t_rr spent in the reduced problem's eigensolver */
+  int jacobi_sweeps;       /* 0: the reduced eigensolver is direct (no Jacobi sweeps) */
   double t_filter_product; /* part of t_filter spent in the product kernels alone (CUDA events
                               around each launch; filters launched as graphs add nothing) */
   double t_graph_build;    /* graph_filter = 1: host seconds spent recording and instantiating

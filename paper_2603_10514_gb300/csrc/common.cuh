@@ -107,9 +107,9 @@ struct DevStatus {
 struct GridBar {
   unsigned count;
   int abort;
-  int sweeps;
-  int pad;
+  int pad[2];
 };
+constexpr int kMaxGridCtas = 1216;  // 8 CTAs of 256 threads on each of the 152 SMs
 constexpr long long kBarWait = 2000000000LL;  // ~1 s of clock64
 
 __device__ inline bool grid_barrier(GridBar* gb, unsigned nblocks, unsigned& k) {

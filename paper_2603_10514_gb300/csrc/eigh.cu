@@ -1,0 +1,714 @@
+// eigh.cu -- direct eigensolver of the Rayleigh-Ritz step (Algorithm 1: solve A~ W = W Lambda~)
+// and of the Lanczos runs' tridiagonals.
+//
+//   1. Householder reduction of the Hermitian H (l x l) to a real tridiagonal T = Q^H H Q, one
+//      cooperative kernel: columns are dealt to the CTAs in turn and stay in shared memory;
+//      per column the owner publishes its reflector v (a flag), every CTA forms its entries of
+//      H v from its own columns (H is Hermitian, so no partial sums cross CTAs), and after one
+//      grid barrier applies H -= v w^H + w v^H to them.
+//   2. Divide and conquer for T = Z Lambda Z^T (stedc.cuh): blocks of up to 32 rows in one CTA
+//      each, then per level five launches over all merges of the level.
+//   3. W = Q Z: one warp per column of W applies the reflectors in turn; columns are
+//      independent, so no CTA waits for another.
+// It replaces a cyclic Jacobi iteration.  GB300 issues 2 FP64 FMAs per clock per SM, which binds
+// both: Jacobi takes ~5 sweeps of ~9 l^3 (complex: x 4) FMAs and l - 1 grid-wide rounds each,
+// this ~4 l^3 for step 1, ~l^3 (real) for 2 and ~2 l^3 for 3, and l grid barriers in all.
+// Measured (random H, GB300): l = 600 complex 124 -> 14.0 ms (8.6 reduction, 2.0 divide and
+// conquer, 3.3 back-transformation), l = 230 complex 31 -> 4.1, l = 600 real 80 -> 8.5, l = 30
+// real 2.0 -> 0.87.
+//
+// Every wait is bounded; a CTA that waits too long raises an abort flag that the others see, and
+// the kernel sets DevStatus.timeout.  Sums are taken in fixed orders: results are reproducible.
+// A non-finite T gives NaN eigenvalues and vectors.
+#include "../../include/chase_gb300.h"
+#include "common.cuh"
+#include "kernels.h"
+#include "stedc.cuh"
+
+#include <type_traits>
+
+#define TRY_EIG(x)           \
+  do {                       \
+    int _rc = (x);           \
+    if (_rc) return _rc;     \
+  } while (0)
+
+namespace chase {
+
+namespace {
+
+constexpr int TNT = 256;          // threads of the reduction kernel
+constexpr int LEAF = 32;          // rows of a divide-and-conquer leaf
+constexpr size_t kSmemMax = 227 * 1024;
+
+__device__ __forceinline__ double warp_add(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_addt(double v) { return warp_add(v); }
+__device__ __forceinline__ z64 warp_addt(z64 v) { return z64{warp_add(v.x), warp_add(v.y)}; }
+
+template <class T> __device__ __forceinline__ T ld_cg(const T* p);
+template <> __device__ __forceinline__ double ld_cg<double>(const double* p) { return __ldcg(p); }
+template <> __device__ __forceinline__ z64 ld_cg<z64>(const z64* p) {
+  const double2 v = __ldcg((const double2*)p);
+  return z64{v.x, v.y};
+}
+
+__device__ __forceinline__ double im_of(double) { return 0.0; }
+__device__ __forceinline__ double im_of(z64 a) { return a.y; }
+
+// ---------------------------------------------------------------------------
+// 1. Reduction to tridiagonal form
+// ---------------------------------------------------------------------------
+struct TriBar {
+  GridBar bar;
+  unsigned ready;  // reflectors published
+  int pad[3];
+};
+
+// Reflector j from column j (rows j .. l - 1 up to date): v into rows j + 1 .. of hcol (global),
+// tau, d[j], e[j].  One CTA; sh: 8 doubles and one T of shared memory.
+template <class T>
+__device__ void make_reflector(int l, int j, const T* col, T* hcol, T* tau, double* d, double* e, double* sh,
+                               T* sh_scale) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double s = 0.0;
+  for (int i = j + 2 + tid; i < l; i += TNT) s += Sc<T>::abs2(col[i]);
+  s = warp_add(s);
+  if (lane == 0) sh[warp] = s;
+  __syncthreads();
+  if (tid == 0) {
+    double x2 = 0.0;
+    for (int w = 0; w < TNT / 32; ++w) x2 += sh[w];
+    d[j] = Sc<T>::re(col[j]);
+    const T alpha = col[j + 1];
+    const double ar = Sc<T>::re(alpha), ai = im_of(alpha);
+    T t = Sc<T>::zero(), sc = Sc<T>::zero();
+    double beta = ar;
+    if (x2 != 0.0 || ai != 0.0) {
+      beta = -copysign(sqrt(ar * ar + ai * ai + x2), ar);
+      const double ib = 1.0 / beta, dr = ar - beta, id = 1.0 / (dr * dr + ai * ai);
+      if constexpr (Sc<T>::cplx) {
+        t = z64{(beta - ar) * ib, -ai * ib};
+        sc = z64{dr * id, -ai * id};
+      } else {
+        t = (beta - ar) * ib;
+        sc = dr * id;
+      }
+    }
+    e[j] = beta;
+    tau[j] = t;
+    *sh_scale = sc;
+  }
+  __syncthreads();
+  const T sc = *sh_scale;
+  for (int i = j + 1 + tid; i < l; i += TNT) hcol[i] = (i == j + 1) ? Sc<T>::one() : Sc<T>::mul(col[i], sc);
+}
+
+// H (l x l, ld ldh): column j is overwritten by reflector j (rows j + 1 ..).  in_smem: this CTA's
+// columns are kept in shared memory, else in place.  STAGE: v and x are copied to shared memory.
+// xb: 2 l elements, part: 2 G elements.
+template <class T, bool STAGE>
+__global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int in_smem, T* tau, double* d,
+                                                      double* e, T* xb, T* part, TriBar* tb,
+                                                      DevStatus* dst) {
+  extern __shared__ __align__(16) unsigned char tri_smem[];
+  const int G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ double sh[TNT / 32];
+  __shared__ T sh_scale, sh_alpha;
+  __shared__ int s_ok;
+  T* vs = (T*)tri_smem;
+  T* xs = vs + (STAGE ? l : 0);
+  T* sx = xs + (STAGE ? l : 0);             // this CTA's terms of x^H v
+  const int nc = me < l ? (l - 1 - me) / G + 1 : 0;  // own columns me, me + G, ...
+  T* S = sx + (l + G - 1) / G;
+  int ldS = l;
+  if (in_smem) {
+    for (int k = 0; k < nc; ++k)
+      for (int i = tid; i < l; i += TNT) S[(size_t)k * l + i] = H[(size_t)i + (size_t)(me + k * G) * ldh];
+  }
+  auto column = [&](int k) -> T* { return in_smem ? S + (size_t)k * ldS : H + (size_t)(me + k * G) * ldh; };
+  __syncthreads();
+  unsigned bars = 0;
+  int par = 0;
+  // publishes reflector j (or the last diagonal entry)
+  auto publish = [&](int j) {
+    if (j < l - 1) {
+      make_reflector<T>(l, j, column(j / G), H + (size_t)j * ldh, tau, d, e, sh, &sh_scale);
+      __syncthreads();
+      if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&tb->ready), "r"(j + 1) : "memory");
+    } else if (tid == 0) {
+      d[j] = Sc<T>::re(column(j / G)[j]);
+    }
+  };
+  if (me == 0) publish(0);
+  for (int j = 0; j + 1 < l; ++j) {
+    if (tid == 0) {
+      int ok = 1;
+      unsigned r;
+      const long long t0 = clock64();
+      while (true) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(&tb->ready) : "memory");
+        if ((int)r > j) break;
+        if (*(volatile int*)&tb->bar.abort) { ok = 0; break; }
+        if (clock64() - t0 > kBarWait) { atomicExch(&tb->bar.abort, 1); ok = 0; break; }
+      }
+      s_ok = ok;
+    }
+    __syncthreads();
+    if (!s_ok) {
+      if (tid == 0) atomicOr(&dst->timeout, 16);
+      return;
+    }
+    const T t = ld_cg(tau + j);
+    const T* vg = H + (size_t)j * ldh;
+    T* xg = xb + (size_t)par * l;
+    const int k0 = (j + 1 <= me) ? 0 : (j + 1 - me + G - 1) / G;  // first own column >= j + 1
+    const bool trivial = Sc<T>::re(t) == 0.0 && im_of(t) == 0.0;
+    if (!trivial) {
+      if (STAGE) {
+        for (int i = j + 1 + tid; i < l; i += TNT) vs[i] = ld_cg(vg + i);
+        __syncthreads();
+      }
+      // x_c = tau (H v)_c for own columns c, one warp each
+      for (int k = k0 + warp; k < nc; k += TNT / 32) {
+        const int c = me + k * G;
+        const T* col = column(k);
+        T s = Sc<T>::zero();
+        for (int i = j + 1 + lane; i < l; i += 32) Sc<T>::fmac(s, col[i], STAGE ? vs[i] : ld_cg(vg + i));
+        s = Sc<T>::mul(t, warp_addt(s));
+        if (lane == 0) {
+          xg[c] = s;
+          sx[k] = Sc<T>::mul(Sc<T>::conj(s), STAGE ? vs[c] : ld_cg(vg + c));
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {
+        T s = Sc<T>::zero();
+        for (int k = k0; k < nc; ++k) s = Sc<T>::add(s, sx[k]);
+        part[(size_t)par * G + me] = s;
+      }
+      if (!grid_barrier(&tb->bar, G, bars)) {
+        if (tid == 0) atomicOr(&dst->timeout, 16);
+        return;
+      }
+      // alpha = -1/2 tau x^H v (every CTA the same sum in the same order)
+      if (warp == 0) {
+        T s = Sc<T>::zero();
+        for (int b = lane; b < G; b += 32) s = Sc<T>::add(s, ld_cg(part + (size_t)par * G + b));
+        s = Sc<T>::scale(Sc<T>::mul(t, warp_addt(s)), -0.5);
+        if (lane == 0) sh_alpha = s;
+      }
+      if (STAGE)
+        for (int i = j + 1 + tid; i < l; i += TNT) xs[i] = ld_cg(xg + i);
+      __syncthreads();
+      par ^= 1;
+    }
+    const T al = sh_alpha;
+    // own column k: H[:, c] -= v conj(w_c) + w conj(v_c), w = x + alpha v
+    auto update = [&](int k, int i0, int step) {
+      const int c = me + k * G;
+      T* col = column(k);
+      const T vc = Sc<T>::conj(STAGE ? vs[c] : ld_cg(vg + c)), xc = Sc<T>::conj(STAGE ? xs[c] : ld_cg(xg + c));
+      // conj(w_c) + alpha conj(v_c) = conj(x_c) + 2 Re(alpha) conj(v_c)
+      const T q = Sc<T>::scale(Sc<T>::add(xc, Sc<T>::scale(vc, 2.0 * Sc<T>::re(al))), -1.0);
+      const T nvc = Sc<T>::scale(vc, -1.0);
+      for (int i = j + 1 + i0; i < l; i += step) {
+        T h = col[i];
+        Sc<T>::fma(h, STAGE ? vs[i] : ld_cg(vg + i), q);
+        Sc<T>::fma(h, STAGE ? xs[i] : ld_cg(xg + i), nvc);
+        col[i] = h;
+      }
+    };
+    int kr = k0;
+    if ((j + 1) % G == me) {  // the next reflector's column first
+      if (!trivial) update(k0, tid, TNT);
+      __syncthreads();
+      publish(j + 1);
+      kr = k0 + 1;
+    }
+    if (!trivial)
+      for (int k = kr + warp; k < nc; k += TNT / 32) update(k, lane, 32);
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// 2. Divide and conquer
+// ---------------------------------------------------------------------------
+struct CtaGroup {
+  int tid, size;
+  double* red;
+  __device__ void sync() const { __syncthreads(); }
+  __device__ double max(double v) const {
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((tid & 31) == 0) red[tid >> 5] = v;
+    __syncthreads();
+    for (int w = 0; w < (size >> 5); ++w) v = fmax(v, red[w]);
+    return v;
+  }
+};
+struct WarpGroup {
+  int tid, size;
+  __device__ void sync() const { __syncwarp(); }
+  __device__ double max(double v) const {
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+  }
+};
+struct Lanes {
+  int lane, width;
+  __device__ double sum(double v) const { return warp_add(v); }
+  __device__ double prod(double v) const {
+    for (int o = 16; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  }
+  __device__ int count(int v) const { return __reduce_add_sync(0xffffffffu, v); }
+};
+
+// Arrays of one problem of order n (offsets of `batch` problems are uniform strides).
+struct DcWork {
+  int n;
+  double* D[2];
+  double *ds, *zs, *dl, *w, *mu, *zh, *lam, *rc, *rs;
+  int *perm, *idx, *defl, *pos, *gat, *org, *rp, *rq, *dest, *cnt;
+  unsigned char *small, *close, *type;
+  double *Q[2], *U;  // n x n
+  int* bad;          // T was not finite
+};
+constexpr int kDcDoubles = 11, kDcInts = 13, kDcBytes = 3;
+
+__host__ __device__ inline size_t dc_align(size_t x) { return (x + 255) & ~(size_t)255; }
+inline size_t dc_bytes(int n) {
+  return dc_align((size_t)n * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)) + 3 * dc_align((size_t)8 * n * n) + 256;
+}
+// Carves the arrays of a problem of order n; with Q == nullptr-sized matrices left out (leaf).
+__host__ __device__ inline DcWork dc_vectors(char* base, int n) {
+  DcWork W{};
+  W.n = n;
+  double* f = (double*)base;
+  double** fs[] = {&W.D[0], &W.D[1], &W.ds, &W.zs, &W.dl, &W.w, &W.mu, &W.zh, &W.lam, &W.rc, &W.rs};
+  for (int i = 0; i < kDcDoubles; ++i) *fs[i] = f + (size_t)i * n;
+  int* q = (int*)(f + (size_t)kDcDoubles * n);
+  int** is[] = {&W.perm, &W.idx, &W.defl, &W.pos, &W.gat, &W.org, &W.rp, &W.rq, &W.dest};
+  for (int i = 0; i < 9; ++i) *is[i] = q + (size_t)i * n;
+  W.cnt = q + (size_t)9 * n;  // 4 n
+  unsigned char* c = (unsigned char*)(q + (size_t)kDcInts * n);
+  W.small = c;
+  W.close = c + n;
+  W.type = c + 2 * (size_t)n;
+  return W;
+}
+inline DcWork dc_carve(char* base, int n) {
+  DcWork W = dc_vectors(base, n);
+  char* p = base + dc_align((size_t)n * (8 * kDcDoubles + 4 * kDcInts + kDcBytes));
+  for (int i = 0; i < 2; ++i) { W.Q[i] = (double*)p; p += dc_align((size_t)8 * n * n); }
+  W.U = (double*)p;
+  p += dc_align((size_t)8 * n * n);
+  W.bad = (int*)p;
+  return W;
+}
+// The arrays of problem b (every array a uniform stride of `stride` bytes further on).
+__device__ inline DcWork dc_at(DcWork W, size_t off) {
+  auto mv = [&](auto*& p) { p = (std::remove_reference_t<decltype(p)>)((char*)p + off); };
+  mv(W.D[0]); mv(W.D[1]); mv(W.ds); mv(W.zs); mv(W.dl); mv(W.w); mv(W.mu); mv(W.zh); mv(W.lam); mv(W.rc); mv(W.rs);
+  mv(W.perm); mv(W.idx); mv(W.defl); mv(W.pos); mv(W.gat); mv(W.org); mv(W.rp); mv(W.rq); mv(W.dest); mv(W.cnt);
+  mv(W.small); mv(W.close); mv(W.type); mv(W.Q[0]); mv(W.Q[1]); mv(W.U); mv(W.bad);
+  return W;
+}
+
+// The merge of rows [s, mid) and [mid, t) of T with off-diagonal e (at mid - 1); input in D[cur].
+__device__ inline dc::Merge dc_merge(const DcWork& W, int cur, int s, int mid, int t, double e) {
+  dc::Merge M;
+  M.m = t - s;
+  M.n1 = mid - s;
+  M.rho = 2.0 * fabs(e);
+  M.sign = e < 0.0 ? -1.0 : 1.0;
+  M.D = W.D[cur] + s;
+  M.ds = W.ds + s; M.zs = W.zs + s; M.dl = W.dl + s; M.w = W.w + s; M.mu = W.mu + s; M.zh = W.zh + s;
+  M.lam = W.lam + s; M.rc = W.rc + s; M.rs = W.rs + s;
+  M.perm = W.perm + s; M.idx = W.idx + s; M.defl = W.defl + s; M.pos = W.pos + s; M.gat = W.gat + s;
+  M.org = W.org + s; M.rp = W.rp + s; M.rq = W.rq + s; M.dest = W.dest + s;
+  M.cnt = W.cnt + 4 * s;
+  M.small = W.small + s; M.close = W.close + s; M.type = W.type + s;
+  return M;
+}
+
+// Rotations of the deflated pairs applied to row i of Q's block (column q at Qb + q ldq).
+__device__ inline void dc_rotate_row(const dc::Merge& M, double* Qb, int ldq, int i) {
+  const int nr = M.cnt[3];
+  for (int r = 0; r < nr; ++r) {
+    double* x = Qb + (size_t)i + (size_t)M.rp[r] * ldq;
+    double* y = Qb + (size_t)i + (size_t)M.rq[r] * ldq;
+    const double a = *x, b = *y;
+    *x = M.rc[r] * a + M.rs[r] * b;
+    *y = M.rc[r] * b - M.rs[r] * a;
+  }
+}
+
+// One merge by one group (a warp or a CTA of nw warps) on local arrays: Q's block is replaced.
+template <class G>
+__device__ inline void dc_merge_local(const G& g, int w, int nw, const dc::Merge& M, double* D, double* Dn,
+                                      double* Qb, double* Qn, double* U, int ldq) {
+  const Lanes L{(int)(threadIdx.x & 31), 32};
+  const int m = M.m;
+  dc::setup(g, M, Qb + M.n1 - 1, Qb + M.n1 + (size_t)M.n1 * ldq, ldq);
+  const int K = M.cnt[0];
+  for (int k = w; k < K; k += nw) dc::root(L, K, k, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+  for (int i = g.tid; i < m; i += g.size) dc_rotate_row(M, Qb, ldq, i);
+  g.sync();
+  for (int k = w; k < K; k += nw) dc::zhat(L, K, k, M.dl, M.w, M.mu, M.org, M.zh);
+  g.sync();
+  for (int k = w; k < K; k += nw) dc::ucol(L, K, k, M.dl, M.zh, M.mu, M.org, M.pos, U, ldq);
+  for (int t = w; t < m; t += nw) dc::place(L, M, K, t);
+  g.sync();
+  for (int u = g.tid; u < m * m; u += g.size) {
+    const int i = u % m, j = u / m;
+    double a = 0.0;
+    if (j < K) {
+      const int p0 = i < M.n1 ? 0 : M.cnt[1], p1 = i < M.n1 ? M.cnt[2] : K;
+      for (int p = p0; p < p1; ++p) a = fma(Qb[(size_t)i + (size_t)M.gat[p] * ldq], U[(size_t)p + (size_t)j * ldq], a);
+    } else {
+      a = Qb[(size_t)i + (size_t)M.perm[M.defl[j - K]] * ldq];
+    }
+    Qn[(size_t)i + (size_t)M.dest[j] * ldq] = a;
+    if (i == 0) Dn[M.dest[j]] = j < K ? M.lam[j] : M.ds[M.defl[j - K]];
+  }
+  g.sync();
+  for (int u = g.tid; u < m * m; u += g.size) Qb[(size_t)(u % m) + (size_t)(u / m) * ldq] = Qn[(size_t)(u % m) + (size_t)(u / m) * ldq];
+  for (int i = g.tid; i < m; i += g.size) D[i] = Dn[i];
+  g.sync();
+}
+
+__host__ __device__ inline int dc_bound(int n, long long i, int depth) { return (int)((i * n) >> depth); }
+
+// Leaf blockIdx.x of 2^depth (at most 32 rows): its eigensystem by merges from single rows up,
+// one warp per merge while a level has at least four, then the whole CTA.
+__global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const double* __restrict__ d0,
+                                                      const double* __restrict__ e0, int ld_de, DcWork W0,
+                                                      size_t stride) {
+  __shared__ double sQ[LEAF * LEAF], sQn[LEAF * LEAF], sU[LEAF * LEAF];
+  __shared__ double s_red[8];
+  __shared__ __align__(16) char s_vec[LEAF * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)];
+  const DcWork W = dc_at(W0, stride * blockIdx.y);
+  const double* d = d0 + (size_t)blockIdx.y * ld_de;
+  const double* e = e0 + (size_t)blockIdx.y * ld_de;
+  const int s = dc_bound(n, blockIdx.x, depth), t = dc_bound(n, blockIdx.x + 1, depth), m = t - s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const DcWork V = dc_vectors(s_vec, LEAF);
+  for (int u = tid; u < LEAF * LEAF; u += 256) sQ[u] = (u % LEAF == u / LEAF) ? 1.0 : 0.0;
+  for (int i = tid; i < m; i += 256) {
+    const int r = s + i;
+    // every off-diagonal is torn at some level
+    const double lo = r > 0 ? fabs(e[r - 1]) : 0.0, up = r + 1 < n ? fabs(e[r]) : 0.0;
+    V.D[0][i] = d[r] - lo - up;
+    if (!isfinite(d[r]) || !isfinite(up)) *W.bad = 1;
+  }
+  __syncthreads();
+  for (int h = 4; h >= 0; --h) {
+    const int parts = 1 << h;
+    const bool by_warp = parts >= 4;
+    for (int q = by_warp ? warp : 0; q < parts; q += by_warp ? 8 : 1) {
+      const long long i0 = ((long long)blockIdx.x << (h + 1)) + 2 * q;
+      const int a = dc_bound(n, i0, depth + h + 1) - s, b = dc_bound(n, i0 + 1, depth + h + 1) - s,
+                c = dc_bound(n, i0 + 2, depth + h + 1) - s;
+      if (b == a || c == b) continue;  // an empty half: nothing to merge
+      const dc::Merge M = dc_merge(V, 0, a, b, c, e[s + b - 1]);
+      double* Qb = sQ + a + a * LEAF;
+      if (by_warp)
+        dc_merge_local(WarpGroup{lane, 32}, 0, 1, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
+                       sU + a + a * LEAF, LEAF);
+      else
+        dc_merge_local(CtaGroup{tid, 256, s_red}, warp, 8, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
+                       sU + a + a * LEAF, LEAF);
+    }
+    __syncthreads();
+  }
+  for (int u = tid; u < m * m; u += 256)
+    W.Q[0][(size_t)(s + u % m) + (size_t)(s + u / m) * n] = sQ[(u % m) + (u / m) * LEAF];
+  for (int i = tid; i < m; i += 256) W.D[0][s + i] = V.D[0][i];
+}
+
+// Merge blockIdx.(y or z) of the level with 2^depth blocks below it; cur: input buffer.
+__device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, int q, const double* e, int* s) {
+  const int a = dc_bound(W.n, 2 * q, depth), b = dc_bound(W.n, 2 * q + 1, depth), c = dc_bound(W.n, 2 * q + 2, depth);
+  *s = a;
+  return dc_merge(W, cur, a, b, c, e[b - 1]);
+}
+
+__global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth,
+                                                       const double* __restrict__ e0, int ld_de) {
+  __shared__ double red[16];
+  const DcWork W = dc_at(W0, stride * blockIdx.y);
+  int s;
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.x, e0 + (size_t)blockIdx.y * ld_de, &s);
+  const double* Qb = W.Q[cur] + s + (size_t)s * W.n;
+  dc::setup(CtaGroup{(int)threadIdx.x, 512, red}, M, Qb + M.n1 - 1, Qb + M.n1 + (size_t)M.n1 * W.n, W.n);
+}
+
+// phase 0: roots, and the rotations of Q's rows; 1: corrected z; 2: U and the new order.
+__global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth,
+                                                       const double* __restrict__ e0, int ld_de, int phase) {
+  const DcWork W = dc_at(W0, stride * blockIdx.z);
+  int s;
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, e0 + (size_t)blockIdx.z * ld_de, &s);
+  const Lanes L{(int)(threadIdx.x & 31), 32};
+  const int w = blockIdx.x * 4 + (threadIdx.x >> 5), nw = gridDim.x * 4;
+  const int K = M.cnt[0];
+  if (phase == 0) {
+    for (int k = w; k < K; k += nw) dc::root(L, K, k, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+    double* Qb = W.Q[cur] + s + (size_t)s * W.n;
+    for (int i = blockIdx.x * 128 + threadIdx.x; i < M.m; i += gridDim.x * 128) dc_rotate_row(M, Qb, W.n, i);
+  } else if (phase == 1) {
+    for (int k = w; k < K; k += nw) dc::zhat(L, K, k, M.dl, M.w, M.mu, M.org, M.zh);
+  } else {
+    double* Ub = W.U + s + (size_t)s * W.n;
+    for (int k = w; k < K; k += nw) dc::ucol(L, K, k, M.dl, M.zh, M.mu, M.org, M.pos, Ub, W.n);
+    for (int t = w; t < M.m; t += nw) dc::place(L, M, K, t);
+  }
+}
+
+// Q_new[:, dest] = Q[:, gathered] U (64 x 32 tiles, FP64), deflated columns copied.
+__global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth,
+                                                      const double* __restrict__ e0, int ld_de, int parts) {
+  const DcWork W = dc_at(W0, stride * (blockIdx.z / parts));
+  int s;
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.z % parts, e0 + (size_t)(blockIdx.z / parts) * ld_de, &s);
+  constexpr int BK = 16;
+  __shared__ double As[BK][64], Bs[BK][33];
+  const int m0 = blockIdx.y * 64, j0 = blockIdx.x * 32, m = M.m, n1 = M.n1, K = M.cnt[0], ld = W.n;
+  if (m0 >= m || j0 >= m) return;
+  const double* Q = W.Q[cur] + s + (size_t)s * ld;
+  const double* U = W.U + s + (size_t)s * ld;
+  double* Qn = W.Q[cur ^ 1] + s + (size_t)s * ld;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  double acc[4][2] = {};
+  if (j0 < K) {
+    const int p0 = m0 >= n1 ? M.cnt[1] : 0, p1 = m0 + 64 <= n1 ? M.cnt[2] : K;
+    for (int pb = p0; pb < p1; pb += BK) {
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = tid & 63, k = (tid >> 6) + 4 * r;
+        As[k][i] = (m0 + i < m && pb + k < p1) ? Q[(size_t)(m0 + i) + (size_t)M.gat[pb + k] * ld] : 0.0;
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int k = tid & 15, j = (tid >> 4) + 16 * r;
+        Bs[k][j] = (j0 + j < K && pb + k < p1) ? U[(size_t)(pb + k) + (size_t)(j0 + j) * ld] : 0.0;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < BK; ++k) {
+        double a[4], b[2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
+        b[0] = Bs[k][tx];
+        b[1] = Bs[k][tx + 16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[i][0] = fma(a[i], b[0], acc[i][0]);
+          acc[i][1] = fma(a[i], b[1], acc[i][1]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int j = j0 + tx + 16 * c;
+    if (j >= m) continue;
+    const int dj = M.dest[j];
+    const double* src = j < K ? nullptr : Q + (size_t)M.perm[M.defl[j - K]] * ld;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = m0 + ty + 16 * i;
+      if (r < m) Qn[(size_t)r + (size_t)dj * ld] = src ? src[r] : acc[i][c];
+    }
+    if (m0 == 0 && ty == 0) W.D[cur ^ 1][s + dj] = j < K ? M.lam[j] : M.ds[M.defl[j - K]];
+  }
+}
+
+int dc_depth(int n) {
+  int depth = 0;
+  while (ceil_div(n, 1 << depth) > LEAF) ++depth;
+  return depth;
+}
+
+// Eigensystems of `batch` tridiagonals (d, e at strides of ld_de) in the arrays W (strides of
+// `stride` bytes); returns the buffer that holds D and Q in *cur.
+int stedc(cudaStream_t st, int n, int batch, const double* d, const double* e, int ld_de, const DcWork& W,
+          size_t stride, int* cur, int* launches) {
+  for (int b = 0; b < batch; ++b) {
+    char* q = (char*)W.Q[0] + stride * b;  // Q[0], Q[1], U and the flag lie one after another
+    CHASE_CUDA_TRY(cudaMemsetAsync(q, 0, 3 * dc_align((size_t)8 * n * n) + sizeof(int), st));
+  }
+  const int depth = dc_depth(n);
+  dc_leaf_kernel<<<dim3(1 << depth, batch), 256, 0, st>>>(n, depth, d, e, ld_de, W, stride);
+  int nl = 1, c = 0;
+  for (int h = depth; h > 0; --h) {
+    const int parts = 1 << (h - 1), m = ceil_div(n, parts);  // rows of a merge, at most
+    dc_setup_kernel<<<dim3(parts, batch), 512, 0, st>>>(W, stride, c, h, e, ld_de);
+    for (int phase = 0; phase < 3; ++phase)
+      dc_phase_kernel<<<dim3(ceil_div(m, 4), parts, batch), 128, 0, st>>>(W, stride, c, h, e, ld_de, phase);
+    dc_gemm_kernel<<<dim3(ceil_div(m, 32), ceil_div(m, 64), parts * batch), 256, 0, st>>>(W, stride, c, h, e,
+                                                                                         ld_de, parts);
+    nl += 5;
+    c ^= 1;
+  }
+  *cur = c;
+  if (launches) *launches += nl;
+  CHASE_CUDA_TRY(cudaGetLastError());
+  return 0;
+}
+
+// ---------------------------------------------------------------------------
+// 3. Back-transformation
+// ---------------------------------------------------------------------------
+// Column c of W = H_0 H_1 ... H_{l-2} Z[:, c]: one warp per column, the column in shared memory
+// (in_smem) or in place; dw = D (NaN if T was not finite).
+template <class T>
+__global__ void backtransform_kernel(int l, const T* __restrict__ H, int ldh, const T* __restrict__ tau,
+                                     const double* __restrict__ Z, const double* __restrict__ D, const int* bad,
+                                     T* Wm, int ldw, double* dw, int in_smem) {
+  extern __shared__ __align__(16) unsigned char bt_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (c >= l) return;
+  T* out = Wm + (size_t)c * ldw;
+  T* z = in_smem ? (T*)bt_smem + (size_t)warp * l : out;
+  if (*bad) {
+    for (int i = lane; i < l; i += 32) out[i] = Sc<T>::from_re(nan(""));
+    if (lane == 0) dw[c] = nan("");
+    return;
+  }
+  for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(Z[(size_t)i + (size_t)c * l]);
+  if (lane == 0) dw[c] = D[c];
+  __syncwarp();
+  for (int j = l - 2; j >= 0; --j) {
+    const T t = tau[j];
+    if (Sc<T>::re(t) == 0.0 && im_of(t) == 0.0) continue;
+    const T* v = H + (size_t)j * ldh;
+    T s = Sc<T>::zero();
+    for (int i = j + 1 + lane; i < l; i += 32) Sc<T>::fmac(s, v[i], z[i]);
+    s = Sc<T>::scale(Sc<T>::mul(t, warp_addt(s)), -1.0);
+    for (int i = j + 1 + lane; i < l; i += 32) {
+      T x = z[i];
+      Sc<T>::fma(x, v[i], s);
+      z[i] = x;
+    }
+    __syncwarp();
+  }
+  if (in_smem)
+    for (int i = lane; i < l; i += 32) out[i] = z[i];
+}
+
+// theta and squared first components of problem blockIdx.x (NaN if its T was not finite)
+__global__ void dc_extract_kernel(DcWork W0, size_t stride, int cur, double* theta, double* weight) {
+  const DcWork W = dc_at(W0, stride * blockIdx.x);
+  for (int i = threadIdx.x; i < W.n; i += blockDim.x) {
+    const double q = W.Q[cur][(size_t)i * W.n];
+    theta[(size_t)blockIdx.x * W.n + i] = *W.bad ? nan("") : W.D[cur][i];
+    weight[(size_t)blockIdx.x * W.n + i] = *W.bad ? nan("") : q * q;
+  }
+}
+// problems of one pass over the tridiagonals: as many as fit about 128 MB, at least one
+int tridiag_pass(int m, int batch) {
+  return (int)std::max<size_t>(1, std::min<size_t>(batch, ((size_t)128 << 20) / dc_align(dc_bytes(m))));
+}
+
+struct EighLayout {
+  size_t tau, d, e, xb, part, tb, dc, total;
+};
+EighLayout eigh_layout(int l, size_t elem) {
+  EighLayout L{};
+  size_t off = 0;
+  auto take = [&](size_t b) { const size_t o = off; off += dc_align(b); return o; };
+  L.tau = take(elem * l);
+  L.d = take(8 * (size_t)l);
+  L.e = take(8 * (size_t)l);
+  L.xb = take(2 * elem * l);
+  L.part = take(2 * elem * kNumSMs);
+  L.tb = take(sizeof(TriBar));
+  L.dc = take(dc_bytes(l));
+  L.total = off;
+  return L;
+}
+
+template <class T>
+int tridiag(cudaStream_t st, int l, T* H, int ldh, T* tau, double* d, double* e, T* xb, T* part, TriBar* tb,
+            DevStatus* dst, int ctas, int* launches) {
+  // CTAs: enough that a column step's FP64 work per SM stays near the barrier's cost
+  const double work = (double)l * l * (Sc<T>::cplx ? 4.0 : 1.0);
+  int G = (int)std::min<double>(kNumSMs, std::max(1.0, work / 6000.0));
+  if (ctas > 0) G = std::min(ctas, kNumSMs);
+  G = std::max(1, std::min(G, l));
+  const size_t own = ceil_div(l, G);
+  const bool stage = (2 * (size_t)l + own) * sizeof(T) <= kSmemMax - 1024;
+  size_t smem = ((stage ? 2 * (size_t)l : 0) + own) * sizeof(T);
+  int in_smem = smem + own * l * sizeof(T) <= kSmemMax - 1024;
+  if (in_smem) smem += own * l * sizeof(T);
+  void (*kern)(int, T*, int, int, T*, double*, double*, T*, T*, TriBar*, DevStatus*) =
+      stage ? tridiag_kernel<T, true> : tridiag_kernel<T, false>;
+  CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
+  CHASE_CUDA_TRY(cudaMemsetAsync(tb, 0, sizeof(TriBar), st));
+  void* args[] = {(void*)&l, (void*)&H, (void*)&ldh, (void*)&in_smem, (void*)&tau, (void*)&d,
+                  (void*)&e, (void*)&xb, (void*)&part, (void*)&tb, (void*)&dst};
+  CHASE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)kern, dim3(G), dim3(TNT), args, smem, st));
+  if (launches) ++*launches;
+  return 0;
+}
+
+}  // namespace
+
+size_t eigh_work_bytes(int l, size_t elem) { return eigh_layout(l, elem).total; }
+
+template <class T>
+int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work, size_t work_bytes,
+         DevStatus* dst, int* launches, int ctas) {
+  if (l <= 0) return 0;
+  const EighLayout L = eigh_layout(l, sizeof(T));
+  if (L.total > work_bytes) return CHASE_ERR_OOM;
+  char* base = (char*)work;
+  T* tau = (T*)(base + L.tau);
+  double *d = (double*)(base + L.d), *e = (double*)(base + L.e);
+  TRY_EIG(tridiag<T>(st, l, H, ldh, tau, d, e, (T*)(base + L.xb), (T*)(base + L.part), (TriBar*)(base + L.tb), dst,
+                     ctas, launches));
+  const DcWork D = dc_carve(base + L.dc, l);
+  int cur = 0;
+  TRY_EIG(stedc(st, l, 1, d, e, 0, D, 0, &cur, launches));
+  const int wpc = (int)std::max<size_t>(1, std::min<size_t>(4, (kSmemMax - 1024) / (sizeof(T) * (size_t)l)));
+  const size_t smem = sizeof(T) * (size_t)l * wpc;
+  const int in_smem = smem <= kSmemMax - 1024;
+  CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)backtransform_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kSmemMax - 1024));
+  backtransform_kernel<T><<<ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, st>>>(l, H, ldh, tau, D.Q[cur], D.D[cur],
+                                                                                 D.bad, W, ldw, dw, in_smem);
+  if (launches) ++*launches;
+  CHASE_CUDA_TRY(cudaGetLastError());
+  return 0;
+}
+
+size_t tridiag_work_bytes(int m, int batch) { return dc_align(dc_bytes(m)) * tridiag_pass(m, batch); }
+
+int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const double* beta, double* theta,
+                 double* weight, void* work, size_t work_bytes, int* launches) {
+  if (m <= 0 || batch <= 0) return 0;
+  if (tridiag_work_bytes(m, batch) > work_bytes) return CHASE_ERR_OOM;
+  const size_t stride = dc_align(dc_bytes(m));
+  const DcWork W = dc_carve((char*)work, m);
+  for (int r = 0, nb = tridiag_pass(m, batch); r < batch; r += nb) {
+    const int cnt = std::min(nb, batch - r);
+    int cur = 0;
+    TRY_EIG(stedc(st, m, cnt, alpha + (size_t)r * m, beta + (size_t)r * m, m, W, stride, &cur, launches));
+    dc_extract_kernel<<<cnt, 128, 0, st>>>(W, stride, cur, theta + (size_t)r * m, weight + (size_t)r * m);
+    if (launches) ++*launches;
+  }
+  CHASE_CUDA_TRY(cudaGetLastError());
+  return 0;
+}
+
+template int eigh<double>(cudaStream_t, int, double*, int, double*, int, double*, void*, size_t, DevStatus*, int*, int);
+template int eigh<z64>(cudaStream_t, int, z64*, int, z64*, int, double*, void*, size_t, DevStatus*, int*, int);
+
+}  // namespace chase

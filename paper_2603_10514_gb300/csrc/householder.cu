@@ -295,8 +295,8 @@ int hh_panel(cudaStream_t st, int n, int j0, int b, T* X, int ldx, T* Vh, int ld
 template <class T>
 size_t hh_panel_coop_bytes(int b) {
   const size_t nent = (size_t)b * (b + 1) / 2;
-  return 256 + 8 * (size_t)(kJacobiMaxCtas + 2) + 2 * sizeof(T) +
-         (size_t)kJacobiMaxCtas * ((size_t)b + nent) * sizeof(T);
+  return 256 + 8 * (size_t)(kMaxGridCtas + 2) + 2 * sizeof(T) +
+         (size_t)kMaxGridCtas * ((size_t)b + nent) * sizeof(T);
 }
 
 template <class T>
@@ -313,7 +313,7 @@ int hh_panel_coop(cudaStream_t st, int n, int j0, int b, T* X, int ldx, T* Vh, i
   const int m = n - j0;
   const int Gmax = per_sm * kNumSMs;
   const int G = std::min(kNumSMs, std::max(ceil_div(m, kHhSliceMax), ceil_div(m, 64)));
-  if (b > 64 || per_sm <= 0 || G > Gmax || G > kJacobiMaxCtas || ceil_div(m, G) > kHhSliceMax ||
+  if (b > 64 || per_sm <= 0 || G > Gmax || G > kMaxGridCtas || ceil_div(m, G) > kHhSliceMax ||
       ws.bytes < hh_panel_coop_bytes<T>(b))
     return CHASE_ERR_UNSUPPORTED;
   GridBar* gb = (GridBar*)ws.ptr;

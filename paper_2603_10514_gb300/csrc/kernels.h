@@ -58,17 +58,20 @@ int hh_build_T(cudaStream_t st, int b, const T* G, int ldg, T* Tm, int ldt, int*
 template <class T>
 int hh_thin_identity(cudaStream_t st, int n, int l, T* X, int ldx, int* launches);
 
-// ---- parallel cyclic Jacobi eigensolver (jacobi.cu) ------------------------
-// Diagonalises the Hermitian H (l x l, overwritten).  Eigenvalues (ascending)
-// go to dw (device) and eigenvectors to W.  Returns sweeps used through *sweeps.
-// One cooperative launch runs every sweep; work: jacobi_work_bytes(l, sizeof(T)) bytes.
-// Returns 5 (CHASE_ERR_TIMEOUT) if a bounded grid-barrier wait ran out.
-constexpr int kJacobiMaxCtas = 1216;  // 8 CTAs of 256 threads on each of the 152 SMs
-size_t jacobi_work_bytes(int l, size_t elem);
-// ctas > 0 fixes the grid size (at most one wave of co-resident CTAs); 0 picks it from l.
+// ---- direct eigensolver (eigh.cu) -------------------------------------------
+// Eigenvalues (ascending, dw on the device) and eigenvectors W of the Hermitian H (l x l,
+// overwritten).  work: eigh_work_bytes(l, sizeof(T)).  A bounded wait that ran out sets
+// dst->timeout.  ctas > 0 fixes the grid of the reduction; 0 picks it from l.
+size_t eigh_work_bytes(int l, size_t elem);
 template <class T>
-int jacobi_eig(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work,
-               size_t work_bytes, int max_sweeps, int* sweeps, int* launches, int ctas = 0);
+int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work, size_t work_bytes,
+         DevStatus* dst, int* launches, int ctas = 0);
+// Eigenvalues (ascending) and squared first eigenvector components of `batch` real symmetric
+// tridiagonals of order m: run r's diagonal at alpha + r m, off-diagonal at beta + r m; theta and
+// weight batch x m (device).
+size_t tridiag_work_bytes(int m, int batch);
+int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const double* beta, double* theta,
+                 double* weight, void* work, size_t work_bytes, int* launches);
 
 // ---- streaming kernels (vec.cu) --------------------------------------------
 template <class T>

@@ -4,8 +4,7 @@
 // nruns runs advance together: one product A * [q_1 ... q_nruns] per step
 // (the FP64 product kernel), column-wise alpha / beta, full
 // re-orthogonalisation of each run's new vector against its own basis, then
-// the m x m tridiagonal of every run is diagonalised by the device Jacobi
-// solver.  The host only reduces the m * nruns Ritz values and weights to the
+// the m x m tridiagonals of all runs are diagonalised together (eigh.cu).  The host only reduces the m * nruns Ritz values and weights to the
 // three bounds:
 //   b_sup      = max_r (theta_max^r + |beta_m^r|)   -- an upper bound of lambda_n
 //   lambda1    = min_r theta_min^r
@@ -114,18 +113,6 @@ __global__ void __launch_bounds__(256) lz_normalize_kernel(int n, const T* __res
   for (int i = threadIdx.x; i < n; i += 256) qn[(size_t)r * n + i] = Sc<T>::scale(w[i], inv);
 }
 
-// Tridiagonal of run r as a dense m x m real matrix (column-major, ld m).
-__global__ void lz_tridiag_kernel(int m, const double* alpha, const double* beta, int r, double* T) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m * m; t += gridDim.x * blockDim.x) {
-    const int i = t % m, k = t / m;
-    double v = 0.0;
-    if (i == k) v = alpha[r * m + i];
-    else if (i == k + 1) v = beta[r * m + k];
-    else if (k == i + 1) v = beta[r * m + i];
-    T[t] = v;
-  }
-}
-
 }  // namespace
 
 template <class T>
@@ -133,7 +120,7 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
                    int m, int ell, double* out, void* work, size_t work_bytes, Scratch scr,
                    int* launches) {
   // workspace: basis (m + 1) x n x nruns | W n x nruns | coef nruns x (m + 1) | alpha, beta |
-  //            T m x m | S m x m | theta m | jacobi work
+  //            theta, weights | work of the tridiagonal eigensolver
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t pstride = (size_t)n * nruns;
   size_t off = 0;
@@ -143,12 +130,9 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   T* coef = (T*)(base + off); off += al(sizeof(T) * (size_t)nruns * (m + 1));
   double* alpha = (double*)(base + off); off += al(sizeof(double) * (size_t)nruns * m);
   double* beta = (double*)(base + off); off += al(sizeof(double) * (size_t)nruns * m);
-  double* Tm = (double*)(base + off); off += al(sizeof(double) * (size_t)m * m);
-  double* Sm = (double*)(base + off); off += al(sizeof(double) * (size_t)m * m);
-  double* th = (double*)(base + off); off += al(sizeof(double) * (size_t)m);
-  void* jw = base + off;
+  double* th = (double*)(base + off); off += al(sizeof(double) * (size_t)nruns * m);
+  double* tw = (double*)(base + off); off += al(sizeof(double) * (size_t)nruns * m);
   if (off > work_bytes) return CHASE_ERR_OOM;
-  const size_t jw_bytes = work_bytes - off;
   int nl = 0;
   // q_0 = v / ||v|| for every run
   TRY_LZ(copy_cols<T>(st, n, nruns, V0, ldv, W, n, &nl));
@@ -173,21 +157,9 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   }
   // Ritz values and weights of each run
   std::vector<double> hth((size_t)nruns * m), htau((size_t)nruns * m), hbeta((size_t)nruns * m);
-  std::vector<double> S1((size_t)m);
-  for (int r = 0; r < nruns; ++r) {
-    lz_tridiag_kernel<<<std::max(1, (m * m + 255) / 256), 256, 0, st>>>(m, alpha, beta, r, Tm);
-    ++nl;
-    int sweeps = 0;
-    int rc = jacobi_eig<double>(st, m, Tm, m, Sm, m, th, jw, jw_bytes, 60, &sweeps, &nl);
-    if (rc) return rc;
-    CHASE_CUDA_TRY(cudaMemcpyAsync(hth.data() + (size_t)r * m, th, sizeof(double) * m,
-                                   cudaMemcpyDeviceToHost, st));
-    // first row of the eigenvector matrix: S[0, i] at stride m
-    CHASE_CUDA_TRY(cudaMemcpy2DAsync(S1.data(), sizeof(double), Sm, sizeof(double) * m,
-                                     sizeof(double), m, cudaMemcpyDeviceToHost, st));
-    CHASE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int i = 0; i < m; ++i) htau[(size_t)r * m + i] = S1[i] * S1[i];
-  }
+  TRY_LZ(tridiag_eigs(st, m, nruns, alpha, beta, th, tw, base + off, work_bytes - off, &nl));
+  CHASE_CUDA_TRY(cudaMemcpyAsync(hth.data(), th, sizeof(double) * (size_t)nruns * m, cudaMemcpyDeviceToHost, st));
+  CHASE_CUDA_TRY(cudaMemcpyAsync(htau.data(), tw, sizeof(double) * (size_t)nruns * m, cudaMemcpyDeviceToHost, st));
   CHASE_CUDA_TRY(cudaMemcpyAsync(hbeta.data(), beta, sizeof(double) * (size_t)nruns * m,
                                  cudaMemcpyDeviceToHost, st));
   CHASE_CUDA_TRY(cudaStreamSynchronize(st));
@@ -217,8 +189,7 @@ size_t lanczos_work_bytes(size_t elem, int n, int nruns, int m) {
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t ps = (size_t)n * nruns;
   return al(elem * ps * (m + 1)) + al(elem * ps) + al(elem * (size_t)nruns * (m + 1)) +
-         2 * al(8 * (size_t)nruns * m) + 2 * al(8 * (size_t)m * m) + al(8 * (size_t)m) +
-         /* jacobi */ al(jacobi_work_bytes(m, sizeof(double))) + 256;
+         4 * al(8 * (size_t)nruns * m) + tridiag_work_bytes(m, nruns);
 }
 
 template int lanczos_bounds<double>(cudaStream_t, int, const double*, int, int, const double*, int,

@@ -133,7 +133,7 @@ int ensure_hbuf(chase_ctx* h, size_t bytes) {
 
 // Workspace carve-up for a problem of order n with block width l.
 struct Layout {
-  size_t V, P, AQ, T2, Xs, G, Ri, H, Wm, jac, dw, dres, scratch, total;
+  size_t V, P, AQ, T2, Xs, G, Ri, H, Wm, eig, dw, dres, scratch, total;
 };
 
 template <class T>
@@ -151,7 +151,7 @@ Layout layout_for(int n, int l) {
   L.Ri = off; off += sq;
   L.H = off; off += sq;
   L.Wm = off; off += sq;
-  L.jac = off; off += align256(jacobi_work_bytes(l, sizeof(T)));
+  L.eig = off; off += align256(eigh_work_bytes(l, sizeof(T)));
   L.dw = off; off += align256(sizeof(double) * (size_t)l);
   L.dres = off; off += align256(sizeof(double) * (size_t)l);
   L.scratch = off; off += kScratchBytes;
@@ -910,8 +910,8 @@ struct Solve final : SolveBase {
   Layout L;
   T *V = nullptr, *P = nullptr, *AQ = nullptr, *T2 = nullptr, *Xs = nullptr, *G = nullptr,
     *Ri = nullptr, *H = nullptr, *Wm = nullptr;
-  void* jac = nullptr;
-  size_t jac_bytes = 0;
+  void* eigw = nullptr;  // the eigensolver's workspace
+  size_t eigw_bytes = 0;
   double *dw = nullptr, *dres = nullptr;
   Scratch scr{nullptr, 0};
   TcBufs tcb;
@@ -964,8 +964,8 @@ struct Solve final : SolveBase {
     Ri = (T*)(base + L.Ri);
     H = (T*)(base + L.H);
     Wm = (T*)(base + L.Wm);
-    jac = base + L.jac;
-    jac_bytes = L.dw - L.jac;
+    eigw = base + L.eig;
+    eigw_bytes = L.dw - L.eig;
     dw = (double*)(base + L.dw);
     dres = (double*)(base + L.dres);
     scr = Scratch{base + L.scratch, kScratchBytes};
@@ -1139,18 +1139,12 @@ struct Solve final : SolveBase {
                    scr, true, false, &h->launches);
     }
     if (!rc) rc = herm_fill_lower<T>(st, nu, H, nu, &h->launches);
-    int sweeps = 0;
     cudaEvent_t j0 = nullptr, j1 = nullptr;
     cudaEventCreate(&j0);
     cudaEventCreate(&j1);
     cudaEventRecord(j0, st);
-    if (!rc) rc = jacobi_eig<T>(st, nu, H, nu, Wm, nu, dw, jac, jac_bytes, 40, &sweeps, &h->launches);
+    if (!rc) rc = eigh<T>(st, nu, H, nu, Wm, nu, dw, eigw, eigw_bytes, h->dstat, &h->launches);
     cudaEventRecord(j1, st);
-    cudaEventSynchronize(j1);
-    S.t_rr_eig += elapsed_s(j0, j1);
-    S.jacobi_sweeps += sweeps;
-    cudaEventDestroy(j0);
-    cudaEventDestroy(j1);
     // V <- Q2 W, AV = AQ W (into P)
     if (rc) {
     } else if (ozq) {
@@ -1164,7 +1158,10 @@ struct Solve final : SolveBase {
                             nullptr, 0, scr, false, false, &h->launches);
       if (!rc) rc = copy_cols<T>(st, n, nu, T2, n, Q2, n, &h->launches);
     }
-    phase_end(S.t_rr);
+    phase_end(S.t_rr);  // synchronises the stream, j1 included
+    S.t_rr_eig += elapsed_s(j0, j1);
+    cudaEventDestroy(j0);
+    cudaEventDestroy(j1);
     if (rc) return rc;
     // --- residuals (eq. res) ---
     double* hw = hstage;      // l Ritz values
@@ -1239,7 +1236,7 @@ struct Solve final : SolveBase {
           hperm[a] = idx[a] - k;
         }
         for (int a = 0; a < l - k; ++a) { deg[k + a] = d2[a]; ritz[k + a] = r2[a]; res[k + a] = s2[a]; }
-        int* dperm = (int*)jac;  // Jacobi workspace is free here
+        int* dperm = (int*)eigw;  // the eigensolver's workspace is free here
         CHASE_CUDA_TRY(cudaMemcpyAsync(dperm, hperm, sizeof(int) * (l - k), cudaMemcpyHostToDevice, st));
         TRY(copy_cols<T>(st, n, l - k, V + (size_t)k * n, n, T2, n, &h->launches));
         TRY(gather_cols<T>(st, n, l - k, T2, n, dperm, V + (size_t)k * n, n, &h->launches));
@@ -1262,7 +1259,7 @@ struct Solve final : SolveBase {
     if (moved) {
       int* hperm = (int*)(hstage + 2 * (size_t)l);
       for (int a = 0; a < l; ++a) hperm[a] = ord[a];
-      int* dperm = (int*)jac;
+      int* dperm = (int*)eigw;
       CHASE_CUDA_TRY(cudaMemcpyAsync(dperm, hperm, sizeof(int) * l, cudaMemcpyHostToDevice, st));
       TRY(copy_cols<T>(st, n, l, V, n, T2, n, &h->launches));
       TRY(gather_cols<T>(st, n, l, T2, n, dperm, V, n, &h->launches));
