@@ -223,8 +223,7 @@ int selftest_wait_timeout(cudaStream_t st, double seconds, DevStatus* dst, int* 
 // out = {lambda1, lambda_ell, b_sup} from nruns runs of m steps started at V0's columns.
 template <class T>
 int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const T* V0, int ldv,
-                   int m, int ell, double* out, void* work, size_t work_bytes, Scratch scr,
-                   int* launches);
+                   int m, int ell, double* out, void* work, size_t work_bytes, int* launches);
 size_t lanczos_work_bytes(size_t elem, int n, int nruns, int m);
 
 }  // namespace chase

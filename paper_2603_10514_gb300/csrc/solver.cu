@@ -1691,16 +1691,15 @@ int lanczos_entry(chase_ctx* h, chase_dtype dtype, int n, const void* dA, int ld
                   const void* dV0, int ldv, int steps, int ell, chase_bounds* out) {
   const size_t elem = (dtype == CHASE_R64) ? sizeof(double) : sizeof(z64);
   const size_t wb = lanczos_work_bytes(elem, n, nruns, steps);
-  TRY(ensure_ws(h, wb + kScratchBytes));
-  Scratch scr{(char*)h->ws + wb, kScratchBytes};
+  TRY(ensure_ws(h, wb));
   double b[3];
   int rc;
   if (dtype == CHASE_R64)
     rc = lanczos_bounds<double>(h->stream, n, (const double*)dA, lda, nruns, (const double*)dV0, ldv,
-                                steps, ell, b, h->ws, wb, scr, &h->launches);
+                                steps, ell, b, h->ws, wb, &h->launches);
   else
     rc = lanczos_bounds<z64>(h->stream, n, (const z64*)dA, lda, nruns, (const z64*)dV0, ldv, steps,
-                             ell, b, h->ws, wb, scr, &h->launches);
+                             ell, b, h->ws, wb, &h->launches);
   if (rc) return rc;
   out->lambda1 = b[0];
   out->lambda_ell = b[1];
