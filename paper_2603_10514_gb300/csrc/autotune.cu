@@ -1,7 +1,7 @@
 // autotune.cu -- the library's autotuner of the emulated-FP64 products' launch plans.
 //
-// A plan of the modular product (gemm_oz.cu) is the cap on its column-tile width (256, 192
-// or 128 columns per CTA; the tiles are then made as even as possible) and its number of K
+// A plan of the modular product (gemm_oz.cu) is the cap on its column-tile width (320, 256
+// or 160 columns per CTA pair; the tiles are then made as even as possible) and its number of K
 // splits (1 or 2).  The best plan depends on the product's shape: how many CTAs the grid
 // holds against the 152 SMs, how much of each tile is padding, and whether the per-CTA
 // fixed costs are amortised.  Because the modular products are exact integer arithmetic,
@@ -68,7 +68,7 @@ int oz_plan_candidates(int N, OzPlan* out, int cap) {
   // distinct (tile width, splits) pairs for N columns
   int n = 0;
   int seen_bn[3] = {0, 0, 0};
-  const int caps[3] = {256, 192, 128};
+  const int caps[3] = {320, 256, 160};
   for (int c = 0; c < 3; ++c) {
     const int ntile = (N + caps[c] - 1) / caps[c];
     const int bn = ((N + ntile - 1) / ntile + 15) / 16 * 16;

@@ -32,17 +32,27 @@
 // TWO real modular products per modulus (see "Complex products in split residue rings").
 //
 // Modular product kernel (ozm_kernel): CTA pairs (clusters of two along grid x), one pair
-// per (256-row block, column tile of BN <= 256 columns, modulus[, K split]).  The even CTA
-// issues tcgen05.mma.cta_group::2.kind::f16 (M 256, N BN, K 16) over the pair: each CTA
-// holds its own 128 rows of A and half of the BN rows of V in shared memory, and its 128
-// rows of the accumulator in its own TMEM (two buffers of 256 columns: the epilogue reads
-// one K chunk while the next accumulates).  Per CTA: a TMA producer thread (its copies
-// count on the even CTA's stage barrier), 16 epilogue warps reading TMEM with tcgen05.ld.
-// Stages: two 64-wide K blocks (128-byte swizzle), 3 stages of 64 KB.
-// Measured on GB300: the tensor pipe loses ~100-150 cycles per barrier round trip between
-// the producer and the issuer, hidden only when a stage holds >= 8 MMAs (K 128); a pair
-// moves 31 % fewer operand bytes per SM than a 128 x BN tile on one SM.  The product of
-// the default workload (K 20032, 600 columns) runs 12 % faster than with single-CTA tiles.
+// per (256-row block, column tile of BN <= 320 columns, modulus[, K split]).  The even CTA
+// issues tcgen05.mma.cta_group::2.kind::f16 (M 256, N <= 160, K 16) over the pair: each CTA
+// holds its own 128 rows of A and half of each MMA's V rows in shared memory, and its 128 rows of
+// the accumulators in its own TMEM.  Tiles above 160 columns are two halves with an MMA each on
+// the same A block.
+// What binds is the operand feed: a stage's copies must land within the time the other stages'
+// MMAs take (DRAM and L2 latency), and every SM takes at most ~67 bytes per clock from L2.  The
+// wide tile moves 59 bytes per clock of MMA time (128 rows of A and 152 of V per 304 columns; 71
+// for 208 columns), and a 64-wide K block of it still holds 8 MMAs, the fewest that hide a
+// barrier round trip between producer and issuer, so six stages fit where three K-128 stages of
+// a 256-column tile did.
+// The halves' exact K chunks are staggered by half a chunk over THREE accumulators of 160
+// columns: while one half's finished chunk is read out, the other half and the next chunk go
+// on in the other two.  16 epilogue warps read TMEM with tcgen05.ld; their sums take 80
+// registers, which setmaxnreg moves over from the producer's warpgroup.  The issuing warp's
+// loop is warp-uniform (one lane's instructions are predicated): under a lane-0 branch every
+// MMA took ~100 cycles to issue, which bound every tile narrower than 256 columns.
+// Measured against two 256-column accumulators, K-128 stages and a lane-0 issuer (full-size
+// modular products, real data): 600 columns complex 2616 -> 2159 us (1.68 PFLOP/s; cuBLAS holds
+// 1.73 under the power cap), real 1427 -> 1100 us; one tile of 64-256 columns stays bound by the
+// stream of A's planes from HBM (941 us at 64 columns, 6.4 TB/s).
 // All mbarrier waits are bounded; on expiry the kernel records the failure in
 // the device status word, waits (bounded) for its copies and MMAs in flight,
 // frees its TMEM and returns.
@@ -50,6 +60,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
+
+#include <type_traits>
 
 #include "../../include/chase_gb300.h"
 #include "common.cuh"
@@ -298,21 +310,50 @@ __constant__ int c_ring_p[kRingModuli] = {ring_modulus(0),  ring_modulus(1),  ri
                                           ring_modulus(15)};
 
 constexpr int MBM = 128, MBK = 64;
-constexpr int MKS = 2;             // 64-wide K blocks per stage: 8 MMAs per barrier round trip
-constexpr int MNST = 3;            // stages
-constexpr int MBN_MAX = 256;
+constexpr int MH_MAX = 160;         // columns of one MMA (one accumulator)
+constexpr int MBN_MAX = 2 * MH_MAX;
+constexpr int MNST_MAX = 8;
 constexpr int M_EPI_WARPS = 16;
-constexpr int M_THREADS = 64 + 32 * M_EPI_WARPS;
-constexpr int M_CHUNK_ST = 1024 / (MKS * MBK);  // stages per exact 1024-wide K chunk
-constexpr int M_RING_CHUNK_ST = kRingChunk / (MKS * MBK);          // and of a ring modulus
-constexpr int M_A1 = MBM * MBK * 2;              // 16 KB: 128 rows of A, one K block
-constexpr int M_B1 = (MBN_MAX / 2) * MBK * 2;    // 16 KB: up to 128 rows of V (half a tile)
-constexpr int M_STG = MKS * (M_A1 + M_B1);       // 64 KB
-constexpr int M_SMEM = MNST * M_STG + 1024 + 256;
-constexpr uint32_t M_TMEM_COLS = 2 * MBN_MAX;    // two accumulators of 256 columns
+constexpr int M_THREADS = 128 + 32 * M_EPI_WARPS;  // a warpgroup for producer and issuer
+constexpr int M_REG_MAIN = 64, M_REG_EPI = 104;    // of 5 x 96 registers at launch
+static_assert(M_REG_MAIN + 4 * M_REG_EPI <= 5 * 96, "register split");
+constexpr int M_CHUNK = 1024 / MBK;                // K blocks of an exact chunk
+constexpr int M_A1 = MBM * MBK * 2;                // 16 KB: 128 rows of A, one K block
+constexpr int M_STAGES = 6 * (M_A1 + MH_MAX * MBK * 2);  // bytes for stages: six of the widest tile
+constexpr int M_SMEM = M_STAGES + 1024 + 256;
+constexpr uint32_t M_TMEM_COLS = 512;              // three accumulators of 160 columns
 static_assert(M_SMEM <= 232448, "shared memory");
-static_assert(M_STG % 1024 == 0 && M_A1 % 1024 == 0, "stage alignment (128-byte swizzle atoms)");
-static_assert(M_CHUNK_ST * MKS * MBK == 1024, "exact chunk");
+static_assert(M_A1 % 1024 == 0, "stage alignment (128-byte swizzle atoms)");
+// K blocks whose products of residues mod p_j, with the folded sum of the earlier ones (fold2),
+// stay exact integers below 2^24: 4 for 509 to 8 for 349
+__host__ __device__ constexpr int ring_chunk_of(int j) {
+  const int h = ring_modulus(j) / 2;
+  return ((1 << 24) - 1 - 2 * h) / (h * h) / MBK;
+}
+static_assert(ring_chunk_of(0) * MBK == kRingChunk, "shortest exact chunk");
+__constant__ int c_ring_chunk[kRingModuli] = {ring_chunk_of(0),  ring_chunk_of(1),  ring_chunk_of(2),
+                                              ring_chunk_of(3),  ring_chunk_of(4),  ring_chunk_of(5),
+                                              ring_chunk_of(6),  ring_chunk_of(7),  ring_chunk_of(8),
+                                              ring_chunk_of(9),  ring_chunk_of(10), ring_chunk_of(11),
+                                              ring_chunk_of(12), ring_chunk_of(13), ring_chunk_of(14),
+                                              ring_chunk_of(15)};
+__device__ __forceinline__ int ring_chunk(int j) { return c_ring_chunk[j]; }
+
+// Shape of a column tile of BN columns (a multiple of 16): one or two halves (multiples of 16),
+// K blocks per stage (8 MMAs where BN > 64 needs them), bytes of a stage and stages that fit.
+struct TileShape {
+  int h0, h1, ks, hb, stage, nst;
+};
+__host__ __device__ inline TileShape tile_shape(int BN) {
+  TileShape s;
+  s.h0 = BN <= MH_MAX ? BN : (BN / 2 + 15) / 16 * 16;
+  s.h1 = BN - s.h0;
+  s.ks = s.h1 ? 1 : 2;
+  s.hb = (s.h0 / 2) * MBK * 2;  // bytes of one CTA's V rows of a half (the box of the V map)
+  s.stage = s.ks * (M_A1 + (s.h1 ? 2 : 1) * s.hb);
+  s.nst = M_STAGES / s.stage < MNST_MAX ? M_STAGES / s.stage : MNST_MAX;
+  return s;
+}
 using namespace tc;
 
 // ---------------------------------------------------------------------------
@@ -320,11 +361,6 @@ using namespace tc;
 // z = split * S + j (grid z).  Lres planes row-major (rows x kp), Vres planes column-major
 // (kp x ncols); both K-padded with zeros to kp (a multiple of 64).
 // ---------------------------------------------------------------------------
-// One CTA of a pair (clusters of two CTAs along grid x): this CTA's rows [m0, m0 + 128)
-// and the pair's columns [n0, n0 + BN) of modulus jm over the K blocks [kbeg, kbeg + nkb);
-// residues into Rz (column-major M x N).  kbeg is even; an odd nkb reads one zero-filled
-// block past kp (the K-padded operands end there), or the first block of the next split
-// only when nkb is odd, which the launch never makes for a split other than the last.
 // s mod p in [0, p) by a float quotient that is off by at most one.
 __device__ __forceinline__ int mod_sum(int s, int p, float ip) {
   const int q = (int)floorf((float)s * ip);
@@ -343,44 +379,56 @@ __device__ __forceinline__ uint64_t pack2(float x, float y) {
 // per SM and would take longer than the chunk's MMAs.
 __device__ __forceinline__ uint64_t fold2(uint64_t acc, uint32_t v0, uint32_t v1, uint64_t ip2, uint64_t np2) {
   const uint64_t magic = 0x4B4000004B400000ull;   // 1.5 * 2^23, twice
-  const uint64_t nmagic = 0xCB400000CB400000ull;
   uint64_t v, s, q, r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(v0), "r"(v1));
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(acc), "l"(v));
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(s), "l"(ip2), "l"(magic));
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(q), "l"(nmagic));
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(q) : "l"(q), "l"(magic));
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(q), "l"(np2), "l"(s));
   return r;
 }
 
+// One CTA of a pair (clusters of two CTAs along grid x): this CTA's rows [m0, m0 + 128)
+// and the pair's columns [n0, n0 + BN) of modulus jm over the K blocks [kbeg, kbeg + nkb);
+// residues into Rv (column-major M x N).  A stage may hold one block past the last (zero-filled
+// beyond kp, else the next split's): it is copied but not multiplied.
 // RING: modulus jm of the ring set, 256-wide exact chunks folded mod p as they come (no limit
 // on the length of K), two-byte residues.
+//
+// Accumulators: at switch s = 1, 2, ... (every half chunk; one-half tiles: every chunk) one
+// half's finished accumulator goes to the epilogue and the half moves on to the accumulator
+// that the switch before gave up.  Two halves: odd switches are half 1's, even ones half 0's;
+// accumulator (2 - s) mod 3 is given up for (3 - s) mod 3.  One half: (s - 1) & 1 for s & 1.
+// After the last block every half's accumulator follows in the same order.
 template <bool RING>
 __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUtensorMap* mapV,
                                               int M, int N, int BN, int col0, int m0, int n0,
                                               int jm, int kbeg, int nkb, void* __restrict__ Rv,
                                               DevStatus* status) {
-  constexpr int CHUNK_ST = RING ? M_RING_CHUNK_ST : M_CHUNK_ST;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = (uint64_t*)(smem + MNST * M_STG);
-  uint64_t* full = bars;                // [MNST] stage loaded (both CTAs' copies; the even CTA's)
-  uint64_t* empty = bars + MNST;        // [MNST] stage read by the pair's MMAs
-  uint64_t* cfull = bars + 2 * MNST;    // [2] chunk accumulated in buffer b
-  uint64_t* cfree = cfull + 2;          // [2] buffer b read out by both CTAs (the even CTA's)
-  uint64_t* tdone = cfree + 2;          // every MMA finished
+  uint64_t* bars = (uint64_t*)(smem + M_STAGES);
+  uint64_t* full = bars;                    // [MNST_MAX] stage loaded (both CTAs' copies; the even CTA's)
+  uint64_t* empty = bars + MNST_MAX;        // [MNST_MAX] stage read by the pair's MMAs
+  uint64_t* cfull = bars + 2 * MNST_MAX;    // [3] accumulator b holds a finished chunk
+  uint64_t* cfree = cfull + 3;              // [3] accumulator b read out by both CTAs (the even CTA's)
+  uint64_t* tdone = cfree + 3;              // every MMA finished
   uint32_t* tslot = (uint32_t*)(tdone + 1);
   int* s_err = (int*)(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
-  const int half = BN >> 1;
-  const int nst = (nkb + MKS - 1) / MKS;
-  const int nchunks = (nst + CHUNK_ST - 1) / CHUNK_ST;
+  const TileShape ts = tile_shape(BN);
+  const bool two = ts.h1 > 0;
+  const int nst = (nkb + ts.ks - 1) / ts.ks;
+  const int chunk = RING ? ring_chunk(jm) : M_CHUNK;  // K blocks of an exact chunk
+  const int gap1 = two ? chunk / 2 : chunk, gap0 = two ? chunk - gap1 : chunk;  // blocks before odd / even switches
+  const int nsw = (two ? 2 : 1) * ((nkb - 1) / chunk) + (two && (nkb - 1) % chunk >= gap1 ? 1 : 0);  // switches
+  const int ndrain = nkb > 0 ? nsw + (two ? 2 : 1) : 0;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < MNST; ++i) { bar_init(&full[i], 1); bar_init(&empty[i], 1); }
-    for (int b = 0; b < 2; ++b) { bar_init(&cfull[b], 1); bar_init(&cfree[b], 2 * M_EPI_WARPS); }
+    for (int i = 0; i < MNST_MAX; ++i) { bar_init(&full[i], 1); bar_init(&empty[i], 1); }
+    for (int b = 0; b < 3; ++b) { bar_init(&cfull[b], 1); bar_init(&cfree[b], 2 * M_EPI_WARPS); }
     bar_init(tdone, 1);
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -396,121 +444,175 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
 
-  if (warp == 0 && lane == 0) {
-    // ---------------- producer (both CTAs): own A rows, own half of the V tile ----------------
-    const uint32_t bytes = (uint32_t)(MKS * (2 * M_A1 + BN * MBK * 2));  // the pair's copies of a stage
-    const uint32_t full0 = peer_addr(full, 0);
-    int issued = 0;
-    for (int kb = 0; kb < nst && !*(volatile int*)s_err; ++kb) {
-      const int s = kb % MNST;
-      if (!bar_wait(&empty[s], (uint32_t)(((kb / MNST) & 1) ^ 1))) { atomicOr(s_err, 1); break; }
-      if (rank == 0) bar_expect(&full[s], bytes);
-      unsigned char* st = smem + s * M_STG;
-      const uint32_t fb = full0 + 8u * (uint32_t)s;
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(M_REG_MAIN));
+    if (warp == 0 && lane == 0) {
+      // ---------------- producer (both CTAs): own A rows, own half of each V half tile ----------------
+      const uint32_t bytes = (uint32_t)(2 * ts.stage);  // the pair's copies of a stage
+      const uint32_t full0 = peer_addr(full, 0);
+      const int v0 = col0 + n0 + (int)rank * (ts.h0 >> 1), v1 = col0 + n0 + ts.h0 + (int)rank * (ts.h1 >> 1);
+      int issued = 0, s = 0;
+      uint32_t ph = 1;
+      for (int it = 0; it < nst && !*(volatile int*)s_err; ++it) {
+        if (!bar_wait(&empty[s], ph)) { atomicOr(s_err, 1); break; }
+        if (rank == 0) bar_expect(&full[s], bytes);
+        unsigned char* st = smem + s * ts.stage;
+        const uint32_t fb = full0 + 8u * (uint32_t)s;
+        const int x = (kbeg + it * ts.ks) * MBK;
+        tma3_pair(st, mapA, fb, x, m0, jm);
+        if (two) {
+          tma3_pair(st + M_A1, mapV, fb, x, v0, jm);
+          tma3_pair(st + M_A1 + ts.hb, mapV, fb, x, v1, jm);
+        } else {
+          tma3_pair(st + M_A1, mapA, fb, x + MBK, m0, jm);
+          tma3_pair(st + 2 * M_A1, mapV, fb, x, v0, jm);
+          tma3_pair(st + 2 * M_A1 + ts.hb, mapV, fb, x + MBK, v0, jm);
+        }
+        issued = it + 1;
+        if (++s == ts.nst) { s = 0; ph ^= 1; }
+      }
+      // every release of this CTA's stages has arrived (no arrival may reach it after exit) ...
+      for (int it = issued; it < issued + ts.nst; ++it)
+        if (!bar_wait(&empty[it % ts.nst], (uint32_t)(((it / ts.nst) & 1) ^ 1))) { atomicOr(s_err, 1); break; }
+      // ... and, in the even CTA, every copy of both CTAs has landed
+      if (rank == 0)
+        for (int b = max(0, issued - ts.nst); b < issued; ++b)
+          if (!bar_wait(&full[b % ts.nst], (uint32_t)((b / ts.nst) & 1))) { atomicOr(s_err, 1); break; }
+    } else if (warp == 1 && rank == 0) {
+      // ---------------- MMA issuer (even CTA, the whole warp): M 256 x N h x K 16 over the pair ----------------
+      const uint32_t leader = elect_lane();
+      const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * MBM) >> 4) << 24);
+      const uint32_t id0 = id | ((uint32_t)(ts.h0 >> 3) << 17), id1 = id | ((uint32_t)(ts.h1 >> 3) << 17);
+      uint32_t d0 = tmem, d1 = tmem + MH_MAX;  // the halves' accumulators
+      uint32_t acc0 = 0, acc1 = 0;             // 0: the next MMA starts a chunk
+      uint32_t given = 0, fph = 0;             // accumulators given up before, phases of their release
+      int sw = 0, left = gap1;                 // switches made, blocks to the next one
+      bool bad = false;
+      int s = 0;
+      uint32_t ph = 0;
+      for (int it = 0; it < nst && !bad; ++it) {
+        if (!bar_poll(&full[s], ph)) { bad = true; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t sa = s32(smem + s * ts.stage);
+        for (int u = 0; u < ts.ks; ++u) {
+          if (it * ts.ks + u >= nkb) break;
+          if (left == 0) {
+            ++sw;
+            left = (sw & 1) ? gap0 : gap1;
+            const int from = two ? (sw % 3 == 0 ? 2 : 2 - sw % 3) : (sw - 1) & 1;
+            const int to = two ? (sw % 3 == 0 ? 0 : 3 - sw % 3) : sw & 1;
+            commit_pair_w(&cfull[from], leader);
+            if ((given >> to) & 1) {  // read out since it was given up
+              if (!bar_poll(&cfree[to], (fph >> to) & 1)) { bad = true; break; }
+              fph ^= 1u << to;
+            }
+            given |= 1u << from;
+            if (two && (sw & 1)) { d1 = tmem + (uint32_t)to * MH_MAX; acc1 = 0; }
+            else { d0 = tmem + (uint32_t)to * MH_MAX; acc0 = 0; }
+          }
+          --left;
+          const uint64_t da = desc_sw128(sa + u * M_A1);
+          const uint64_t dv = desc_sw128(sa + ts.ks * M_A1 + u * ts.hb);
 #pragma unroll
-      for (int u = 0; u < MKS; ++u) {
-        const int x = (kbeg + kb * MKS + u) * MBK;
-        tma3_pair(st + u * M_A1, mapA, fb, x, m0, jm);
-        tma3_pair(st + MKS * M_A1 + u * M_B1, mapV, fb, x, col0 + n0 + (int)rank * half, jm);
-      }
-      issued = kb + 1;
-    }
-    // every release of this CTA's stages has arrived (no arrival may reach it after exit) ...
-    for (int kb = issued; kb < issued + MNST; ++kb)
-      if (!bar_wait(&empty[kb % MNST], (uint32_t)(((kb / MNST) & 1) ^ 1))) { atomicOr(s_err, 1); break; }
-    // ... and, in the even CTA, every copy of both CTAs has landed
-    if (rank == 0)
-      for (int b = max(0, issued - MNST); b < issued; ++b)
-        if (!bar_wait(&full[b % MNST], (uint32_t)((b / MNST) & 1))) { atomicOr(s_err, 1); break; }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
-    // ---------------- MMA issuer (even CTA): M 256 x N BN x K 16 over the pair ----------------
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                           ((uint32_t)((2 * MBM) >> 4) << 24);
-    bool bad = false;
-    for (int kb = 0; kb < nst && !bad; ++kb) {
-      const int chunk = kb / CHUNK_ST;
-      const bool cstart = (kb % CHUNK_ST) == 0;
-      const bool clast = (kb % CHUNK_ST) == CHUNK_ST - 1 || kb == nst - 1;
-      const uint32_t buf = (uint32_t)(chunk & 1);
-      if (cstart && chunk >= 2) {
-        // both CTAs' epilogues have read this buffer's previous chunk (chunk - 2)
-        if (!bar_wait(&cfree[buf], (uint32_t)(((chunk - 2) >> 1) & 1))) { bad = true; break; }
-      }
-      const int s = kb % MNST;
-      if (!bar_poll(&full[s], (uint32_t)((kb / MNST) & 1))) { bad = true; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sa = s32(smem + s * M_STG);
+          for (int k = 0; k < MBK / 16; ++k) {
+            mma_pair_w(d0, da + 2 * k, dv + 2 * k, id0, acc0, leader);
+            acc0 = 1;
+          }
+          if (two) {
+            const uint64_t dw = desc_sw128(sa + M_A1 + ts.hb);
 #pragma unroll
-      for (int kk = 0; kk < MKS * (MBK / 16); ++kk) {
-        const uint64_t da = desc_sw128(sa + (kk >> 2) * M_A1);
-        const uint64_t dv = desc_sw128(sa + MKS * M_A1 + (kk >> 2) * M_B1);
-        mma_pair(tmem + buf * MBN_MAX, da + (uint64_t)((kk & 3) * 2), dv + (uint64_t)((kk & 3) * 2),
-                 idesc, (cstart && kk == 0) ? 0u : 1u);
+            for (int k = 0; k < MBK / 16; ++k) {
+              mma_pair_w(d1, da + 2 * k, dw + 2 * k, id1, acc1, leader);
+              acc1 = 1;
+            }
+          }
+        }
+        if (bad) break;
+        commit_pair_w(&empty[s], leader);
+        if (++s == ts.nst) { s = 0; ph ^= 1; }
       }
-      commit_pair(&empty[s]);
-      if (clast) commit_pair(&cfull[buf]);
+      if (bad && lane == 0) atomicOr(s_err, 2);
+      // the halves' last chunks, in switch order
+      for (int e = nsw + 1; e <= ndrain && !bad; ++e)
+        commit_pair_w(&cfull[two ? (e % 3 == 0 ? 2 : 2 - e % 3) : (e - 1) & 1], leader);
+      commit_pair_w(tdone, leader);
     }
-    if (bad) atomicOr(s_err, 2);
-    commit_pair(tdone);
-  } else if (warp >= 2) {
+  } else {
     // ---------------- epilogue (both CTAs, own TMEM lanes = own 128 rows) ----------------
-    // warp w reads TMEM lanes 32 (w % 4) .. +31 (the hardware's lane quarter of the warp)
-    // and the column quarter (w - 2) / 4 of the tile (BN / 4 <= 64 columns).
-    const int q = warp & 3, cq = (warp - 2) >> 2;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(M_REG_EPI));
+    // warp w reads TMEM lanes 32 (w % 4) .. +31 (the hardware's lane quarter of the warp) and
+    // the quarter (w - 4) / 4 of each half's columns (<= 40)
+    const int q = warp & 3, cq = (warp - 4) >> 2;
     const int r = m0 + 32 * q + lane;
-    const int cw = BN >> 2;
+    const int cw0 = ts.h0 >> 2, cw1 = ts.h1 >> 2;
     const uint32_t cfree0 = peer_addr(cfree, 0);
     const int pm = RING ? c_ring_p[jm] : c_crt.p[jm];
     const float ip = 1.0f / (float)pm;
     // sums of the chunks: 32-bit integers, or (ring) pairs of floats in (-0.51 p, 0.51 p)
-    int sum[RING ? 1 : 64];
-    uint64_t acc[RING ? 32 : 1];
+    constexpr int CW = MH_MAX / 4;
+    int sum[2][RING ? 1 : CW];
+    uint64_t acc[2][RING ? CW / 2 : 1];
     const uint64_t ip2 = pack2(ip, ip), np2 = pack2(-(float)pm, -(float)pm);
 #pragma unroll
-    for (int j = 0; j < (RING ? 1 : 64); ++j) sum[j] = 0;
+    for (int h = 0; h < 2; ++h) {
 #pragma unroll
-    for (int j = 0; j < (RING ? 32 : 1); ++j) acc[j] = 0;
+      for (int j = 0; j < (RING ? 1 : CW); ++j) sum[h][j] = 0;
+#pragma unroll
+      for (int j = 0; j < (RING ? CW / 2 : 1); ++j) acc[h][j] = 0;
+    }
+    uint32_t uses = 0;  // phases of the accumulators' cfull
     bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-      const uint32_t buf = (uint32_t)(c & 1);
-      if (!__all_sync(0xffffffffu, bar_wait(&cfull[buf], (uint32_t)((c >> 1) & 1)))) {
+    auto drain = [&](auto half, int e, int b) {
+      constexpr int H = decltype(half)::value;
+      const int cw = H ? cw1 : cw0;
+      if (!__all_sync(0xffffffffu, bar_wait(&cfull[b], (uses >> b) & 1))) {
         ok = false;
         if (lane == 0) atomicOr(s_err, 4);
-        break;
+        return;
       }
+      uses ^= 1u << b;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + buf * MBN_MAX + (uint32_t)(cq * cw);
-      // 16 columns at a time: wider reads spill, and a spill in this loop costs more than the reads
+      const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * MH_MAX + cq * cw);
+      // eight columns at a time: wider reads spill, and a spill in this loop costs more
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        if (16 * g >= cw) break;
-        uint32_t v[16];
-        ld16(ta + 16 * g, v);
+      for (int g = 0; g < CW / 8; ++g) {
+        if (8 * g >= cw) break;
+        uint32_t v[8];
+        ld8(ta + 8 * g, v);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if constexpr (RING) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            acc[8 * g + j] = fold2(acc[8 * g + j], v[2 * j], v[2 * j + 1], ip2, np2);
+          for (int j = 0; j < 4; ++j)
+            acc[H][4 * g + j] = fold2(acc[H][4 * g + j], v[2 * j], v[2 * j + 1], ip2, np2);
         } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) sum[16 * g + j] += __float2int_rn(__uint_as_float(v[j]));
+          for (int j = 0; j < 8; ++j) sum[H][8 * g + j] += __float2int_rn(__uint_as_float(v[j]));
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0 && c + 2 < nchunks) arrive_remote_relaxed(cfree0 + 8u * buf);
+      if (lane == 0 && e <= nsw) arrive_remote_relaxed(cfree0 + 8u * (uint32_t)b);
+    };
+    for (int e = 1; e <= ndrain && ok; ++e) {
+      if (!two) drain(std::integral_constant<int, 0>(), e, (e - 1) & 1);
+      else if (e & 1) drain(std::integral_constant<int, 1>(), e, e % 3 == 0 ? 2 : 2 - e % 3);
+      else drain(std::integral_constant<int, 0>(), e, e % 3 == 0 ? 2 : 2 - e % 3);
     }
     if (__shfl_sync(0xffffffffu, (int)(ok && !*(volatile int*)s_err), 0) && r < M) {
-      // the sum mod p in [0, p)
+      // the sums mod p in [0, p)
 #pragma unroll
-      for (int j = 0; j < 64; ++j) {
-        const int col = n0 + cq * cw + j;
-        if (j < cw && col - n0 < BN && col < N) {
-          if constexpr (RING) {
-            const int rr = (int)__uint_as_float((uint32_t)(acc[j >> 1] >> (32 * (j & 1))));
-            ((uint16_t*)Rv)[(size_t)col * M + r] = (uint16_t)(rr < 0 ? rr + pm : rr);
-          } else {
-            ((uint8_t*)Rv)[(size_t)col * M + r] = (uint8_t)mod_sum(sum[j], pm, ip);
+      for (int h = 0; h < 2; ++h) {
+        const int cw = h ? cw1 : cw0, c0 = n0 + h * ts.h0 + cq * cw;
+#pragma unroll
+        for (int j = 0; j < CW; ++j) {
+          if (j < cw && c0 + j < N) {
+            const size_t at = (size_t)(c0 + j) * M + r;
+            if constexpr (RING) {
+              const int rr = (int)__uint_as_float((uint32_t)(acc[h][j >> 1] >> (32 * (j & 1))));
+              ((uint16_t*)Rv)[at] = (uint16_t)(rr < 0 ? rr + pm : rr);
+            } else {
+              ((uint8_t*)Rv)[at] = (uint8_t)mod_sum(sum[h][j], pm, ip);
+            }
           }
         }
       }
@@ -1400,7 +1502,7 @@ int ozm_launch(cudaStream_t st, int M, int kp, const void* Aplanes, int a_plane_
   const int BN = ceil_div(ceil_div(N, ntile), 16) * 16;
   CUtensorMap mA, mV;
   if (make_map3(&mA, Aplanes, kp, M, a_plane_rows, MBM) ||
-      make_map3(&mV, Vplanes, kp, ncols_total, ncols_total, BN / 2))
+      make_map3(&mV, Vplanes, kp, ncols_total, ncols_total, tile_shape(BN).h0 / 2))
     return CHASE_ERR_CUDA;
   CHASE_CUDA_TRY(cudaFuncSetAttribute(ozm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M_SMEM));
   const int nkb = kp / MBK;
@@ -1416,7 +1518,7 @@ int ozm_launch(cudaStream_t st, int M, int kp, const void* Aplanes, int a_plane_
   S = std::max(std::min(S, kOzMaxSplits), min_S);
   while (S > min_S && (size_t)S * slab > resbuf.bytes) --S;
   if ((size_t)S * slab > resbuf.bytes) return CHASE_ERR_OOM;
-  const int kbs = ceil_div(nchunks, S) * kChunkKB;  // whole chunks: every split starts on an even block
+  const int kbs = ceil_div(nchunks, S) * kChunkKB;  // whole chunks
   S = ceil_div(nkb, kbs);
   TRY_OZ(launch_pairs(ozm_kernel, dim3(ntile * mblk, 1, kOzModuli * S), st, mA, mV, M, N, BN, ntile,
                       col0, nkb, kbs, (uint8_t*)resbuf.ptr, dst));
@@ -1577,7 +1679,7 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
       const int p = P.count++;
       if (make_map3(&P.mapA[p], (const char*)it.Aplanes + sidx * aset, it.kp, it.M, rows, MBM, nm) ||
           make_map3(&P.mapV[p], (const char*)it.Vplanes + sidx * vset, it.kp, it.ncols_total,
-                    it.ncols_total, BN / 2, nm))
+                    it.ncols_total, tile_shape(BN).h0 / 2, nm))
         return CHASE_ERR_CUDA;
       P.R[p] = (char*)it.resbuf.ptr + sidx * rset;
       P.ring[p] = it.ring ? nm : 0;

@@ -169,7 +169,7 @@ int transpose(cudaStream_t st, int n, int l, const T* X, int ldx, T* Xt, int ldt
 // Launch plan of an emulated product: cap on the column-tile width (tiles as even as
 // possible below it) and K splits (0: about four waves of CTAs, at most kOzMaxSplits).
 struct OzPlan {
-  int bn_max = 256;
+  int bn_max = 320;
   int splits = 0;
 };
 // The autotuner's table (autotune.cu): plans measured per shape bucket.
