@@ -501,7 +501,7 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
             left = (sw & 1) ? gap0 : gap1;
             const int from = two ? (sw % 3 == 0 ? 2 : 2 - sw % 3) : (sw - 1) & 1;
             const int to = two ? (sw % 3 == 0 ? 0 : 3 - sw % 3) : sw & 1;
-            commit_pair_w(&cfull[from], leader);
+            commit_pair(&cfull[from], leader);
             if ((given >> to) & 1) {  // read out since it was given up
               if (!bar_poll(&cfree[to], (fph >> to) & 1)) { bad = true; break; }
               fph ^= 1u << to;
@@ -515,27 +515,27 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
           const uint64_t dv = desc_sw128(sa + ts.ks * M_A1 + u * ts.hb);
 #pragma unroll
           for (int k = 0; k < MBK / 16; ++k) {
-            mma_pair_w(d0, da + 2 * k, dv + 2 * k, id0, acc0, leader);
+            mma_pair(d0, da + 2 * k, dv + 2 * k, id0, acc0, leader);
             acc0 = 1;
           }
           if (two) {
             const uint64_t dw = desc_sw128(sa + M_A1 + ts.hb);
 #pragma unroll
             for (int k = 0; k < MBK / 16; ++k) {
-              mma_pair_w(d1, da + 2 * k, dw + 2 * k, id1, acc1, leader);
+              mma_pair(d1, da + 2 * k, dw + 2 * k, id1, acc1, leader);
               acc1 = 1;
             }
           }
         }
         if (bad) break;
-        commit_pair_w(&empty[s], leader);
+        commit_pair(&empty[s], leader);
         if (++s == ts.nst) { s = 0; ph ^= 1; }
       }
       if (bad && lane == 0) atomicOr(s_err, 2);
       // the halves' last chunks, in switch order
       for (int e = nsw + 1; e <= ndrain && !bad; ++e)
-        commit_pair_w(&cfull[two ? (e % 3 == 0 ? 2 : 2 - e % 3) : (e - 1) & 1], leader);
-      commit_pair_w(tdone, leader);
+        commit_pair(&cfull[two ? (e % 3 == 0 ? 2 : 2 - e % 3) : (e - 1) & 1], leader);
+      commit_pair(tdone, leader);
     }
   } else {
     // ---------------- epilogue (both CTAs, own TMEM lanes = own 128 rows) ----------------
@@ -591,7 +591,7 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0 && e <= nsw) arrive_remote_relaxed(cfree0 + 8u * (uint32_t)b);
+      if (lane == 0 && e <= nsw) arrive_remote(cfree0 + 8u * (uint32_t)b);
     };
     for (int e = 1; e <= ndrain && ok; ++e) {
       if (!two) drain(std::integral_constant<int, 0>(), e, (e - 1) & 1);

@@ -19,8 +19,9 @@
 // each CTA); each CTA loads its own 128 rows of Ah and Al and half of the tile's rows of Vh
 // and Vl (TMA, 128-byte swizzle, 64-wide K blocks, three 64 KB stages: 12 MMAs per barrier
 // round trip); 16 epilogue warps per CTA read TMEM (tcgen05.ld), apply the FP64 three-term
-// update and write the BF16 split of the result.  Same structure as the modular-product
-// kernel of gemm_oz.cu (and its measured reasons).
+// update and write the BF16 split of the result.  Bound: the MMAs, and the epilogue's FP64
+// operations (2 per clock per SM).  Complex n = 4000, 240 columns, 20 steps: 4.17 -> 2.71 ms by
+// the warp-uniform issuer, tiles that fill the SMs and splitting each part of A once.
 // Every mbarrier wait is bounded (~2 s of clock64); on expiry the kernel sets a flag in the
 // device status word, drains, frees its TMEM and returns.
 #include <cuda.h>
@@ -116,14 +117,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (rank == 0)
       for (int b = max(0, issued - TSTAGES); b < issued; ++b)
         if (!bar_wait(&full[b % TSTAGES], (uint32_t)((b / TSTAGES) & 1))) { atomicOr(s_err, 1); break; }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
+  } else if (warp == 1 && rank == 0) {
     // ---------------- MMA issuer (even CTA): M 256 x N BN x K 16, three per K step ----------------
+    // (the whole warp, one lane's instructions predicated: see tcgen05.cuh)
+    const uint32_t leader = elect_lane();
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)((2 * TBM) >> 4) << 24);
     bool bad = false;
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % TSTAGES;
-      if (!bar_poll(&full[s], (uint32_t)((kb / TSTAGES) & 1))) { bad = true; break; }
+      if (!bar_poll(&full[s], ph)) { bad = true; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sa = s32(smem + s * STAGE_BYTES);
       const uint64_t dAh = desc_sw128(sa), dAl = desc_sw128(sa + T_A1);
@@ -131,14 +135,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
       for (int kk = 0; kk < TBK / 16; ++kk) {
         const uint64_t off = (uint64_t)(kk * 2);  // 32 bytes per K = 16 step
-        mma_pair(tmem, dAh + off, dVh + off, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-        mma_pair(tmem, dAh + off, dVl + off, idesc, 1u);
-        mma_pair(tmem, dAl + off, dVh + off, idesc, 1u);
+        mma_pair(tmem, dAh + off, dVh + off, idesc, (kb > 0 || kk > 0) ? 1u : 0u, leader);
+        mma_pair(tmem, dAh + off, dVl + off, idesc, 1u, leader);
+        mma_pair(tmem, dAl + off, dVh + off, idesc, 1u, leader);
       }
-      commit_pair(&empty[s]);
+      commit_pair(&empty[s], leader);
+      if (++s == TSTAGES) { s = 0; ph ^= 1; }
     }
-    if (bad) atomicOr(s_err, 2);
-    commit_pair(tfull);
+    if (bad && lane == 0) atomicOr(s_err, 2);
+    commit_pair(tfull, leader);
   } else if (warp >= 2) {
     // ---------------- epilogue (both CTAs: own TMEM lanes = own 128 rows) ----------------
     const int q = warp & 3, cq = (warp - 2) >> 2;  // lane quarter, column quarter
@@ -187,31 +192,45 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // ---------------- operand preparation ----------------
 
 // Stacked real A (row-major, K contiguous, ld kp) split into BF16 hi / lo.
-// Complex: Ahat = [[Ar, -Ai], [Ai, Ar]] (symmetric because A is Hermitian).
+// Complex: Ahat = [[Ar, -Ai], [Ai, Ar]] (symmetric because A is Hermitian): each part is split
+// once and written to its two places (the splits' FP64 conversions and subtraction, at 2 per
+// clock per SM, bind).  Row blockIdx.y of A, K along x; the last column block pads to kp.
 template <class T>
-__global__ void split_A_kernel(int n, const T* __restrict__ A, int lda, int kp,
-                               __nv_bfloat16* Ah, __nv_bfloat16* Al) {
+__global__ void __launch_bounds__(256) split_A_kernel(int n, const T* __restrict__ A, int lda, int kp,
+                                                      __nv_bfloat16* Ah, __nv_bfloat16* Al) {
   const int M = Sc<T>::cplx ? 2 * n : n;
-  const size_t total = (size_t)M * kp;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(t % kp), m = (int)(t / kp);
-    double x = 0.0;
-    if (k < M) {
-      // Ahat[m, k] = Ahat[k, m] (symmetric): read column m of Ahat, contiguous in k
+  auto split = [](double x, __nv_bfloat16* hi, __nv_bfloat16* lo) {
+    *hi = __double2bfloat16(x);
+    *lo = __double2bfloat16(x - (double)__bfloat162float(*hi));
+  };
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  for (int m = blockIdx.y; m < n; m += gridDim.y) {
+    const size_t row = (size_t)m * kp, row2 = (size_t)(n + m) * kp;
+    if (k < n) {
+      const T a = A[(size_t)k + (size_t)m * lda];
+      __nv_bfloat16 h, l;
+      split(Sc<T>::re(a), &h, &l);
+      Ah[row + k] = h;
+      Al[row + k] = l;
       if constexpr (Sc<T>::cplx) {
-        const int kk = k % n, mm = m % n;
-        const bool kre = k < n, mre = m < n;
-        const z64 a = A[(size_t)kk + (size_t)mm * lda];  // A[kk, mm]
-        // Ahat[k, m]: block (k-half, m-half): (re,re) Ar, (re,im) -Ai, (im,re) Ai, (im,im) Ar
-        x = (kre == mre) ? a.x : (kre ? -a.y : a.y);
-      } else {
-        x = A[(size_t)k + (size_t)m * lda];
+        Ah[row2 + n + k] = h;
+        Al[row2 + n + k] = l;
+        split(a.y, &h, &l);
+        Ah[row + n + k] = h;
+        Al[row + n + k] = l;
+        Ah[row2 + k] = __hneg(h);
+        Al[row2 + k] = __hneg(l);
       }
     }
-    const __nv_bfloat16 hi = __double2bfloat16(x);
-    Ah[t] = hi;
-    Al[t] = __double2bfloat16(x - (double)__bfloat162float(hi));
+    if (k < kp - M) {  // (kp - M < 64)
+      const __nv_bfloat16 z = __float2bfloat16(0.f);
+      Ah[row + M + k] = z;
+      Al[row + M + k] = z;
+      if (Sc<T>::cplx) {
+        Ah[row2 + M + k] = z;
+        Al[row2 + M + k] = z;
+      }
+    }
   }
 }
 
@@ -300,9 +319,8 @@ int tc_kpad(int M) { return ((M + TBK - 1) / TBK) * TBK; }
 template <class T>
 int tc_split_A(cudaStream_t st, int n, const T* A, int lda, int kp, void* Ah, void* Al,
                int* launches) {
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  split_A_kernel<T><<<grid_for((size_t)M * kp), 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)Ah,
-                                                              (__nv_bfloat16*)Al);
+  const dim3 grid(ceil_div(n, 256), std::min(n, 65535));
+  split_A_kernel<T><<<grid, 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)Ah, (__nv_bfloat16*)Al);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -335,10 +353,20 @@ int tc_filter_step(cudaStream_t st, int M, int kp, const void* Ah, const void* A
                    double* out64, int ldv, void* Vh_out, void* Vl_out, DevStatus* dst,
                    int* launches) {
   if (N <= 0) return 0;
-  // column tiles of at most 256 (a multiple of 16), as even as possible; CTA pairs over
-  // 256-row blocks
-  const int ntile = ceil_div(N, TBN_MAX);
-  const int BN = ceil_div(ceil_div(N, ntile), 16) * 16;
+  // CTA pairs over 256-row blocks and column tiles of BN <= 256 (a multiple of 16), as even as
+  // possible: the count of tiles with the least waves x (MMAs + FP64 epilogue of a tile), in
+  // clocks: three MMAs of BN / 2 (at least 48) per K step and ~4 FP64 operations for each of
+  // 128 BN outputs per CTA at 2 per clock.  M = 8000, N = 240: 32 pairs of 240 columns leave
+  // half of the SMs idle, 64 of 128 take 0.6 of the time.
+  int ntile = ceil_div(N, TBN_MAX), BN = 0;
+  double best = 1e300;
+  for (int nt = ntile; nt <= ceil_div(N, 48) || nt == ntile; ++nt) {
+    const int bn = ceil_div(ceil_div(N, nt), 16) * 16;
+    const double waves = ceil_div((long long)ceil_div(M, 2 * TBM) * ceil_div(N, bn), kNumSMs / 2);
+    const double cost = waves * (kp / 16 * 3.0 * std::max(bn / 2, 48) + 256.0 * bn + 8000.0);
+    if (cost < best * 0.98) { best = cost; BN = bn; }
+  }
+  ntile = ceil_div(N, BN);
   CUtensorMap mAh, mAl, mVh, mVl;
   if (make_map(&mAh, Ah, kp, M, TBM) || make_map(&mAl, Al, kp, M, TBM) ||
       make_map(&mVh, Vh_in, kp, ncols_total, BN / 2) || make_map(&mVl, Vl_in, kp, ncols_total, BN / 2))

@@ -76,12 +76,8 @@ __device__ __forceinline__ void cluster_sync() {
 // Arrival that hands a TMEM buffer back (after tcgen05.wait::ld and fence::before_thread_sync:
 // the loaded values are in registers and no other memory is passed on, so it is relaxed: a
 // release at cluster scope costs a memory barrier per arrival).
-__device__ __forceinline__ void arrive_remote_relaxed(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
-               : "memory");
-}
 __device__ __forceinline__ void arrive_remote(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
                : "memory");
 }
 // TMA tile load into this CTA's shared memory whose completion is counted on a barrier of
@@ -109,26 +105,7 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t a) {
   return (uint64_t)((a >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// Arrive on the barrier at this offset in both CTAs of the pair once the pair's MMAs issued
-// so far have completed.
-__device__ __forceinline__ void commit_pair(uint64_t* b) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(s32(b)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-// D[256 x N] (+)= A[256 x 16] B[16 x N] over a CTA pair: rows 0-127 of A and D in the
-// even CTA (the issuer), rows 128-255 in the odd one; B's first N/2 rows (K-major) in the
-// even CTA, the rest in the odd one, at the same shared-memory offsets.
-__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-// The forms for an issuing WARP: every lane runs the loop and the instruction is predicated on
+// The issuing WARP runs its loop with every lane and the instructions below are predicated on
 // one lane (leader: elect_lane() there), so that descriptors and addresses stay in uniform
 // registers.  Under a lane-0 branch each MMA cost the issuer ~100 cycles.
 __device__ __forceinline__ uint32_t elect_lane() {
@@ -136,7 +113,9 @@ __device__ __forceinline__ uint32_t elect_lane() {
   asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void commit_pair_w(uint64_t* b, uint32_t leader) {
+// Arrive on the barrier at this offset in both CTAs of the pair once the pair's MMAs issued
+// so far have completed.
+__device__ __forceinline__ void commit_pair(uint64_t* b, uint32_t leader) {
   asm volatile(
       "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %2, 0;\n\t"
       "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
@@ -144,7 +123,10 @@ __device__ __forceinline__ void commit_pair_w(uint64_t* b, uint32_t leader) {
       "h"((uint16_t)3), "r"(leader)
       : "memory");
 }
-__device__ __forceinline__ void mma_pair_w(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc,
+// D[256 x N] (+)= A[256 x 16] B[16 x N] over a CTA pair: rows 0-127 of A and D in the
+// even CTA (the issuer), rows 128-255 in the odd one; B's first N/2 rows (K-major) in the
+// even CTA, the rest in the odd one, at the same shared-memory offsets.
+__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc,
                                            uint32_t leader) {
   asm volatile(
       "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
