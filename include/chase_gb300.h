@@ -258,8 +258,8 @@ int chase_qr(chase_handle h, chase_dtype dtype, int n, int ncols, void* dX, int 
  *                   that precision).
  * The Cholesky factor, its inverse and the Householder fallback stay FP64.
  * Other precisions return -9.  In the emulated mode the workspace grows by the
- * products' residue planes, residues and FP64 staging: about 450 n ncols bytes
- * (complex) or 150 n ncols bytes (real).
+ * products' residue planes and residues: about 240 n ncols bytes (complex) or 150 n ncols
+ * bytes (real).
  */
 int chase_qr_prec(chase_handle h, chase_dtype dtype, int n, int ncols, void* dX, int ldx,
                   double est_cond, int qr_force, chase_precision prec, int* variant_used,

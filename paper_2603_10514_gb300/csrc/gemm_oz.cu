@@ -807,17 +807,23 @@ __device__ __forceinline__ double crt_value(const uint8_t* __restrict__ R, size_
   return crt_combine(rj, shift_out);
 }
 
+// x 2^E with |x| in [2^63, 2^64]: one exact multiply by the power of two 2^E built from its
+// exponent field when that is a normal number (ldexp otherwise).
+__device__ __forceinline__ double crt_scale(double x, int E) {
+  return (E > -1022 && E < 1024) ? x * __longlong_as_double((long long)(E + 1023) << 52) : ldexp(x, E);
+}
+__device__ __forceinline__ void crt_store_z(double re, int sre, double im, int sim, int e, z64* out, int sub) {
+  z64 v{crt_scale(re, sre + e - 2 * OZ_KBITS), crt_scale(im, sim + e - 2 * OZ_KBITS)};
+  if (sub) v = z64{out->x - v.x, out->y - v.y};
+  *out = v;
+}
 // The epilogue of one reconstructed entry: v = alpha 2^E x + beta X64 + gamma Z64.
 __device__ __forceinline__ void crt_store(double x, int sh, int r, int c, const int* __restrict__ rowexp,
                                           const int* __restrict__ colexp, int col0, double alpha,
                                           double beta, const double* X64, double gamma,
                                           const double* Z64, double* out64, int ldo, int er = -1) {
-  // x 2^E with |x| in [2^63, 2^64]: one exact multiply by the power of two 2^E built from
-  // its exponent field when that is a normal number (ldexp otherwise); er: the row whose
-  // exponent scales the entry (r by default)
-  const int E = sh + rowexp[er < 0 ? r : er] + colexp[col0 + c] - 2 * OZ_KBITS;
-  const double v0 = (E > -1022 && E < 1024) ? x * __longlong_as_double((long long)(E + 1023) << 52)
-                                            : ldexp(x, E);
+  // er: the row whose exponent scales the entry (r by default)
+  const double v0 = crt_scale(x, sh + rowexp[er < 0 ? r : er] + colexp[col0 + c] - 2 * OZ_KBITS);
   const size_t idx = (size_t)r + (size_t)(col0 + c) * ldo;
   double v = alpha * v0;
   if (beta != 0.0) v = fma(beta, X64[idx], v);
@@ -904,7 +910,7 @@ __global__ void __launch_bounds__(256) crt_ring_kernel(int n, int N, const uint1
                                                        const int* __restrict__ colexp, int col0,
                                                        double alpha, double beta, const double* X64,
                                                        double gamma, const double* Z64, double* out64,
-                                                       int ldo) {
+                                                       int ldo, z64* zout, int zsub) {
   const size_t total = (size_t)n * N, quads = total / 4;
   const uint2* R4 = (const uint2*)R;
   const size_t stride4 = total / 4, set4 = (size_t)NM * stride4;
@@ -929,6 +935,10 @@ __global__ void __launch_bounds__(256) crt_ring_kernel(int n, int N, const uint1
       double re, im;
       int sre, sim;
       ring_combine<NM>(u, w, &re, &sre, &im, &sim);
+      if (zout) {
+        crt_store_z(re, sre, im, sim, rowexp[r] + colexp[col0 + c], zout + (size_t)r + (size_t)(col0 + c) * ldo, zsub);
+        continue;
+      }
       crt_store(re, sre, r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo);
       crt_store(im, sim, n + r, c, rowexp, colexp, col0, alpha, beta, X64, gamma, Z64, out64, ldo, r);
     }
@@ -946,6 +956,8 @@ struct CrtGroupParams {
   long long out0[kOzGroupMax + 1];  // first output index of each problem
   int M[kOzGroupMax], N[kOzGroupMax], col0[kOzGroupMax], ldo[kOzGroupMax];
   int ring[kOzGroupMax];  // ring moduli (0: a real problem): M = n, residues of U | W, stacked output
+  z64* zout[kOzGroupMax]; // complex output instead of the stacked one
+  int zsub[kOzGroupMax];
   int count;
 };
 static_assert(sizeof(CrtGroupParams) <= 32000, "kernel parameter space");
@@ -964,6 +976,11 @@ __device__ __forceinline__ void crt_ring_entry(const CrtGroupParams& P, int p, l
   double re, im;
   int sre, sim;
   ring_combine<NM>(ru, rw, &re, &sre, &im, &sim);
+  if (P.zout[p]) {
+    crt_store_z(re, sre, im, sim, P.rowexp[p][r] + P.colexp[p][P.col0[p] + c],
+                P.zout[p] + (size_t)r + (size_t)(P.col0[p] + c) * P.ldo[p], P.zsub[p]);
+    return;
+  }
   crt_store(re, sre, r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
             P.gamma[p], P.Z64[p], P.out64[p], P.ldo[p]);
   crt_store(im, sim, M + r, c, P.rowexp[p], P.colexp[p], P.col0[p], P.alpha[p], P.beta[p], P.X64[p],
@@ -990,9 +1007,7 @@ __global__ void __launch_bounds__(256) crt_group_kernel(const __grid_constant__ 
     }
     int sh;
     const double x = crt_value((const uint8_t*)P.R[p], (size_t)M * P.N[p], (size_t)u, 1, &sh);
-    const int E = sh + P.rowexp[p][r] + P.colexp[p][P.col0[p] + c] - 2 * OZ_KBITS;
-    const double v0 = (E > -1022 && E < 1024) ? x * __longlong_as_double((long long)(E + 1023) << 52)
-                                              : ldexp(x, E);
+    const double v0 = crt_scale(x, sh + P.rowexp[p][r] + P.colexp[p][P.col0[p] + c] - 2 * OZ_KBITS);
     const size_t idx = (size_t)r + (size_t)(P.col0[p] + c) * P.ldo[p];
     double v = P.alpha[p] * v0;
     if (P.beta[p] != 0.0) v = fma(P.beta[p], P.X64[p][idx], v);
@@ -1287,108 +1302,122 @@ __global__ void stack_V_kernel(int n, int ncols, const T* __restrict__ V, int ld
   }
 }
 
-// Xt (l x n, ld ldt) is the transpose of a column-major X (n x l): row m of X is column m
-// of Xt.  Residues of the rows of the stacked operator [[Xr, -Xi], [Xi, Xr]] (2n x 2l;
-// real: X itself, n x l) into planes (row-major, ld kp), row exponents into rowexp.
-template <class T>
-__global__ void __launch_bounds__(256) oz_slice_rows_kernel(int n, int l, const T* __restrict__ Xt,
-                                                            int ldt, int kp, __nv_bfloat16* planes,
-                                                            size_t plane, int* rowexp) {
+// Column blockIdx.x of a complex block Y (n x q, ld ldy): its exponent (over Re and Im) and its
+// two plane rows (u | w), ld kp; entries past n are zero.
+template <int NM>
+__global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z64* __restrict__ Y, int ldy, int kp,
+                                                                 __nv_bfloat16* planes, size_t plane,
+                                                                 int* colexp) {
+  __shared__ unsigned long long red[8];
+  const int c = blockIdx.x;
+  const z64* col = Y + (size_t)c * ldy;
+  unsigned long long amax = 0;
+  for (int k = threadIdx.x; k < n; k += 256) {
+    const unsigned long long b = max(abs_bits(col[k].x), abs_bits(col[k].y));
+    amax = b > amax ? b : amax;
+  }
+  const int e = exp_bound(block_max(amax, red));
+  if (threadIdx.x == 0) colexp[c] = e;
+  for (int k = 4 * threadIdx.x; k < kp; k += 1024) {
+    long long xr[4], xi[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      const z64 a = (k + d < n) ? col[k + d] : z64{0.0, 0.0};
+      xr[d] = oz_int(a.x, e);
+      xi[d] = oz_int(a.y, e);
+    }
+    write_ring4<NM>(xr, xi, planes, (size_t)c * kp + k, plane);
+  }
+}
+
+// Row exponents (over Re and Im) of a column-major complex X (n x l): 32 rows per CTA, eight
+// column groups.
+__global__ void __launch_bounds__(256) oz_row_exp_kernel(int n, int l, const z64* __restrict__ X, int ldx,
+                                                         int* rowexp) {
+  __shared__ unsigned long long red[8][32];
+  const int i = threadIdx.x & 31, g = threadIdx.x >> 5, r = blockIdx.x * 32 + i;
+  unsigned long long m = 0;
+  if (r < n)
+    for (int k = g; k < l; k += 8) {
+      const z64 a = X[(size_t)r + (size_t)k * ldx];
+      const unsigned long long b = max(abs_bits(a.x), abs_bits(a.y));
+      m = b > m ? b : m;
+    }
+  red[g][i] = m;
+  __syncthreads();
+  if (g == 0 && r < n) {
+    for (int j = 1; j < 8; ++j) m = red[j][i] > m ? red[j][i] : m;
+    rowexp[r] = exp_bound(m);
+  }
+}
+
+// Rows of a column-major complex X (n x l) as plane rows (u | w, ld kp, K contiguous): 32 rows
+// x 64 of K per CTA through shared memory, so that X is read along its columns and the planes
+// are written along K.
+template <int NM>
+__global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, const z64* __restrict__ X, int ldx,
+                                                                 int kp, __nv_bfloat16* planes, size_t plane,
+                                                                 const int* __restrict__ rowexp) {
+  __shared__ z64 tile[64][33];
+  const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
+  const int i = threadIdx.x & 31, g = threadIdx.x >> 5;
+  for (int k = g; k < 64; k += 8)
+    tile[k][i] = (r0 + i < n && k0 + k < l) ? X[(size_t)(r0 + i) + (size_t)(k0 + k) * ldx] : z64{0.0, 0.0};
+  __syncthreads();
+  for (int t = threadIdx.x; t < 512; t += 256) {
+    const int row = t >> 4, k = 4 * (t & 15);
+    if (r0 + row >= n) continue;
+    const int e = rowexp[r0 + row];
+    long long xr[4], xi[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      const z64 a = tile[k + d][row];
+      xr[d] = oz_int(a.x, e);
+      xi[d] = oz_int(a.y, e);
+    }
+    write_ring4<NM>(xr, xi, planes, (size_t)(r0 + row) * kp + k0 + k, plane);
+  }
+}
+
+// Xt (l x n, ld ldt) is the transpose of a real column-major X (n x l): row m of X is column m
+// of Xt.  Residues of the rows into planes (row-major, ld kp), row exponents into rowexp.
+__global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double* __restrict__ Xt, int ldt, int kp,
+                                                            __nv_bfloat16* planes, size_t plane, int* rowexp) {
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
-  const int mm = Sc<T>::cplx ? (m % n) : m;
-  const bool mre = !Sc<T>::cplx || m < n;
-  const int K = Sc<T>::cplx ? 2 * l : l;
-  const T* row = Xt + (size_t)mm * ldt;  // X[mm, 0..l)
-  auto elem = [&](int k) -> double {
-    if constexpr (Sc<T>::cplx) {
-      const z64 x = row[k % l];
-      const bool kre = k < l;
-      // [[Xr, -Xi], [Xi, Xr]]
-      return mre ? (kre ? x.x : -x.y) : (kre ? x.y : x.x);
-    } else {
-      return row[k];
-    }
-  };
+  const double* row = Xt + (size_t)m * ldt;  // X[m, 0..l)
   unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < K; k += 256) {
-    const unsigned long long b = abs_bits(elem(k));
+  for (int k = threadIdx.x; k < l; k += 256) {
+    const unsigned long long b = abs_bits(row[k]);
     amax = b > amax ? b : amax;
   }
   const int e = exp_bound(block_max(amax, red));
   if (threadIdx.x == 0) rowexp[m] = e;
-  for (int k = threadIdx.x; k < kp; k += 256) {
-    const double x = (k < K) ? elem(k) : 0.0;
-    write_residues(x, e, planes, (size_t)m * kp + k, plane);
-  }
+  for (int k = threadIdx.x; k < kp; k += 256)
+    write_residues(k < l ? row[k] : 0.0, e, planes, (size_t)m * kp + k, plane);
 }
 
-// Residues of the columns of a block Y (n x q, ld ldy) in stacked form: plane column j < q
-// holds [Re Y; Im Y][:, j]; with `pair` (complex only) plane column q + j holds the stacked
-// -i Y[:, j] = [Im Y; -Re Y][:, j].  Then, with X's columns as the left operand's rows,
-// Xhat^T [Yhat | stack(-i Y)] = [Re(X^H Y) | Im(X^H Y)].  Both columns of a pair share the
-// exponent of Y[:, j].  Planes column-major (ld kp; rows >= M are zero).
-template <class T>
-__global__ void __launch_bounds__(512) oz_slice_cols_kernel(int n, int q, const T* __restrict__ Y,
-                                                            int ldy, int kp, bool pair,
-                                                            __nv_bfloat16* planes, size_t plane,
-                                                            int* colexp) {
+// Residues of the columns of a real block Y (n x q, ld ldy): planes column-major (ld kp; rows
+// >= n are zero), column exponents.
+__global__ void __launch_bounds__(512) oz_slice_cols_kernel(int n, const double* __restrict__ Y, int ldy, int kp,
+                                                            __nv_bfloat16* planes, size_t plane, int* colexp) {
   __shared__ unsigned long long red[16];
   const int j = blockIdx.x;
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  const T* col = Y + (size_t)j * ldy;
+  const double* col = Y + (size_t)j * ldy;
   unsigned long long amax = 0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    unsigned long long b;
-    if constexpr (Sc<T>::cplx) {
-      const unsigned long long b0 = abs_bits(col[i].x), b1 = abs_bits(col[i].y);
-      b = b0 > b1 ? b0 : b1;
-    } else {
-      b = abs_bits(col[i]);
-    }
+    const unsigned long long b = abs_bits(col[i]);
     amax = b > amax ? b : amax;
   }
   const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) {
-    colexp[j] = e;
-    if (pair) colexp[q + j] = e;
-  }
-  for (int k = threadIdx.x; k < kp; k += blockDim.x) {
-    double x = 0.0, y = 0.0;
-    if (k < M) {
-      if constexpr (Sc<T>::cplx) {
-        const z64 v = col[k % n];
-        x = (k < n) ? v.x : v.y;
-        y = (k < n) ? v.y : -v.x;
-      } else {
-        x = col[k];
-      }
-    }
-    write_residues(x, e, planes, (size_t)j * kp + k, plane);
-    if (pair) write_residues(y, e, planes, (size_t)(q + j) * kp + k, plane);
-  }
+  if (threadIdx.x == 0) colexp[j] = e;
+  for (int k = threadIdx.x; k < kp; k += blockDim.x)
+    write_residues(k < n ? col[k] : 0.0, e, planes, (size_t)j * kp + k, plane);
 }
 
-// out (l x 2l FP64, ld ldo) -> G (l x l, ld ldg) with G = out[:, :l] + i out[:, l:] (real: copy)
-template <class T>
-__global__ void gram_assemble_kernel(int qx, int qy, const double* __restrict__ out, int ldo, T* G,
-                                     int ldg) {
-  const size_t total = (size_t)qx * qy;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
-       t += (size_t)gridDim.x * blockDim.x) {
-    const int p = (int)(t % qx), q = (int)(t / qx);
-    if constexpr (Sc<T>::cplx) {
-      G[(size_t)p + (size_t)q * ldg] = z64{out[(size_t)p + (size_t)q * ldo], out[(size_t)p + (size_t)(q + qy) * ldo]};
-    } else {
-      G[(size_t)p + (size_t)q * ldg] = out[(size_t)p + (size_t)q * ldo];
-    }
-  }
-}
-
-// Xt = X^T (plain transpose, no conjugation): X n x l (ld ldx) -> Xt l x n (ld ldt).
-template <class T>
-__global__ void transpose_kernel(int n, int l, const T* __restrict__ X, int ldx, T* Xt, int ldt) {
-  __shared__ T tile[32][33];
+// Xt = X^T: real X n x l (ld ldx) -> Xt l x n (ld ldt).
+__global__ void transpose_kernel(int n, int l, const double* __restrict__ X, int ldx, double* Xt, int ldt) {
+  __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
     const int i = i0 + threadIdx.x, j = j0 + r;
@@ -1626,7 +1655,86 @@ int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* 
   return 0;
 }
 
-int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatus* dst, int* launches) {
+namespace {
+
+// Appends the modular products of one item (its one or two plane sets) to a grouped launch.
+int ozm_append(OzmGroupParams& P, int& tiles, const OzGroupItem& it, int bn_max) {
+  const int sets = it.ring ? 2 : 1;  // ring products: U, W
+  const int nm = it.ring ? ring_moduli(it.kp) : kOzModuli;
+  const int ntile = ceil_div(it.N, std::min(bn_max, MBN_MAX));
+  const int BN = ceil_div(ceil_div(it.N, ntile), 16) * 16;
+  const int rows = std::max(it.a_plane_rows, it.M);
+  const size_t rset = (size_t)nm * (it.ring ? 2 : 1) * it.M * it.N;  // residue bytes of one set
+  const size_t aset = (size_t)nm * rows * it.kp * 2;                 // bytes of one A plane set
+  const size_t vset = (size_t)nm * it.ncols_total * it.kp * 2;       // of one V plane set
+  if (sets * rset > it.resbuf.bytes) return CHASE_ERR_OOM;
+  for (int sidx = 0; sidx < sets; ++sidx) {
+    const int p = P.count++;
+    if (make_map3(&P.mapA[p], (const char*)it.Aplanes + (sidx ^ it.aswap) * aset, it.kp, it.M, rows, MBM, nm) ||
+        make_map3(&P.mapV[p], (const char*)it.Vplanes + sidx * vset, it.kp, it.ncols_total,
+                  it.ncols_total, tile_shape(BN).h0 / 2, nm))
+      return CHASE_ERR_CUDA;
+    P.R[p] = (char*)it.resbuf.ptr + sidx * rset;
+    P.ring[p] = it.ring ? nm : 0;
+    P.tile0[p] = tiles;
+    P.M[p] = it.M;
+    P.N[p] = it.N;
+    P.BN[p] = BN;
+    P.col0[p] = it.col0;
+    P.ntile[p] = ntile;
+    P.nkb[p] = it.kp / MBK;
+    tiles += ntile * ceil_div(it.M, 2 * MBM) * 2;  // CTA pairs over 256-row blocks
+  }
+  return 0;
+}
+
+int ozm_launch_group(cudaStream_t st, OzmGroupParams& P, int tiles, DevStatus* dst, int* launches) {
+  P.tile0[P.count] = tiles;
+  int planes = 0;  // moduli of the longest set in the launch
+  for (int p = 0; p < P.count; ++p) planes = std::max(planes, P.ring[p] ? P.ring[p] : kOzModuli);
+  TRY_OZ(launch_pairs(ozm_group_kernel, dim3(tiles, 1, planes), st, P, dst));
+  if (launches) ++*launches;
+  return 0;
+}
+
+// Times one item's modular products with every candidate tile width (they read only the
+// residue planes and all yield the same exact residues) and records the fastest.
+int tune_group_item(cudaStream_t st, const OzGroupItem& it, DevStatus* dst, int* launches, int* trials) {
+  OzPlan cand[6];
+  const int all = oz_plan_candidates(it.N, cand, 6);
+  int nc = 0;
+  for (int i = 0; i < all; ++i)
+    if (cand[i].splits == 1) cand[nc++] = cand[i];  // K is not split in a grouped launch
+  cudaEvent_t ev[7];
+  for (int i = 0; i <= nc; ++i) CHASE_CUDA_TRY(cudaEventCreate(&ev[i]));
+  int rc = 0;
+  cudaEventRecord(ev[0], st);
+  for (int i = 0; i < nc && !rc; ++i) {
+    OzmGroupParams P{};
+    int tiles = 0;
+    rc = ozm_append(P, tiles, it, cand[i].bn_max);
+    if (!rc) rc = ozm_launch_group(st, P, tiles, dst, launches);
+    cudaEventRecord(ev[i + 1], st);
+  }
+  if (!rc && cudaEventSynchronize(ev[nc]) == cudaSuccess) {
+    int best = 0;
+    float tbest = 1e30f;
+    for (int i = 0; i < nc; ++i) {
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, ev[i], ev[i + 1]);
+      if (ms < tbest) { tbest = ms; best = i; }
+    }
+    oz_plan_store(it.M, it.N, it.kp, cand[best], tbest * 1e-3);
+    if (trials) *trials += nc;
+  }
+  for (int i = 0; i <= nc; ++i) cudaEventDestroy(ev[i]);
+  return rc;
+}
+
+}  // namespace
+
+int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatus* dst, int* launches, int tune,
+                  int* trials) {
   CHASE_CUDA_TRY(cudaFuncSetAttribute(ozm_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M_SMEM));
   OzmGroupParams P{};
   CrtGroupParams C{};
@@ -1635,18 +1743,14 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
   // one launch of the modular products and one of the reconstructions for what is gathered
   auto flush = [&]() -> int {
     if (P.count == 0) return 0;
-    P.tile0[P.count] = tiles;
+    TRY_OZ(ozm_launch_group(st, P, tiles, dst, launches));
     C.out0[C.count] = outs;
-    int planes = 0;  // moduli of the longest set in the launch
-    for (int p = 0; p < P.count; ++p) planes = std::max(planes, P.ring[p] ? P.ring[p] : kOzModuli);
-    TRY_OZ(launch_pairs(ozm_group_kernel, dim3(tiles, 1, planes), st, P, dst));
-    if (launches) ++*launches;
     if (C.count == 1 && C.ring[0] && outs % 4 == 0) {  // one complex problem: the vector form
       const int b4 = (int)std::max<long long>(1, std::min<long long>((outs / 4 + 255) / 256, (long long)kNumSMs * 16));
       auto kern = C.ring[0] == kRingShort ? crt_ring_kernel<kRingShort> : crt_ring_kernel<kRingModuli>;
       kern<<<b4, 256, 0, st>>>(C.M[0], C.N[0], (const uint16_t*)C.R[0], C.rowexp[0], C.colexp[0],
                                C.col0[0], C.alpha[0], C.beta[0], C.X64[0], C.gamma[0], C.Z64[0],
-                               C.out64[0], C.ldo[0]);
+                               C.out64[0], C.ldo[0], C.zout[0], C.zsub[0]);
     } else {
       const int blocks = (int)std::max<long long>(1, std::min<long long>((outs + 255) / 256, (long long)kNumSMs * 16));
       crt_group_kernel<<<blocks, 256, 0, st>>>(C);
@@ -1663,35 +1767,16 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     const OzGroupItem& it = items[i];
     if (it.N <= 0 || it.M <= 0) continue;
     if (it.kp % MBK != 0 || it.kp > kOzSplitMaxK) return CHASE_ERR_UNSUPPORTED;  // K is not split here
-    const int sets = it.ring ? 2 : 1;  // ring products: U, W
-    const int nm = it.ring ? ring_moduli(it.kp) : kOzModuli;
-    const size_t rset = (size_t)nm * (it.ring ? 2 : 1) * it.M * it.N;  // residue bytes of one set
-    if (sets * rset > it.resbuf.bytes) return CHASE_ERR_OOM;
-    if (P.count + sets > kOzGroupMax || C.count + 1 > kOzGroupMax) TRY_OZ(flush());
+    if (P.count + (it.ring ? 2 : 1) > kOzGroupMax || C.count + 1 > kOzGroupMax) TRY_OZ(flush());
     OzPlan plan;  // the autotuner's tile width for this shape, if it measured one
-    oz_plan_lookup(it.M, it.N, it.kp, &plan);
-    const int ntile = ceil_div(it.N, std::min(plan.bn_max, MBN_MAX));
-    const int BN = ceil_div(ceil_div(it.N, ntile), 16) * 16;
-    const int rows = std::max(it.a_plane_rows, it.M);
-    const size_t aset = (size_t)nm * rows * it.kp * 2;             // bytes of one A plane set
-    const size_t vset = (size_t)nm * it.ncols_total * it.kp * 2;   // of one V plane set
-    for (int sidx = 0; sidx < sets; ++sidx) {
-      const int p = P.count++;
-      if (make_map3(&P.mapA[p], (const char*)it.Aplanes + sidx * aset, it.kp, it.M, rows, MBM, nm) ||
-          make_map3(&P.mapV[p], (const char*)it.Vplanes + sidx * vset, it.kp, it.ncols_total,
-                    it.ncols_total, tile_shape(BN).h0 / 2, nm))
-        return CHASE_ERR_CUDA;
-      P.R[p] = (char*)it.resbuf.ptr + sidx * rset;
-      P.ring[p] = it.ring ? nm : 0;
-      P.tile0[p] = tiles;
-      P.M[p] = it.M;
-      P.N[p] = it.N;
-      P.BN[p] = BN;
-      P.col0[p] = it.col0;
-      P.ntile[p] = ntile;
-      P.nkb[p] = it.kp / MBK;
-      tiles += ntile * ceil_div(it.M, 2 * MBM) * 2;  // CTA pairs over 256-row blocks
+    bool known = oz_plan_lookup(it.M, it.N, it.kp, &plan);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (tune && !known && count == 1 && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
+        cs == cudaStreamCaptureStatusNone) {
+      TRY_OZ(tune_group_item(st, it, dst, launches, trials));
+      oz_plan_lookup(it.M, it.N, it.kp, &plan);
     }
+    TRY_OZ(ozm_append(P, tiles, it, plan.bn_max));
     const int c = C.count++;
     C.R[c] = it.resbuf.ptr;
     C.rowexp[c] = it.rowexp;
@@ -1707,7 +1792,9 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     C.N[c] = it.N;
     C.col0[c] = it.col0;
     C.ldo[c] = it.ldo;
-    C.ring[c] = it.ring ? nm : 0;
+    C.ring[c] = it.ring ? ring_moduli(it.kp) : 0;
+    C.zout[c] = it.zout;
+    C.zsub[c] = it.zsub;
     outs += (long long)it.M * it.N;
   }
   return flush();
@@ -1726,60 +1813,45 @@ int oz_stack_V(cudaStream_t st, int n, int ncols, const T* V, int ldv, double* V
   return 0;
 }
 
-template <class T>
-int oz_slice_rows(cudaStream_t st, int n, int l, const T* Xt, int ldt, int kp, void* planes,
-                  int* rowexp, int* launches) {
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  oz_slice_rows_kernel<T><<<M, 256, 0, st>>>(n, l, Xt, ldt, kp, (__nv_bfloat16*)planes,
-                                             (size_t)M * kp, rowexp);
-  if (launches) ++*launches;
-  CHASE_CUDA_TRY(cudaGetLastError());
-  return 0;
-}
-
-template <class T>
-int oz_slice_cols(cudaStream_t st, int n, int q, const T* Y, int ldy, int kp, bool pair,
-                  void* planes, int* colexp, int* launches) {
+int oz_slice_cols_ring(cudaStream_t st, int n, int q, const z64* Y, int ldy, int kp, void* planes, int* colexp,
+                       int* launches) {
   if (q <= 0) return 0;
-  pair = pair && Sc<T>::cplx;
-  const size_t ncols_total = pair ? 2 * (size_t)q : (size_t)q;
-  oz_slice_cols_kernel<T><<<q, 512, 0, st>>>(n, q, Y, ldy, kp, pair, (__nv_bfloat16*)planes,
-                                             ncols_total * kp, colexp);
+  auto kern = ring_moduli(kp) == kRingShort ? oz_slice_cols_ring_kernel<kRingShort> : oz_slice_cols_ring_kernel<kRingModuli>;
+  kern<<<q, 256, 0, st>>>(n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
 }
 
-template <class T>
-int oz_gram_assemble(cudaStream_t st, int qx, int qy, const double* out, int ldo, T* G, int ldg,
-                     int* launches) {
-  const size_t work = (size_t)qx * qy;
-  if (work == 0) return 0;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((work + 255) / 256, (size_t)kNumSMs * 16));
-  gram_assemble_kernel<T><<<blocks, 256, 0, st>>>(qx, qy, out, ldo, G, ldg);
-  if (launches) ++*launches;
+int oz_slice_rows_ring(cudaStream_t st, int n, int l, const z64* X, int ldx, int kp, void* planes, int* rowexp,
+                       int* launches) {
+  if (n <= 0) return 0;
+  oz_row_exp_kernel<<<ceil_div(n, 32), 256, 0, st>>>(n, l, X, ldx, rowexp);
+  auto kern = ring_moduli(kp) == kRingShort ? oz_slice_rows_ring_kernel<kRingShort> : oz_slice_rows_ring_kernel<kRingModuli>;
+  kern<<<dim3(ceil_div(n, 32), kp / 64), 256, 0, st>>>(n, l, X, ldx, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  if (launches) *launches += 2;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
 }
 
-template <class T>
-int transpose(cudaStream_t st, int n, int l, const T* X, int ldx, T* Xt, int ldt, int* launches) {
-  dim3 grid(ceil_div(n, 32), ceil_div(l, 32)), block(32, 8);
-  transpose_kernel<T><<<grid, block, 0, st>>>(n, l, X, ldx, Xt, ldt);
-  if (launches) ++*launches;
+int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, double* Xt, int kp, void* planes,
+                  int* rowexp, int* launches) {
+  if (n <= 0) return 0;
+  transpose_kernel<<<dim3(ceil_div(n, 32), ceil_div(l, 32)), dim3(32, 8), 0, st>>>(n, l, X, ldx, Xt, l);
+  oz_slice_rows_kernel<<<n, 256, 0, st>>>(l, Xt, l, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  if (launches) *launches += 2;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
 }
 
-#define OZ_INST(T)                                                                                \
-  template int oz_slice_rows<T>(cudaStream_t, int, int, const T*, int, int, void*, int*, int*);   \
-  template int oz_slice_cols<T>(cudaStream_t, int, int, const T*, int, int, bool, void*, int*,   \
-                                int*);                                                            \
-  template int oz_gram_assemble<T>(cudaStream_t, int, int, const double*, int, T*, int, int*);    \
-  template int transpose<T>(cudaStream_t, int, int, const T*, int, T*, int, int*);
-OZ_INST(double)
-OZ_INST(z64)
-#undef OZ_INST
+int oz_slice_cols(cudaStream_t st, int n, int q, const double* Y, int ldy, int kp, void* planes, int* colexp,
+                  int* launches) {
+  if (q <= 0) return 0;
+  oz_slice_cols_kernel<<<q, 512, 0, st>>>(n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
+  if (launches) ++*launches;
+  CHASE_CUDA_TRY(cudaGetLastError());
+  return 0;
+}
 
 template int oz_stack_V<double>(cudaStream_t, int, int, const double*, int, double*, int, int*);
 template int oz_stack_V<z64>(cudaStream_t, int, int, const z64*, int, double*, int, int*);

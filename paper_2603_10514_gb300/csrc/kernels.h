@@ -150,22 +150,18 @@ int oz_slice_V(cudaStream_t st, int M, int c0, int c1, const double* V64, int ld
 template <class T>
 int oz_stack_V(cudaStream_t st, int n, int ncols, const T* V, int ldv, double* V64, int ldo,
                int* launches);
-// Row residues of the stacked operator of a general X given as Xt = X^T (l x n, ld ldt).
-template <class T>
-int oz_slice_rows(cudaStream_t st, int n, int l, const T* Xt, int ldt, int kp, void* planes,
+// Operands of the QR's and Rayleigh-Ritz's products: columns of a block Y (n x q) and rows of a
+// tall X (n x l) as residue planes; ring residues (u | w) for complex ones.  The plane rows of
+// X^H are the columns of X with u and w exchanged (OzGroupItem::aswap).
+int oz_slice_cols_ring(cudaStream_t st, int n, int q, const z64* Y, int ldy, int kp, void* planes, int* colexp,
+                       int* launches);
+int oz_slice_rows_ring(cudaStream_t st, int n, int l, const z64* X, int ldx, int kp, void* planes, int* rowexp,
+                       int* launches);
+int oz_slice_cols(cudaStream_t st, int n, int q, const double* Y, int ldy, int kp, void* planes, int* colexp,
+                  int* launches);
+// (through Xt = X^T, l x n)
+int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, double* Xt, int kp, void* planes,
                   int* rowexp, int* launches);
-// Column residues of a block Y (n x q): plane column j = stacked Y[:, j] and, with pair
-// (complex only), plane column q + j = stacked (-i Y[:, j]); plane stride (q or 2q) * kp.
-template <class T>
-int oz_slice_cols(cudaStream_t st, int n, int q, const T* Y, int ldy, int kp, bool pair,
-                  void* planes, int* colexp, int* launches);
-// G = out[:, :qy] + i out[:, qy:] (complex) or out (real); out qx x 2qy (or qx x qy), ld ldo;
-// G qx x qy.
-template <class T>
-int oz_gram_assemble(cudaStream_t st, int qx, int qy, const double* out, int ldo, T* G, int ldg,
-                     int* launches);
-template <class T>
-int transpose(cudaStream_t st, int n, int l, const T* X, int ldx, T* Xt, int ldt, int* launches);
 // Launch plan of an emulated product: cap on the column-tile width (tiles as even as
 // possible below it) and K splits (0: about four waves of CTAs, at most kOzMaxSplits).
 struct OzPlan {
@@ -210,9 +206,14 @@ struct OzGroupItem {
   // complex problem in ring residues: M = n, Aplanes / Vplanes hold two plane sets (u | w),
   // V64_in / X64 / Z64 / out64 are the stacked [Re; Im] blocks
   int ring = 0;
+  int aswap = 0;        // ring: the left operand's u and w sets are exchanged (its conjugate)
+  z64* zout = nullptr;  // ring: plain product to a complex block (ld ldo) instead of the update
+  int zsub = 0;         // and subtracted from it
 };
 int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* launches);
-int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatus* dst, int* launches);
+// tune, trials: as oz_gemm (one item only).
+int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatus* dst, int* launches,
+                  int tune = 0, int* trials = nullptr);
 
 // ---- failure path of the bounded device waits (selftest.cu) ----------------
 // One thread waits (at most `seconds`) on an mbarrier nothing arrives on and sets

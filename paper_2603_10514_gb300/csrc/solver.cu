@@ -539,104 +539,120 @@ int filter_oz_graph(chase_ctx* h, int n, const T* A, int lda, bool split_A, int 
 
 // AQ = A Q (n x nu, both ld n) by the Ozaki-scheme product; A's planes must be ready.
 template <class T>
-int aq_oz(chase_ctx* h, int n, const T* Q, int nu, T* AQ, OzBufs& B, Scratch scr) {
+int aq_oz(chase_ctx* h, int n, const T* Q, int nu, T* AQ, OzBufs& B) {
   cudaStream_t st = h->stream;
   if (nu <= 0) return 0;
-  TRY(oz_stack_V<T>(st, n, nu, Q, n, B.V64[0], B.kp, &h->launches));
-  if (B.ring) {
-    const OzGroupItem it = oz_item(B, B.ncols, 0, nu, 1.0, 0.0, nullptr, 0.0, nullptr, B.V64[1], B.V64[0]);
-    TRY(oz_slice_V_group(st, 1, &it, &h->launches));
-    TRY(oz_gemm_group(st, 1, &it, h->dstat, &h->launches));
+  if constexpr (Sc<T>::cplx) {
+    TRY(oz_slice_cols_ring(st, n, nu, Q, n, B.kpn, B.Vp, B.colexp, &h->launches));
+    OzGroupItem it = oz_item(B, nu, 0, nu, 1.0, 0.0, nullptr, 0.0, nullptr, nullptr, nullptr);
+    it.zout = AQ;
+    it.ldo = n;
+    TRY(oz_gemm_group(st, 1, &it, h->dstat, &h->launches, h->autotune, &h->tune_trials));
   } else {
-    TRY(oz_slice_V(st, B.M, 0, nu, B.V64[0], B.kp, B.kp, B.ncols, B.Vp, B.colexp, &h->launches));
-    TRY(oz_gemm(st, B.M, B.kp, B.Ap, B.rowexp, 0, B.Vp, B.colexp, B.ncols, 0, nu, 1.0, 0.0, nullptr,
-                0.0, nullptr, B.V64[1], B.kp, h->dstat, B.res, &h->launches, h->autotune,
-                &h->tune_trials));
+    TRY(oz_slice_cols(st, n, nu, Q, n, B.kp, B.Vp, B.colexp, &h->launches));
+    TRY(oz_gemm(st, B.M, B.kp, B.Ap, B.rowexp, 0, B.Vp, B.colexp, nu, 0, nu, 1.0, 0.0, nullptr, 0.0, nullptr,
+                AQ, n, h->dstat, B.res, &h->launches, h->autotune, &h->tune_trials));
   }
-  TRY(tc_unstack_V<T>(st, n, 0, nu, B.V64[1], B.kp, AQ, n, &h->launches));
   return 0;
 }
 
 // ---------------------------------------------------------------------------
 // FP64-accurate products of the QR and Rayleigh-Ritz steps by the Ozaki scheme:
-//   Gram    G = X^H Y (l x l; X's columns are the left operand's rows, Y and
-//           -i Y the right operand's columns, K = n or 2n);
-//   tall    Y = X B  (X n x kl sliced by rows of its stacked operator
-//           [[Xr, -Xi], [Xi, Xr]], B kl x N stacked as [Br; Bi]).
+//   xhy     W = X^H Y (qx x qy, K = n; X's columns are the left operand's rows);
+//   tall    Y = X B  (X n x kl sliced by rows, B kl x N by columns).
+// Complex products run in split residue rings, straight to complex results.
 // ---------------------------------------------------------------------------
 struct OzProd {
-  int n = 0, l = 0, M = 0, kp = 0, kpl = 0;
-  void* Gp = nullptr;  int* gexp = nullptr;   // kp x 2l column planes (Y | -iY)
-  void* Lp = nullptr;  int* lexp = nullptr;   // kp x l column planes (X, when X != Y)
-  void* Rp = nullptr;  int* rexp = nullptr;   // M x kpl row planes of a tall X
-  void* Bp = nullptr;  int* bexp = nullptr;   // kpl x l column planes of a small factor
-  double* B64 = nullptr;                      // kpl x l stacked small factor
-  double* out = nullptr;                      // FP64 result staging, max(M, 2l) x l
-  void* Xt = nullptr;                         // X^T (l x n)
+  int n = 0, l = 0, kp = 0, kpl = 0;          // K of xhy and of tall, padded
+  void* Gp = nullptr;  int* gexp = nullptr;   // column planes of Y (kp x l)
+  void* Lp = nullptr;  int* lexp = nullptr;   // column planes of X, when X != Y
+  void* Rp = nullptr;  int* rexp = nullptr;   // row planes of a tall X (n x kpl)
+  void* Bp = nullptr;  int* bexp = nullptr;   // column planes of a small factor (kpl x l)
+  void* Xt = nullptr;                         // X^T (real: l x n)
+  double* out = nullptr;                      // real tall results before they are subtracted
   Scratch res{nullptr, 0};                    // residues of the modular products
 };
 
+// Bytes of planes per operand element of a product with K padded to kp.
 template <class T>
-size_t ozp_bytes(int n, int l) {
-  const int M = Sc<T>::cplx ? 2 * n : n;
-  const size_t kp = (size_t)tc_kpad(M);
-  const size_t kpl = (size_t)tc_kpad(Sc<T>::cplx ? 2 * l : l);
-  const size_t wl = Sc<T>::cplx ? 2 * (size_t)l : (size_t)l;
-  return align256(kOzPlaneBytes * kp * wl) + align256(4 * wl) + align256(kOzPlaneBytes * kp * l) + align256(4 * (size_t)l) +
-         align256(kOzPlaneBytes * (size_t)M * kpl) + align256(4 * (size_t)M) + align256(kOzPlaneBytes * kpl * l) +
-         align256(4 * (size_t)l) + align256(8 * kpl * l) +
-         align256(8 * std::max<size_t>(M, wl) * l) + align256(sizeof(T) * (size_t)n * l) +
-         align256(oz_residue_bytes((int)std::max<size_t>(M, wl), l));
-}
+size_t oz_plane_bytes(int kp) { return Sc<T>::cplx ? ring_plane_bytes(kp) : kOzPlaneBytes; }
 
 template <class T>
-OzProd ozp_carve(char* base, int n, int l) {
+OzProd ozp_carve(char* base, int n, int l, size_t* total = nullptr) {
   OzProd P;
   P.n = n; P.l = l;
-  P.M = Sc<T>::cplx ? 2 * n : n;
-  P.kp = tc_kpad(P.M);
-  P.kpl = tc_kpad(Sc<T>::cplx ? 2 * l : l);
-  const size_t wl = Sc<T>::cplx ? 2 * (size_t)l : (size_t)l;
+  P.kp = tc_kpad(n);
+  P.kpl = tc_kpad(l);
   size_t off = 0;
   auto take = [&](size_t b) { char* p = base + off; off += align256(b); return p; };
-  P.Gp = take(kOzPlaneBytes * (size_t)P.kp * wl);
-  P.gexp = (int*)take(4 * wl);
-  P.Lp = take(kOzPlaneBytes * (size_t)P.kp * l);
+  const size_t pb = oz_plane_bytes<T>(P.kp), pbl = oz_plane_bytes<T>(P.kpl);
+  P.Gp = take(pb * (size_t)P.kp * l);
+  P.gexp = (int*)take(4 * (size_t)l);
+  P.Lp = take(pb * (size_t)P.kp * l);
   P.lexp = (int*)take(4 * (size_t)l);
-  P.Rp = take(kOzPlaneBytes * (size_t)P.M * P.kpl);
-  P.rexp = (int*)take(4 * (size_t)P.M);
-  P.Bp = take(kOzPlaneBytes * (size_t)P.kpl * l);
+  P.Rp = take(pbl * (size_t)n * P.kpl);
+  P.rexp = (int*)take(4 * (size_t)n);
+  P.Bp = take(pbl * (size_t)P.kpl * l);
   P.bexp = (int*)take(4 * (size_t)l);
-  P.B64 = (double*)take(8 * (size_t)P.kpl * l);
-  P.out = (double*)take(8 * std::max<size_t>(P.M, wl) * l);
-  P.Xt = take(sizeof(T) * (size_t)n * l);
-  const size_t rb = oz_residue_bytes((int)std::max<size_t>(P.M, wl), l);
+  if (!Sc<T>::cplx) {
+    P.Xt = take(sizeof(T) * (size_t)n * l);
+    P.out = (double*)take(8 * (size_t)n * l);
+  }
+  const int m = std::max(n, l);
+  const size_t rb = Sc<T>::cplx ? std::max(ring_residue_bytes(n, P.kpl, l), ring_residue_bytes(l, P.kp, l))
+                                : oz_residue_bytes(m, l);
   P.res = Scratch{take(rb), rb};
+  if (total) *total = off;
   return P;
 }
 
-// G = X^H Y (q x q, ld ldg) for X, Y n x q; X == Y uses one slicing for both sides.
 template <class T>
-int oz_gram(chase_ctx* h, OzProd& P, int q, const T* X, int ldx, const T* Y, int ldy, T* G, int ldg,
-            Scratch scr) {
+size_t ozp_bytes(int n, int l) {
+  size_t b = 0;
+  ozp_carve<T>((char*)256, n, l, &b);  // (sizes only)
+  return b;
+}
+
+// W = X^H Y (qx x qy, ld ldw) for X n x qx and Y n x qy; X == Y uses one slicing for both sides.
+template <class T>
+int oz_xhy(chase_ctx* h, OzProd& P, int qx, const T* X, int ldx, int qy, const T* Y, int ldy, T* W, int ldw) {
   cudaStream_t st = h->stream;
-  if (q <= 0) return 0;
-  const bool cplx = Sc<T>::cplx;
-  const int wq = cplx ? 2 * q : q;
-  TRY(oz_slice_cols<T>(st, P.n, q, Y, ldy, P.kp, true, P.Gp, P.gexp, &h->launches));
-  const void* left = P.Gp;
-  const int* lexp = P.gexp;
-  int plane_rows = wq;
-  if (X != Y) {
-    TRY(oz_slice_cols<T>(st, P.n, q, X, ldx, P.kp, false, P.Lp, P.lexp, &h->launches));
-    left = P.Lp;
-    lexp = P.lexp;
-    plane_rows = q;
+  if (qx <= 0 || qy <= 0) return 0;
+  auto slice = [&](int q, const T* Z, int ldz, void* planes, int* exps) -> int {
+    if constexpr (Sc<T>::cplx) return oz_slice_cols_ring(st, P.n, q, Z, ldz, P.kp, planes, exps, &h->launches);
+    else return oz_slice_cols(st, P.n, q, Z, ldz, P.kp, planes, exps, &h->launches);
+  };
+  const bool same = X == Y && qx == qy && ldx == ldy;
+  TRY(slice(qy, Y, ldy, P.Gp, P.gexp));
+  if (!same) TRY(slice(qx, X, ldx, P.Lp, P.lexp));
+  const void* left = same ? P.Gp : P.Lp;
+  const int* lexp = same ? P.gexp : P.lexp;
+  if constexpr (Sc<T>::cplx) {
+    OzGroupItem it;
+    it.ring = 1;
+    it.aswap = 1;
+    it.M = qx;
+    it.kp = P.kp;
+    it.a_plane_rows = qx;
+    it.Aplanes = left;
+    it.rowexp = lexp;
+    it.Vplanes = P.Gp;
+    it.colexp = P.gexp;
+    it.ncols_total = it.N = qy;
+    it.zout = W;
+    it.ldo = ldw;
+    it.resbuf = P.res;
+    return oz_gemm_group(st, 1, &it, h->dstat, &h->launches, h->autotune, &h->tune_trials);
+  } else {
+    return oz_gemm(st, qx, P.kp, left, lexp, qx, P.Gp, P.gexp, qy, 0, qy, 1.0, 0.0, nullptr, 0.0, nullptr, W, ldw,
+                   h->dstat, P.res, &h->launches, h->autotune, &h->tune_trials);
   }
-  TRY(oz_gemm(st, q, P.kp, left, lexp, plane_rows, P.Gp, P.gexp, wq, 0, wq, 1.0, 0.0, nullptr, 0.0,
-              nullptr, P.out, q, h->dstat, P.res, &h->launches, h->autotune, &h->tune_trials));
-  TRY(oz_gram_assemble<T>(st, q, q, P.out, q, G, ldg, &h->launches));
-  return 0;
+}
+
+// G = X^H Y (q x q, ld ldg).
+template <class T>
+int oz_gram(chase_ctx* h, OzProd& P, int q, const T* X, int ldx, const T* Y, int ldy, T* G, int ldg) {
+  return oz_xhy<T>(h, P, q, X, ldx, q, Y, ldy, G, ldg);
 }
 
 // Residue planes of the small right factor B (kl x N, ld ldb) for oz_tall.  kpk: padded K of
@@ -644,44 +660,46 @@ int oz_gram(chase_ctx* h, OzProd& P, int q, const T* X, int ldx, const T* Y, int
 // that the modular products do not run over zero padding).
 template <class T>
 int oz_prep_factor(chase_ctx* h, OzProd& P, int kl, int N, const T* B, int ldb, int kpk = 0) {
-  cudaStream_t st = h->stream;
-  const int K = Sc<T>::cplx ? 2 * kl : kl;
   if (kpk <= 0) kpk = P.kpl;
-  TRY(oz_stack_V<T>(st, kl, N, B, ldb, P.B64, kpk, &h->launches));
-  TRY(oz_slice_V(st, K, 0, N, P.B64, kpk, kpk, N, P.Bp, P.bexp, &h->launches));
-  return 0;
+  if constexpr (Sc<T>::cplx)
+    return oz_slice_cols_ring(h->stream, kl, N, B, ldb, kpk, P.Bp, P.bexp, &h->launches);
+  else
+    return oz_slice_cols(h->stream, kl, N, B, ldb, kpk, P.Bp, P.bexp, &h->launches);
 }
 
 // Y = X B (n x N, ld ldy), or Y -= X B with subtract, with X n x kl (ld ldx) and B prepared
 // by oz_prep_factor with the same kpk.  Y may alias X: X is fully sliced before Y is written.
 template <class T>
-int oz_tall(chase_ctx* h, OzProd& P, int kl, const T* X, int ldx, int N, T* Y, int ldy, Scratch scr,
-            int kpk = 0, bool subtract = false) {
+int oz_tall(chase_ctx* h, OzProd& P, int kl, const T* X, int ldx, int N, T* Y, int ldy, int kpk = 0,
+            bool subtract = false) {
   cudaStream_t st = h->stream;
   if (N <= 0) return 0;
   if (kpk <= 0) kpk = P.kpl;
-  T* Xt = (T*)P.Xt;
-  TRY(transpose<T>(st, P.n, kl, X, ldx, Xt, kl, &h->launches));
-  TRY(oz_slice_rows<T>(st, P.n, kl, Xt, kl, kpk, P.Rp, P.rexp, &h->launches));
-  TRY(oz_gemm(st, P.M, kpk, P.Rp, P.rexp, 0, P.Bp, P.bexp, N, 0, N, 1.0, 0.0, nullptr, 0.0,
-              nullptr, P.out, P.M, h->dstat, P.res, &h->launches, h->autotune, &h->tune_trials));
-  TRY(tc_unstack_V<T>(st, P.n, 0, N, P.out, P.M, Y, ldy, &h->launches, subtract));
-  return 0;
-}
-
-// W = X^H Y (qx x qy, ld ldw) for X n x qx and Y n x qy (the rectangular form of oz_gram).
-template <class T>
-int oz_xhy(chase_ctx* h, OzProd& P, int qx, const T* X, int ldx, int qy, const T* Y, int ldy, T* W,
-           int ldw) {
-  cudaStream_t st = h->stream;
-  if (qx <= 0 || qy <= 0) return 0;
-  const int wqy = Sc<T>::cplx ? 2 * qy : qy;
-  TRY(oz_slice_cols<T>(st, P.n, qy, Y, ldy, P.kp, true, P.Gp, P.gexp, &h->launches));
-  TRY(oz_slice_cols<T>(st, P.n, qx, X, ldx, P.kp, false, P.Lp, P.lexp, &h->launches));
-  TRY(oz_gemm(st, qx, P.kp, P.Lp, P.lexp, qx, P.Gp, P.gexp, wqy, 0, wqy, 1.0, 0.0, nullptr, 0.0,
-              nullptr, P.out, qx, h->dstat, P.res, &h->launches, h->autotune, &h->tune_trials));
-  TRY(oz_gram_assemble<T>(st, qx, qy, P.out, qx, W, ldw, &h->launches));
-  return 0;
+  if constexpr (Sc<T>::cplx) {
+    TRY(oz_slice_rows_ring(st, P.n, kl, X, ldx, kpk, P.Rp, P.rexp, &h->launches));
+    OzGroupItem it;
+    it.ring = 1;
+    it.M = P.n;
+    it.kp = kpk;
+    it.a_plane_rows = P.n;
+    it.Aplanes = P.Rp;
+    it.rowexp = P.rexp;
+    it.Vplanes = P.Bp;
+    it.colexp = P.bexp;
+    it.ncols_total = it.N = N;
+    it.zout = Y;
+    it.zsub = subtract ? 1 : 0;
+    it.ldo = ldy;
+    it.resbuf = P.res;
+    return oz_gemm_group(st, 1, &it, h->dstat, &h->launches, h->autotune, &h->tune_trials);
+  } else {
+    TRY(oz_slice_rows(st, P.n, kl, X, ldx, (double*)P.Xt, kpk, P.Rp, P.rexp, &h->launches));
+    TRY(oz_gemm(st, P.n, kpk, P.Rp, P.rexp, 0, P.Bp, P.bexp, N, 0, N, 1.0, 0.0, nullptr, 0.0, nullptr,
+                subtract ? P.out : Y, subtract ? P.n : ldy, h->dstat, P.res, &h->launches, h->autotune,
+                &h->tune_trials));
+    if (subtract) TRY(tc_unstack_V<T>(st, P.n, 0, N, P.out, P.n, Y, ldy, &h->launches, true));
+    return 0;
+  }
 }
 
 // One CholeskyQR pass (Algorithm 2 body): X <- X R^{-1} with R = chol(X^H X [+ sI]).
@@ -692,7 +710,7 @@ int cholqr_pass(chase_ctx* h, int n, int l, T* X, int ldx, T* Xtmp, T* G, T* Ri,
                 Scratch scr, int* info, OzProd* oz) {
   cudaStream_t st = h->stream;
   if (oz)
-    TRY(oz_gram<T>(h, *oz, l, X, ldx, X, ldx, G, l, scr));
+    TRY(oz_gram<T>(h, *oz, l, X, ldx, X, ldx, G, l));
   else
     TRY(gemm<T>(st, true, l, l, n, X, ldx, X, ldx, G, l, 1.0, 0.0, nullptr, 0, 0.0, nullptr, 0, scr,
                 true, false, &h->launches));
@@ -709,7 +727,7 @@ int cholqr_pass(chase_ctx* h, int n, int l, T* X, int ldx, T* Xtmp, T* G, T* Ri,
   TRY(trtri_upper<T>(st, l, G, l, Ri, l, &h->launches));
   if (oz) {
     TRY(oz_prep_factor<T>(h, *oz, l, l, Ri, l));
-    TRY(oz_tall<T>(h, *oz, l, X, ldx, l, X, ldx, scr));
+    TRY(oz_tall<T>(h, *oz, l, X, ldx, l, X, ldx));
     return 0;
   }
   TRY(gemm<T>(st, false, n, l, l, X, ldx, Ri, l, Xtmp, n, 1.0, 0.0, nullptr, 0, 0.0, nullptr, 0,
@@ -734,9 +752,9 @@ int wy_apply(chase_ctx* h, int n, int j0, int b, const T* V, const T* Tm, int ld
   TRY(gemm<T>(st, trans, b, nc, b, Tm, ldt, W, b, W2, b, 1.0, 0.0, nullptr, 0, 0.0, nullptr, 0, scr,
               false, false, &h->launches));
   if (oz) {
-    const int kpk = tc_kpad(Sc<T>::cplx ? 2 * b : b);
+    const int kpk = tc_kpad(b);
     TRY(oz_prep_factor<T>(h, *oz, b, nc, W2, b, kpk));
-    TRY(oz_tall<T>(h, *oz, b, V, n, nc, C, ldc, scr, kpk, true));
+    TRY(oz_tall<T>(h, *oz, b, V, n, nc, C, ldc, kpk, true));
   } else {
     TRY(gemm<T>(st, false, n - j0, nc, b, V + j0, n, W2, b, C + j0, ldc, -1.0, 1.0, C + j0, ldc, 0.0,
                 nullptr, 0, scr, false, false, &h->launches));
@@ -1126,14 +1144,14 @@ struct Solve final : SolveBase {
     if (emu) {
       if (!A_oz) rc = oz_slice_A_bufs<T>(h, n, A, lda, ozb);
       A_oz = true;
-      if (!rc) rc = aq_oz<T>(h, n, Q2, nu, AQ, ozb, scr);
+      if (!rc) rc = aq_oz<T>(h, n, Q2, nu, AQ, ozb);
     } else {
       rc = gemm<T>(st, false, n, nu, n, A, lda, Q2, n, AQ, n, 1.0, 0.0, nullptr, 0, 0.0, nullptr,
                    0, scr, false, false, &h->launches);
     }
     if (rc) {
     } else if (ozq) {
-      rc = oz_gram<T>(h, ozp, nu, Q2, n, AQ, n, H, nu, scr);
+      rc = oz_gram<T>(h, ozp, nu, Q2, n, AQ, n, H, nu);
     } else {
       rc = gemm<T>(st, true, nu, nu, n, Q2, n, AQ, n, H, nu, 1.0, 0.0, nullptr, 0, 0.0, nullptr, 0,
                    scr, true, false, &h->launches);
@@ -1149,8 +1167,8 @@ struct Solve final : SolveBase {
     if (rc) {
     } else if (ozq) {
       rc = oz_prep_factor<T>(h, ozp, nu, nu, Wm, nu);
-      if (!rc) rc = oz_tall<T>(h, ozp, nu, AQ, n, nu, P, n, scr);
-      if (!rc) rc = oz_tall<T>(h, ozp, nu, Q2, n, nu, Q2, n, scr);
+      if (!rc) rc = oz_tall<T>(h, ozp, nu, AQ, n, nu, P, n);
+      if (!rc) rc = oz_tall<T>(h, ozp, nu, Q2, n, nu, Q2, n);
     } else {
       rc = gemm<T>(st, false, n, nu, nu, Q2, n, Wm, nu, T2, n, 1.0, 0.0, nullptr, 0, 0.0, nullptr, 0,
                    scr, false, false, &h->launches);

@@ -158,3 +158,30 @@ def test_ring_product_beyond_the_short_range(cl):
     """K = 32832 > 2^15: 16 moduli."""
     torch.cuda.empty_cache()
     assert step_error(cl, 32800, 3, 5) <= 1.0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("n,l", [(1, 1), (31, 3), (33, 32), (64, 64), (65, 33), (257, 65), (700, 257), (1025, 321)])
+def test_qr_products_at_the_edges(cl, complex_, n, l):
+    """CholeskyQR2 of a well-conditioned block: both its products (X^H X and X R^-1) at the edges
+    of slicing tiles (32 rows x 64 of K), row pairs and column tiles.  Q is the unique factor with
+    positive diagonal R: within 64 n 2^-53 of torch's, orthonormal to the same."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + l)
+    dt = torch.complex128 if complex_ else torch.float64
+    U = torch.linalg.qr(torch.randn(n, l, generator=g, device="cuda", dtype=dt))[0]
+    M = torch.linalg.qr(torch.randn(l, l, generator=g, device="cuda", dtype=dt))[0]
+    X = cl.colmajor((U * torch.linspace(1.0, 2.0, l, device="cuda", dtype=torch.float64)) @ M)
+    Q0, R0 = torch.linalg.qr(X)
+    d = torch.diagonal(R0)
+    Q0 = Q0 * (d / d.abs())
+    h = cl.Handle(0)
+    try:
+        rc, v, info = cl.chase_qr(h, X, 1.0, qr_force=2, prec=cl.CHASE_FP64_EMU)
+    finally:
+        h.close()
+    tol = 64 * max(n, 16) * 2.0 ** -53
+    assert rc == 0 and v == 2 and info == 0
+    assert float((X - Q0).abs().max()) <= tol
+    assert float((X.mH @ X - torch.eye(l, device="cuda", dtype=dt)).abs().max()) <= tol
