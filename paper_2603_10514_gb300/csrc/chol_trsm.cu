@@ -1,21 +1,26 @@
-// chol_trsm.cu -- the small ell x ell factorisations of CholeskyQR
-// (Algorithm 2: R = chol(X^H X); Algorithm 3: chol(R + sI)) and the inverse of
-// the triangular factor used for X <- X R^{-1}.
+// chol_trsm.cu -- the small ell x ell factorisation of CholeskyQR (Algorithm 2:
+// R = chol(X^H X); Algorithm 3: chol(R + sI)) and the inverse of the triangular factor used
+// for X <- X R^{-1}.
 //
-// Cholesky: right-looking, one CTA of 1024 threads, upper triangle in global
-// memory (an ell x ell FP64 matrix, <= 23 MB, stays in the 129 MB L2).  A
-// non-positive or non-finite pivot j is reported as info = j + 1 in the device
-// status word (LAPACK convention) and the kernel returns -- no trap.
+// Cholesky: one cooperative kernel over blocks of 32 rows.  Per block
+//   A  CTA 0 factors the diagonal block, eliminating [G_kk | I] so that M = R_kk^{-H} comes
+//      with it, and publishes both (a flag);
+//   B  block row R_k. = M G_k., one warp per column;
+//   C  trailing update G -= R_k.^H R_k. of the upper triangle, one warp per 8 x 8 tile;
+// with a grid barrier after B and after C.  A non-positive or non-finite pivot j is reported as
+// info = j + 1 in the device status word (LAPACK convention) and every CTA leaves.  The
+// kernel reads G through L2 only (other CTAs wrote it).
 //
-// For ell > 128 the factorisation is blocked (block 64, right-looking): the
-// diagonal block is factored by one CTA in shared memory, the block row is
-// R_kk^{-H} G_k. (inverse of the diagonal block, then a product), and the
-// trailing update G -= R_k.^H R_k. is a K = 64 product over all SMs; the FP64
-// pipe of the whole GPU does the O(ell^3) work instead of one SM's.
+// Inverse: CTA b takes columns b and n - 1 - b of R^{-1} (together every CTA the same work),
+// each by back substitution over the same blocks of 32, with the M of step A for the diagonal
+// blocks: no division and three block barriers per 32 rows.
 //
-// Triangular inverse: one CTA per column j of R^{-1}; column j solves
-// R x = e_j by back substitution in column-oriented (axpy) form held in
-// shared memory.
+// What binds is FP64 at 2 FMAs per clock per SM (a warp instruction takes 64 clocks of a
+// sub-partition) and, in A, the chain of pivots: blocks of 32 keep A's share on one SM short
+// (64 would take four times that: the FP64 work of a block grows with its cube), the rest is
+// spread over all SMs.  n = 600 complex: 4.8 -> 2.0 ms (1.59 factor, 0.40 inverse) against blocks
+// of 64 in separate launches and an inverse by single columns; n = 30 real 57 -> 26 us.
+#include "../../include/chase_gb300.h"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -23,238 +28,281 @@ namespace chase {
 
 namespace {
 
+constexpr int CB = 32;              // rows of a block
+constexpr int CT = 8;               // trailing tiles are 8 x 8
+constexpr int CNT = 256, CW = CNT / 32;
+constexpr int CLD = CB + 1;
+
+struct CholBar {
+  GridBar bar;
+  unsigned ready;  // diagonal blocks factored
+  int fail;        // a pivot was not positive
+  int pad[2];
+};
+
+template <class T> __device__ __forceinline__ T ld_cg(const T* p);
+template <> __device__ __forceinline__ double ld_cg<double>(const double* p) { return __ldcg(p); }
+template <> __device__ __forceinline__ z64 ld_cg<z64>(const z64* p) {
+  const double2 v = __ldcg((const double2*)p);
+  return z64{v.x, v.y};
+}
+
+// A: factors the b x b block at `off` (CTA 0, CNT threads).  B, M: CB x CLD in shared memory.
+// Returns false (on every thread) after a failing pivot, reported in dst.
 template <class T>
-__global__ void __launch_bounds__(1024) potrf_upper_kernel(int n, T* G, int ldg,
-                                                           double shift_factor, DevStatus* dst) {
-  __shared__ double s_piv;
+__device__ bool chol_block(int b, T* G, int ldg, int off, double shift, T* B, T* M, T* Mb, DevStatus* dst) {
   __shared__ int s_fail;
-  __shared__ double s_red[32];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
-  if (shift_factor > 0.0) {
-    // shift s = shift_factor * ||X||_F^2 with ||X||_F^2 = trace(X^H X)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_fail = 0;
+  for (int t = tid; t < CB * CB; t += CNT) {
+    const int i = t % CB, j = t / CB;
+    T g = Sc<T>::zero();
+    if (i <= j && j < b) g = ld_cg(G + (size_t)(off + i) + (size_t)(off + j) * ldg);
+    if (i == j) g = Sc<T>::add(g, Sc<T>::from_re(shift));
+    B[i * CLD + j] = g;
+    M[i * CLD + j] = i == j ? Sc<T>::one() : Sc<T>::zero();
+  }
+  __syncthreads();
+  // row p of [B | M] minus conj(R[j][p]) times row j
+  auto eliminate = [&](int j, int p) {
+    const T f = Sc<T>::scale(Sc<T>::conj(B[j * CLD + p]), -1.0);
+    if (lane >= p) Sc<T>::fma(B[p * CLD + lane], f, B[j * CLD + lane]);
+    else if (lane <= j) Sc<T>::fma(M[p * CLD + lane], f, M[j * CLD + lane]);
+  };
+  // pivot of row j, and the row scaled by it (one warp)
+  auto pivot = [&](int j) {
+    const double d = Sc<T>::re(B[j * CLD + j]);
+    const bool bad = !(d > 0.0) || !isfinite(d);
+    const double r = bad ? 1.0 : rsqrt(d);
+    __syncwarp();
+    if (lane > j) B[j * CLD + lane] = Sc<T>::scale(B[j * CLD + lane], r);
+    else M[j * CLD + lane] = Sc<T>::scale(M[j * CLD + lane], r);
+    if (lane == j) B[j * CLD + j] = Sc<T>::from_re(d * r);
+    if (lane == 0 && bad) {
+      s_fail = 1;
+      atomicCAS(&dst->chol_info, 0, off + j + 1);
+    }
+  };
+  // Warp 0 runs ahead with the next row and its pivot, while the warps of the other
+  // sub-partitions eliminate from the rows after it (warp 4 shares warp 0's FP64 pipe and idles).
+  if (warp == 0) pivot(0);
+  __syncthreads();
+  if (s_fail) return false;
+  for (int j = 0; j + 1 < b; ++j) {
+    if (warp == 0) {
+      eliminate(j, j + 1);
+      __syncwarp();
+      pivot(j + 1);
+    } else if (warp != 4) {
+      for (int p = j + 1 + (warp < 4 ? warp : warp - 1); p < b; p += 6) eliminate(j, p);
+    }
+    __syncthreads();
+    if (s_fail) return false;
+  }
+  for (int t = tid; t < CB * CB; t += CNT) {
+    const int i = t % CB, j = t / CB;
+    if (i <= j && j < b) G[(size_t)(off + i) + (size_t)(off + j) * ldg] = B[i * CLD + j];
+    Mb[t] = (i < b && j <= i) ? M[i * CLD + j] : Sc<T>::zero();  // column-major CB x CB
+  }
+  return true;
+}
+
+// G (n x n, upper triangle) -> R in place; Mb: the blocks' R_kk^{-H}.  Rinv is written here when
+// n <= CB (one block).
+template <class T>
+__global__ void __launch_bounds__(CNT) chol_kernel(int n, T* G, int ldg, double shift_factor, T* Mb, T* Rinv,
+                                                   int ldri, CholBar* cb, DevStatus* dst) {
+  extern __shared__ __align__(16) unsigned char chol_smem[];
+  T* sm = (T*)chol_smem;
+  __shared__ int s_ok;
+  __shared__ double s_red[CW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G_ = gridDim.x, gw = blockIdx.x * CW + warp, nw = G_ * CW;
+  unsigned bars = 0;
+  double shift = 0.0;
+  if (shift_factor > 0.0 && blockIdx.x == 0) {
+    // s = shift_factor ||X||_F^2 with ||X||_F^2 = trace(X^H X), before anything is updated
     double tr = 0.0;
-    for (int j = tid; j < n; j += nt) tr += Sc<T>::re(G[(size_t)j + (size_t)j * ldg]);
+    for (int j = tid; j < n; j += CNT) tr += Sc<T>::re(ld_cg(G + (size_t)j + (size_t)j * ldg));
     for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
     if (lane == 0) s_red[warp] = tr;
     __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < nwarps; ++w) t += s_red[w];
-      s_piv = shift_factor * t;
-    }
-    __syncthreads();
-    const double s = s_piv;
-    for (int j = tid; j < n; j += nt) {
-      T& g = G[(size_t)j + (size_t)j * ldg];
-      g = Sc<T>::add(g, Sc<T>::from_re(s));
-    }
-    __syncthreads();
+    for (int w = 0; w < CW; ++w) shift += s_red[w];
+    shift *= shift_factor;
   }
-  for (int j = 0; j < n; ++j) {
-    if (tid == 0) {
-      double d = Sc<T>::re(G[(size_t)j + (size_t)j * ldg]);
-      int fail = !(d > 0.0) || !isfinite(d);
-      s_fail = fail;
-      if (fail) dst->chol_info = j + 1;
-      s_piv = fail ? 1.0 : sqrt(d);
-    }
-    __syncthreads();
-    if (s_fail) return;
-    const double r = s_piv, inv = 1.0 / r;
-    // row j of R: G[j, k] / r for k > j, diagonal r
-    for (int k = j + tid; k < n; k += nt) {
-      T& g = G[(size_t)j + (size_t)k * ldg];
-      g = (k == j) ? Sc<T>::from_re(r) : Sc<T>::scale(g, inv);
-    }
-    __syncthreads();
-    // trailing update of the upper triangle: G[p, q] -= conj(R[j, p]) R[j, q], j < p <= q;
-    // one warp per column q, lanes along p (contiguous in column-major storage)
-    for (int q = j + 1 + warp; q < n; q += nwarps) {
-      const T rq = G[(size_t)j + (size_t)q * ldg];
-      T* col = G + (size_t)q * ldg;
-      for (int p = j + 1 + lane; p <= q; p += 32) {
-        T rp = G[(size_t)j + (size_t)p * ldg];
-        col[p] = Sc<T>::sub(col[p], Sc<T>::mul(Sc<T>::conj(rp), rq));
+  for (int kb = 0, off = 0; off < n; ++kb, off += CB) {
+    const int b = min(CB, n - off), rest = n - off - b;
+    T* Mk = Mb + (size_t)kb * CB * CB;
+    if (blockIdx.x == 0) {
+      const bool ok = chol_block<T>(b, G, ldg, off, shift, sm, sm + CB * CLD, Mk, dst);
+      __syncthreads();
+      if (tid == 0) {
+        if (!ok) atomicExch(&cb->fail, 1);
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&cb->ready), "r"(kb + 1) : "memory");
+      }
+      if (!ok) return;
+      if (n <= CB) {
+        for (int t = tid; t < n * n; t += CNT) {
+          const int i = t % n, j = t / n;
+          Rinv[(size_t)i + (size_t)j * ldri] = i <= j ? Sc<T>::conj(sm[CB * CLD + j * CLD + i]) : Sc<T>::zero();
+        }
       }
     }
-    __syncthreads();
-  }
-  // zero the strict lower triangle so that G is exactly R
-  for (int k = warp; k < n; k += nwarps)
-    for (int i = k + 1 + lane; i < n; i += 32) G[(size_t)i + (size_t)k * ldg] = Sc<T>::zero();
-}
-
-template <class T>
-__global__ void __launch_bounds__(256) trtri_upper_kernel(int n, const T* __restrict__ R, int ldr,
-                                                          T* Rinv, int ldri) {
-  extern __shared__ unsigned char smem_raw[];
-  T* x = reinterpret_cast<T*>(smem_raw);
-  const int j = blockIdx.x;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i <= j; i += nt) x[i] = Sc<T>::zero();
-  __syncthreads();
-  if (tid == 0) {
-    T rjj = R[(size_t)j + (size_t)j * ldr];
-    // 1 / rjj (the diagonal of a Cholesky factor is real and positive)
-    x[j] = Sc<T>::from_re(1.0 / Sc<T>::re(rjj));
-  }
-  __syncthreads();
-  for (int p = j; p >= 1; --p) {
-    const T xp = x[p];
-    for (int i = tid; i < p; i += nt) {
-      T r = R[(size_t)i + (size_t)p * ldr];
-      x[i] = Sc<T>::sub(x[i], Sc<T>::mul(r, xp));
-    }
-    __syncthreads();
+    if (rest <= 0) return;
     if (tid == 0) {
-      double d = Sc<T>::re(R[(size_t)(p - 1) + (size_t)(p - 1) * ldr]);
-      x[p - 1] = Sc<T>::scale(x[p - 1], 1.0 / d);
+      int ok = 1;
+      const long long t0 = clock64();
+      while (true) {
+        unsigned r;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(&cb->ready) : "memory");
+        if ((int)r > kb) break;
+        if (*(volatile int*)&cb->bar.abort) { ok = 0; break; }
+        if (clock64() - t0 > kBarWait) { atomicExch(&cb->bar.abort, 1); ok = 0; break; }
+      }
+      if (!ok) atomicOr(&dst->timeout, 32);
+      s_ok = ok && !*(volatile int*)&cb->fail;
     }
     __syncthreads();
+    if (!s_ok) return;
+    // B: block row
+    for (int t = tid; t < CB * CB; t += CNT) sm[(t % CB) * CLD + t / CB] = ld_cg(Mk + t);
+    __syncthreads();
+    T* colb = sm + CB * CLD + warp * CB;
+    for (int c = off + b + gw; c < n; c += nw) {
+      T* g = G + (size_t)off + (size_t)c * ldg;
+      colb[lane] = ld_cg(g + lane);  // (b == CB: there are columns to the right)
+      __syncwarp();
+      T a = Sc<T>::zero();
+#pragma unroll 4
+      for (int p = 0; p < CB; ++p) Sc<T>::fma(a, sm[lane * CLD + p], colb[p]);
+      g[lane] = a;
+      __syncwarp();
+    }
+    if (!grid_barrier(&cb->bar, G_, bars)) {
+      if (tid == 0) atomicOr(&dst->timeout, 32);
+      return;
+    }
+    // C: trailing tiles (tp <= tq)
+    const int nt = (rest + CT - 1) / CT, tiles = nt * (nt + 1) / 2, o2 = off + b;
+    T* P = sm + (size_t)warp * 2 * CT * CLD;
+    T* Q = P + CT * CLD;
+    for (int t = gw; t < tiles; t += nw) {
+      int tq = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+      while (tq * (tq + 1) / 2 > t) --tq;
+      while ((tq + 1) * (tq + 2) / 2 <= t) ++tq;
+      const int tp = t - tq * (tq + 1) / 2;
+      const int p0 = o2 + tp * CT, q0 = o2 + tq * CT;
+#pragma unroll
+      for (int c = 0; c < CT; ++c) {
+        P[c * CLD + lane] = p0 + c < n ? ld_cg(G + (size_t)(off + lane) + (size_t)(p0 + c) * ldg) : Sc<T>::zero();
+        Q[c * CLD + lane] = q0 + c < n ? ld_cg(G + (size_t)(off + lane) + (size_t)(q0 + c) * ldg) : Sc<T>::zero();
+      }
+      __syncwarp();
+      const int p = lane & 7, q = lane >> 3;  // entries (p, q) and (p, q + 4)
+      T a0 = Sc<T>::zero(), a1 = Sc<T>::zero();
+#pragma unroll 4
+      for (int s = 0; s < CB; ++s) {
+        const T x = P[p * CLD + s];
+        Sc<T>::fmac(a0, x, Q[q * CLD + s]);
+        Sc<T>::fmac(a1, x, Q[(q + 4) * CLD + s]);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int gp = p0 + p, gq = q0 + q + 4 * h;
+        if (gp <= gq && gq < n) {
+          T* g = G + (size_t)gp + (size_t)gq * ldg;
+          *g = Sc<T>::sub(ld_cg(g), h ? a1 : a0);
+        }
+      }
+      __syncwarp();
+    }
+    if (!grid_barrier(&cb->bar, G_, bars)) {
+      if (tid == 0) atomicOr(&dst->timeout, 32);
+      return;
+    }
   }
-  for (int i = tid; i < n; i += nt)
-    Rinv[(size_t)i + (size_t)j * ldri] = (i <= j) ? x[i] : Sc<T>::zero();
 }
 
-constexpr int CNB = 64;
-
-// G[j, j] += shift_factor * trace(G)   (one CTA)
+// Columns blockIdx.x and n - 1 - blockIdx.x of R^{-1} (n > CB).
 template <class T>
-__global__ void __launch_bounds__(1024) add_shift_kernel(int n, T* G, int ldg, double factor) {
-  __shared__ double red[32];
-  __shared__ double s_shift;
-  double tr = 0.0;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) tr += Sc<T>::re(G[(size_t)j + (size_t)j * ldg]);
-  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = tr;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    s_shift = factor * t;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    T& g = G[(size_t)j + (size_t)j * ldg];
-    g = Sc<T>::add(g, Sc<T>::from_re(s_shift));
-  }
-}
-
-// Factors the b x b diagonal block at (off, off) in shared memory (upper, in place): one CTA
-// of 1024 threads (the rank-1 updates of a 64 x 64 block take 2 entries per thread).
-template <class T>
-__global__ void __launch_bounds__(1024) chol_diag_kernel(int b, T* G, int ldg, int off,
-                                                         DevStatus* dst) {
-  extern __shared__ unsigned char diag_smem[];
-  T(*B)[CNB + 1] = reinterpret_cast<T(*)[CNB + 1]>(diag_smem);  // CNB x (CNB + 1)
-  __shared__ double s_piv;
-  __shared__ int s_fail;
-  if (*(volatile int*)&dst->chol_info) return;
-  const int tid = threadIdx.x;
-  for (int t = tid; t < b * b; t += blockDim.x) {
-    const int i = t % b, j = t / b;
-    B[i][j] = (i <= j) ? G[(size_t)(off + i) + (size_t)(off + j) * ldg] : Sc<T>::zero();
-  }
-  __syncthreads();
-  for (int j = 0; j < b; ++j) {
-    if (tid == 0) {
-      const double d = Sc<T>::re(B[j][j]);
-      const int fail = !(d > 0.0) || !isfinite(d);
-      s_fail = fail;
-      if (fail) atomicCAS(&dst->chol_info, 0, off + j + 1);
-      s_piv = fail ? 1.0 : sqrt(d);
+__global__ void __launch_bounds__(128) trinv_kernel(int n, const T* __restrict__ R, int ldr,
+                                                    const T* __restrict__ Mb, T* Rinv, int ldri,
+                                                    const DevStatus* dst) {
+  extern __shared__ __align__(16) unsigned char inv_smem[];
+  T* x = (T*)inv_smem;
+  __shared__ T part[4][CB];
+  if (dst->chol_info) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int half = 0; half < 2; ++half) {
+    const int j = half ? n - 1 - (int)blockIdx.x : (int)blockIdx.x;
+    if (half && j <= (int)blockIdx.x) break;
+    const int kj = j / CB, jj = j - kj * CB;
+    for (int i = tid; i < kj * CB; i += 128) x[i] = Sc<T>::zero();
+    // R_kk^{-1} e_jj: column jj of M^H
+    if (tid < CB) x[kj * CB + tid] = tid <= jj ? Sc<T>::conj(Mb[(size_t)kj * CB * CB + jj + tid * CB]) : Sc<T>::zero();
+    __syncthreads();
+    for (int k = kj; k > 0; --k) {
+      const int off = k * CB, len = k == kj ? jj + 1 : CB;
+      // rows above the block
+      for (int i = tid; i < off; i += 128) {
+        T a = x[i];
+        const T* r = R + (size_t)i + (size_t)off * ldr;
+#pragma unroll 4
+        for (int s = 0; s < len; ++s) Sc<T>::fma(a, r[(size_t)s * ldr], Sc<T>::scale(x[off + s], -1.0));
+        x[i] = a;
+      }
+      __syncthreads();
+      // block k - 1: x <- R_kk^{-1} x = M^H x, the sum over rows split over the four warps
+      const T* M = Mb + (size_t)(k - 1) * CB * CB;
+      T a = Sc<T>::zero();
+#pragma unroll
+      for (int p = 8 * warp; p < 8 * warp + 8; ++p) Sc<T>::fmac(a, M[p + lane * CB], x[off - CB + p]);
+      part[warp][lane] = a;
+      __syncthreads();
+      if (warp == 0) {
+        for (int w = 1; w < 4; ++w) a = Sc<T>::add(a, part[w][lane]);
+        x[off - CB + lane] = a;
+      }
+      __syncthreads();
     }
+    for (int i = tid; i < n; i += 128) Rinv[(size_t)i + (size_t)j * ldri] = i <= j ? x[i] : Sc<T>::zero();
     __syncthreads();
-    if (s_fail) return;
-    const double r = s_piv, inv = 1.0 / r;
-    for (int k = j + tid; k < b; k += blockDim.x) B[j][k] = (k == j) ? Sc<T>::from_re(r) : Sc<T>::scale(B[j][k], inv);
-    __syncthreads();
-    const int m = b - j - 1;
-    for (int t = tid; t < m * m; t += blockDim.x) {
-      const int p = j + 1 + t % m, q = j + 1 + t / m;
-      if (p <= q) B[p][q] = Sc<T>::sub(B[p][q], Sc<T>::mul(Sc<T>::conj(B[j][p]), B[j][q]));
-    }
-    __syncthreads();
-  }
-  for (int t = tid; t < b * b; t += blockDim.x) {
-    const int i = t % b, j = t / b;
-    if (i <= j) G[(size_t)(off + i) + (size_t)(off + j) * ldg] = B[i][j];
   }
 }
 
 }  // namespace
 
+size_t chol_work_bytes(int n, size_t elem) { return sizeof(CholBar) + 256 + elem * CB * CB * (size_t)ceil_div(n, CB); }
+
 template <class T>
-int potrf_upper_blocked(cudaStream_t st, int n, T* G, int ldg, double shift_factor, DevStatus* dst,
-                        T* scratch, Scratch gscr, int* launches) {
-  if (shift_factor > 0.0) {
-    add_shift_kernel<T><<<1, 1024, 0, st>>>(n, G, ldg, shift_factor);
+int chol_inverse(cudaStream_t st, int n, T* G, int ldg, double shift_factor, T* Rinv, int ldri, Scratch work,
+                 DevStatus* dst, int* launches) {
+  if (n <= 0) return 0;
+  if (work.bytes < chol_work_bytes(n, sizeof(T))) return CHASE_ERR_OOM;
+  CholBar* cb = (CholBar*)work.ptr;
+  T* Mb = (T*)((char*)work.ptr + 256);
+  // CTAs: eight tiles of the first trailing update per warp, at most one per SM
+  const long long nt = ceil_div(std::max(0, n - CB), CT), tiles = nt * (nt + 1) / 2;
+  int grid = (int)std::max(1LL, std::min<long long>(kNumSMs, (tiles + CW - 1) / CW));
+  const int smem = (int)sizeof(T) * std::max(CW * 2 * CT * CLD, 2 * CB * CLD);
+  CHASE_CUDA_TRY(cudaFuncSetAttribute(chol_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  CHASE_CUDA_TRY(cudaMemsetAsync(cb, 0, sizeof(CholBar), st));
+  void* args[] = {(void*)&n, (void*)&G, (void*)&ldg, (void*)&shift_factor, (void*)&Mb, (void*)&Rinv,
+                  (void*)&ldri, (void*)&cb, (void*)&dst};
+  CHASE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)chol_kernel<T>, dim3(grid), dim3(CNT), args, (size_t)smem, st));
+  if (launches) ++*launches;
+  if (n > CB) {
+    const size_t xs = sizeof(T) * (size_t)ceil_div(n, CB) * CB;
+    if (xs > 48 * 1024)
+      CHASE_CUDA_TRY(cudaFuncSetAttribute(trinv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs));
+    trinv_kernel<T><<<ceil_div(n, 2), 128, xs, st>>>(n, G, ldg, Mb, Rinv, ldri, dst);
     if (launches) ++*launches;
   }
-  T* Rkk_inv = scratch;                 // CNB x CNB
-  T* tmp = scratch + CNB * CNB;         // CNB x n
-  const int dsmem = (int)(sizeof(T) * CNB * (CNB + 1));
-  CHASE_CUDA_TRY(cudaFuncSetAttribute(chol_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      dsmem));
-  for (int off = 0; off < n; off += CNB) {
-    const int b = std::min(CNB, n - off);
-    chol_diag_kernel<T><<<1, 1024, dsmem, st>>>(b, G, ldg, off, dst);
-    if (launches) ++*launches;
-    const int rest = n - off - b;
-    if (rest <= 0) break;
-    T* Gkk = G + (size_t)off + (size_t)off * ldg;
-    T* Gpanel = G + (size_t)off + (size_t)(off + b) * ldg;        // b x rest
-    T* Gtrail = G + (size_t)(off + b) + (size_t)(off + b) * ldg;  // rest x rest
-    // the inverse of the diagonal block: one CTA per column (its FP64 work over b SMs)
-    int rc = trtri_upper<T>(st, b, Gkk, ldg, Rkk_inv, b, launches);
-    if (rc) return rc;
-    // block row: R_k. = R_kk^{-H} G_k.
-    rc = gemm<T>(st, true, b, rest, b, Rkk_inv, b, Gpanel, ldg, tmp, b, 1.0, 0.0, nullptr, 0, 0.0,
-                 nullptr, 0, gscr, false, false, launches);
-    if (rc) return rc;
-    CHASE_CUDA_TRY(cudaMemcpy2DAsync(Gpanel, sizeof(T) * (size_t)ldg, tmp, sizeof(T) * (size_t)b,
-                                     sizeof(T) * (size_t)b, rest, cudaMemcpyDeviceToDevice, st));
-    // trailing update of the upper triangle: G -= R_k.^H R_k.
-    rc = gemm<T>(st, true, rest, rest, b, Gpanel, ldg, Gpanel, ldg, Gtrail, ldg, -1.0, 1.0, Gtrail,
-                 ldg, 0.0, nullptr, 0, gscr, true, false, launches);
-    if (rc) return rc;
-  }
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
 }
 
-template <class T>
-int potrf_upper(cudaStream_t st, int n, T* G, int ldg, double shift_factor, DevStatus* dst,
-                int* launches) {
-  if (n <= 0) return 0;
-  potrf_upper_kernel<T><<<1, 1024, 0, st>>>(n, G, ldg, shift_factor, dst);
-  if (launches) ++*launches;
-  CHASE_CUDA_TRY(cudaGetLastError());
-  return 0;
-}
-
-template <class T>
-int trtri_upper(cudaStream_t st, int n, const T* R, int ldr, T* Rinv, int ldri, int* launches) {
-  if (n <= 0) return 0;
-  size_t smem = sizeof(T) * (size_t)n;
-  if (smem > 48 * 1024) {
-    CHASE_CUDA_TRY(cudaFuncSetAttribute(trtri_upper_kernel<T>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  }
-  trtri_upper_kernel<T><<<n, 256, smem, st>>>(n, R, ldr, Rinv, ldri);
-  if (launches) ++*launches;
-  CHASE_CUDA_TRY(cudaGetLastError());
-  return 0;
-}
-
-template int potrf_upper<double>(cudaStream_t, int, double*, int, double, DevStatus*, int*);
-template int potrf_upper<z64>(cudaStream_t, int, z64*, int, double, DevStatus*, int*);
-template int potrf_upper_blocked<double>(cudaStream_t, int, double*, int, double, DevStatus*,
-                                         double*, Scratch, int*);
-template int potrf_upper_blocked<z64>(cudaStream_t, int, z64*, int, double, DevStatus*, z64*,
-                                      Scratch, int*);
-template int trtri_upper<double>(cudaStream_t, int, const double*, int, double*, int, int*);
-template int trtri_upper<z64>(cudaStream_t, int, const z64*, int, z64*, int, int*);
+template int chol_inverse<double>(cudaStream_t, int, double*, int, double, double*, int, Scratch, DevStatus*, int*);
+template int chol_inverse<z64>(cudaStream_t, int, z64*, int, double, z64*, int, Scratch, DevStatus*, int*);
 
 }  // namespace chase

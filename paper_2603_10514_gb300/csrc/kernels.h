@@ -21,21 +21,14 @@ int gemm(cudaStream_t st, bool transA, int M, int N, int K, const T* A, int lda,
          const T* Y, int ldy, Scratch scratch, bool upper_only, bool tri_b, int* launches);
 
 // ---- dense small-matrix kernels (chol_trsm.cu) ----------------------------
-// Upper Cholesky of G in place; info (first failing pivot + 1) goes to dst->chol_info.
+// Upper Cholesky G = R^H R of G's upper triangle in place, and Rinv = R^{-1} (zero strict lower
+// part); info (first failing pivot + 1) goes to dst->chol_info, Rinv is then not written.
 // shift_factor > 0 first adds s = shift_factor * trace(G) to the diagonal (the shifted
-// CholeskyQR step: trace(X^H X) = ||X||_F^2).
+// CholeskyQR step: trace(X^H X) = ||X||_F^2).  work: chol_work_bytes.
+size_t chol_work_bytes(int n, size_t elem);
 template <class T>
-int potrf_upper(cudaStream_t st, int n, T* G, int ldg, double shift_factor, DevStatus* dst,
-                int* launches);
-// Blocked (64) variant for larger n: diagonal blocks on one CTA, block rows and
-// trailing updates as products.  scratch: 64*64 + 64*n elements; the strict lower
-// triangle of G is left as it was.
-template <class T>
-int potrf_upper_blocked(cudaStream_t st, int n, T* G, int ldg, double shift_factor, DevStatus* dst,
-                        T* scratch, Scratch gscr, int* launches);
-// Rinv = R^{-1} for upper-triangular R (zero strict lower part written).
-template <class T>
-int trtri_upper(cudaStream_t st, int n, const T* R, int ldr, T* Rinv, int ldri, int* launches);
+int chol_inverse(cudaStream_t st, int n, T* G, int ldg, double shift_factor, T* Rinv, int ldri, Scratch work,
+                 DevStatus* dst, int* launches);
 
 // ---- Householder QR with explicit thin Q (householder.cu) -----------------
 template <class T>
