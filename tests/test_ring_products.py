@@ -185,3 +185,33 @@ def test_qr_products_at_the_edges(cl, complex_, n, l):
     assert rc == 0 and v == 2 and info == 0
     assert float((X - Q0).abs().max()) <= tol
     assert float((X.mH @ X - torch.eye(l, device="cuda", dtype=dt)).abs().max()) <= tol
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("n,ncols", [(96, 8), (97, 9)])
+@pytest.mark.parametrize("scale", [-1060, -1000, 0, 900])
+def test_reconstruction_over_the_exponent_range(cl, complex_, n, ncols, scale):
+    """Results from the subnormal range up to 2^900, one zero column: within the scheme's bound of
+    the product of the unscaled operands (and one subnormal unit for each rounding)."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    dt = torch.complex128 if complex_ else torch.float64
+    A = torch.randn(n, n, generator=g, device="cuda", dtype=dt)
+    A = cl.colmajor(A + A.mH)
+    V = cl.colmajor(torch.randn(n, ncols, generator=g, device="cuda", dtype=dt))
+    V[:, ncols // 2] = 0.0
+    c, e, l1 = 0.0, 1.0, -2.0  # one step: out = A V / l1
+    half = 2.0 ** (scale // 2)
+    h = cl.Handle(0)
+    try:
+        got = cl.chase_filter(h, cl.colmajor(A * half), cl.colmajor(V * half), [1] * ncols, c, e, l1,
+                              prec=cl.CHASE_FP64_EMU)
+    finally:
+        h.close()
+    parts = lambda x: torch.view_as_real(x) if complex_ else x
+    ref = (A @ V) / l1
+    bound = 2 * n * 2.0 ** -53 * 2.0 * parts(A).abs().max() * parts(V).abs().max()
+    err = (parts(got) / half / half if scale > -1000 else parts(got * 2.0 ** 500) * 2.0 ** (-scale - 500)) - parts(ref)
+    assert float(err.abs().max()) <= float(bound) + 4 * 2.0 ** (-1074 - min(scale, 0))
+    assert torch.equal(got[:, ncols // 2], torch.zeros_like(got[:, 0]))
