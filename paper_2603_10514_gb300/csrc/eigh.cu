@@ -2,10 +2,11 @@
 // and of the Lanczos runs' tridiagonals.
 //
 //   1. Householder reduction of the Hermitian H (l x l) to a real tridiagonal T = Q^H H Q, one
-//      cooperative kernel: columns are dealt to the CTAs in turn and stay in shared memory;
-//      per column the owner publishes its reflector v (a flag), every CTA forms its entries of
-//      H v from its own columns (H is Hermitian, so no partial sums cross CTAs), and after one
-//      grid barrier applies H -= v w^H + w v^H to them.
+//      cooperative kernel: columns are dealt to the CTAs in turn and stay in shared memory.
+//      Per column every CTA forms its entries of H v from its own columns (H is Hermitian, so
+//      no partial sums cross CTAs); after the step's one grid barrier every CTA forms
+//      w itself, the owner's next raw column was published beside it, and the next reflector
+//      is formed by every CTA from that while its other warps apply H -= v w^H + w v^H.
 //   2. Divide and conquer for T = Z Lambda Z^T (stedc.cuh): blocks of up to 32 rows in one CTA
 //      each, then per level five launches over all merges of the level.
 //   3. W = Q Z: one warp per column of W applies the reflectors in turn; columns are
@@ -13,9 +14,9 @@
 // It replaces a cyclic Jacobi iteration.  GB300 issues 2 FP64 FMAs per clock per SM, which binds
 // both: Jacobi takes ~5 sweeps of ~9 l^3 (complex: x 4) FMAs and l - 1 grid-wide rounds each,
 // this ~4 l^3 for step 1, ~l^3 (real) for 2 and ~2 l^3 for 3, and l grid barriers in all.
-// Measured (random H, GB300): l = 600 complex 124 -> 14.0 ms (8.6 reduction, 2.0 divide and
-// conquer, 3.3 back-transformation), l = 230 complex 31 -> 4.1, l = 600 real 80 -> 8.5, l = 30
-// real 2.0 -> 0.87.
+// Measured (random H, GB300): l = 600 complex 124 -> 11.8 ms (6.5 reduction, 1.8 divide and
+// conquer, 3.5 back-transformation), l = 230 complex 31 -> 3.5, l = 600 real 80 -> 7.8, l = 30
+// real 2.0 -> 0.48.
 //
 // Every wait is bounded; a CTA that waits too long raises an abort flag that the others see, and
 // the kernel sets DevStatus.timeout.  Sums are taken in fixed orders: results are reproducible.
@@ -61,34 +62,52 @@ __device__ __forceinline__ double im_of(z64 a) { return a.y; }
 // ---------------------------------------------------------------------------
 // 1. Reduction to tridiagonal form
 // ---------------------------------------------------------------------------
-struct TriBar {
-  GridBar bar;
-  unsigned ready;  // reflectors published
-  int pad[3];
-};
-
-// Reflector j from column j (rows j .. l - 1 up to date): v into rows j + 1 .. of hcol (global),
-// tau, d[j], e[j].  One CTA; sh: 8 doubles and one T of shared memory.
+// H (l x l, ld ldh): column j is overwritten by reflector j (rows j + 1 ..).  in_smem: this CTA's
+// columns are kept in shared memory, else in place.  Per column j, with v = v_j and tau known to
+// every CTA:
+//   x_c = tau (H v)_c for the own columns c; the owner of column j + 1 publishes it as it is;
+//   grid barrier; alpha = -1/2 tau x^H v (real: -1/2 |tau|^2 v^H H v) from the CTAs' parts;
+//   every CTA updates column j + 1 for itself and forms reflector j + 1 from it -- a few l FMAs
+//   more on every SM, but no second wait on its owner -- and while one warp takes the reflector's
+//   square root and divisions (~35 dependent FP64 instructions), the others apply
+//   H -= v w^H + w v^H, w = x + alpha v, to the own columns.
+// xb, cb: 2 l elements, part: 2 G doubles; scr: 3 l elements per CTA where they do not fit
+// shared memory (else null).
 template <class T>
-__device__ void make_reflector(int l, int j, const T* col, T* hcol, T* tau, double* d, double* e, double* sh,
-                               T* sh_scale) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double s = 0.0;
-  for (int i = j + 2 + tid; i < l; i += TNT) s += Sc<T>::abs2(col[i]);
-  s = warp_add(s);
-  if (lane == 0) sh[warp] = s;
-  __syncthreads();
-  if (tid == 0) {
+__global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int in_smem, T* tau, double* d,
+                                                      double* e, T* xb, T* cb, double* part, T* scr, GridBar* gb,
+                                                      DevStatus* dst) {
+  extern __shared__ __align__(16) unsigned char tri_smem[];
+  const int G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = TNT / 32;
+  __shared__ double sh[NW];
+  __shared__ T sh_tau, sh_scale;
+  __shared__ double sh_alpha;
+  const int own = (l + G - 1) / G;                     // columns me, me + G, ...
+  const int nc = me < l ? (l - 1 - me) / G + 1 : 0;
+  T* sp = (T*)tri_smem;                                // 4 partial sums per own column
+  T* sq = sp + 4 * own;                                // the update's two factors per own column
+  T* vec = scr ? scr + (size_t)me * 3 * l : sq + 2 * own;
+  T *vs = vec, *xs = vec + l, *us = vec + 2 * (size_t)l;
+  T* S = scr ? sq + 2 * own : vec + 3 * (size_t)l;
+  auto column = [&](int k) -> T* { return in_smem ? S + (size_t)k * l : H + (size_t)(me + k * G) * ldh; };
+  if (in_smem)
+    for (int k = 0; k < nc; ++k)
+      for (int i = tid; i < l; i += TNT) S[(size_t)k * l + i] = H[(size_t)i + (size_t)(me + k * G) * ldh];
+
+  // Reflector j from u (rows j .. of the updated column j): its scalars, by one thread.
+  auto scalars = [&](int j, const T* u) {
     double x2 = 0.0;
-    for (int w = 0; w < TNT / 32; ++w) x2 += sh[w];
-    d[j] = Sc<T>::re(col[j]);
-    const T alpha = col[j + 1];
+    for (int w = 0; w < NW; ++w) x2 += sh[w];
+    const T alpha = u[j + 1];
     const double ar = Sc<T>::re(alpha), ai = im_of(alpha);
     T t = Sc<T>::zero(), sc = Sc<T>::zero();
     double beta = ar;
-    if (x2 != 0.0 || ai != 0.0) {
-      beta = -copysign(sqrt(ar * ar + ai * ai + x2), ar);
-      const double ib = 1.0 / beta, dr = ar - beta, id = 1.0 / (dr * dr + ai * ai);
+    const double nn = ar * ar + ai * ai + x2;
+    if ((x2 != 0.0 || ai != 0.0) && !(nn < 1e-300)) {  // (below: nothing is left, and 1 / nn overflows)
+      const double rn = rsqrt(nn);
+      beta = -copysign(nn * rn, ar);
+      const double ib = -copysign(rn, ar), dr = ar - beta, id = 1.0 / (dr * dr + ai * ai);
       if constexpr (Sc<T>::cplx) {
         t = z64{(beta - ar) * ib, -ai * ib};
         sc = z64{dr * id, -ai * id};
@@ -97,139 +116,168 @@ __device__ void make_reflector(int l, int j, const T* col, T* hcol, T* tau, doub
         sc = dr * id;
       }
     }
-    e[j] = beta;
-    tau[j] = t;
-    *sh_scale = sc;
-  }
-  __syncthreads();
-  const T sc = *sh_scale;
-  for (int i = j + 1 + tid; i < l; i += TNT) hcol[i] = (i == j + 1) ? Sc<T>::one() : Sc<T>::mul(col[i], sc);
-}
-
-// H (l x l, ld ldh): column j is overwritten by reflector j (rows j + 1 ..).  in_smem: this CTA's
-// columns are kept in shared memory, else in place.  STAGE: v and x are copied to shared memory.
-// xb: 2 l elements, part: 2 G elements.
-template <class T, bool STAGE>
-__global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int in_smem, T* tau, double* d,
-                                                      double* e, T* xb, T* part, TriBar* tb,
-                                                      DevStatus* dst) {
-  extern __shared__ __align__(16) unsigned char tri_smem[];
-  const int G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ double sh[TNT / 32];
-  __shared__ T sh_scale, sh_alpha;
-  __shared__ int s_ok;
-  T* vs = (T*)tri_smem;
-  T* xs = vs + (STAGE ? l : 0);
-  T* sx = xs + (STAGE ? l : 0);             // this CTA's terms of x^H v
-  const int nc = me < l ? (l - 1 - me) / G + 1 : 0;  // own columns me, me + G, ...
-  T* S = sx + (l + G - 1) / G;
-  int ldS = l;
-  if (in_smem) {
-    for (int k = 0; k < nc; ++k)
-      for (int i = tid; i < l; i += TNT) S[(size_t)k * l + i] = H[(size_t)i + (size_t)(me + k * G) * ldh];
-  }
-  auto column = [&](int k) -> T* { return in_smem ? S + (size_t)k * ldS : H + (size_t)(me + k * G) * ldh; };
-  __syncthreads();
-  unsigned bars = 0;
-  int par = 0;
-  // publishes reflector j (or the last diagonal entry)
-  auto publish = [&](int j) {
-    if (j < l - 1) {
-      make_reflector<T>(l, j, column(j / G), H + (size_t)j * ldh, tau, d, e, sh, &sh_scale);
-      __syncthreads();
-      if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&tb->ready), "r"(j + 1) : "memory");
-    } else if (tid == 0) {
-      d[j] = Sc<T>::re(column(j / G)[j]);
+    sh_tau = t;
+    sh_scale = sc;
+    if (j % G == me) {
+      d[j] = Sc<T>::re(u[j]);
+      e[j] = beta;
+      tau[j] = t;
     }
   };
-  if (me == 0) publish(0);
+  auto norm_part = [&](double s) {  // sum of squares below the subdiagonal, a part per warp
+    s = warp_add(s);
+    if (lane == 0) sh[warp] = s;
+  };
+  // v = u scaled (in u's place), kept in H by its owner
+  auto finish_reflector = [&](int j, T* u) {
+    const T sc = sh_scale;
+    T* hcol = H + (size_t)j * ldh;
+    for (int i = j + 1 + tid; i < l; i += TNT) {
+      const T v = (i == j + 1) ? Sc<T>::one() : Sc<T>::mul(u[i], sc);
+      u[i] = v;
+      if (j % G == me) hcol[i] = v;
+    }
+  };
+
+  // reflector 0, by every CTA from the matrix (read before any column is overwritten: its owner
+  // writes it after the first barrier's worth of work is published, see below)
+  {
+    double s = 0.0;
+    for (int i = tid; i < l; i += TNT) {
+      const T h = H[i];
+      us[i] = h;
+      if (i >= 2) s += Sc<T>::abs2(h);
+    }
+    norm_part(s);
+  }
+  __syncthreads();
+  if (l == 1) {
+    if (me == 0 && tid == 0) d[0] = Sc<T>::re(us[0]);
+    return;
+  }
+  unsigned bars = 0;
+  int par = 0;
+  if (G > 1 && !grid_barrier(gb, G, bars)) {  // column 0 has been read everywhere
+    if (tid == 0) atomicOr(&dst->timeout, 16);
+    return;
+  }
+  if (tid == 0) scalars(0, us);
+  __syncthreads();
+  finish_reflector(0, us);
+  __syncthreads();
   for (int j = 0; j + 1 < l; ++j) {
-    if (tid == 0) {
-      int ok = 1;
-      unsigned r;
-      const long long t0 = clock64();
-      while (true) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(&tb->ready) : "memory");
-        if ((int)r > j) break;
-        if (*(volatile int*)&tb->bar.abort) { ok = 0; break; }
-        if (clock64() - t0 > kBarWait) { atomicExch(&tb->bar.abort, 1); ok = 0; break; }
-      }
-      s_ok = ok;
-    }
-    __syncthreads();
-    if (!s_ok) {
-      if (tid == 0) atomicOr(&dst->timeout, 16);
-      return;
-    }
-    const T t = ld_cg(tau + j);
-    const T* vg = H + (size_t)j * ldh;
-    T* xg = xb + (size_t)par * l;
-    const int k0 = (j + 1 <= me) ? 0 : (j + 1 - me + G - 1) / G;  // first own column >= j + 1
+    { T* q = vs; vs = us; us = q; }  // v_j
+    const T t = sh_tau;
+    const int k0 = (j + 1 <= me) ? 0 : (j + 1 - me + G - 1) / G, na = nc - k0;  // own columns >= j + 1
     const bool trivial = Sc<T>::re(t) == 0.0 && im_of(t) == 0.0;
+    T *xg = xb + (size_t)par * l, *cg = cb + (size_t)par * l;
+    const bool next_mine = (j + 1) % G == me;
+    // x = tau H v on the own columns, each split over enough warps to use every sub-partition
     if (!trivial) {
-      if (STAGE) {
-        for (int i = j + 1 + tid; i < l; i += TNT) vs[i] = ld_cg(vg + i);
-        __syncthreads();
-      }
-      // x_c = tau (H v)_c for own columns c, one warp each
-      for (int k = k0 + warp; k < nc; k += TNT / 32) {
-        const int c = me + k * G;
+      const int parts = na <= 2 ? 4 : na <= 4 ? 2 : 1;
+      for (int w = warp; w < na * parts; w += NW) {
+        const int k = k0 + w / parts, p = w - (k - k0) * parts;
         const T* col = column(k);
         T s = Sc<T>::zero();
-        for (int i = j + 1 + lane; i < l; i += 32) Sc<T>::fmac(s, col[i], STAGE ? vs[i] : ld_cg(vg + i));
-        s = Sc<T>::mul(t, warp_addt(s));
-        if (lane == 0) {
-          xg[c] = s;
-          sx[k] = Sc<T>::mul(Sc<T>::conj(s), STAGE ? vs[c] : ld_cg(vg + c));
-        }
+        for (int i = j + 1 + 32 * p + lane; i < l; i += 32 * parts) Sc<T>::fmac(s, col[i], vs[i]);
+        s = warp_addt(s);
+        if (lane == 0) sp[(size_t)k * 4 + p] = s;
       }
       __syncthreads();
-      if (tid == 0) {
-        T s = Sc<T>::zero();
-        for (int k = k0; k < nc; ++k) s = Sc<T>::add(s, sx[k]);
-        part[(size_t)par * G + me] = s;
+      if (warp == 0) {
+        double a = 0.0;
+        for (int k = k0 + lane; k < nc; k += 32) {
+          T s = sp[(size_t)k * 4];
+          for (int p = 1; p < parts; ++p) s = Sc<T>::add(s, sp[(size_t)k * 4 + p]);
+          s = Sc<T>::mul(t, s);
+          const int c = me + k * G;
+          if (G > 1) xg[c] = s;
+          else xs[c] = s;
+          a += Sc<T>::re(Sc<T>::mul(t, Sc<T>::mul(Sc<T>::conj(s), vs[c])));
+        }
+        if (na <= 1) a = __shfl_sync(0xffffffffu, a, 0);
+        else a = warp_add(a);
+        if (lane == 0) {
+          if (G > 1) part[(size_t)par * G + me] = a;
+          else sh_alpha = -0.5 * a;
+        }
       }
-      if (!grid_barrier(&tb->bar, G, bars)) {
+    }
+    if (G > 1) {
+      if (next_mine)
+        for (int i = j + 1 + tid; i < l; i += TNT) cg[i] = column(k0)[i];
+      if (!grid_barrier(gb, G, bars)) {
         if (tid == 0) atomicOr(&dst->timeout, 16);
         return;
       }
-      // alpha = -1/2 tau x^H v (every CTA the same sum in the same order)
       if (warp == 0) {
-        T s = Sc<T>::zero();
-        for (int b = lane; b < G; b += 32) s = Sc<T>::add(s, ld_cg(part + (size_t)par * G + b));
-        s = Sc<T>::scale(Sc<T>::mul(t, warp_addt(s)), -0.5);
-        if (lane == 0) sh_alpha = s;
+        if (!trivial) {
+          double a = 0.0;
+          for (int b = lane; b < G; b += 32) a += __ldcg(part + (size_t)par * G + b);
+          a = warp_add(a);
+          if (lane == 0) sh_alpha = -0.5 * a;
+        }
+      } else {
+        for (int i = j + 1 + tid - 32; i < l; i += TNT - 32) {
+          if (!trivial) xs[i] = ld_cg(xg + i);
+          us[i] = ld_cg(cg + i);
+        }
       }
-      if (STAGE)
-        for (int i = j + 1 + tid; i < l; i += TNT) xs[i] = ld_cg(xg + i);
-      __syncthreads();
       par ^= 1;
-    }
-    const T al = sh_alpha;
-    // own column k: H[:, c] -= v conj(w_c) + w conj(v_c), w = x + alpha v
-    auto update = [&](int k, int i0, int step) {
-      const int c = me + k * G;
-      T* col = column(k);
-      const T vc = Sc<T>::conj(STAGE ? vs[c] : ld_cg(vg + c)), xc = Sc<T>::conj(STAGE ? xs[c] : ld_cg(xg + c));
-      // conj(w_c) + alpha conj(v_c) = conj(x_c) + 2 Re(alpha) conj(v_c)
-      const T q = Sc<T>::scale(Sc<T>::add(xc, Sc<T>::scale(vc, 2.0 * Sc<T>::re(al))), -1.0);
-      const T nvc = Sc<T>::scale(vc, -1.0);
-      for (int i = j + 1 + i0; i < l; i += step) {
-        T h = col[i];
-        Sc<T>::fma(h, STAGE ? vs[i] : ld_cg(vg + i), q);
-        Sc<T>::fma(h, STAGE ? xs[i] : ld_cg(xg + i), nvc);
-        col[i] = h;
-      }
-    };
-    int kr = k0;
-    if ((j + 1) % G == me) {  // the next reflector's column first
-      if (!trivial) update(k0, tid, TNT);
+    } else {
       __syncthreads();
-      publish(j + 1);
-      kr = k0 + 1;
+      for (int i = j + 1 + tid; i < l; i += TNT) us[i] = column(k0)[i];
     }
-    if (!trivial)
-      for (int k = kr + warp; k < nc; k += TNT / 32) update(k, lane, 32);
+    __syncthreads();
+    const double al = trivial ? 0.0 : sh_alpha;
+    // H[:, c] -= v conj(w_c) + w conj(v_c) = v q + x p with q = -(conj(x_c) + 2 alpha conj(v_c)),
+    // p = -conj(v_c)
+    auto factors = [&](int c, T* q, T* p) {
+      const T vc = Sc<T>::conj(vs[c]);
+      *q = Sc<T>::scale(Sc<T>::add(Sc<T>::conj(xs[c]), Sc<T>::scale(vc, 2.0 * al)), -1.0);
+      *p = Sc<T>::scale(vc, -1.0);
+    };
+    if (!trivial) {
+      T q, p;
+      factors(j + 1, &q, &p);
+      double s = 0.0;
+      for (int i = j + 1 + tid; i < l; i += TNT) {
+        T h = us[i];
+        Sc<T>::fma(h, vs[i], q);
+        Sc<T>::fma(h, xs[i], p);
+        us[i] = h;
+        if (i >= j + 3) s += Sc<T>::abs2(h);
+      }
+      norm_part(s);
+      for (int k = k0 + tid; k < nc; k += TNT) factors(me + k * G, sq + 2 * k, sq + 2 * k + 1);
+    } else {
+      double s = 0.0;
+      for (int i = j + 3 + tid; i < l; i += TNT) s += Sc<T>::abs2(us[i]);
+      norm_part(s);
+    }
+    __syncthreads();
+    if (j + 2 == l) {  // the last diagonal entry
+      if (next_mine && tid == 0) d[j + 1] = Sc<T>::re(us[j + 1]);
+      return;
+    }
+    if (tid == 0) scalars(j + 1, us);
+    if (!trivial && warp != 0 && warp != NW / 2) {  // (warp NW / 2 shares warp 0's FP64 pipe)
+      // chunks of 32 rows of every own column after j + 1, over the other warps
+      const int wi = warp < NW / 2 ? warp - 1 : warp - 2, kf = k0 + (next_mine ? 1 : 0);
+      const int ch = (l - j - 1 + 31) / 32;
+      for (int w = wi; w < (nc - kf) * ch; w += NW - 2) {
+        const int k = kf + w / ch, i = j + 1 + 32 * (w - (k - kf) * ch) + lane;
+        if (i < l) {
+          T* col = column(k);
+          T h = col[i];
+          Sc<T>::fma(h, vs[i], sq[2 * k]);
+          Sc<T>::fma(h, xs[i], sq[2 * k + 1]);
+          col[i] = h;
+        }
+      }
+    }
+    __syncthreads();
+    finish_reflector(j + 1, us);
     __syncthreads();
   }
 }
@@ -258,15 +306,33 @@ struct WarpGroup {
     return v;
   }
 };
+// `width` lanes (a power of two) of a warp, `group` of them counted.
 struct Lanes {
-  int lane, width;
-  __device__ double sum(double v) const { return warp_add(v); }
-  __device__ double prod(double v) const {
-    for (int o = 16; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
+  int lane, width, group;
+  __device__ explicit Lanes(int w) : lane(threadIdx.x & (w - 1)), width(w), group((threadIdx.x & 31) / w) {}
+  __device__ double sum(double v) const {
+    for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
   }
-  __device__ int count(int v) const { return __reduce_add_sync(0xffffffffu, v); }
+  __device__ double prod(double v) const {
+    for (int o = width >> 1; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  }
+  __device__ int count(int v) const {
+    for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  }
+  __device__ bool any(bool v) const { return __any_sync(0xffffffffu, v); }
 };
+// f(i, write) for the items [0, n) of a merge, one per group of lanes: warp w of nw.
+template <class F>
+__device__ __forceinline__ void for_items(const Lanes& L, int w, int nw, int n, const F& f) {
+  const int per = 32 / L.width;
+  for (int i0 = w * per; i0 < n; i0 += nw * per) {
+    const int i = i0 + L.group;
+    f(min(i, n - 1), i < n);
+  }
+}
 
 // Arrays of one problem of order n (offsets of `batch` problems are uniform strides).
 struct DcWork {
@@ -349,20 +415,24 @@ __device__ inline void dc_rotate_row(const dc::Merge& M, double* Qb, int ldq, in
 }
 
 // One merge by one group (a warp or a CTA of nw warps) on local arrays: Q's block is replaced.
+// width: lanes per root, so that the roots of a merge fill the group's warps (an iteration's
+// scalar FP64 work, ~40 instructions of 64 clocks, is then shared by 32 / width roots).
 template <class G>
-__device__ inline void dc_merge_local(const G& g, int w, int nw, const dc::Merge& M, double* D, double* Dn,
+__device__ inline void dc_merge_local(const G& g, int w, int nw, int width, const dc::Merge& M, double* D, double* Dn,
                                       double* Qb, double* Qn, double* U, int ldq) {
-  const Lanes L{(int)(threadIdx.x & 31), 32};
+  const Lanes L(width);
   const int m = M.m;
   dc::setup(g, M, Qb + M.n1 - 1, Qb + M.n1 + (size_t)M.n1 * ldq, ldq);
   const int K = M.cnt[0];
-  for (int k = w; k < K; k += nw) dc::root(L, K, k, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+  for_items(L, w, nw, K, [&](int k, bool wr) {
+    dc::root(L, K, k, wr, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+  });
   for (int i = g.tid; i < m; i += g.size) dc_rotate_row(M, Qb, ldq, i);
   g.sync();
-  for (int k = w; k < K; k += nw) dc::zhat(L, K, k, M.dl, M.w, M.mu, M.org, M.zh);
+  for_items(L, w, nw, K, [&](int k, bool wr) { dc::zhat(L, K, k, wr, M.dl, M.w, M.mu, M.org, M.zh); });
   g.sync();
-  for (int k = w; k < K; k += nw) dc::ucol(L, K, k, M.dl, M.zh, M.mu, M.org, M.pos, U, ldq);
-  for (int t = w; t < m; t += nw) dc::place(L, M, K, t);
+  for_items(L, w, nw, K, [&](int k, bool wr) { dc::ucol(L, K, k, wr, M.dl, M.zh, M.mu, M.org, M.pos, U, ldq); });
+  for_items(L, w, nw, m, [&](int t, bool wr) { dc::place(L, M, K, t, wr); });
   g.sync();
   for (int u = g.tid; u < m * m; u += g.size) {
     const int i = u % m, j = u / m;
@@ -418,10 +488,10 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
       const dc::Merge M = dc_merge(V, 0, a, b, c, e[s + b - 1]);
       double* Qb = sQ + a + a * LEAF;
       if (by_warp)
-        dc_merge_local(WarpGroup{lane, 32}, 0, 1, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
+        dc_merge_local(WarpGroup{lane, 32}, 0, 1, h == 4 ? 16 : h == 3 ? 8 : 4, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
                        sU + a + a * LEAF, LEAF);
       else
-        dc_merge_local(CtaGroup{tid, 256, s_red}, warp, 8, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
+        dc_merge_local(CtaGroup{tid, 256, s_red}, warp, 8, h == 1 ? 16 : 8, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
                        sU + a + a * LEAF, LEAF);
     }
     __syncthreads();
@@ -454,19 +524,19 @@ __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride,
   const DcWork W = dc_at(W0, stride * blockIdx.z);
   int s;
   const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, e0 + (size_t)blockIdx.z * ld_de, &s);
-  const Lanes L{(int)(threadIdx.x & 31), 32};
+  const Lanes L(32);
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5), nw = gridDim.x * 4;
   const int K = M.cnt[0];
   if (phase == 0) {
-    for (int k = w; k < K; k += nw) dc::root(L, K, k, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+    for (int k = w; k < K; k += nw) dc::root(L, K, k, true, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
     double* Qb = W.Q[cur] + s + (size_t)s * W.n;
     for (int i = blockIdx.x * 128 + threadIdx.x; i < M.m; i += gridDim.x * 128) dc_rotate_row(M, Qb, W.n, i);
   } else if (phase == 1) {
-    for (int k = w; k < K; k += nw) dc::zhat(L, K, k, M.dl, M.w, M.mu, M.org, M.zh);
+    for (int k = w; k < K; k += nw) dc::zhat(L, K, k, true, M.dl, M.w, M.mu, M.org, M.zh);
   } else {
     double* Ub = W.U + s + (size_t)s * W.n;
-    for (int k = w; k < K; k += nw) dc::ucol(L, K, k, M.dl, M.zh, M.mu, M.org, M.pos, Ub, W.n);
-    for (int t = w; t < M.m; t += nw) dc::place(L, M, K, t);
+    for (int k = w; k < K; k += nw) dc::ucol(L, K, k, true, M.dl, M.zh, M.mu, M.org, M.pos, Ub, W.n);
+    for (int t = w; t < M.m; t += nw) dc::place(L, M, K, t, true);
   }
 }
 
@@ -618,8 +688,11 @@ int tridiag_pass(int m, int batch) {
 }
 
 struct EighLayout {
-  size_t tau, d, e, xb, part, tb, dc, total;
+  size_t tau, d, e, xb, cb, part, scr, tb, dc, total;
 };
+// Shared memory of the reduction: partial sums and factors of the own columns, three vectors.
+size_t tri_fixed_smem(int l, int own, size_t elem) { return elem * (6 * (size_t)own + 3 * (size_t)l); }
+bool tri_vec_smem(int l, size_t elem) { return tri_fixed_smem(l, ceil_div(l, kNumSMs), elem) <= kSmemMax - 1024; }
 EighLayout eigh_layout(int l, size_t elem) {
   EighLayout L{};
   size_t off = 0;
@@ -628,33 +701,46 @@ EighLayout eigh_layout(int l, size_t elem) {
   L.d = take(8 * (size_t)l);
   L.e = take(8 * (size_t)l);
   L.xb = take(2 * elem * l);
-  L.part = take(2 * elem * kNumSMs);
-  L.tb = take(sizeof(TriBar));
+  L.cb = take(2 * elem * l);
+  L.part = take(2 * 8 * kNumSMs);
+  L.scr = take(tri_vec_smem(l, elem) ? 0 : elem * 3 * (size_t)l * kNumSMs);
+  L.tb = take(sizeof(GridBar));
   L.dc = take(dc_bytes(l));
   L.total = off;
   return L;
 }
 
 template <class T>
-int tridiag(cudaStream_t st, int l, T* H, int ldh, T* tau, double* d, double* e, T* xb, T* part, TriBar* tb,
-            DevStatus* dst, int ctas, int* launches) {
-  // CTAs: enough that a column step's FP64 work per SM stays near the barrier's cost
+int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout& L, DevStatus* dst, int ctas,
+            int* launches) {
+  T *tau = (T*)(base + L.tau), *xb = (T*)(base + L.xb), *cb = (T*)(base + L.cb);
+  double *d = (double*)(base + L.d), *e = (double*)(base + L.e), *part = (double*)(base + L.part);
+  GridBar* gb = (GridBar*)(base + L.tb);
+  // CTAs: one for every 1000 elements (complex: x 4), one alone below 3000, where a column's
+  // FP64 work costs less than the grid barrier (measured: l = 30 real 0.142 ms on one CTA, 0.171
+  // on four; l = 60 real 0.417 and 0.343; l = 230 complex 1.95 on 38, 1.73 on 76)
   const double work = (double)l * l * (Sc<T>::cplx ? 4.0 : 1.0);
-  int G = (int)std::min<double>(kNumSMs, std::max(1.0, work / 6000.0));
+  int G = work < 3000.0 ? 1 : (int)std::min<double>(kNumSMs, work / 1000.0);
   if (ctas > 0) G = std::min(ctas, kNumSMs);
+  const bool vec = tri_vec_smem(l, sizeof(T));
+  if (!vec) G = kNumSMs;
   G = std::max(1, std::min(G, l));
-  const size_t own = ceil_div(l, G);
-  const bool stage = (2 * (size_t)l + own) * sizeof(T) <= kSmemMax - 1024;
-  size_t smem = ((stage ? 2 * (size_t)l : 0) + own) * sizeof(T);
-  int in_smem = smem + own * l * sizeof(T) <= kSmemMax - 1024;
-  if (in_smem) smem += own * l * sizeof(T);
-  void (*kern)(int, T*, int, int, T*, double*, double*, T*, T*, TriBar*, DevStatus*) =
-      stage ? tridiag_kernel<T, true> : tridiag_kernel<T, false>;
-  CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
-  CHASE_CUDA_TRY(cudaMemsetAsync(tb, 0, sizeof(TriBar), st));
-  void* args[] = {(void*)&l, (void*)&H, (void*)&ldh, (void*)&in_smem, (void*)&tau, (void*)&d,
-                  (void*)&e, (void*)&xb, (void*)&part, (void*)&tb, (void*)&dst};
-  CHASE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)kern, dim3(G), dim3(TNT), args, smem, st));
+  size_t smem;
+  for (;; ++G) {  // (fewer CTAs own more columns each)
+    smem = vec ? tri_fixed_smem(l, ceil_div(l, G), sizeof(T)) : sizeof(T) * 6 * (size_t)ceil_div(l, G);
+    if (smem <= kSmemMax - 1024 || G >= std::min(l, kNumSMs)) break;
+  }
+  if (smem > kSmemMax - 1024) return CHASE_ERR_UNSUPPORTED;
+  T* scr = vec ? nullptr : (T*)(base + L.scr);
+  const size_t cols = sizeof(T) * (size_t)ceil_div(l, G) * l;
+  int in_smem = smem + cols <= kSmemMax - 1024;
+  if (in_smem) smem += cols;
+  CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)tridiag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kSmemMax - 1024));
+  CHASE_CUDA_TRY(cudaMemsetAsync(gb, 0, sizeof(GridBar), st));
+  void* args[] = {(void*)&l,  (void*)&H,  (void*)&ldh,  (void*)&in_smem, (void*)&tau, (void*)&d,  (void*)&e,
+                  (void*)&xb, (void*)&cb, (void*)&part, (void*)&scr,     (void*)&gb,  (void*)&dst};
+  CHASE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)tridiag_kernel<T>, dim3(G), dim3(TNT), args, smem, st));
   if (launches) ++*launches;
   return 0;
 }
@@ -672,8 +758,7 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   char* base = (char*)work;
   T* tau = (T*)(base + L.tau);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e);
-  TRY_EIG(tridiag<T>(st, l, H, ldh, tau, d, e, (T*)(base + L.xb), (T*)(base + L.part), (TriBar*)(base + L.tb), dst,
-                     ctas, launches));
+  TRY_EIG(tridiag<T>(st, l, H, ldh, base, L, dst, ctas, launches));
   const DcWork D = dc_carve(base + L.dc, l);
   int cur = 0;
   TRY_EIG(stedc(st, l, 1, d, e, 0, D, 0, &cur, launches));

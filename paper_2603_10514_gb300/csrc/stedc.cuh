@@ -4,10 +4,11 @@
 // the secular equation's roots (Li's middle way inside a bracket), and the vector z that makes
 // the computed roots exact, so that the eigenvectors are orthogonal to working precision.
 //
-// Every step is written for a group of threads G (tid, size, sync, max over the group) or for a
-// warp L (lane, width, sums and products over its lanes); eigh.cu runs them over a warp, a CTA
-// or a grid.  All loops are bounded, and every index written is below m whatever the data
-// (NaN included).
+// Every step is written for a group of threads G (tid, size, sync, max over the group) or for
+// `width` lanes L of a warp (sums and products over them, any over the whole warp); eigh.cu runs
+// them over a warp, a CTA or a grid.  The groups of one warp call the L steps together: one that
+// has no item of its own takes another's and writes nothing (write = false).  All loops are
+// bounded, and every index written is below m whatever the data (NaN included).
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -151,42 +152,46 @@ DC_FN void setup(const G& g, const Merge& M, const double* q_last, const double*
 
 // Root k of 1 / rho + sum_i w_i^2 / (d_i - x) = 0 as mu = x - d_org, d_org the nearer pole.
 template <class L>
-DC_FN void root(const L& l, int K, int k, const double* dl, const double* w, double rho, double* mu_out,
-                int* org_out, double* lam_out) {
-  const double ri = 1.0 / rho;
-  int org, a, b;  // origin; the two poles of the interpolation
-  double lo, hi, mu;
+DC_FN void root(const L& l, int K, int k, bool write, const double* dl, const double* w, double rho,
+                double* mu_out, int* org_out, double* lam_out) {
   if (K == 1) {
-    if (l.lane == 0) { *mu_out = rho * w[0] * w[0]; *org_out = 0; *lam_out = dl[0] + rho * w[0] * w[0]; }
+    if (l.lane == 0 && write) { *mu_out = rho * w[0] * w[0]; *org_out = 0; *lam_out = dl[0] + rho * w[0] * w[0]; }
     return;
   }
-  if (k < K - 1) {
-    a = k; b = k + 1;
-    const double gap = dl[b] - dl[a], h = 0.5 * gap;
-    double s = 0.0;
-    for (int i = l.lane; i < K; i += l.width)
-      if (i != a && i != b) s += w[i] * (w[i] / ((dl[i] - dl[a]) - h));
-    const double c = ri + l.sum(s), wa = w[a] * w[a], wb = w[b] * w[b];
-    if (c + (wb - wa) / h > 0.0) {  // f(middle) > 0: the root lies in the left half
-      org = a; lo = 0.0; hi = h;
-      const double A = c * gap + wa + wb, B = wa * gap, q = sqrt(fabs(A * A - 4.0 * B * c));
+  const double ri = 1.0 / rho;
+  const bool inner = k < K - 1;
+  const int a = inner ? k : K - 2, b = a + 1;  // the two poles of the interpolation
+  const double gap = dl[b] - dl[a], h = 0.5 * gap;
+  // inner: the other terms of f in the middle of the interval; last: |w|^2
+  double s = 0.0;
+  for (int i = l.lane; i < K; i += l.width) {
+    const double t = inner ? w[i] / ((dl[i] - dl[a]) - h) : w[i];
+    if (!inner || (i != a && i != b)) s += w[i] * t;
+  }
+  s = l.sum(s);
+  int org = b;
+  double lo = 0.0, hi, mu;
+  if (inner) {
+    const double c = ri + s, wa = w[a] * w[a], wb = w[b] * w[b];
+    const bool left = c + (wb - wa) / h > 0.0;  // f(middle) > 0: the root lies in the left half
+    const double A = left ? c * gap + wa + wb : c * gap - wa - wb, B = left ? wa * gap : wb * gap;
+    const double q = sqrt(fabs(A * A + (left ? -4.0 : 4.0) * B * c));
+    if (left) {
+      org = a;
+      hi = h;
       mu = A > 0.0 ? 2.0 * B / (A + q) : (A - q) / (2.0 * c);
     } else {
-      org = b; lo = -h; hi = 0.0;
-      const double A = c * gap - wa - wb, B = wb * gap, q = sqrt(fabs(A * A + 4.0 * B * c));
+      lo = -h;
+      hi = 0.0;
       mu = A < 0.0 ? 2.0 * B / (A - q) : -(A + q) / (2.0 * c);
     }
   } else {
-    a = K - 2; b = K - 1;
-    org = b;
-    double s = 0.0;
-    for (int i = l.lane; i < K; i += l.width) s += w[i] * w[i];
-    lo = 0.0;
-    hi = rho * l.sum(s) * (1.0 + 4.0 * kEps);
+    hi = rho * s * (1.0 + 4.0 * kEps);
     mu = 0.5 * hi;
   }
   if (!(mu > lo && mu < hi)) mu = 0.5 * (lo + hi);
   const double dorg = dl[org];
+  bool act = true;
   for (int it = 0; it < 80; ++it) {
     double psi = 0.0, phi = 0.0, dpsi = 0.0, dphi = 0.0;
     for (int i = l.lane; i < K; i += l.width) {
@@ -196,35 +201,36 @@ DC_FN void root(const L& l, int K, int k, const double* dl, const double* w, dou
     }
     psi = l.sum(psi); phi = l.sum(phi); dpsi = l.sum(dpsi); dphi = l.sum(dphi);
     const double f = ri + psi + phi, df = dpsi + dphi;
-    if (!(fabs(f) > kEps * (8.0 * (fabs(psi) + fabs(phi)) + ri + fabs(mu) * df))) break;
-    if (f > 0.0) hi = mu; else lo = mu;
-    const double Da = (dl[a] - dorg) - mu, Db = (dl[b] - dorg) - mu;
-    double c = f - Da * dpsi - Db * dphi;
-    const double A = (Da + Db) * f - Da * Db * df, B = Da * Db * f;
-    double eta;
-    if (k < K - 1) {
+    act = act && fabs(f) > kEps * (8.0 * (fabs(psi) + fabs(phi)) + ri + fabs(mu) * df);
+    if (!l.any(act)) break;
+    if (act) {
+      if (f > 0.0) hi = mu; else lo = mu;
+      const double Da = (dl[a] - dorg) - mu, Db = (dl[b] - dorg) - mu;
+      double c = f - Da * dpsi - Db * dphi;
+      const double A = (Da + Db) * f - Da * Db * df, B = Da * Db * f;
+      // the middle way's step: inner roots (A - q) / 2c, the last one (A + q) / 2|c|
+      double sg = 1.0;
+      if (inner) sg = -1.0;
+      else c = fabs(c);
       const double q = sqrt(fabs(A * A - 4.0 * B * c));
-      if (c == 0.0) eta = B / A;
-      else eta = A <= 0.0 ? (A - q) / (2.0 * c) : 2.0 * B / (A + q);
-    } else {
-      c = fabs(c);
-      const double q = sqrt(fabs(A * A - 4.0 * B * c));
-      if (c == 0.0) eta = hi - mu;
-      else eta = A >= 0.0 ? (A + q) / (2.0 * c) : 2.0 * B / (A - q);
+      const bool direct = inner ? A <= 0.0 : A >= 0.0;
+      const double num = direct ? A + sg * q : 2.0 * B, den = direct ? 2.0 * c : A - sg * q;
+      double eta = num / den;
+      if (c == 0.0) eta = inner ? B / A : hi - mu;
+      if (!(f * eta < 0.0)) eta = -f / df;
+      double nx = mu + eta;
+      if (!(nx > lo && nx < hi)) nx = 0.5 * (lo + hi);
+      if (nx == mu || !(nx > lo && nx < hi)) act = false;  // the bracket is down to neighbours
+      else mu = nx;
     }
-    if (!(f * eta < 0.0)) eta = -f / df;
-    double nx = mu + eta;
-    if (!(nx > lo && nx < hi)) nx = 0.5 * (lo + hi);
-    if (nx == mu || !(nx > lo && nx < hi)) break;  // the bracket is down to neighbours
-    mu = nx;
   }
-  if (l.lane == 0) { *mu_out = mu; *org_out = org; *lam_out = dorg + mu; }
+  if (l.lane == 0 && write) { *mu_out = mu; *org_out = org; *lam_out = dorg + mu; }
 }
 
 // z_i for which the computed roots are the exact ones (Loewner's formula).
 template <class L>
-DC_FN void zhat(const L& l, int K, int i, const double* dl, const double* w, const double* mu, const int* org,
-                double* zh) {
+DC_FN void zhat(const L& l, int K, int i, bool write, const double* dl, const double* w, const double* mu,
+                const int* org, double* zh) {
   const double di = dl[i];
   double p = 1.0;
   for (int j = l.lane; j < K; j += l.width) {
@@ -232,13 +238,13 @@ DC_FN void zhat(const L& l, int K, int i, const double* dl, const double* w, con
     p *= (j == i) ? t : t / (di - dl[j]);
   }
   p = l.prod(p);
-  if (l.lane == 0) zh[i] = copysign(sqrt(fabs(p)), w[i]);
+  if (l.lane == 0 && write) zh[i] = copysign(sqrt(fabs(p)), w[i]);
 }
 
 // Column j of U (eigenvector of the rank-one update), rows in gather order, unit length.
 template <class L>
-DC_FN void ucol(const L& l, int K, int j, const double* dl, const double* zh, const double* mu, const int* org,
-                const int* pos, double* U, int ldu) {
+DC_FN void ucol(const L& l, int K, int j, bool write, const double* dl, const double* zh, const double* mu,
+                const int* org, const int* pos, double* U, int ldu) {
   const double dorg = dl[org[j]], m = mu[j];
   double s = 0.0;
   for (int i = l.lane; i < K; i += l.width) {
@@ -246,12 +252,13 @@ DC_FN void ucol(const L& l, int K, int j, const double* dl, const double* zh, co
     s += u * u;
   }
   const double r = 1.0 / sqrt(l.sum(s));
-  for (int i = l.lane; i < K; i += l.width) U[(size_t)pos[i] + (size_t)j * ldu] = zh[i] / ((dl[i] - dorg) - m) * r;
+  if (write)
+    for (int i = l.lane; i < K; i += l.width) U[(size_t)pos[i] + (size_t)j * ldu] = zh[i] / ((dl[i] - dorg) - m) * r;
 }
 
 // New position of value t (t < K: root t; else the deflated value t - K).
 template <class L>
-DC_FN void place(const L& l, const Merge& M, int K, int t) {
+DC_FN void place(const L& l, const Merge& M, int K, int t, bool write) {
   const int nd = M.m - K;
   int n = 0;
   double v;
@@ -269,7 +276,7 @@ DC_FN void place(const L& l, const Merge& M, int K, int t) {
     }
     n = l.count(n);
   }
-  if (l.lane == 0) M.dest[t] = n;
+  if (l.lane == 0 && write) M.dest[t] = n;
 }
 
 }  // namespace dc

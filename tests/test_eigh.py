@@ -30,7 +30,8 @@ DRIVER = r"""
 using namespace chase::dc;
 struct One { int tid = 0, size = 1; void sync() const {} double max(double v) const { return v; } };
 struct Lane { int lane = 0, width = 1; double sum(double v) const { return v; }
-              double prod(double v) const { return v; } int count(int v) const { return v; } };
+              double prod(double v) const { return v; } int count(int v) const { return v; }
+              bool any(bool v) const { return v; } };
 extern "C" void dc_solve(int n, const double* d, const double* e, double* D, double* Q) {
   std::vector<double> U((size_t)n * n), out((size_t)n * n);
   for (int i = 0; i < n; ++i) {
@@ -56,16 +57,16 @@ extern "C" void dc_solve(int n, const double* d, const double* e, double* D, dou
       double* B = Q + s + (size_t)s * n;
       setup(One(), M, B + M.n1 - 1, B + M.n1 + (size_t)M.n1 * n, n);
       const int K = cnt[0];
-      for (int k = 0; k < K; ++k) root(Lane(), K, k, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
+      for (int k = 0; k < K; ++k) root(Lane(), K, k, true, M.dl, M.w, M.rho, M.mu + k, M.org + k, M.lam + k);
       for (int r = 0; r < cnt[3]; ++r)
         for (int i = 0; i < m; ++i) {
           double &x = B[i + (size_t)M.rp[r] * n], &y = B[i + (size_t)M.rq[r] * n], a = x;
           x = M.rc[r] * a + M.rs[r] * y;
           y = M.rc[r] * y - M.rs[r] * a;
         }
-      for (int k = 0; k < K; ++k) zhat(Lane(), K, k, M.dl, M.w, M.mu, M.org, M.zh);
-      for (int k = 0; k < K; ++k) ucol(Lane(), K, k, M.dl, M.zh, M.mu, M.org, M.pos, U.data(), n);
-      for (int t = 0; t < m; ++t) place(Lane(), M, K, t);
+      for (int k = 0; k < K; ++k) zhat(Lane(), K, k, true, M.dl, M.w, M.mu, M.org, M.zh);
+      for (int k = 0; k < K; ++k) ucol(Lane(), K, k, true, M.dl, M.zh, M.mu, M.org, M.pos, U.data(), n);
+      for (int t = 0; t < m; ++t) place(Lane(), M, K, t, true);
       for (int j = 0; j < m; ++j)
         for (int i = 0; i < m; ++i) {
           double a = 0;
