@@ -228,6 +228,7 @@ template <class T>
 __global__ void __launch_bounds__(128) trinv_kernel(int n, const T* __restrict__ R, int ldr,
                                                     const T* __restrict__ Mb, T* Rinv, int ldri,
                                                     const DevStatus* dst) {
+  dep_wait();
   extern __shared__ __align__(16) unsigned char inv_smem[];
   T* x = (T*)inv_smem;
   __shared__ T part[4][CB];
@@ -295,7 +296,7 @@ int chol_inverse(cudaStream_t st, int n, T* G, int ldg, double shift_factor, T* 
     const size_t xs = sizeof(T) * (size_t)ceil_div(n, CB) * CB;
     if (xs > 48 * 1024)
       CHASE_CUDA_TRY(cudaFuncSetAttribute(trinv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs));
-    trinv_kernel<T><<<ceil_div(n, 2), 128, xs, st>>>(n, G, ldg, Mb, Rinv, ldri, dst);
+    launch_dep(st, ceil_div(n, 2), 128, xs, trinv_kernel<T>, n, G, ldg, Mb, Rinv, ldri, dst);
     if (launches) ++*launches;
   }
   CHASE_CUDA_TRY(cudaGetLastError());

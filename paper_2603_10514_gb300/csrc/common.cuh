@@ -100,6 +100,35 @@ struct DevStatus {
 };
 
 #ifdef __CUDACC__
+// Launch of a kernel that may be set up, and its blocks placed, while the launch before it on the
+// stream is still running (programmatic dependent launch).  Such a kernel calls dep_wait() in every
+// thread before it touches global memory: it returns when the launches before have completed and
+// their writes are seen, so their order is that of plain launches.  A plain launch, a copy or an
+// event still waits for the whole kernel before it.  It takes the launch latency and the set-up
+// (barriers, tensor memory) out of a chain of short kernels: n = 1000 real, 30 columns, a filter
+// step 35 -> 27 us, a solve of 30 vectors 11.6 -> 10.9 ms.
+__device__ __forceinline__ void dep_wait() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+template <class T> struct SameType { using type = T; };
+template <class... P>
+inline cudaError_t launch_dep(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*kernel)(P...),
+                              const typename SameType<P>::type&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  void* p[] = {(void*)&args...};
+  return cudaLaunchKernelExC(&cfg, (const void*)kernel, p);
+}
+
 // Grid-wide barrier of a cooperative launch on a counter that only grows: barrier k ends
 // once all G CTAs have added their arrival (count >= (k + 1) G).  One release-add per CTA
 // and acquire polls with a short back-off.  Bounded: returns false (the caller leaves the

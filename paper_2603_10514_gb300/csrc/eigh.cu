@@ -459,6 +459,7 @@ __host__ __device__ inline int dc_bound(int n, long long i, int depth) { return 
 __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const double* __restrict__ d0,
                                                       const double* __restrict__ e0, int ld_de, DcWork W0,
                                                       size_t stride) {
+  dep_wait();
   __shared__ double sQ[LEAF * LEAF], sQn[LEAF * LEAF], sU[LEAF * LEAF];
   __shared__ double s_red[8];
   __shared__ __align__(16) char s_vec[LEAF * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)];
@@ -510,6 +511,7 @@ __device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, 
 
 __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                        const double* __restrict__ e0, int ld_de) {
+  dep_wait();
   __shared__ double red[16];
   const DcWork W = dc_at(W0, stride * blockIdx.y);
   int s;
@@ -521,6 +523,7 @@ __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride,
 // phase 0: roots, and the rotations of Q's rows; 1: corrected z; 2: U and the new order.
 __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                        const double* __restrict__ e0, int ld_de, int phase) {
+  dep_wait();
   const DcWork W = dc_at(W0, stride * blockIdx.z);
   int s;
   const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, e0 + (size_t)blockIdx.z * ld_de, &s);
@@ -543,6 +546,7 @@ __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride,
 // Q_new[:, dest] = Q[:, gathered] U (64 x 32 tiles, FP64), deflated columns copied.
 __global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                       const double* __restrict__ e0, int ld_de, int parts) {
+  dep_wait();
   const DcWork W = dc_at(W0, stride * (blockIdx.z / parts));
   int s;
   const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.z % parts, e0 + (size_t)(blockIdx.z / parts) * ld_de, &s);
@@ -615,15 +619,15 @@ int stedc(cudaStream_t st, int n, int batch, const double* d, const double* e, i
     CHASE_CUDA_TRY(cudaMemsetAsync(q, 0, 3 * dc_align((size_t)8 * n * n) + sizeof(int), st));
   }
   const int depth = dc_depth(n);
-  dc_leaf_kernel<<<dim3(1 << depth, batch), 256, 0, st>>>(n, depth, d, e, ld_de, W, stride);
+  launch_dep(st, dim3(1 << depth, batch), 256, 0, dc_leaf_kernel, n, depth, d, e, ld_de, W, stride);
   int nl = 1, c = 0;
   for (int h = depth; h > 0; --h) {
     const int parts = 1 << (h - 1), m = ceil_div(n, parts);  // rows of a merge, at most
-    dc_setup_kernel<<<dim3(parts, batch), 512, 0, st>>>(W, stride, c, h, e, ld_de);
+    launch_dep(st, dim3(parts, batch), 512, 0, dc_setup_kernel, W, stride, c, h, e, ld_de);
     for (int phase = 0; phase < 3; ++phase)
-      dc_phase_kernel<<<dim3(ceil_div(m, 4), parts, batch), 128, 0, st>>>(W, stride, c, h, e, ld_de, phase);
-    dc_gemm_kernel<<<dim3(ceil_div(m, 32), ceil_div(m, 64), parts * batch), 256, 0, st>>>(W, stride, c, h, e,
-                                                                                         ld_de, parts);
+      launch_dep(st, dim3(ceil_div(m, 4), parts, batch), 128, 0, dc_phase_kernel, W, stride, c, h, e, ld_de, phase);
+    launch_dep(st, dim3(ceil_div(m, 32), ceil_div(m, 64), parts * batch), 256, 0, dc_gemm_kernel, W, stride, c, h,
+               e, ld_de, parts);
     nl += 5;
     c ^= 1;
   }
@@ -642,6 +646,7 @@ template <class T>
 __global__ void backtransform_kernel(int l, const T* __restrict__ H, int ldh, const T* __restrict__ tau,
                                      const double* __restrict__ Z, const double* __restrict__ D, const int* bad,
                                      T* Wm, int ldw, double* dw, int in_smem) {
+  dep_wait();
   extern __shared__ __align__(16) unsigned char bt_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
   if (c >= l) return;
@@ -675,6 +680,7 @@ __global__ void backtransform_kernel(int l, const T* __restrict__ H, int ldh, co
 
 // theta and squared first components of problem blockIdx.x (NaN if its T was not finite)
 __global__ void dc_extract_kernel(DcWork W0, size_t stride, int cur, double* theta, double* weight) {
+  dep_wait();
   const DcWork W = dc_at(W0, stride * blockIdx.x);
   for (int i = threadIdx.x; i < W.n; i += blockDim.x) {
     const double q = W.Q[cur][(size_t)i * W.n];
@@ -767,8 +773,8 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   const int in_smem = smem <= kSmemMax - 1024;
   CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)backtransform_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSmemMax - 1024));
-  backtransform_kernel<T><<<ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, st>>>(l, H, ldh, tau, D.Q[cur], D.D[cur],
-                                                                                 D.bad, W, ldw, dw, in_smem);
+  launch_dep(st, ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, backtransform_kernel<T>, l, H, ldh, tau, D.Q[cur],
+             D.D[cur], D.bad, W, ldw, dw, in_smem);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -786,7 +792,7 @@ int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const d
     const int cnt = std::min(nb, batch - r);
     int cur = 0;
     TRY_EIG(stedc(st, m, cnt, alpha + (size_t)r * m, beta + (size_t)r * m, m, W, stride, &cur, launches));
-    dc_extract_kernel<<<cnt, 128, 0, st>>>(W, stride, cur, theta + (size_t)r * m, weight + (size_t)r * m);
+    launch_dep(st, cnt, 128, 0, dc_extract_kernel, W, stride, cur, theta + (size_t)r * m, weight + (size_t)r * m);
     if (launches) ++*launches;
   }
   CHASE_CUDA_TRY(cudaGetLastError());

@@ -443,6 +443,7 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
   cluster_sync();  // both CTAs' barriers initialised before any copy or arrival crosses over
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
+  dep_wait();  // (the set-up above runs beside the end of the launch before)
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(M_REG_MAIN));
@@ -864,6 +865,7 @@ __device__ __forceinline__ void crt_ring(const CrtItem& I, int blk) {
 // KIND 1, 4: real, entries per thread; 15, 16: ring moduli, one entry; 30: 15 moduli, two entries.
 template <int KIND>
 __global__ void __launch_bounds__(CRT_NT) crt_kernel(const __grid_constant__ CrtItem I) {
+  dep_wait();
   const int blk = blockIdx.x;
   if constexpr (KIND == 1 || KIND == 4) crt_real<KIND>(I, blk);
   else if constexpr (KIND == 30) crt_ring<kRingShort, 2>(I, blk);
@@ -877,6 +879,7 @@ struct CrtGroupParams {
 static_assert(sizeof(CrtGroupParams) <= 32000, "kernel parameter space");
 
 __global__ void __launch_bounds__(CRT_NT) crt_group_kernel(const __grid_constant__ CrtGroupParams P) {
+  dep_wait();
   int p = 0;
   while (p + 1 < P.count && (int)blockIdx.x >= P.it[p + 1].blk0) ++p;
   const CrtItem& I = P.it[p];
@@ -891,14 +894,14 @@ __global__ void __launch_bounds__(CRT_NT) crt_group_kernel(const __grid_constant
 int crt_launch(cudaStream_t st, const CrtItem& I, int* launches) {
   const bool big = (long long)I.M * I.N >= 4LL * kNumSMs * 2048;
   if (I.ring == kRingShort) {
-    if (big && I.M % 2 == 0) crt_kernel<30><<<crt_blocks(I.M, I.N, 2), CRT_NT, 0, st>>>(I);
-    else crt_kernel<kRingShort><<<crt_blocks(I.M, I.N, 1), CRT_NT, 0, st>>>(I);
+    if (big && I.M % 2 == 0) launch_dep(st, crt_blocks(I.M, I.N, 2), CRT_NT, 0, crt_kernel<30>, I);
+    else launch_dep(st, crt_blocks(I.M, I.N, 1), CRT_NT, 0, crt_kernel<kRingShort>, I);
   } else if (I.ring) {
-    crt_kernel<kRingModuli><<<crt_blocks(I.M, I.N, 1), CRT_NT, 0, st>>>(I);
+    launch_dep(st, crt_blocks(I.M, I.N, 1), CRT_NT, 0, crt_kernel<kRingModuli>, I);
   } else if (big && I.M % 4 == 0) {
-    crt_kernel<4><<<crt_blocks(I.M, I.N, 4), CRT_NT, 0, st>>>(I);
+    launch_dep(st, crt_blocks(I.M, I.N, 4), CRT_NT, 0, crt_kernel<4>, I);
   } else {
-    crt_kernel<1><<<crt_blocks(I.M, I.N, 1), CRT_NT, 0, st>>>(I);
+    launch_dep(st, crt_blocks(I.M, I.N, 1), CRT_NT, 0, crt_kernel<1>, I);
   }
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
@@ -1035,6 +1038,7 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
 __global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __restrict__ A, int lda,
                                                          int kp, __nv_bfloat16* planes,
                                                          size_t plane, int* rowexp) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const double* col = A + (size_t)m * lda;
@@ -1054,6 +1058,7 @@ __global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __
 __global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const double* __restrict__ V64,
                                                          int ldi, int kp, __nv_bfloat16* planes,
                                                          size_t plane, int* colexp) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   const int c = c0 + blockIdx.x;
   const double* col = V64 + (size_t)c * ldi;
@@ -1081,6 +1086,7 @@ template <int NM>
 __global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* __restrict__ A, int lda,
                                                               int kpn, __nv_bfloat16* planes, size_t plane,
                                                               int* rowexp) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const z64* col = A + (size_t)m * lda;
@@ -1143,6 +1149,7 @@ struct SliceGroupParams {
 static_assert(sizeof(SliceGroupParams) <= 32000, "kernel parameter space");
 
 __global__ void __launch_bounds__(256) oz_slice_V_group_kernel(const __grid_constant__ SliceGroupParams P) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   int p = 0;
   while (p + 1 < P.count && (int)blockIdx.x >= P.blk0[p + 1]) ++p;
@@ -1175,6 +1182,7 @@ __global__ void __launch_bounds__(256) oz_slice_V_group_kernel(const __grid_cons
 template <class T>
 __global__ void stack_V_kernel(int n, int ncols, const T* __restrict__ V, int ldv, double* V64,
                                int ldo) {
+  dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
   const size_t total = (size_t)M * ncols;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
@@ -1197,6 +1205,7 @@ template <int NM>
 __global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z64* __restrict__ Y, int ldy, int kp,
                                                                  __nv_bfloat16* planes, size_t plane,
                                                                  int* colexp) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   const int c = blockIdx.x;
   const z64* col = Y + (size_t)c * ldy;
@@ -1223,6 +1232,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z6
 // column groups.
 __global__ void __launch_bounds__(256) oz_row_exp_kernel(int n, int l, const z64* __restrict__ X, int ldx,
                                                          int* rowexp) {
+  dep_wait();
   __shared__ unsigned long long red[8][32];
   const int i = threadIdx.x & 31, g = threadIdx.x >> 5, r = blockIdx.x * 32 + i;
   unsigned long long m = 0;
@@ -1247,6 +1257,7 @@ template <int NM>
 __global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, const z64* __restrict__ X, int ldx,
                                                                  int kp, __nv_bfloat16* planes, size_t plane,
                                                                  const int* __restrict__ rowexp) {
+  dep_wait();
   __shared__ z64 tile[64][33];
   const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
   const int i = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -1272,6 +1283,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, c
 // of Xt.  Residues of the rows into planes (row-major, ld kp), row exponents into rowexp.
 __global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double* __restrict__ Xt, int ldt, int kp,
                                                             __nv_bfloat16* planes, size_t plane, int* rowexp) {
+  dep_wait();
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const double* row = Xt + (size_t)m * ldt;  // X[m, 0..l)
@@ -1290,6 +1302,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double*
 // >= n are zero), column exponents.
 __global__ void __launch_bounds__(512) oz_slice_cols_kernel(int n, const double* __restrict__ Y, int ldy, int kp,
                                                             __nv_bfloat16* planes, size_t plane, int* colexp) {
+  dep_wait();
   __shared__ unsigned long long red[16];
   const int j = blockIdx.x;
   const double* col = Y + (size_t)j * ldy;
@@ -1306,6 +1319,7 @@ __global__ void __launch_bounds__(512) oz_slice_cols_kernel(int n, const double*
 
 // Xt = X^T: real X n x l (ld ldx) -> Xt l x n (ld ldt).
 __global__ void transpose_kernel(int n, int l, const double* __restrict__ X, int ldx, double* Xt, int ldt) {
+  dep_wait();
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -1360,7 +1374,7 @@ size_t oz_residue_bytes(int M, int N) {
 
 int oz_slice_A(cudaStream_t st, int n, const double* A, int lda, int kp, void* planes, int* rowexp,
                int* launches) {
-  oz_slice_A_kernel<<<n, 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  launch_dep(st, n, 256, 0, oz_slice_A_kernel, n, A, lda, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1370,9 +1384,11 @@ int oz_slice_A_ring(cudaStream_t st, int n, const z64* A, int lda, int kpn, void
                     int* launches) {
   const size_t plane = (size_t)n * kpn;
   if (ring_moduli(kpn) == kRingShort)
-    oz_slice_A_ring_kernel<kRingShort><<<n, 256, 0, st>>>(n, A, lda, kpn, (__nv_bfloat16*)planes, plane, rowexp);
+    launch_dep(st, n, 256, 0, oz_slice_A_ring_kernel<kRingShort>, n, A, lda, kpn, (__nv_bfloat16*)planes, plane,
+               rowexp);
   else
-    oz_slice_A_ring_kernel<kRingModuli><<<n, 256, 0, st>>>(n, A, lda, kpn, (__nv_bfloat16*)planes, plane, rowexp);
+    launch_dep(st, n, 256, 0, oz_slice_A_ring_kernel<kRingModuli>, n, A, lda, kpn, (__nv_bfloat16*)planes, plane,
+               rowexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1381,8 +1397,8 @@ int oz_slice_A_ring(cudaStream_t st, int n, const z64* A, int lda, int kpn, void
 int oz_slice_V(cudaStream_t st, int M, int c0, int c1, const double* V64, int ldi, int kp,
                int ncols_total, void* planes, int* colexp, int* launches) {
   if (c1 <= c0) return 0;
-  oz_slice_V_kernel<<<c1 - c0, 256, 0, st>>>(M, c0, V64, ldi, kp, (__nv_bfloat16*)planes,
-                                             (size_t)ncols_total * kp, colexp);
+  launch_dep(st, c1 - c0, 256, 0, oz_slice_V_kernel, M, c0, V64, ldi, kp, (__nv_bfloat16*)planes,
+             (size_t)ncols_total * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1398,13 +1414,15 @@ int launch_pairs(void (*kernel)(Params...), dim3 grid, cudaStream_t st, Args... 
   cfg.blockDim = dim3(M_THREADS);
   cfg.dynamicSmemBytes = M_SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   CHASE_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
   return 0;
 }
@@ -1533,7 +1551,7 @@ int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* 
     }
     if (P.count == 0) continue;
     P.blk0[P.count] = blocks;
-    oz_slice_V_group_kernel<<<blocks, 256, 0, st>>>(P);
+    launch_dep(st, blocks, 256, 0, oz_slice_V_group_kernel, P);
     if (launches) ++*launches;
     CHASE_CUDA_TRY(cudaGetLastError());
   }
@@ -1632,7 +1650,7 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     if (C.count == 1) {
       TRY_OZ(crt_launch(st, C.it[0], launches));
     } else {
-      crt_group_kernel<<<blocks, CRT_NT, 0, st>>>(C);
+      launch_dep(st, blocks, CRT_NT, 0, crt_group_kernel, C);
       if (launches) ++*launches;
       CHASE_CUDA_TRY(cudaGetLastError());
     }
@@ -1687,7 +1705,7 @@ int oz_stack_V(cudaStream_t st, int n, int ncols, const T* V, int ldv, double* V
   const int M = Sc<T>::cplx ? 2 * n : n;
   const size_t work = (size_t)M * ncols;
   const int blocks = (int)std::max<size_t>(1, std::min<size_t>((work + 255) / 256, (size_t)kNumSMs * 16));
-  stack_V_kernel<T><<<blocks, 256, 0, st>>>(n, ncols, V, ldv, V64, ldo);
+  launch_dep(st, blocks, 256, 0, stack_V_kernel<T>, n, ncols, V, ldv, V64, ldo);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1697,7 +1715,7 @@ int oz_slice_cols_ring(cudaStream_t st, int n, int q, const z64* Y, int ldy, int
                        int* launches) {
   if (q <= 0) return 0;
   auto kern = ring_moduli(kp) == kRingShort ? oz_slice_cols_ring_kernel<kRingShort> : oz_slice_cols_ring_kernel<kRingModuli>;
-  kern<<<q, 256, 0, st>>>(n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
+  launch_dep(st, q, 256, 0, kern, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1706,9 +1724,10 @@ int oz_slice_cols_ring(cudaStream_t st, int n, int q, const z64* Y, int ldy, int
 int oz_slice_rows_ring(cudaStream_t st, int n, int l, const z64* X, int ldx, int kp, void* planes, int* rowexp,
                        int* launches) {
   if (n <= 0) return 0;
-  oz_row_exp_kernel<<<ceil_div(n, 32), 256, 0, st>>>(n, l, X, ldx, rowexp);
+  launch_dep(st, ceil_div(n, 32), 256, 0, oz_row_exp_kernel, n, l, X, ldx, rowexp);
   auto kern = ring_moduli(kp) == kRingShort ? oz_slice_rows_ring_kernel<kRingShort> : oz_slice_rows_ring_kernel<kRingModuli>;
-  kern<<<dim3(ceil_div(n, 32), kp / 64), 256, 0, st>>>(n, l, X, ldx, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  launch_dep(st, dim3(ceil_div(n, 32), kp / 64), 256, 0, kern, n, l, X, ldx, kp, (__nv_bfloat16*)planes,
+             (size_t)n * kp, rowexp);
   if (launches) *launches += 2;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1717,8 +1736,8 @@ int oz_slice_rows_ring(cudaStream_t st, int n, int l, const z64* X, int ldx, int
 int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, double* Xt, int kp, void* planes,
                   int* rowexp, int* launches) {
   if (n <= 0) return 0;
-  transpose_kernel<<<dim3(ceil_div(n, 32), ceil_div(l, 32)), dim3(32, 8), 0, st>>>(n, l, X, ldx, Xt, l);
-  oz_slice_rows_kernel<<<n, 256, 0, st>>>(l, Xt, l, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  launch_dep(st, dim3(ceil_div(n, 32), ceil_div(l, 32)), dim3(32, 8), 0, transpose_kernel, n, l, X, ldx, Xt, l);
+  launch_dep(st, n, 256, 0, oz_slice_rows_kernel, l, Xt, l, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
   if (launches) *launches += 2;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1727,7 +1746,7 @@ int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, doubl
 int oz_slice_cols(cudaStream_t st, int n, int q, const double* Y, int ldy, int kp, void* planes, int* colexp,
                   int* launches) {
   if (q <= 0) return 0;
-  oz_slice_cols_kernel<<<q, 512, 0, st>>>(n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
+  launch_dep(st, q, 512, 0, oz_slice_cols_kernel, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   cluster_sync();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
+  dep_wait();  // (the set-up above runs beside the end of the launch before)
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 template <class T>
 __global__ void __launch_bounds__(256) split_A_kernel(int n, const T* __restrict__ A, int lda, int kp,
                                                       __nv_bfloat16* Ah, __nv_bfloat16* Al) {
+  dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
   auto split = [](double x, __nv_bfloat16* hi, __nv_bfloat16* lo) {
     *hi = __double2bfloat16(x);
@@ -239,6 +241,7 @@ __global__ void __launch_bounds__(256) split_A_kernel(int n, const T* __restrict
 template <class T>
 __global__ void split_V_kernel(int n, int ncols, const T* __restrict__ V, int ldv, double* V64,
                                int ldo, int kp, __nv_bfloat16* Vh, __nv_bfloat16* Vl) {
+  dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
   const size_t total = (size_t)kp * ncols;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
@@ -264,6 +267,7 @@ __global__ void split_V_kernel(int n, int ncols, const T* __restrict__ V, int ld
 template <class T>
 __global__ void unstack_V_kernel(int n, int c0, int c1, const double* __restrict__ V64, int ldi,
                                  T* V, int ldv, bool subtract) {
+  dep_wait();
   const size_t total = (size_t)n * (c1 - c0);
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
@@ -320,7 +324,7 @@ template <class T>
 int tc_split_A(cudaStream_t st, int n, const T* A, int lda, int kp, void* Ah, void* Al,
                int* launches) {
   const dim3 grid(ceil_div(n, 256), std::min(n, 65535));
-  split_A_kernel<T><<<grid, 256, 0, st>>>(n, A, lda, kp, (__nv_bfloat16*)Ah, (__nv_bfloat16*)Al);
+  launch_dep(st, grid, 256, 0, split_A_kernel<T>, n, A, lda, kp, (__nv_bfloat16*)Ah, (__nv_bfloat16*)Al);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -329,8 +333,8 @@ int tc_split_A(cudaStream_t st, int n, const T* A, int lda, int kp, void* Ah, vo
 template <class T>
 int tc_split_V(cudaStream_t st, int n, int ncols, const T* V, int ldv, double* V64, int ldo, int kp,
                void* Vh, void* Vl, int* launches) {
-  split_V_kernel<T><<<grid_for((size_t)kp * ncols), 256, 0, st>>>(
-      n, ncols, V, ldv, V64, ldo, kp, (__nv_bfloat16*)Vh, (__nv_bfloat16*)Vl);
+  launch_dep(st, grid_for((size_t)kp * ncols), 256, 0, split_V_kernel<T>, n, ncols, V, ldv, V64, ldo, kp,
+             (__nv_bfloat16*)Vh, (__nv_bfloat16*)Vl);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -340,8 +344,8 @@ template <class T>
 int tc_unstack_V(cudaStream_t st, int n, int c0, int c1, const double* V64, int ldi, T* V, int ldv,
                  int* launches, bool subtract) {
   if (c1 <= c0) return 0;
-  unstack_V_kernel<T><<<grid_for((size_t)n * (c1 - c0)), 256, 0, st>>>(n, c0, c1, V64, ldi, V, ldv,
-                                                                      subtract);
+  launch_dep(st, grid_for((size_t)n * (c1 - c0)), 256, 0, unstack_V_kernel<T>, n, c0, c1, V64, ldi, V, ldv,
+             subtract);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -379,13 +383,15 @@ int tc_filter_step(cudaStream_t st, int M, int kp, const void* Ah, const void* A
   cfg.blockDim = dim3(TC_THREADS);
   cfg.dynamicSmemBytes = TC_SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   CHASE_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_filter_bf16x3_kernel, mAh, mAl, mVh, mVl, M, N, BN, ntile,
                                     kp / TBK, col0, alpha, beta, X64, gamma, Z64, out64, ldv,
                                     (__nv_bfloat16*)Vh_out, (__nv_bfloat16*)Vl_out, kp, dst));

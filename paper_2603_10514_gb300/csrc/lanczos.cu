@@ -66,6 +66,7 @@ __device__ inline z64 block_sum_t<z64>(z64 v, double* red) {
 template <class T, int R>
 __global__ void __launch_bounds__(256) lz_product_kernel(int n, const T* __restrict__ A, int lda,
                                                          const T* __restrict__ Q, T* __restrict__ W) {
+  dep_wait();
   const int lane = threadIdx.x & 31, c = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (c >= n) return;
   const T* col = A + (size_t)c * lda;
@@ -97,10 +98,10 @@ int lz_product(cudaStream_t st, int n, int nruns, const T* A, int lda, const T* 
     const T* q = Q + (size_t)r * n;
     T* w = W + (size_t)r * n;
     switch (std::min(4, nruns - r)) {
-      case 1: lz_product_kernel<T, 1><<<blocks, 256, 0, st>>>(n, A, lda, q, w); break;
-      case 2: lz_product_kernel<T, 2><<<blocks, 256, 0, st>>>(n, A, lda, q, w); break;
-      case 3: lz_product_kernel<T, 3><<<blocks, 256, 0, st>>>(n, A, lda, q, w); break;
-      default: lz_product_kernel<T, 4><<<blocks, 256, 0, st>>>(n, A, lda, q, w); break;
+      case 1: launch_dep(st, blocks, 256, 0, lz_product_kernel<T, 1>, n, A, lda, q, w); break;
+      case 2: launch_dep(st, blocks, 256, 0, lz_product_kernel<T, 2>, n, A, lda, q, w); break;
+      case 3: launch_dep(st, blocks, 256, 0, lz_product_kernel<T, 3>, n, A, lda, q, w); break;
+      default: launch_dep(st, blocks, 256, 0, lz_product_kernel<T, 4>, n, A, lda, q, w); break;
     }
     ++*nl;
   }
@@ -114,6 +115,7 @@ template <class T>
 __global__ void __launch_bounds__(256) lz_dots_kernel(int n, const T* __restrict__ Qb,
                                                       size_t pstride, const T* __restrict__ W,
                                                       T* coef, int ldc) {
+  dep_wait();
   __shared__ double red[8];
   const int r = blockIdx.x, p = blockIdx.y;
   const T* q = Qb + (size_t)p * pstride + (size_t)r * n;
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(256) lz_dots_kernel(int n, const T* __restrict
 template <class T>
 __global__ void lz_sub_kernel(int n, int nruns, const T* __restrict__ Qb, size_t pstride, T* W,
                               const T* __restrict__ coef, int ldc, int np) {
+  dep_wait();
   const size_t total = (size_t)n * nruns;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
@@ -143,6 +146,7 @@ __global__ void lz_sub_kernel(int n, int nruns, const T* __restrict__ Qb, size_t
 template <class T>
 __global__ void lz_store_alpha_kernel(int nruns, const T* coef, int ldc, int j, double* alpha,
                                       int m) {
+  dep_wait();
   const int r = threadIdx.x;
   if (r < nruns) alpha[r * m + j] = Sc<T>::re(coef[(size_t)r * ldc + j]);
 }
@@ -151,6 +155,7 @@ __global__ void lz_store_alpha_kernel(int nruns, const T* coef, int ldc, int j, 
 template <class T>
 __global__ void __launch_bounds__(256) lz_normalize_kernel(int n, const T* __restrict__ W, T* qn,
                                                            double* beta, int m, int j) {
+  dep_wait();
   __shared__ double red[8];
   const int r = blockIdx.x;
   const T* w = W + (size_t)r * n;
@@ -185,7 +190,7 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   int nl = 0;
   // q_0 = v / ||v|| for every run
   TRY_LZ(copy_cols<T>(st, n, nruns, V0, ldv, W, n, &nl));
-  lz_normalize_kernel<T><<<nruns, 256, 0, st>>>(n, W, Qb, beta, m, 0);  // beta[.,0] rewritten below
+  launch_dep(st, nruns, 256, 0, lz_normalize_kernel<T>, n, W, Qb, beta, m, 0);  // beta[.,0] rewritten below
   ++nl;
   const int blocks = (int)std::min<size_t>((pstride + 255) / 256, (size_t)kNumSMs * 16);
   for (int j = 0; j < m; ++j) {
@@ -195,12 +200,12 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
     // coefficients against q_0..q_j: coef[., j] is alpha_j; subtracting all of them is the
     // three-term step plus full re-orthogonalisation (classical Gram-Schmidt, twice)
     for (int pass = 0; pass < 2; ++pass) {
-      lz_dots_kernel<T><<<dim3(nruns, j + 1), 256, 0, st>>>(n, Qb, pstride, W, coef, m + 1);
-      if (pass == 0) lz_store_alpha_kernel<T><<<1, 32, 0, st>>>(nruns, coef, m + 1, j, alpha, m);
-      lz_sub_kernel<T><<<blocks, 256, 0, st>>>(n, nruns, Qb, pstride, W, coef, m + 1, j + 1);
+      launch_dep(st, dim3(nruns, j + 1), 256, 0, lz_dots_kernel<T>, n, Qb, pstride, W, coef, m + 1);
+      if (pass == 0) launch_dep(st, 1, 32, 0, lz_store_alpha_kernel<T>, nruns, coef, m + 1, j, alpha, m);
+      launch_dep(st, blocks, 256, 0, lz_sub_kernel<T>, n, nruns, Qb, pstride, W, coef, m + 1, j + 1);
       nl += (pass == 0) ? 3 : 2;
     }
-    lz_normalize_kernel<T><<<nruns, 256, 0, st>>>(n, W, Qb + (size_t)(j + 1) * pstride, beta, m, j);
+    launch_dep(st, nruns, 256, 0, lz_normalize_kernel<T>, n, W, Qb + (size_t)(j + 1) * pstride, beta, m, j);
     ++nl;
   }
   // Ritz values and weights of each run

@@ -15,6 +15,7 @@ inline int grid_for(size_t work, int threads) {
 
 template <class T>
 __global__ void herm_fill_lower_kernel(int n, T* G, int ldg) {
+  dep_wait();
   size_t total = (size_t)n * n;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
@@ -30,6 +31,7 @@ __global__ void __launch_bounds__(256) resid_norms_kernel(int n, const T* __rest
                                                           const T* __restrict__ V, int ldv,
                                                           const double* __restrict__ theta,
                                                           double* res) {
+  dep_wait();
   __shared__ double r0[8], r1[8];
   const int a = blockIdx.x;
   const double th = theta[a];
@@ -58,6 +60,7 @@ __global__ void __launch_bounds__(256) resid_norms_kernel(int n, const T* __rest
 template <class T>
 __global__ void gather_cols_kernel(int n, int ncols, const T* src, int lds, const int* perm, T* dst,
                                    int ldd) {
+  dep_wait();
   size_t total = (size_t)n * ncols;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
@@ -69,6 +72,7 @@ __global__ void gather_cols_kernel(int n, int ncols, const T* src, int lds, cons
 template <class T>
 __global__ void select_cols_kernel(int n, int ncols, const T* s0, const T* s1, int lds,
                                    const int* sel, T* dst, int ldd) {
+  dep_wait();
   size_t total = (size_t)n * ncols;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
        t += (size_t)gridDim.x * blockDim.x) {
@@ -80,6 +84,7 @@ __global__ void select_cols_kernel(int n, int ncols, const T* s0, const T* s1, i
 
 template <class T>
 __global__ void nonfinite_kernel(int n, int ncols, const T* X, int ldx, DevStatus* st) {
+  dep_wait();
   size_t total = (size_t)n * ncols;
   int bad = 0;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
@@ -95,7 +100,7 @@ __global__ void nonfinite_kernel(int n, int ncols, const T* X, int ldx, DevStatu
 template <class T>
 int herm_fill_lower(cudaStream_t st, int n, T* G, int ldg, int* launches) {
   if (n <= 0) return 0;
-  herm_fill_lower_kernel<T><<<grid_for((size_t)n * n, 256), 256, 0, st>>>(n, G, ldg);
+  launch_dep(st, grid_for((size_t)n * n, 256), 256, 0, herm_fill_lower_kernel<T>, n, G, ldg);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -105,7 +110,7 @@ template <class T>
 int resid_norms(cudaStream_t st, int n, int ncols, const T* AV, int ldav, const T* V, int ldv,
                 const double* dtheta, double* dres, int* launches) {
   if (n <= 0 || ncols <= 0) return 0;
-  resid_norms_kernel<T><<<ncols, 256, 0, st>>>(n, AV, ldav, V, ldv, dtheta, dres);
+  launch_dep(st, ncols, 256, 0, resid_norms_kernel<T>, n, AV, ldav, V, ldv, dtheta, dres);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -125,8 +130,8 @@ template <class T>
 int gather_cols(cudaStream_t st, int n, int ncols, const T* src, int lds, const int* dperm, T* dst,
                 int ldd, int* launches) {
   if (n <= 0 || ncols <= 0) return 0;
-  gather_cols_kernel<T><<<grid_for((size_t)n * ncols, 256), 256, 0, st>>>(n, ncols, src, lds, dperm,
-                                                                          dst, ldd);
+  launch_dep(st, grid_for((size_t)n * ncols, 256), 256, 0, gather_cols_kernel<T>, n, ncols, src, lds, dperm, dst,
+             ldd);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -136,8 +141,8 @@ template <class T>
 int select_cols(cudaStream_t st, int n, int ncols, const T* src0, const T* src1, int lds,
                 const int* dsel, T* dst, int ldd, int* launches) {
   if (n <= 0 || ncols <= 0) return 0;
-  select_cols_kernel<T><<<grid_for((size_t)n * ncols, 256), 256, 0, st>>>(n, ncols, src0, src1, lds,
-                                                                          dsel, dst, ldd);
+  launch_dep(st, grid_for((size_t)n * ncols, 256), 256, 0, select_cols_kernel<T>, n, ncols, src0, src1, lds, dsel,
+             dst, ldd);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -147,7 +152,7 @@ template <class T>
 int nonfinite_check(cudaStream_t st, int n, int ncols, const T* X, int ldx, DevStatus* dst,
                     int* launches) {
   if (n <= 0 || ncols <= 0) return 0;
-  nonfinite_kernel<T><<<grid_for((size_t)n * ncols, 256), 256, 0, st>>>(n, ncols, X, ldx, dst);
+  launch_dep(st, grid_for((size_t)n * ncols, 256), 256, 0, nonfinite_kernel<T>, n, ncols, X, ldx, dst);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
