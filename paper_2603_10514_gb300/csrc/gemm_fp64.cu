@@ -9,162 +9,147 @@
 // thread that then writes the same element of C, which is what lets the filter
 // write V_i over V_{i-2} in place.
 //
-// GB300 has 2 FP64 FMA lanes per SM per clock (~1.2 TFLOP/s for the whole GPU,
-// measured), so these products are bound by the FP64 pipe, not by HBM: a
-// 64 x (16|32) register-tiled SIMT kernel keeps that pipe busy, and the design
-// work goes into load balance across the 152 SMs.  Work is cut into
-// (row tile, column tile, K chunk) units, with enough K chunks (split-K) that
-// every SM receives ~8 units; partial sums go to scratch memory and a second
-// kernel reduces them in a fixed order (deterministic results) and applies the
-// epilogue.
+// GB300 issues 2 FP64 FMAs per SM per clock (~1.2 TFLOP/s for the whole GPU, measured), so a warp's
+// FP64 instruction holds its sub-partition for 64 clocks and nothing else binds these products:
+// not HBM, not shared memory.  What counts is that every sub-partition has the same number of
+// them and that none is spent on padding.
+//   - Tiles of 64 rows by up to 64 columns, the columns shared out evenly over the tiles.  A warp
+//     takes 32 rows and every fourth column, so a tile costs its own columns, not a multiple of
+//     16 or 32; the odd columns fall on other sub-partitions in every second CTA.
+//   - One wave of two CTAs per SM, each with the same number of single K steps, over tile borders
+//     (gemm_split.h): no last wave.  Tiles shared by CTAs have their parts summed in a fixed order
+//     by a second kernel, which applies the epilogue.
+// Against tiles of 64 x 32 (64 x 16) cut into equal K chunks, a step of the filter: n = 1531 complex,
+// 57 columns 1022 -> 903 us (the pipe alone: 916 at 1.92 GHz), 33 columns 1016 -> 535, 17 columns
+// 536 -> 293; n = 1000 real, 1 column 63 -> 23, 30 columns 106 -> 80; n = 5000 complex, 300 columns
+// 54.8 -> 48.8 ms.
 #include "common.cuh"
+#include "gemm_split.h"
 #include "kernels.h"
+
+#include <utility>
 
 namespace chase {
 
 namespace {
 
-constexpr int BM = 64;
-constexpr int BK = 16;
-constexpr int TM = 4;
+constexpr int BM = kGemmRows;
+constexpr int BK = 8;
 constexpr int NT = 256;
+constexpr int TN = kGemmCols / 4;  // columns of a thread (one row)
 
-template <class T, bool TRANS_A, int TN>
-__global__ void __launch_bounds__(NT) gemm_kernel(int M, int N, int K, const T* __restrict__ A,
-                                                  int lda, const T* __restrict__ B, int ldb, T* C,
-                                                  int ldc, double alpha, double beta, const T* X,
-                                                  int ldx, double gamma, const T* Y, int ldy,
-                                                  int kchunk, T* __restrict__ partial,
-                                                  int upper_only, int tri_b) {
-  constexpr int BN = 16 * TN;
-  __shared__ T As[BK][BM];
-  __shared__ T Bs[BK][BN];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  // column tiles vary fastest so that the CTAs in flight share A's row panels in L2
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
-  if (upper_only && m0 > n0 + BN - 1) return;
-  const int kb = blockIdx.z * kchunk;
-  int ke = min(K, kb + kchunk);
-  if (tri_b) ke = min(ke, n0 + BN);  // B[k, j] = 0 for k > j
-
-  T acc[TM][TN];
+// acc[j] += sum over kn steps of K of a b[4 j], j < nc: a loop of its own for every nc, since an
+// FP64 instruction that is predicated off holds the pipe as long as one that is not.
+template <class T, int NC>
+__device__ __forceinline__ void block_fma_n(const T* a, const T* b, int kn, T* acc) {
+#pragma unroll 2
+  for (int kk = 0; kk < kn; ++kk) {
+    const T x = a[kk * (BM + 1)];
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = Sc<T>::zero();
-
-  // register prefetch of the next tile
-  T ra[4], rb[TN];
-  auto load_tiles = [&](int k0) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int i, kk;
-      if (!TRANS_A) { i = tid & 63; kk = (tid >> 6) + 4 * r; }
-      else          { kk = tid & 15; i = (tid >> 4) + 16 * r; }
-      int gi = m0 + i, gk = k0 + kk;
-      T v = Sc<T>::zero();
-      if (gi < M && gk < ke) {
-        v = TRANS_A ? Sc<T>::conj(A[(size_t)gk + (size_t)gi * lda]) : A[(size_t)gi + (size_t)gk * lda];
-      }
-      ra[r] = v;
-    }
-#pragma unroll
-    for (int r = 0; r < TN; ++r) {
-      int kk = tid & 15, j = (tid >> 4) + 16 * r;
-      int gj = n0 + j, gk = k0 + kk;
-      T v = Sc<T>::zero();
-      if (gj < N && gk < ke) v = B[(size_t)gk + (size_t)gj * ldb];
-      rb[r] = v;
-    }
-  };
-  auto store_tiles = [&]() {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int i, kk;
-      if (!TRANS_A) { i = tid & 63; kk = (tid >> 6) + 4 * r; }
-      else          { kk = tid & 15; i = (tid >> 4) + 16 * r; }
-      As[kk][i] = ra[r];
-    }
-#pragma unroll
-    for (int r = 0; r < TN; ++r) {
-      int kk = tid & 15, j = (tid >> 4) + 16 * r;
-      Bs[kk][j] = rb[r];
-    }
-  };
-
-  if (kb < ke) load_tiles(kb);
-  for (int k0 = kb; k0 < ke; k0 += BK) {
-    __syncthreads();
-    store_tiles();
-    __syncthreads();
-    if (k0 + BK < ke) load_tiles(k0 + BK);
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], b[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) Sc<T>::fma(acc[i][j], a[i], b[j]);
-    }
+    for (int j = 0; j < NC; ++j) Sc<T>::fma(acc[j], x, b[kk * kGemmCols + 4 * j]);
   }
+}
+template <class T, int... J>
+__device__ __forceinline__ void block_fma(std::integer_sequence<int, J...>, int nc, const T* a, const T* b, int kn,
+                                          T* acc) {
+  (void)((nc == J + 1 && (block_fma_n<T, J + 1>(a, b, kn, acc), true)) || ...);
+}
 
-  if (partial) {
-    T* P = partial + (size_t)blockIdx.z * M * N;
+template <class T, bool TRANS_A>
+__global__ void __launch_bounds__(NT, 2) gemm_kernel(GemmSplit sp, const T* __restrict__ A, int lda,
+                                                     const T* __restrict__ B, int ldb, T* C, int ldc,
+                                                     double alpha, double beta, const T* X, int ldx,
+                                                     double gamma, const T* Y, int ldy,
+                                                     T* __restrict__ partial) {
+  __shared__ T As[2][BK][BM + 1];
+  __shared__ T Bs[2][BK][kGemmCols];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = blockIdx.x;
+  const int row = 32 * (warp & 1) + lane;
+  const int grp = ((warp >> 1) + g + g / kNumSMs) & 3;  // first column: rotated, see above
+  long long w = sp.whole ? 0 : sp.begin(g);
+  const long long w1 = sp.whole ? 0 : sp.begin(g + 1);
+  do {
+    const GemmTile t = sp.whole ? sp.tile(g) : sp.at(w);
+    const int kb = sp.whole ? 0 : (int)(w - t.w0);
+    const int ke = sp.whole ? t.kt : (int)min((long long)t.kt, kb + (w1 - w));
+    const int nc = (t.nb - grp + 3) >> 2;
+    T acc[TN];
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+    for (int j = 0; j < TN; ++j) acc[j] = Sc<T>::zero();
+
+    T ra[2], rb[2];  // the next block of K
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int i = TRANS_A ? (tid >> 3) + 32 * r : tid & 63;
+        const int ka = k0 + (TRANS_A ? tid & 7 : (tid >> 6) + 4 * r), gi = t.m0 + i;
+        ra[r] = Sc<T>::zero();
+        if (gi < sp.M && ka < ke)
+          ra[r] = TRANS_A ? Sc<T>::conj(A[(size_t)ka + (size_t)gi * lda]) : A[(size_t)gi + (size_t)ka * lda];
+        const int j = (tid >> 3) + 32 * r, kk = k0 + (tid & 7);
+        rb[r] = Sc<T>::zero();
+        if (j < t.nb && kk < ke) rb[r] = B[(size_t)kk + (size_t)(t.n0 + j) * ldb];
+      }
+    };
+    int s = 0;
+    if (kb < ke) load(kb);
+    for (int k0 = kb; k0 < ke; k0 += BK, s ^= 1) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        if (TRANS_A) As[s][tid & 7][(tid >> 3) + 32 * r] = ra[r];
+        else As[s][(tid >> 6) + 4 * r][tid & 63] = ra[r];
+        Bs[s][tid & 7][(tid >> 3) + 32 * r] = rb[r];
+      }
+      __syncthreads();  // (the other buffer is written only after this block's barrier: one is enough)
+      if (k0 + BK < ke) load(k0 + BK);
+      block_fma<T>(std::make_integer_sequence<int, TN>(), nc, &As[s][0][row], &Bs[s][0][grp], min(BK, ke - k0), acc);
+    }
+    __syncthreads();  // before the next tile's first block
+
+    if (ke - kb < t.kt) {
+      T* P = partial + (long long)(g + t.t) * sp.slot_elems();
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+        if (j < nc) P[(grp + 4 * j) * BM + row] = acc[j];
+    } else {
+      const int gi = t.m0 + row;
 #pragma unroll
       for (int j = 0; j < TN; ++j) {
-        int gi = m0 + ty + 16 * i, gj = n0 + tx + 16 * j;
-        if (gi < M && gj < N) P[(size_t)gi + (size_t)gj * M] = acc[i][j];
-      }
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      int gi = m0 + ty + 16 * i, gj = n0 + tx + 16 * j;
-      if (gi < M && gj < N) {
-        T v = Sc<T>::scale(acc[i][j], alpha);
-        if (beta != 0.0) v = Sc<T>::add(v, Sc<T>::scale(X[(size_t)gi + (size_t)gj * ldx], beta));
-        if (gamma != 0.0) v = Sc<T>::add(v, Sc<T>::scale(Y[(size_t)gi + (size_t)gj * ldy], gamma));
-        C[(size_t)gi + (size_t)gj * ldc] = v;
+        const int gj = t.n0 + grp + 4 * j;
+        if (j < nc && gi < sp.M && !(sp.upper && gi > gj)) {
+          T v = Sc<T>::scale(acc[j], alpha);
+          if (beta != 0.0) v = Sc<T>::add(v, Sc<T>::scale(X[(size_t)gi + (size_t)gj * ldx], beta));
+          if (gamma != 0.0) v = Sc<T>::add(v, Sc<T>::scale(Y[(size_t)gi + (size_t)gj * ldy], gamma));
+          C[(size_t)gi + (size_t)gj * ldc] = v;
+        }
       }
     }
+    w += ke - kb;
+  } while (w < w1);
 }
 
-// Sums the split-K partials in a fixed order and applies the epilogue.
+// Sums the parts of the tiles that CTAs shared, in their order, and applies the epilogue.
+// blockIdx.x: tile, blockIdx.y: columns y, y + gridDim.y, ...
 template <class T>
-__global__ void splitk_reduce_kernel(int M, int N, int S, const T* __restrict__ partial, T* C,
-                                     int ldc, double alpha, double beta, const T* X, int ldx,
-                                     double gamma, const T* Y, int ldy, int upper_only) {
-  size_t total = (size_t)M * N;
-  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    int i = (int)(idx % M), j = (int)(idx / M);
-    if (upper_only && i > j) continue;
-    T s = partial[idx];
-    for (int z = 1; z < S; ++z) s = Sc<T>::add(s, partial[idx + (size_t)z * total]);
-    T v = Sc<T>::scale(s, alpha);
-    if (beta != 0.0) v = Sc<T>::add(v, Sc<T>::scale(X[(size_t)i + (size_t)j * ldx], beta));
-    if (gamma != 0.0) v = Sc<T>::add(v, Sc<T>::scale(Y[(size_t)i + (size_t)j * ldy], gamma));
-    C[(size_t)i + (size_t)j * ldc] = v;
+__global__ void __launch_bounds__(128) split_reduce_kernel(GemmSplit sp, const T* __restrict__ partial, T* C,
+                                                           int ldc, double alpha, double beta, const T* X, int ldx,
+                                                           double gamma, const T* Y, int ldy) {
+  const GemmTile t = sp.tile(blockIdx.x);
+  const int g0 = sp.owner(t.w0), g1 = sp.owner(t.w0 + t.kt - 1);
+  if (g0 == g1) return;
+  const int row = threadIdx.x & 63, gi = t.m0 + row;
+  if (gi >= sp.M) return;
+  for (int j = 2 * blockIdx.y + (threadIdx.x >> 6); j < t.nb; j += 2 * gridDim.y) {
+    const int gj = t.n0 + j;
+    if (sp.upper && gi > gj) continue;
+    const T* p = partial + j * BM + row;
+    T v = p[(g0 + t.t) * sp.slot_elems()];
+    for (int g = g0 + 1; g <= g1; ++g) v = Sc<T>::add(v, p[(g + t.t) * sp.slot_elems()]);
+    v = Sc<T>::scale(v, alpha);
+    if (beta != 0.0) v = Sc<T>::add(v, Sc<T>::scale(X[(size_t)gi + (size_t)gj * ldx], beta));
+    if (gamma != 0.0) v = Sc<T>::add(v, Sc<T>::scale(Y[(size_t)gi + (size_t)gj * ldy], gamma));
+    C[(size_t)gi + (size_t)gj * ldc] = v;
   }
-}
-
-template <class T, bool TRANS_A, int TN>
-void launch_gemm(cudaStream_t st, dim3 grid, int M, int N, int K, const T* A, int lda, const T* B,
-                 int ldb, T* C, int ldc, double alpha, double beta, const T* X, int ldx,
-                 double gamma, const T* Y, int ldy, int kchunk, T* partial, int upper_only,
-                 int tri_b) {
-  gemm_kernel<T, TRANS_A, TN><<<grid, NT, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, X,
-                                                  ldx, gamma, Y, ldy, kchunk, partial, upper_only,
-                                                  tri_b);
 }
 
 }  // namespace
@@ -174,48 +159,21 @@ int gemm(cudaStream_t st, bool transA, int M, int N, int K, const T* A, int lda,
          int ldb, T* C, int ldc, double alpha, double beta, const T* X, int ldx, double gamma,
          const T* Y, int ldy, Scratch scratch, bool upper_only, bool tri_b, int* launches) {
   if (M <= 0 || N <= 0) return 0;
-  // 64 x 32 tiles; 64 x 16 when N <= 16, or when a short product (K <= 256, no room for
-  // split-K) would otherwise leave SMs idle: twice the CTAs, each with half the FP64 work
-  int TN = (N > 16) ? 2 : 1;
-  if (TN == 2 && K <= 256) {
-    long long t2 = (long long)ceil_div(M, BM) * ceil_div(N, 32);
-    if (upper_only) t2 = (t2 + ceil_div(M, BM)) / 2;
-    if (t2 < 2LL * kNumSMs) TN = 1;
-  }
-  const int BN = 16 * TN;
-  const int tm = ceil_div(M, BM), tn = ceil_div(N, BN);
-  long long tiles = (long long)tm * tn;
-  if (upper_only) tiles = (tiles + tm) / 2;
-  // split-K so that every SM gets about 8 work units
-  int S = 1;
-  if (K > 0) {
-    long long target = 8LL * kNumSMs;
-    S = (int)std::max(1LL, (target + tiles - 1) / tiles);
-    S = std::min(S, std::max(1, K / 64));
-    size_t need = (size_t)S * M * N * sizeof(T);
-    while (S > 1 && need > scratch.bytes) { --S; need = (size_t)S * M * N * sizeof(T); }
-  }
-  int kchunk = K;
-  if (S > 1) {
-    kchunk = ceil_div(ceil_div(K, S), BK) * BK;
-    S = ceil_div(K, kchunk);
-  }
-  if (K <= 0) { S = 1; kchunk = 0; }
-  T* partial = (S > 1) ? (T*)scratch.ptr : nullptr;
-  dim3 grid(tn, tm, S);
-  if (transA) {
-    if (TN == 2) launch_gemm<T, true, 2>(st, grid, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy, kchunk, partial, upper_only, tri_b);
-    else         launch_gemm<T, true, 1>(st, grid, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy, kchunk, partial, upper_only, tri_b);
-  } else {
-    if (TN == 2) launch_gemm<T, false, 2>(st, grid, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy, kchunk, partial, upper_only, tri_b);
-    else         launch_gemm<T, false, 1>(st, grid, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy, kchunk, partial, upper_only, tri_b);
-  }
+  // kmin: a CTA with fewer K steps of a tile costs about as much to start as it computes (a step is
+  // up to 2 us in complex arithmetic, 0.5 in real; a launch and the second kernel ~3)
+  const GemmSplit sp = gemm_split(M, N, K, upper_only, tri_b, 2 * kNumSMs, Sc<T>::cplx ? 8 : 16,
+                                  (long long)(scratch.bytes / sizeof(T)));
+  T* partial = sp.whole ? nullptr : (T*)scratch.ptr;
+  if (transA)
+    gemm_kernel<T, true><<<sp.G, NT, 0, st>>>(sp, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy,
+                                              partial);
+  else
+    gemm_kernel<T, false><<<sp.G, NT, 0, st>>>(sp, A, lda, B, ldb, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy,
+                                               partial);
   if (launches) ++*launches;
-  if (S > 1) {
-    size_t total = (size_t)M * N;
-    int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)kNumSMs * 16);
-    splitk_reduce_kernel<T><<<blocks, 256, 0, st>>>(M, N, S, partial, C, ldc, alpha, beta, X, ldx,
-                                                    gamma, Y, ldy, upper_only);
+  if (!sp.whole) {
+    split_reduce_kernel<T><<<dim3(sp.T, std::max(1, ceil_div(sp.bn, 8))), 128, 0, st>>>(
+        sp, partial, C, ldc, alpha, beta, X, ldx, gamma, Y, ldy);
     if (launches) ++*launches;
   }
   CHASE_CUDA_TRY(cudaGetLastError());
