@@ -947,24 +947,31 @@ __device__ __forceinline__ long long oz_int(double x, int e) {
   return X;
 }
 
-// Residues of an integer X (|X| < 2^59) mod p_j in symmetric range, stored as BF16 (exact:
-// integers of magnitude <= 128) in plane j.
-__device__ __forceinline__ void write_residues_int(long long X, __nv_bfloat16* base, size_t idx,
-                                                   size_t plane) {
-  // |X| = U1 2^29 + U0 with U0 < 2^29 and U1 < 2^30: |X| mod p = ((U1 mod p) (2^29 mod p) +
-  // U0 mod p) mod p in 32-bit arithmetic (remainders by compile-time constants; the product
-  // stays below 2^16)
-  const unsigned long long U = (unsigned long long)(X < 0 ? -X : X);
-  const uint32_t U1 = (uint32_t)(U >> 29), U0 = (uint32_t)(U & ((1u << 29) - 1));
+// Residues of four adjacent K entries (|X| < 2^58) mod p_j in [-(p/2), p - 1 - p/2], stored as BF16
+// (exact: magnitudes <= 128), 8-byte words.  Cut up as in write_ring4 (below): one unreduced
+// 31-bit sum and one division by a constant per residue (before: three divisions per residue and
+// 2-byte stores).  Integer-issue-bound.  n = 4999, A 430 -> 235 us; a filter of 299 columns 9.95 ->
+// 8.95 ms together with the split of columns below.
+__device__ __forceinline__ void write_real4(const long long* x, __nv_bfloat16* base, size_t idx, size_t plane) {
+  uint32_t x0[4], x1[4], x2[4];
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    const unsigned long long X = (unsigned long long)(x[d] + (1LL << 58));
+    x0[d] = (uint32_t)X & 0x7FFFFu;
+    x1[d] = (uint32_t)(X >> 19) & 0x7FFFFu;
+    x2[d] = (uint32_t)(X >> 38);
+  }
 #pragma unroll
   for (int j = 0; j < kOzModuli; ++j) {
     const uint32_t p = (uint32_t)oz_modulus(j);
-    const uint32_t k29 = (uint32_t)((1ull << 29) % p);
-    const uint32_t u = ((U1 % p) * k29 + U0 % p) % p;   // |X| mod p in [0, p)
-    int rr = X < 0 ? -(int)u : (int)u;                   // X mod p in (-p, p), sign of X
-    if (rr > (int)p / 2) rr -= (int)p;
-    else if (rr < -((int)p / 2)) rr += (int)p;
-    base[idx + (size_t)j * plane] = __int2bfloat16_rn(rr);  // exact: |rr| <= 128
+    const uint32_t k19 = (uint32_t)((1ull << 19) % p), k38 = (uint32_t)((1ull << 38) % p), half = p / 2;
+    const uint32_t off = p - (uint32_t)((1ull << 58) % p) + half;
+    float f[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d)  // < 2^21 2^8 + 2^19 2^8 + 2^19 + 2^9 < 2^30
+      f[d] = (float)((int)((x2[d] * k38 + x1[d] * k19 + x0[d] + off) % p) - (int)half);
+    __nv_bfloat162 pk[2] = {__floats2bfloat162_rn(f[0], f[1]), __floats2bfloat162_rn(f[2], f[3])};
+    *(uint2*)(base + idx + (size_t)j * plane) = *(const uint2*)pk;
   }
 }
 
@@ -1014,11 +1021,6 @@ __device__ __forceinline__ void write_ring4(const long long* xr, const long long
   }
 }
 
-__device__ __forceinline__ void write_residues(double x, int e, __nv_bfloat16* base, size_t idx,
-                                               size_t plane) {
-  write_residues_int(oz_int(x, e), base, idx, plane);
-}
-
 __device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* red) {
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
@@ -1033,6 +1035,36 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
   return mx;
 }
 
+// Exponent of n values, by the whole block.
+__device__ __forceinline__ int column_exp(const double* __restrict__ col, int n, unsigned long long* red) {
+  unsigned long long amax = 0;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const unsigned long long b = abs_bits(col[k]);
+    amax = b > amax ? b : amax;
+  }
+  return exp_bound(block_max(amax, red));
+}
+
+// Residues of entries [k0, k1) of a column of n values (multiples of 4; zero from n on), at idx + k.
+__device__ __forceinline__ void slice_real(const double* __restrict__ col, int n, int k0, int k1, int e,
+                                           __nv_bfloat16* planes, size_t idx, size_t plane) {
+  for (int k = k0 + 4 * threadIdx.x; k < k1; k += 4 * blockDim.x) {
+    long long x[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) x[d] = oz_int(k + d < n ? col[k + d] : 0.0, e);
+    write_real4(x, planes, idx + k, plane);
+  }
+}
+
+// A column is sliced by `parts` blocks, each of which takes its exponent for itself (an L2 read of
+// the column): one block per column leaves most of the SMs' warps empty for few columns, and half of
+// them at 600.  A part is at least 1024 rows, four per thread.
+__host__ __device__ inline int slice_part(int kp, int parts) { return (kp / 64 + parts - 1) / parts * 64; }
+inline int slice_parts(int kp, int cols) {
+  return std::max(1, std::min(kp / 1024, 8 * kNumSMs / std::max(1, cols)));
+}
+
 // Real A (n x n): residues of row m (column m of A: symmetric) into planes (row-major, ld kp),
 // row exponent into rowexp[m].
 __global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __restrict__ A, int lda,
@@ -1042,15 +1074,9 @@ __global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const double* col = A + (size_t)m * lda;
-  unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < n; k += 256) {
-    const unsigned long long b = abs_bits(col[k]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
+  const int e = column_exp(col, n, red);
   if (threadIdx.x == 0) rowexp[m] = e;
-  for (int k = threadIdx.x; k < kp; k += 256)
-    write_residues(k < n ? col[k] : 0.0, e, planes, (size_t)m * kp + k, plane);
+  slice_real(col, n, 0, kp, e, planes, (size_t)m * kp, plane);
 }
 
 // FP64 stacked block V64 (M x ncols, ld ldi): residues of column c into planes
@@ -1060,19 +1086,11 @@ __global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const do
                                                          size_t plane, int* colexp) {
   dep_wait();
   __shared__ unsigned long long red[8];
-  const int c = c0 + blockIdx.x;
+  const int c = c0 + blockIdx.x, part = slice_part(kp, gridDim.y), k0 = blockIdx.y * part;
   const double* col = V64 + (size_t)c * ldi;
-  unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < M; k += 256) {
-    const unsigned long long b = abs_bits(col[k]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) colexp[c] = e;
-  for (int k = threadIdx.x; k < kp; k += 256) {
-    const double x = (k < M) ? col[k] : 0.0;
-    write_residues(x, e, planes, (size_t)c * kp + k, plane);
-  }
+  const int e = column_exp(col, M, red);
+  if (threadIdx.x == 0 && blockIdx.y == 0) colexp[c] = e;
+  slice_real(col, M, k0, min(kp, k0 + part), e, planes, (size_t)c * kp, plane);
 }
 
 // ---- operands of the ring products ----
@@ -1113,17 +1131,12 @@ __global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* 
 // both halves, then its two plane rows (u | w), ld kpn.
 template <int NM>
 __device__ __forceinline__ void slice_V_ring_column(int n, int c, const double* __restrict__ V64, int ldi,
-                                                    int kpn, __nv_bfloat16* planes, size_t plane,
-                                                    int* colexp, unsigned long long* red) {
+                                                    int kpn, int k0, int k1, __nv_bfloat16* planes,
+                                                    size_t plane, int* colexp, unsigned long long* red) {
   const double* col = V64 + (size_t)c * ldi;
-  unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < 2 * n; k += 256) {
-    const unsigned long long b = abs_bits(col[k]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) colexp[c] = e;
-  for (int k = 4 * threadIdx.x; k < kpn; k += 1024) {
+  const int e = column_exp(col, 2 * n, red);
+  if (threadIdx.x == 0 && k0 == 0) colexp[c] = e;
+  for (int k = k0 + 4 * threadIdx.x; k < k1; k += 1024) {
     long long xr[4], xi[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
@@ -1135,7 +1148,7 @@ __device__ __forceinline__ void slice_V_ring_column(int n, int c, const double* 
   }
 }
 
-// Grouped form of oz_slice_V_kernel: one block per sliced column of every problem.
+// Grouped form of oz_slice_V_kernel: parts[p] blocks per sliced column of every problem.
 struct SliceGroupParams {
   const double* V64[kOzGroupMax];
   __nv_bfloat16* planes[kOzGroupMax];
@@ -1144,6 +1157,7 @@ struct SliceGroupParams {
   int blk0[kOzGroupMax + 1];  // first block of each problem
   int M[kOzGroupMax], c0[kOzGroupMax], ldi[kOzGroupMax], kp[kOzGroupMax];
   int ring[kOzGroupMax];  // ring moduli of a complex problem (M = n); 0: real
+  int parts[kOzGroupMax];
   int count;
 };
 static_assert(sizeof(SliceGroupParams) <= 32000, "kernel parameter space");
@@ -1153,29 +1167,22 @@ __global__ void __launch_bounds__(256) oz_slice_V_group_kernel(const __grid_cons
   __shared__ unsigned long long red[8];
   int p = 0;
   while (p + 1 < P.count && (int)blockIdx.x >= P.blk0[p + 1]) ++p;
-  const int c = P.c0[p] + (blockIdx.x - P.blk0[p]);
+  const int b = blockIdx.x - P.blk0[p], c = P.c0[p] + b / P.parts[p];
   const int M = P.M[p], kp = P.kp[p];
+  const int part = slice_part(kp, P.parts[p]), k0 = b % P.parts[p] * part, k1 = min(kp, k0 + part);
   if (P.ring[p]) {
     if (P.ring[p] == kRingShort)
-      slice_V_ring_column<kRingShort>(M, c, P.V64[p], P.ldi[p], kp, P.planes[p], (size_t)P.plane[p],
+      slice_V_ring_column<kRingShort>(M, c, P.V64[p], P.ldi[p], kp, k0, k1, P.planes[p], (size_t)P.plane[p],
                                       P.colexp[p], red);
     else
-      slice_V_ring_column<kRingModuli>(M, c, P.V64[p], P.ldi[p], kp, P.planes[p], (size_t)P.plane[p],
+      slice_V_ring_column<kRingModuli>(M, c, P.V64[p], P.ldi[p], kp, k0, k1, P.planes[p], (size_t)P.plane[p],
                                        P.colexp[p], red);
     return;
   }
   const double* col = P.V64[p] + (size_t)c * P.ldi[p];
-  unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < M; k += 256) {
-    const unsigned long long b = abs_bits(col[k]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) P.colexp[p][c] = e;
-  for (int k = threadIdx.x; k < kp; k += 256) {
-    const double x = (k < M) ? col[k] : 0.0;
-    write_residues(x, e, P.planes[p], (size_t)c * kp + k, (size_t)P.plane[p]);
-  }
+  const int e = column_exp(col, M, red);
+  if (threadIdx.x == 0 && k0 == 0) P.colexp[p][c] = e;
+  slice_real(col, M, k0, k1, e, P.planes[p], (size_t)c * kp, (size_t)P.plane[p]);
 }
 
 // Caller's block V (n x ncols, ld ldv) -> stacked FP64 (M x ncols, ld ldo).
@@ -1207,16 +1214,17 @@ __global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z6
                                                                  int* colexp) {
   dep_wait();
   __shared__ unsigned long long red[8];
-  const int c = blockIdx.x;
+  const int c = blockIdx.x, part = slice_part(kp, gridDim.y), k0 = blockIdx.y * part, k1 = min(kp, k0 + part);
   const z64* col = Y + (size_t)c * ldy;
   unsigned long long amax = 0;
+#pragma unroll 4
   for (int k = threadIdx.x; k < n; k += 256) {
     const unsigned long long b = max(abs_bits(col[k].x), abs_bits(col[k].y));
     amax = b > amax ? b : amax;
   }
   const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) colexp[c] = e;
-  for (int k = 4 * threadIdx.x; k < kp; k += 1024) {
+  if (threadIdx.x == 0 && k0 == 0) colexp[c] = e;
+  for (int k = k0 + 4 * threadIdx.x; k < k1; k += 1024) {
     long long xr[4], xi[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
@@ -1287,34 +1295,22 @@ __global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double*
   __shared__ unsigned long long red[8];
   const int m = blockIdx.x;
   const double* row = Xt + (size_t)m * ldt;  // X[m, 0..l)
-  unsigned long long amax = 0;
-  for (int k = threadIdx.x; k < l; k += 256) {
-    const unsigned long long b = abs_bits(row[k]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
+  const int e = column_exp(row, l, red);
   if (threadIdx.x == 0) rowexp[m] = e;
-  for (int k = threadIdx.x; k < kp; k += 256)
-    write_residues(k < l ? row[k] : 0.0, e, planes, (size_t)m * kp + k, plane);
+  slice_real(row, l, 0, kp, e, planes, (size_t)m * kp, plane);
 }
 
 // Residues of the columns of a real block Y (n x q, ld ldy): planes column-major (ld kp; rows
 // >= n are zero), column exponents.
-__global__ void __launch_bounds__(512) oz_slice_cols_kernel(int n, const double* __restrict__ Y, int ldy, int kp,
+__global__ void __launch_bounds__(256) oz_slice_cols_kernel(int n, const double* __restrict__ Y, int ldy, int kp,
                                                             __nv_bfloat16* planes, size_t plane, int* colexp) {
   dep_wait();
-  __shared__ unsigned long long red[16];
-  const int j = blockIdx.x;
+  __shared__ unsigned long long red[8];
+  const int j = blockIdx.x, part = slice_part(kp, gridDim.y), k0 = blockIdx.y * part;
   const double* col = Y + (size_t)j * ldy;
-  unsigned long long amax = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const unsigned long long b = abs_bits(col[i]);
-    amax = b > amax ? b : amax;
-  }
-  const int e = exp_bound(block_max(amax, red));
-  if (threadIdx.x == 0) colexp[j] = e;
-  for (int k = threadIdx.x; k < kp; k += blockDim.x)
-    write_residues(k < n ? col[k] : 0.0, e, planes, (size_t)j * kp + k, plane);
+  const int e = column_exp(col, n, red);
+  if (threadIdx.x == 0 && k0 == 0) colexp[j] = e;
+  slice_real(col, n, k0, min(kp, k0 + part), e, planes, (size_t)j * kp, plane);
 }
 
 // Xt = X^T: real X n x l (ld ldx) -> Xt l x n (ld ldt).
@@ -1397,7 +1393,7 @@ int oz_slice_A_ring(cudaStream_t st, int n, const z64* A, int lda, int kpn, void
 int oz_slice_V(cudaStream_t st, int M, int c0, int c1, const double* V64, int ldi, int kp,
                int ncols_total, void* planes, int* colexp, int* launches) {
   if (c1 <= c0) return 0;
-  launch_dep(st, c1 - c0, 256, 0, oz_slice_V_kernel, M, c0, V64, ldi, kp, (__nv_bfloat16*)planes,
+  launch_dep(st, dim3(c1 - c0, slice_parts(kp, c1 - c0)), 256, 0, oz_slice_V_kernel, M, c0, V64, ldi, kp, (__nv_bfloat16*)planes,
              (size_t)ncols_total * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
@@ -1531,7 +1527,8 @@ int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* 
   for (int g0 = 0; g0 < count; g0 += kOzGroupMax) {
     const int cnt = std::min(kOzGroupMax, count - g0);
     SliceGroupParams P{};
-    int blocks = 0;
+    int blocks = 0, cols = 0;
+    for (int i = 0; i < cnt; ++i) cols += std::max(0, items[g0 + i].N);
     P.count = 0;
     for (int i = 0; i < cnt; ++i) {
       const OzGroupItem& it = items[g0 + i];
@@ -1542,12 +1539,13 @@ int oz_slice_V_group(cudaStream_t st, int count, const OzGroupItem* items, int* 
       P.colexp[p] = const_cast<int*>(it.colexp);
       P.plane[p] = (long long)it.ncols_total * it.kp;
       P.blk0[p] = blocks;
+      P.parts[p] = slice_parts(it.kp, cols);
       P.M[p] = it.M;
       P.c0[p] = it.col0;
       P.ldi[p] = it.ldi;
       P.kp[p] = it.kp;
       P.ring[p] = it.ring ? ring_moduli(it.kp) : 0;
-      blocks += it.N;
+      blocks += it.N * P.parts[p];
     }
     if (P.count == 0) continue;
     P.blk0[P.count] = blocks;
@@ -1715,7 +1713,7 @@ int oz_slice_cols_ring(cudaStream_t st, int n, int q, const z64* Y, int ldy, int
                        int* launches) {
   if (q <= 0) return 0;
   auto kern = ring_moduli(kp) == kRingShort ? oz_slice_cols_ring_kernel<kRingShort> : oz_slice_cols_ring_kernel<kRingModuli>;
-  launch_dep(st, q, 256, 0, kern, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
+  launch_dep(st, dim3(q, slice_parts(kp, q)), 256, 0, kern, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1737,7 +1735,9 @@ int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, doubl
                   int* rowexp, int* launches) {
   if (n <= 0) return 0;
   launch_dep(st, dim3(ceil_div(n, 32), ceil_div(l, 32)), dim3(32, 8), 0, transpose_kernel, n, l, X, ldx, Xt, l);
-  launch_dep(st, n, 256, 0, oz_slice_rows_kernel, l, Xt, l, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
+  // (a thread takes four entries of a row)
+  const int threads = std::min(256, std::max(32, ceil_div(kp / 4, 32) * 32));
+  launch_dep(st, n, threads, 0, oz_slice_rows_kernel, l, Xt, l, kp, (__nv_bfloat16*)planes, (size_t)n * kp, rowexp);
   if (launches) *launches += 2;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1746,7 +1746,7 @@ int oz_slice_rows(cudaStream_t st, int n, int l, const double* X, int ldx, doubl
 int oz_slice_cols(cudaStream_t st, int n, int q, const double* Y, int ldy, int kp, void* planes, int* colexp,
                   int* launches) {
   if (q <= 0) return 0;
-  launch_dep(st, q, 512, 0, oz_slice_cols_kernel, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
+  launch_dep(st, dim3(q, slice_parts(kp, q)), 256, 0, oz_slice_cols_kernel, n, Y, ldy, kp, (__nv_bfloat16*)planes, (size_t)q * kp, colexp);
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;
