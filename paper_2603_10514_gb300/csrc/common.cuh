@@ -106,10 +106,13 @@ struct DevStatus {
 // their writes are seen, so their order is that of plain launches.  A plain launch, a copy or an
 // event still waits for the whole kernel before it.  It takes the launch latency and the set-up
 // (barriers, tensor memory) out of a chain of short kernels: n = 1000 real, 30 columns, a filter
-// step 35 -> 27 us, a solve of 30 vectors 11.6 -> 10.9 ms.
-__device__ __forceinline__ void dep_wait() {
+// step 35 -> 27 us, a solve of 30 vectors 11.6 -> 10.9 ms.  early = false: the next launch's blocks
+// are placed only when this one's have left (blocks placed beside them are spread unevenly, which
+// costs a launch of about one long block per SM more than its latency: divide and conquer and
+// back-transformation of l = 600 complex 5.3 ms so, 7.0 placed early; no difference at l = 30 to 230).
+__device__ __forceinline__ void dep_wait(bool early = true) {
   cudaGridDependencySynchronize();
-  cudaTriggerProgrammaticLaunchCompletion();
+  if (early) cudaTriggerProgrammaticLaunchCompletion();
 }
 template <class T> struct SameType { using type = T; };
 template <class... P>

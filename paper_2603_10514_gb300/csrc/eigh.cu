@@ -9,14 +9,14 @@
 //      is formed by every CTA from that while its other warps apply H -= v w^H + w v^H.
 //   2. Divide and conquer for T = Z Lambda Z^T (stedc.cuh): blocks of up to 32 rows in one CTA
 //      each, then per level five launches over all merges of the level.
-//   3. W = Q Z: one warp per column of W applies the reflectors in turn; columns are
+//   3. W = Q Z: one warp per column of W applies the reflectors, eight at a time; columns are
 //      independent, so no CTA waits for another.
 // It replaces a cyclic Jacobi iteration.  GB300 issues 2 FP64 FMAs per clock per SM, which binds
 // both: Jacobi takes ~5 sweeps of ~9 l^3 (complex: x 4) FMAs and l - 1 grid-wide rounds each,
 // this ~4 l^3 for step 1, ~l^3 (real) for 2 and ~2 l^3 for 3, and l grid barriers in all.
-// Measured (random H, GB300): l = 600 complex 124 -> 11.8 ms (6.5 reduction, 1.8 divide and
-// conquer, 3.5 back-transformation), l = 230 complex 31 -> 3.5, l = 600 real 80 -> 7.8, l = 30
-// real 2.0 -> 0.48.
+// Measured (random H, GB300): l = 600 complex 124 -> 10.3 ms (6.4 reduction, 1.75 divide and
+// conquer, 2.05 back-transformation), l = 230 complex 31 -> 3.0, l = 600 real 80 -> 6.7, l = 30
+// real 2.0 -> 0.41.
 //
 // Every wait is bounded; a CTA that waits too long raises an abort flag that the others see, and
 // the kernel sets DevStatus.timeout.  Sums are taken in fixed orders: results are reproducible.
@@ -298,6 +298,20 @@ struct CtaGroup {
     return v;
   }
 };
+// `size` threads of a CTA (whole warps, in a row) with a barrier of their own.
+struct PartGroup {
+  int tid, size, id;
+  double* red;
+  __device__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(size) : "memory"); }
+  __device__ double max(double v) const {
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    sync();
+    if ((tid & 31) == 0) red[tid >> 5] = v;
+    sync();
+    for (int w = 0; w < (size >> 5); ++w) v = fmax(v, red[w]);
+    return v;
+  }
+};
 struct WarpGroup {
   int tid, size;
   __device__ void sync() const { __syncwarp(); }
@@ -454,12 +468,35 @@ __device__ inline void dc_merge_local(const G& g, int w, int nw, int width, cons
 
 __host__ __device__ inline int dc_bound(int n, long long i, int depth) { return (int)((i * n) >> depth); }
 
-// Leaf blockIdx.x of 2^depth (at most 32 rows): its eigensystem by merges from single rows up,
-// one warp per merge while a level has at least four, then the whole CTA.
+// Eigensystem of the pair [x0 + |e|, e; e, x1 + |e|] (x: diagonal entries with e torn off), by one
+// rotation: D ascending, vectors in q (ld ldq).
+__device__ inline void dc_pair(double e, double* D, double* q, int ldq) {
+  const double a = D[0] + fabs(e), b = D[1] + fabs(e);
+  double c = 1.0, s = 0.0, t = 0.0;
+  if (e != 0.0) {
+    const double tau = (b - a) / (2.0 * e);
+    t = copysign(1.0 / (fabs(tau) + sqrt(1.0 + tau * tau)), tau);
+    c = 1.0 / sqrt(1.0 + t * t);
+    s = t * c;
+  }
+  const double la = a - t * e, lb = b + t * e;  // of (c, -s) and (s, c)
+  const bool swap = la > lb;
+  D[0] = swap ? lb : la;
+  D[1] = swap ? la : lb;
+  q[0] = swap ? s : c;
+  q[1] = swap ? c : -s;
+  q[ldq] = swap ? c : s;
+  q[ldq + 1] = swap ? -s : c;
+}
+
+// Leaf blockIdx.x of 2^depth (at most 32 rows): its eigensystem by merges from pairs of rows up,
+// the merges of a level at once with 8, 4, 2 or 1 of the warps each.  Latency-bound: a chain of
+// divisions and square roots per root.  l = 30: 252 -> 195 us against merges from single rows
+// with one warp or the whole CTA each.
 __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const double* __restrict__ d0,
                                                       const double* __restrict__ e0, int ld_de, DcWork W0,
                                                       size_t stride) {
-  dep_wait();
+  dep_wait(false);
   __shared__ double sQ[LEAF * LEAF], sQn[LEAF * LEAF], sU[LEAF * LEAF];
   __shared__ double s_red[8];
   __shared__ __align__(16) char s_vec[LEAF * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)];
@@ -478,22 +515,26 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
     if (!isfinite(d[r]) || !isfinite(up)) *W.bad = 1;
   }
   __syncthreads();
-  for (int h = 4; h >= 0; --h) {
-    const int parts = 1 << h;
-    const bool by_warp = parts >= 4;
-    for (int q = by_warp ? warp : 0; q < parts; q += by_warp ? 8 : 1) {
-      const long long i0 = ((long long)blockIdx.x << (h + 1)) + 2 * q;
-      const int a = dc_bound(n, i0, depth + h + 1) - s, b = dc_bound(n, i0 + 1, depth + h + 1) - s,
-                c = dc_bound(n, i0 + 2, depth + h + 1) - s;
-      if (b == a || c == b) continue;  // an empty half: nothing to merge
+  if (tid < 16) {  // single rows: at most one each side
+    const long long i0 = ((long long)blockIdx.x << 5) + 2 * tid;
+    const int a = dc_bound(n, i0, depth + 5) - s, b = dc_bound(n, i0 + 1, depth + 5) - s,
+              c = dc_bound(n, i0 + 2, depth + 5) - s;
+    if (b > a && c > b) dc_pair(e[s + b - 1], V.D[0] + a, sQ + a + a * LEAF, LEAF);
+  }
+  __syncthreads();
+  for (int h = 3; h >= 0; --h) {
+    const int nw = 8 >> h, q = warp / nw, wq = warp - q * nw;  // warps per merge, this warp's merge
+    const long long i0 = ((long long)blockIdx.x << (h + 1)) + 2 * q;
+    const int a = dc_bound(n, i0, depth + h + 1) - s, b = dc_bound(n, i0 + 1, depth + h + 1) - s,
+              c = dc_bound(n, i0 + 2, depth + h + 1) - s;
+    if (b > a && c > b) {  // (an empty half: nothing to merge)
       const dc::Merge M = dc_merge(V, 0, a, b, c, e[s + b - 1]);
-      double* Qb = sQ + a + a * LEAF;
-      if (by_warp)
-        dc_merge_local(WarpGroup{lane, 32}, 0, 1, h == 4 ? 16 : h == 3 ? 8 : 4, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
-                       sU + a + a * LEAF, LEAF);
+      const int at = a + a * LEAF;
+      if (h == 3)
+        dc_merge_local(WarpGroup{lane, 32}, 0, 1, 8, M, V.D[0] + a, V.D[1] + a, sQ + at, sQn + at, sU + at, LEAF);
       else
-        dc_merge_local(CtaGroup{tid, 256, s_red}, warp, 8, h == 1 ? 16 : 8, M, V.D[0] + a, V.D[1] + a, Qb, sQn + a + a * LEAF,
-                       sU + a + a * LEAF, LEAF);
+        dc_merge_local(PartGroup{tid - 32 * nw * q, 32 * nw, 1 + q, s_red + nw * q}, wq, nw, 8, M, V.D[0] + a,
+                       V.D[1] + a, sQ + at, sQn + at, sU + at, LEAF);
     }
     __syncthreads();
   }
@@ -511,7 +552,7 @@ __device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, 
 
 __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                        const double* __restrict__ e0, int ld_de) {
-  dep_wait();
+  dep_wait(false);
   __shared__ double red[16];
   const DcWork W = dc_at(W0, stride * blockIdx.y);
   int s;
@@ -523,7 +564,7 @@ __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride,
 // phase 0: roots, and the rotations of Q's rows; 1: corrected z; 2: U and the new order.
 __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                        const double* __restrict__ e0, int ld_de, int phase) {
-  dep_wait();
+  dep_wait(false);
   const DcWork W = dc_at(W0, stride * blockIdx.z);
   int s;
   const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, e0 + (size_t)blockIdx.z * ld_de, &s);
@@ -546,7 +587,7 @@ __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride,
 // Q_new[:, dest] = Q[:, gathered] U (64 x 32 tiles, FP64), deflated columns copied.
 __global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth,
                                                       const double* __restrict__ e0, int ld_de, int parts) {
-  dep_wait();
+  dep_wait(false);
   const DcWork W = dc_at(W0, stride * (blockIdx.z / parts));
   int s;
   const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.z % parts, e0 + (size_t)(blockIdx.z / parts) * ld_de, &s);
@@ -640,13 +681,144 @@ int stedc(cudaStream_t st, int n, int batch, const double* d, const double* e, i
 // ---------------------------------------------------------------------------
 // 3. Back-transformation
 // ---------------------------------------------------------------------------
+// 3. Back-transformation.  H_a ... H_{a+7} = I - V T V^H with an upper triangular T (8 x 8): block
+// blockIdx.x of eight reflectors, T row by row into Tb.
+constexpr int BTK = 8;
+constexpr int BT_MIN = 24;  // rows from which the blocked form is used (l = 30 real: the same 25 us;
+                            // l = 60 real 58 -> 26 us, l = 600 complex 3.5 -> 2.05 ms)
+
+template <class T>
+__global__ void __launch_bounds__(256) bt_factor_kernel(int l, const T* __restrict__ H, int ldh,
+                                                        const T* __restrict__ tau, T* __restrict__ Tb) {
+  dep_wait(false);
+  __shared__ T G[BTK][BTK], S[BTK][BTK];
+  const int a = blockIdx.x * BTK, kb = min(BTK, l - 1 - a), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < BTK * BTK) S[threadIdx.x / BTK][threadIdx.x % BTK] = Sc<T>::zero();
+  for (int u = warp; u < BTK * BTK; u += 8) {  // G[i][j] = v_i^H v_j, i < j
+    const int i = u / BTK, j = u % BTK;
+    if (i >= j || j >= kb) continue;
+    T s = Sc<T>::zero();
+    for (int r = a + j + 1 + lane; r < l; r += 32)
+      Sc<T>::fmac(s, H[(size_t)r + (size_t)(a + i) * ldh], H[(size_t)r + (size_t)(a + j) * ldh]);
+    s = warp_addt(s);
+    if (lane == 0) G[i][j] = s;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    for (int j = 0; j < kb; ++j) {  // column j: tau_j, above it -tau_j T G[:, j]
+      const T t = tau[a + j];
+      if (lane < j) {
+        T s = Sc<T>::zero();
+        for (int k = lane; k < j; ++k) Sc<T>::fma(s, S[lane][k], G[k][j]);
+        S[lane][j] = Sc<T>::scale(Sc<T>::mul(t, s), -1.0);
+      } else if (lane == j) {
+        S[j][j] = t;
+      }
+      __syncwarp();
+    }
+    for (int u = lane; u < BTK * BTK; u += 32) Tb[(size_t)blockIdx.x * BTK * BTK + u] = S[u / BTK][u % BTK];
+  }
+}
+
+// Sums over the warp of the eight values of every lane: lane 4 i .. 4 i + 3 gets value i.  Halves
+// are exchanged, so it takes 9 additions (complex 18) instead of 40 (80): each holds the FP64 pipe
+// for 64 clocks.
+__device__ __forceinline__ double sum8(const double* v, int lane) {
+  double a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double keep = lane & 16 ? v[k + 4] : v[k], send = lane & 16 ? v[k] : v[k + 4];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double keep = lane & 8 ? a[k + 2] : a[k], send = lane & 8 ? a[k] : a[k + 2];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+  double c = (lane & 4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+__device__ __forceinline__ double sum8t(const double* s, int lane) { return sum8(s, lane); }
+__device__ __forceinline__ z64 sum8t(const z64* s, int lane) {
+  double re[8], im[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) { re[j] = s[j].x; im[j] = s[j].y; }
+  return z64{sum8(re, lane), sum8(im, lane)};
+}
+__device__ __forceinline__ double shfl_t(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ z64 shfl_t(z64 v, int src) { return z64{shfl_t(v.x, src), shfl_t(v.y, src)}; }
+
+// Column c of W = H_0 H_1 ... H_{l-2} Z[:, c], eight reflectors at a time: z -= V (T (V^H z)).  One
+// warp per column, z in shared memory, the next 32 rows of V loaded ahead of their use; dw = D (NaN
+// if T was not finite).  FP64-bound (8 l^2 / 2 FMAs of a complex column on one sub-partition): one
+// reflector at a time waited for each one's loads and for 10 additions of the warp's sum.
+template <class T>
+__global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* __restrict__ H, int ldh,
+                                                       const T* __restrict__ Tb, const double* __restrict__ Z,
+                                                       const double* __restrict__ D, const int* bad, T* Wm, int ldw,
+                                                       double* dw) {
+  dep_wait(false);
+  extern __shared__ __align__(16) unsigned char bt_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (c >= l) return;
+  const bool nan_out = *bad != 0;
+  T* z = (T*)bt_smem + (size_t)warp * l;
+  for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(nan_out ? nan("") : Z[(size_t)i + (size_t)c * l]);
+  if (lane == 0) dw[c] = nan_out ? nan("") : D[c];
+  __syncwarp();
+  const int nb = nan_out ? 0 : (l - 1 + BTK - 1) / BTK;
+  for (int b = nb - 1; b >= 0; --b) {
+    const int a = b * BTK, kb = min(BTK, l - 1 - a), r0 = (a + 1) & ~31;
+    T x[BTK], y[BTK], s[BTK];
+    auto load = [&](int i) {
+#pragma unroll
+      for (int j = 0; j < BTK; ++j)
+        y[j] = (j < kb && i > a + j && i < l) ? H[(size_t)i + (size_t)(a + j) * ldh] : Sc<T>::zero();
+    };
+    const int ti = lane >> 2, tk = lane & 3;
+    const T t0 = Tb[(size_t)b * BTK * BTK + ti * BTK + tk], t1 = Tb[(size_t)b * BTK * BTK + ti * BTK + tk + 4];
+#pragma unroll
+    for (int j = 0; j < BTK; ++j) s[j] = Sc<T>::zero();
+    load(r0 + lane);
+    for (int i = r0 + lane; i - lane < l; i += 32) {
+#pragma unroll
+      for (int j = 0; j < BTK; ++j) x[j] = y[j];
+      if (i - lane + 32 < l) load(i + 32);
+      const T zi = i < l ? z[i] : Sc<T>::zero();
+#pragma unroll
+      for (int j = 0; j < BTK; ++j) Sc<T>::fmac(s[j], x[j], zi);
+    }
+    load(r0 + lane);
+    const T q = sum8t(s, lane);  // of reflector lane / 4
+    T u = Sc<T>::mul(t0, shfl_t(q, 4 * tk));
+    Sc<T>::fma(u, t1, shfl_t(q, 4 * (tk + 4)));
+    u = Sc<T>::add(u, shfl_t(u, lane ^ 1));
+    u = Sc<T>::scale(Sc<T>::add(u, shfl_t(u, lane ^ 2)), -1.0);
+#pragma unroll
+    for (int j = 0; j < BTK; ++j) s[j] = shfl_t(u, 4 * j);
+    for (int i = r0 + lane; i - lane < l; i += 32) {
+#pragma unroll
+      for (int j = 0; j < BTK; ++j) x[j] = y[j];
+      if (i - lane + 32 < l) load(i + 32);
+      T zi = i < l ? z[i] : Sc<T>::zero();
+#pragma unroll
+      for (int j = 0; j < BTK; ++j) Sc<T>::fma(zi, x[j], s[j]);
+      if (i < l) z[i] = zi;
+    }
+  }
+  T* out = Wm + (size_t)c * ldw;
+  for (int i = lane; i < l; i += 32) out[i] = z[i];
+}
+
+// The same one reflector at a time, for few rows and for columns that do not fit shared memory.
 // Column c of W = H_0 H_1 ... H_{l-2} Z[:, c]: one warp per column, the column in shared memory
 // (in_smem) or in place; dw = D (NaN if T was not finite).
 template <class T>
 __global__ void backtransform_kernel(int l, const T* __restrict__ H, int ldh, const T* __restrict__ tau,
                                      const double* __restrict__ Z, const double* __restrict__ D, const int* bad,
                                      T* Wm, int ldw, double* dw, int in_smem) {
-  dep_wait();
+  dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
   if (c >= l) return;
@@ -773,8 +945,18 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   const int in_smem = smem <= kSmemMax - 1024;
   CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)backtransform_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSmemMax - 1024));
-  launch_dep(st, ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, backtransform_kernel<T>, l, H, ldh, tau, D.Q[cur],
-             D.D[cur], D.bad, W, ldw, dw, in_smem);
+  if (in_smem && l >= BT_MIN) {
+    T* Tb = (T*)D.U;  // free by now: l^2 doubles for 8 (l + 7) elements
+    launch_dep(st, ceil_div(l - 1, BTK), 256, 0, bt_factor_kernel<T>, l, H, ldh, tau, Tb);
+    CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)bt_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kSmemMax - 1024));
+    launch_dep(st, ceil_div(l, wpc), 32 * wpc, smem, bt_block_kernel<T>, l, H, ldh, Tb, D.Q[cur], D.D[cur], D.bad, W,
+               ldw, dw);
+    if (launches) ++*launches;
+  } else {
+    launch_dep(st, ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, backtransform_kernel<T>, l, H, ldh, tau, D.Q[cur],
+               D.D[cur], D.bad, W, ldw, dw, in_smem);
+  }
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());
   return 0;

@@ -137,7 +137,7 @@ def cl():
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("complex_", [False, True])
-@pytest.mark.parametrize("n", [1, 2, 3, 31, 32, 33, 63, 64, 65, 129, 257, 601])
+@pytest.mark.parametrize("n", [1, 2, 3, 23, 24, 31, 32, 33, 63, 64, 65, 129, 257, 601])
 @pytest.mark.parametrize("spectrum", ["uniform", "multiple", "diagonal"])
 def test_whole_space_rayleigh_ritz(cl, complex_, n, spectrum):
     """nev = n, nex = 0: after one iteration (degree 1, far from the damped interval) the Ritz
