@@ -39,34 +39,49 @@ int fail_cuda(cudaError_t e, const char* what, const char* file, int line) {
 using namespace chase;
 
 // CUDA-event time of selected launches on one stream (the filter's product kernels):
-// event pairs around each launch, summed once the stream has been synchronised.
+// event pairs around each launch, summed once the stream has been synchronised.  Of short launches
+// (`few_us`) every eighth is timed and stands for eight: an event takes a few microseconds between
+// two launches, and launch_dep's overlap with it (a filter step of n = 1000, 30 columns: 34 us
+// with two events in every step, 25 without).
 struct LaunchTimer {
   std::vector<cudaEvent_t> ev;
   size_t used = 0;
   bool enabled = true;  // off while a stream is being captured into a graph
-  void begin(cudaStream_t st) {
+  bool open = false;
+  std::vector<char> few;            // per pair: a short launch
+  size_t few_all = 0, few_timed = 0;
+  void begin(cudaStream_t st, bool few_us = false) {
     if (!enabled) return;
+    if (few_us && few_all++ % 8) return;
     while (ev.size() < used + 2) {
       cudaEvent_t e;
       if (cudaEventCreate(&e) != cudaSuccess) return;
       ev.push_back(e);
     }
     cudaEventRecord(ev[used], st);
+    few.resize(used / 2);
+    few.push_back(few_us);
+    few_timed += few_us;
+    open = true;
   }
   void end(cudaStream_t st) {
-    if (!enabled || ev.size() < used + 2) return;
+    if (!open) return;
     cudaEventRecord(ev[used + 1], st);
     used += 2;
+    open = false;
   }
   double collect() {  // seconds; call after the stream has been synchronised
-    double s = 0.0;
+    double s = 0.0, f = 0.0;
     for (size_t i = 0; i + 1 < used; i += 2) {
       float ms = 0.f;
-      if (cudaEventElapsedTime(&ms, ev[i], ev[i + 1]) == cudaSuccess) s += ms;
+      if (cudaEventElapsedTime(&ms, ev[i], ev[i + 1]) == cudaSuccess) (few[i / 2] ? f : s) += ms;
     }
-    used = 0;
+    if (few_timed) s += f * ((double)few_all / (double)few_timed);
+    used = few_all = few_timed = 0;
     return s * 1e-3;
   }
+  // a product of fewer operations takes under ~100 us (the emulated one 60 us at 2e10)
+  static constexpr double kFewUsFlops = 2e10;
   ~LaunchTimer() {
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   }
@@ -299,7 +314,7 @@ int filter_mixed(chase_ctx* h, int n, const T* A, int lda, bool split_A, int nco
       gamma = -sigma * sn;
       sigma = sn;
     }
-    h->product_timer.begin(st);
+    h->product_timer.begin(st, per_col * act < LaunchTimer::kFewUsFlops);
     TRY(tc_filter_step(st, M, kp, B.Ah, B.Al, B.Vh[in], B.Vl[in], ncols, first, act, alpha, beta,
                        B.V64[in], gamma, B.V64[out], B.V64[out], kp, B.Vh[out], B.Vl[out],
                        h->dstat, &h->launches));
@@ -456,12 +471,12 @@ int filter_oz_enqueue(chase_ctx* h, int n, const T* A, int lda, bool split_A, in
       const OzGroupItem it = oz_item(B, ncols, first, act, alpha, beta, B.V64[in], gamma, B.V64[out],
                                      B.V64[out], B.V64[in]);
       TRY(oz_slice_V_group(st, 1, &it, &h->launches));
-      h->product_timer.begin(st);
+      h->product_timer.begin(st, per_col * act < LaunchTimer::kFewUsFlops);
       TRY(oz_gemm_group(st, 1, &it, h->dstat, &h->launches));
       h->product_timer.end(st);
     } else {
       TRY(oz_slice_V(st, M, first, ncols, B.V64[in], kp, kp, ncols, B.Vp, B.colexp, &h->launches));
-      h->product_timer.begin(st);
+      h->product_timer.begin(st, per_col * act < LaunchTimer::kFewUsFlops);
       TRY(oz_gemm(st, M, kp, B.Ap, B.rowexp, 0, B.Vp, B.colexp, ncols, first, act, alpha, beta,
                   B.V64[in], gamma, B.V64[out], B.V64[out], kp, h->dstat, B.res, &h->launches,
                   h->autotune, &h->tune_trials));
