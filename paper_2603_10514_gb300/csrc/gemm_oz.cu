@@ -443,7 +443,10 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
   cluster_sync();  // both CTAs' barriers initialised before any copy or arrival crosses over
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
-  dep_wait();  // (the set-up above runs beside the end of the launch before)
+  // (the set-up above runs beside the end of the launch before; the reconstruction after it is not
+  // placed early, on the few SMs that the last tiles leave free: n = 1000 real, 30 columns, a filter
+  // of 20 steps 492 -> 444 us, a solve 9.1 -> 8.1 ms)
+  dep_wait(false);
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(M_REG_MAIN));
