@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(CNT) chol_kernel(int n, T* G, int ldg, double 
 
 // Columns blockIdx.x and n - 1 - blockIdx.x of R^{-1} (n > CB).
 template <class T>
-__global__ void __launch_bounds__(128) trinv_kernel(int n, const T* __restrict__ R, int ldr,
-                                                    const T* __restrict__ Mb, T* Rinv, int ldri,
+__global__ void __launch_bounds__(128) trinv_kernel(int n, const T* R, int ldr,
+                                                    const T* Mb, T* Rinv, int ldri,
                                                     const DevStatus* dst) {
   dep_wait();
   extern __shared__ __align__(16) unsigned char inv_smem[];

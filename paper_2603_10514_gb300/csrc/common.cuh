@@ -103,7 +103,8 @@ struct DevStatus {
 // Launch of a kernel that may be set up, and its blocks placed, while the launch before it on the
 // stream is still running (programmatic dependent launch).  Such a kernel calls dep_wait() in every
 // thread before it touches global memory: it returns when the launches before have completed and
-// their writes are seen, so their order is that of plain launches.  A plain launch, a copy or an
+// their writes are seen, so their order is that of plain launches.  Its pointer parameters are not
+// `const __restrict__`: loads through those count as invariant, and may be moved above the wait.  A plain launch, a copy or an
 // event still waits for the whole kernel before it.  It takes the launch latency and the set-up
 // (barriers, tensor memory) out of a chain of short kernels: n = 1000 real, 30 columns, a filter
 // step 35 -> 27 us, a solve of 30 vectors 11.6 -> 10.9 ms.  early = false: the next launch's blocks
@@ -111,8 +112,8 @@ struct DevStatus {
 // costs a launch of about one long block per SM more than its latency: divide and conquer and
 // back-transformation of l = 600 complex 5.3 ms so, 7.0 placed early; no difference at l = 30 to 230).
 __device__ __forceinline__ void dep_wait(bool early = true) {
-  cudaGridDependencySynchronize();
-  if (early) cudaTriggerProgrammaticLaunchCompletion();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <class T> struct SameType { using type = T; };
 template <class... P>
@@ -132,6 +133,25 @@ inline cudaError_t launch_dep(cudaStream_t st, dim3 grid, dim3 block, size_t sme
   return cudaLaunchKernelExC(&cfg, (const void*)kernel, p);
 }
 
+// Sums over the warp of the eight values of every lane: lane 4 i .. 4 i + 3 gets value i.  Halves
+// are exchanged, so it takes 9 additions (complex 18) instead of 40 (80): each holds the FP64 pipe
+// for 64 clocks.
+__device__ __forceinline__ double sum8(const double* v, int lane) {
+  double a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double keep = lane & 16 ? v[k + 4] : v[k], send = lane & 16 ? v[k] : v[k + 4];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const double keep = lane & 8 ? a[k + 2] : a[k], send = lane & 8 ? a[k] : a[k + 2];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+  double c = (lane & 4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
 // Grid-wide barrier of a cooperative launch on a counter that only grows: barrier k ends
 // once all G CTAs have added their arrival (count >= (k + 1) G).  One release-add per CTA
 // and acquire polls with a short back-off.  Bounded: returns false (the caller leaves the

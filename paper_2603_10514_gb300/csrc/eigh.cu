@@ -493,8 +493,8 @@ __device__ inline void dc_pair(double e, double* D, double* q, int ldq) {
 // the merges of a level at once with 8, 4, 2 or 1 of the warps each.  Latency-bound: a chain of
 // divisions and square roots per root.  l = 30: 252 -> 195 us against merges from single rows
 // with one warp or the whole CTA each.
-__global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const double* __restrict__ d0,
-                                                      const double* __restrict__ e0, int ld_de, DcWork W0,
+__global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const double* d0,
+                                                      const double* e0, int ld_de, DcWork W0,
                                                       size_t stride) {
   dep_wait(false);
   __shared__ double sQ[LEAF * LEAF], sQn[LEAF * LEAF], sU[LEAF * LEAF];
@@ -551,7 +551,7 @@ __device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, 
 }
 
 __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                       const double* __restrict__ e0, int ld_de) {
+                                                       const double* e0, int ld_de) {
   dep_wait(false);
   __shared__ double red[16];
   const DcWork W = dc_at(W0, stride * blockIdx.y);
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride,
 
 // phase 0: roots, and the rotations of Q's rows; 1: corrected z; 2: U and the new order.
 __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                       const double* __restrict__ e0, int ld_de, int phase) {
+                                                       const double* e0, int ld_de, int phase) {
   dep_wait(false);
   const DcWork W = dc_at(W0, stride * blockIdx.z);
   int s;
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride,
 
 // Q_new[:, dest] = Q[:, gathered] U (64 x 32 tiles, FP64), deflated columns copied.
 __global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                      const double* __restrict__ e0, int ld_de, int parts) {
+                                                      const double* e0, int ld_de, int parts) {
   dep_wait(false);
   const DcWork W = dc_at(W0, stride * (blockIdx.z / parts));
   int s;
@@ -688,8 +688,8 @@ constexpr int BT_MIN = 24;  // rows from which the blocked form is used (l = 30 
                             // l = 60 real 58 -> 26 us, l = 600 complex 3.5 -> 2.05 ms)
 
 template <class T>
-__global__ void __launch_bounds__(256) bt_factor_kernel(int l, const T* __restrict__ H, int ldh,
-                                                        const T* __restrict__ tau, T* __restrict__ Tb) {
+__global__ void __launch_bounds__(256) bt_factor_kernel(int l, const T* H, int ldh,
+                                                        const T* tau, T* Tb) {
   dep_wait(false);
   __shared__ T G[BTK][BTK], S[BTK][BTK];
   const int a = blockIdx.x * BTK, kb = min(BTK, l - 1 - a), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -720,25 +720,6 @@ __global__ void __launch_bounds__(256) bt_factor_kernel(int l, const T* __restri
   }
 }
 
-// Sums over the warp of the eight values of every lane: lane 4 i .. 4 i + 3 gets value i.  Halves
-// are exchanged, so it takes 9 additions (complex 18) instead of 40 (80): each holds the FP64 pipe
-// for 64 clocks.
-__device__ __forceinline__ double sum8(const double* v, int lane) {
-  double a[4], b[2];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const double keep = lane & 16 ? v[k + 4] : v[k], send = lane & 16 ? v[k] : v[k + 4];
-    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const double keep = lane & 8 ? a[k + 2] : a[k], send = lane & 8 ? a[k] : a[k + 2];
-    b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  double c = (lane & 4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? b[0] : b[1], 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  return c + __shfl_xor_sync(0xffffffffu, c, 1);
-}
 __device__ __forceinline__ double sum8t(const double* s, int lane) { return sum8(s, lane); }
 __device__ __forceinline__ z64 sum8t(const z64* s, int lane) {
   double re[8], im[8];
@@ -754,9 +735,9 @@ __device__ __forceinline__ z64 shfl_t(z64 v, int src) { return z64{shfl_t(v.x, s
 // if T was not finite).  FP64-bound (8 l^2 / 2 FMAs of a complex column on one sub-partition): one
 // reflector at a time waited for each one's loads and for 10 additions of the warp's sum.
 template <class T>
-__global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* __restrict__ H, int ldh,
-                                                       const T* __restrict__ Tb, const double* __restrict__ Z,
-                                                       const double* __restrict__ D, const int* bad, T* Wm, int ldw,
+__global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ldh,
+                                                       const T* Tb, const double* Z,
+                                                       const double* D, const int* bad, T* Wm, int ldw,
                                                        double* dw) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
@@ -815,8 +796,8 @@ __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* __restric
 // Column c of W = H_0 H_1 ... H_{l-2} Z[:, c]: one warp per column, the column in shared memory
 // (in_smem) or in place; dw = D (NaN if T was not finite).
 template <class T>
-__global__ void backtransform_kernel(int l, const T* __restrict__ H, int ldh, const T* __restrict__ tau,
-                                     const double* __restrict__ Z, const double* __restrict__ D, const int* bad,
+__global__ void backtransform_kernel(int l, const T* H, int ldh, const T* tau,
+                                     const double* Z, const double* D, const int* bad,
                                      T* Wm, int ldw, double* dw, int in_smem) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];

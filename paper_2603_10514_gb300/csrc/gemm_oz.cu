@@ -644,7 +644,7 @@ __device__ __forceinline__ void pair_tile_coords(int x, int ntile, int BN, int* 
 __global__ void __launch_bounds__(M_THREADS, 1)
     ozm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapV,
                int M, int N, int BN, int ntile, int col0, int nkb_total, int kbs,
-               uint8_t* __restrict__ R, DevStatus* status) {
+               uint8_t* R, DevStatus* status) {
   const int jm = blockIdx.z % kOzModuli, split = blockIdx.z / kOzModuli;
   const int kbeg = split * kbs;
   const int nkb = max(0, min(kbs, nkb_total - kbeg));
@@ -1070,7 +1070,7 @@ inline int slice_parts(int kp, int cols) {
 
 // Real A (n x n): residues of row m (column m of A: symmetric) into planes (row-major, ld kp),
 // row exponent into rowexp[m].
-__global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __restrict__ A, int lda,
+__global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* A, int lda,
                                                          int kp, __nv_bfloat16* planes,
                                                          size_t plane, int* rowexp) {
   dep_wait();
@@ -1084,7 +1084,7 @@ __global__ void __launch_bounds__(256) oz_slice_A_kernel(int n, const double* __
 
 // FP64 stacked block V64 (M x ncols, ld ldi): residues of column c into planes
 // (column-major, ld kp; rows >= M zero), column exponent into colexp[c].
-__global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const double* __restrict__ V64,
+__global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const double* V64,
                                                          int ldi, int kp, __nv_bfloat16* planes,
                                                          size_t plane, int* colexp) {
   dep_wait();
@@ -1104,7 +1104,7 @@ __global__ void __launch_bounds__(256) oz_slice_V_kernel(int M, int c0, const do
 // Row m of A (complex Hermitian, column-major): its integer row from column m of A
 // (A[m, k] = conj(A[k, m])): Ar[m, k] = Re A[k, m], Ai[m, k] = -Im A[k, m].
 template <int NM>
-__global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* __restrict__ A, int lda,
+__global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* A, int lda,
                                                               int kpn, __nv_bfloat16* planes, size_t plane,
                                                               int* rowexp) {
   dep_wait();
@@ -1190,7 +1190,7 @@ __global__ void __launch_bounds__(256) oz_slice_V_group_kernel(const __grid_cons
 
 // Caller's block V (n x ncols, ld ldv) -> stacked FP64 (M x ncols, ld ldo).
 template <class T>
-__global__ void stack_V_kernel(int n, int ncols, const T* __restrict__ V, int ldv, double* V64,
+__global__ void stack_V_kernel(int n, int ncols, const T* V, int ldv, double* V64,
                                int ldo) {
   dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
@@ -1212,7 +1212,7 @@ __global__ void stack_V_kernel(int n, int ncols, const T* __restrict__ V, int ld
 // Column blockIdx.x of a complex block Y (n x q, ld ldy): its exponent (over Re and Im) and its
 // two plane rows (u | w), ld kp; entries past n are zero.
 template <int NM>
-__global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z64* __restrict__ Y, int ldy, int kp,
+__global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z64* Y, int ldy, int kp,
                                                                  __nv_bfloat16* planes, size_t plane,
                                                                  int* colexp) {
   dep_wait();
@@ -1241,7 +1241,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols_ring_kernel(int n, const z6
 
 // Row exponents (over Re and Im) of a column-major complex X (n x l): 32 rows per CTA, eight
 // column groups.
-__global__ void __launch_bounds__(256) oz_row_exp_kernel(int n, int l, const z64* __restrict__ X, int ldx,
+__global__ void __launch_bounds__(256) oz_row_exp_kernel(int n, int l, const z64* X, int ldx,
                                                          int* rowexp) {
   dep_wait();
   __shared__ unsigned long long red[8][32];
@@ -1265,9 +1265,9 @@ __global__ void __launch_bounds__(256) oz_row_exp_kernel(int n, int l, const z64
 // x 64 of K per CTA through shared memory, so that X is read along its columns and the planes
 // are written along K.
 template <int NM>
-__global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, const z64* __restrict__ X, int ldx,
+__global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, const z64* X, int ldx,
                                                                  int kp, __nv_bfloat16* planes, size_t plane,
-                                                                 const int* __restrict__ rowexp) {
+                                                                 const int* rowexp) {
   dep_wait();
   __shared__ z64 tile[64][33];
   const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
@@ -1292,7 +1292,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows_ring_kernel(int n, int l, c
 
 // Xt (l x n, ld ldt) is the transpose of a real column-major X (n x l): row m of X is column m
 // of Xt.  Residues of the rows into planes (row-major, ld kp), row exponents into rowexp.
-__global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double* __restrict__ Xt, int ldt, int kp,
+__global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double* Xt, int ldt, int kp,
                                                             __nv_bfloat16* planes, size_t plane, int* rowexp) {
   dep_wait();
   __shared__ unsigned long long red[8];
@@ -1305,7 +1305,7 @@ __global__ void __launch_bounds__(256) oz_slice_rows_kernel(int l, const double*
 
 // Residues of the columns of a real block Y (n x q, ld ldy): planes column-major (ld kp; rows
 // >= n are zero), column exponents.
-__global__ void __launch_bounds__(256) oz_slice_cols_kernel(int n, const double* __restrict__ Y, int ldy, int kp,
+__global__ void __launch_bounds__(256) oz_slice_cols_kernel(int n, const double* Y, int ldy, int kp,
                                                             __nv_bfloat16* planes, size_t plane, int* colexp) {
   dep_wait();
   __shared__ unsigned long long red[8];
@@ -1317,7 +1317,7 @@ __global__ void __launch_bounds__(256) oz_slice_cols_kernel(int n, const double*
 }
 
 // Xt = X^T: real X n x l (ld ldx) -> Xt l x n (ld ldt).
-__global__ void transpose_kernel(int n, int l, const double* __restrict__ X, int ldx, double* Xt, int ldt) {
+__global__ void transpose_kernel(int n, int l, const double* X, int ldx, double* Xt, int ldt) {
   dep_wait();
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;

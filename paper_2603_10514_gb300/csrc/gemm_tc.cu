@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // once and written to its two places (the splits' FP64 conversions and subtraction, at 2 per
 // clock per SM, bind).  Row blockIdx.y of A, K along x; the last column block pads to kp.
 template <class T>
-__global__ void __launch_bounds__(256) split_A_kernel(int n, const T* __restrict__ A, int lda, int kp,
+__global__ void __launch_bounds__(256) split_A_kernel(int n, const T* A, int lda, int kp,
                                                       __nv_bfloat16* Ah, __nv_bfloat16* Al) {
   dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(256) split_A_kernel(int n, const T* __restrict
 // Complex/real block V (n x ncols, ld ldv) -> stacked FP64 (M x ncols, ld ldo) and its
 // BF16 hi/lo split (ld kp, rows >= M zero).
 template <class T>
-__global__ void split_V_kernel(int n, int ncols, const T* __restrict__ V, int ldv, double* V64,
+__global__ void split_V_kernel(int n, int ncols, const T* V, int ldv, double* V64,
                                int ldo, int kp, __nv_bfloat16* Vh, __nv_bfloat16* Vl) {
   dep_wait();
   const int M = Sc<T>::cplx ? 2 * n : n;
@@ -265,7 +265,7 @@ __global__ void split_V_kernel(int n, int ncols, const T* __restrict__ V, int ld
 
 // Stacked FP64 columns [c0, c1) back into the caller's layout.
 template <class T>
-__global__ void unstack_V_kernel(int n, int c0, int c1, const double* __restrict__ V64, int ldi,
+__global__ void unstack_V_kernel(int n, int c0, int c1, const double* V64, int ldi,
                                  T* V, int ldv, bool subtract) {
   dep_wait();
   const size_t total = (size_t)n * (c1 - c0);

@@ -27,9 +27,9 @@ __global__ void herm_fill_lower_kernel(int n, T* G, int ldg) {
 
 // One CTA per column: r_a = ||AV[:,a] - theta_a V[:,a]|| / ||V[:,a]||.
 template <class T>
-__global__ void __launch_bounds__(256) resid_norms_kernel(int n, const T* __restrict__ AV, int ldav,
-                                                          const T* __restrict__ V, int ldv,
-                                                          const double* __restrict__ theta,
+__global__ void __launch_bounds__(256) resid_norms_kernel(int n, const T* AV, int ldav,
+                                                          const T* V, int ldv,
+                                                          const double* theta,
                                                           double* res) {
   dep_wait();
   __shared__ double r0[8], r1[8];
