@@ -714,7 +714,7 @@ def main():
         pipe = tc_flops / nl / dur_launch / 1e12 if dur_launch > 0 else None
         traffic = (OZ_TRAFFIC_PER_LAUNCH if (OZ_TRAFFIC_PER_LAUNCH and lp == 0 and args.n == 10000
                                              and args.prec == "fp64_emu") else None)
-        roof = {"kernel": "ozm_group_kernel + crt_ring_kernel (Ozaki scheme II FP64 product: 15 "
+        roof = {"kernel": "ozm_group_kernel + crt_kernel (Ozaki scheme II FP64 product: 15 "
                           "moduli x 2 modular BF16 tcgen05 products, CRT reconstruction)" +
                           (" + tc_filter_bf16x3_kernel" if lp > 0 else ""),
                 "bound": "tensor", "achieved": achieved, "peak": BF16_SUSTAINED_TFLOPS,
