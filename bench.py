@@ -54,8 +54,9 @@ BF16_PEAK_TFLOPS, BF16_SUSTAINED_TFLOPS = _measured_peaks()
 RING_MODULI = 15
 OZAKI_PAIRS = RING_MODULI * 0.5   # the default workload is complex
 # DRAM bytes (read + write) of one emulated product of the default workload (complex
-# n = 10000, 600 active columns) by an ncu capture; None until one of these kernels is taken.
-OZ_TRAFFIC_PER_LAUNCH = None
+# n = 10000, 600 active columns), by ncu in one pass: ozm_group_kernel 6.78 + 0.36 GB, crt_kernel
+# 0.46 + 0.08 GB.
+OZ_TRAFFIC_PER_LAUNCH = 7.67e9
 # Column MatVecs of one complete solve of the default workload as counted by the GPU path
 # (filter MatVecs plus the 2 (ell - k) products of Rayleigh-Ritz and residuals per
 # iteration); used to scale the oracle's timed sample to a whole solve.  Measured on a
