@@ -256,26 +256,25 @@ DC_FN void ucol(const L& l, int K, int j, bool write, const double* dl, const do
     for (int i = l.lane; i < K; i += l.width) U[(size_t)pos[i] + (size_t)j * ldu] = zh[i] / ((dl[i] - dorg) - m) * r;
 }
 
-// New position of value t (t < K: root t; else the deflated value t - K).
+// New position of value t (t < K: root t; else the deflated value t - K).  One count for both kinds:
+// the groups of a warp may hold both, and its lanes have to meet in the same shuffles.
 template <class L>
 DC_FN void place(const L& l, const Merge& M, int K, int t, bool write) {
   const int nd = M.m - K;
+  const bool is_root = t < K;
+  const double v = is_root ? M.lam[t] : M.ds[M.defl[t - K]];
   int n = 0;
-  double v;
-  if (t < K) {
-    v = M.lam[t];
+  if (is_root) {
     for (int u = l.lane; u < nd; u += l.width) n += M.ds[M.defl[u]] < v;
-    n = l.count(n) + t;
   } else {
     const int me = t - K;
-    v = M.ds[M.defl[me]];
     for (int k = l.lane; k < K; k += l.width) n += M.lam[k] <= v;
     for (int u = l.lane; u < nd; u += l.width) {
       const double x = M.ds[M.defl[u]];
       n += x < v || (x == v && u < me);
     }
-    n = l.count(n);
   }
+  n = l.count(n) + (is_root ? t : 0);
   if (l.lane == 0 && write) M.dest[t] = n;
 }
 
