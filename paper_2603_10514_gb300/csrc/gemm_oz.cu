@@ -507,7 +507,9 @@ __device__ __forceinline__ void ozm_pair_tile(const CUtensorMap* mapA, const CUt
             const int to = two ? (sw % 3 == 0 ? 0 : 3 - sw % 3) : sw & 1;
             commit_pair(&cfull[from], leader);
             if ((given >> to) & 1) {  // read out since it was given up
-              if (!bar_poll(&cfree[to], (fph >> to) & 1)) { bad = true; break; }
+              if (!bar_poll_cluster(&cfree[to], (fph >> to) & 1)) { bad = true; break; }
+              // the stage's fence was before this wait: the MMAs below overwrite what was read out
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               fph ^= 1u << to;
             }
             given |= 1u << from;

@@ -58,6 +58,25 @@ __device__ __forceinline__ bool bar_poll(uint64_t* b, uint32_t ph) {
     if (clock64() - t0 > kTcWait) return false;
   }
 }
+// The same for a barrier that threads of the other CTA arrive on (arrive_remote).
+__device__ __forceinline__ bool bar_test_cluster(uint64_t* b, uint32_t ph) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(s32(b)), "r"(ph)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool bar_poll_cluster(uint64_t* b, uint32_t ph) {
+  if (bar_test_cluster(b, ph)) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (bar_test_cluster(b, ph)) return true;
+    if (clock64() - t0 > kTcWait) return false;
+  }
+}
 // The same shared-memory offset in CTA `rank` of the cluster, as a shared::cluster address.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
   uint32_t r;
@@ -73,11 +92,11 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
-// Arrival that hands a TMEM buffer back (after tcgen05.wait::ld and fence::before_thread_sync:
-// the loaded values are in registers and no other memory is passed on, so it is relaxed: a
-// release at cluster scope costs a memory barrier per arrival).
+// Arrival that hands a TMEM buffer back, after tcgen05.wait::ld and fence::before_thread_sync of
+// every lane.  The waiting side (bar_poll_cluster) puts a fence::after_thread_sync before the MMAs
+// that overwrite the buffer.
 __device__ __forceinline__ void arrive_remote(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
                : "memory");
 }
 // TMA tile load into this CTA's shared memory whose completion is counted on a barrier of

@@ -1,0 +1,44 @@
+"""Orderings that a kernel has to ask for and that no result shows reliably, read off the sources:
+a wait that hands an accumulator in tensor memory over is followed by a tcgen05 fence before the
+next MMA, and the arrival that it waits for releases."""
+import os
+import re
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2603_10514_gb300", "csrc")
+
+
+def code(name):
+    """A source file without its comments."""
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"/\*.*?\*/", "", re.sub(r"//[^\n]*", "", text), flags=re.S)
+
+
+def function(text, head):
+    """The body of the function that starts with `head`."""
+    at = text.index("{", text.index(head))
+    depth, i = 0, at
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[at:i + 1]
+        i += 1
+
+
+def test_issuer_fences_after_every_wait():
+    text = code("gemm_oz.cu")
+    issuer = text[text.index("elect_lane()"):]
+    issuer = issuer[:issuer.index("setmaxnreg.inc")]
+    waits = [m.start() for m in re.finditer(r"bar_poll\w*\(", issuer)]
+    assert len(waits) == 2  # a stage, an accumulator
+    for w in waits:
+        rest = issuer[w:]
+        assert rest.index("tcgen05.fence::after_thread_sync") < rest.index("mma_pair("), rest[:60]
+
+
+def test_accumulator_release_and_acquire_reach_the_cluster():
+    helpers = code("tcgen05.cuh")
+    assert "mbarrier.arrive.release.cluster" in function(helpers, "void arrive_remote(")
+    assert "acquire.cluster" in function(helpers, "bool bar_test_cluster(")
+    oz = code("gemm_oz.cu")
+    assert re.search(r"bar_poll_cluster\(&cfree\[", oz)
