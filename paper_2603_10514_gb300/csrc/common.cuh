@@ -103,8 +103,9 @@ struct DevStatus {
 // Launch of a kernel that may be set up, and its blocks placed, while the launch before it on the
 // stream is still running (programmatic dependent launch).  Such a kernel calls dep_wait() in every
 // thread before it touches global memory: it returns when the launches before have completed and
-// their writes are seen, so their order is that of plain launches.  Its pointer parameters are not
-// `const __restrict__`: loads through those count as invariant, and may be moved above the wait.  A plain launch, a copy or an
+// their writes are seen, so their order is that of plain launches.  No load of such a kernel may be
+// an invariant one, which may be moved above the wait: its pointers, and those of the functions it
+// calls, are not `const __restrict__`, and it uses no __ldg.  A plain launch, a copy or an
 // event still waits for the whole kernel before it.  It takes the launch latency and the set-up
 // (barriers, tensor memory) out of a chain of short kernels: n = 1000 real, 30 columns, a filter
 // step 35 -> 27 us, a solve of 30 vectors 11.6 -> 10.9 ms.  early = false: the next launch's blocks

@@ -798,11 +798,11 @@ __device__ __forceinline__ void crt_real(const CrtItem& I, int blk) {
 #pragma unroll
   for (int j = 0; j < kOzModuli; ++j) {
     if constexpr (E == 4) {
-      w[j] = __ldg((const uint32_t*)(R + (size_t)j * plane));
-      w2[j] = I.splits > 1 ? __ldg((const uint32_t*)(R + (size_t)(kOzModuli + j) * plane)) : 0u;
+      w[j] = *(const uint32_t*)(R + (size_t)j * plane);
+      w2[j] = I.splits > 1 ? *(const uint32_t*)(R + (size_t)(kOzModuli + j) * plane) : 0u;
     } else {
-      w[j] = __ldg(R + (size_t)j * plane);
-      w2[j] = I.splits > 1 ? __ldg(R + (size_t)(kOzModuli + j) * plane) : 0u;
+      w[j] = R[(size_t)j * plane];
+      w2[j] = I.splits > 1 ? R[(size_t)(kOzModuli + j) * plane] : 0u;
     }
   }
   const int ec = I.colexp[I.col0 + c] - 2 * OZ_KBITS;
@@ -832,11 +832,11 @@ __device__ __forceinline__ void crt_ring(const CrtItem& I, int blk) {
 #pragma unroll
   for (int j = 0; j < NM; ++j) {
     if constexpr (E == 2) {
-      u[j] = __ldg((const uint32_t*)(R + (size_t)j * plane));
-      w[j] = __ldg((const uint32_t*)(R + (size_t)(NM + j) * plane));
+      u[j] = *(const uint32_t*)(R + (size_t)j * plane);
+      w[j] = *(const uint32_t*)(R + (size_t)(NM + j) * plane);
     } else {
-      u[j] = __ldg(R + (size_t)j * plane);
-      w[j] = __ldg(R + (size_t)(NM + j) * plane);
+      u[j] = R[(size_t)j * plane];
+      w[j] = R[(size_t)(NM + j) * plane];
     }
   }
   const int ec = I.colexp[I.col0 + c] - 2 * OZ_KBITS;
@@ -1041,7 +1041,7 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
 }
 
 // Exponent of n values, by the whole block.
-__device__ __forceinline__ int column_exp(const double* __restrict__ col, int n, unsigned long long* red) {
+__device__ __forceinline__ int column_exp(const double* col, int n, unsigned long long* red) {
   unsigned long long amax = 0;
 #pragma unroll 4
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
@@ -1052,7 +1052,7 @@ __device__ __forceinline__ int column_exp(const double* __restrict__ col, int n,
 }
 
 // Residues of entries [k0, k1) of a column of n values (multiples of 4; zero from n on), at idx + k.
-__device__ __forceinline__ void slice_real(const double* __restrict__ col, int n, int k0, int k1, int e,
+__device__ __forceinline__ void slice_real(const double* col, int n, int k0, int k1, int e,
                                            __nv_bfloat16* planes, size_t idx, size_t plane) {
   for (int k = k0 + 4 * threadIdx.x; k < k1; k += 4 * blockDim.x) {
     long long x[4];
@@ -1135,7 +1135,7 @@ __global__ void __launch_bounds__(256) oz_slice_A_ring_kernel(int n, const z64* 
 // Column c of the stacked FP64 block V64 ([Re V; Im V], 2n rows, ld ldi): its exponent over
 // both halves, then its two plane rows (u | w), ld kpn.
 template <int NM>
-__device__ __forceinline__ void slice_V_ring_column(int n, int c, const double* __restrict__ V64, int ldi,
+__device__ __forceinline__ void slice_V_ring_column(int n, int c, const double* V64, int ldi,
                                                     int kpn, int k0, int k1, __nv_bfloat16* planes,
                                                     size_t plane, int* colexp, unsigned long long* red) {
   const double* col = V64 + (size_t)c * ldi;

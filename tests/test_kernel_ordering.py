@@ -42,3 +42,18 @@ def test_accumulator_release_and_acquire_reach_the_cluster():
     assert "acquire.cluster" in function(helpers, "bool bar_test_cluster(")
     oz = code("gemm_oz.cu")
     assert re.search(r"bar_poll_cluster\(&cfree\[", oz)
+
+
+def test_dependent_kernels_make_no_invariant_loads():
+    """A kernel that may be placed before the launch before it has ended (it calls dep_wait) reads
+    what that launch writes: an invariant load (__ldg, or through const __restrict__, also of a
+    function that it calls) may be moved above the wait."""
+    seen = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = code(name)
+        if name == "common.cuh" or "dep_wait(" not in text:
+            continue
+        seen += 1
+        assert "__ldg(" not in text, name
+        assert not re.search(r"const\s+\w+(<\w+>)?\s*\*\s*__restrict__", text), name
+    assert seen >= 6
