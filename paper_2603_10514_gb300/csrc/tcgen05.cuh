@@ -92,11 +92,16 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
-// Arrival that hands a TMEM buffer back, after tcgen05.wait::ld and fence::before_thread_sync of
-// every lane.  The waiting side (bar_poll_cluster) puts a fence::after_thread_sync before the MMAs
-// that overwrite the buffer.
+// Arrival that hands a TMEM buffer back, by one lane after tcgen05.wait::ld and
+// tcgen05.fence::before_thread_sync of the whole warp and __syncwarp; the waiting side
+// (bar_poll_cluster) puts tcgen05.fence::after_thread_sync before the MMAs that overwrite the
+// buffer.  The two fences order the tensor memory accesses around the barrier, and nothing else is
+// passed on, so the arrival is relaxed, as in the PTX ISA's canonical synchronization pattern for
+// tcgen05.ld and tcgen05.mma in different threads.  A release at cluster scope would wait for the
+// thread's global stores: n = 10000 complex, 600 columns, a filter 72 -> 108 ms (95 ms with one
+// releasing thread per CTA).
 __device__ __forceinline__ void arrive_remote(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr)
                : "memory");
 }
 // TMA tile load into this CTA's shared memory whose completion is counted on a barrier of

@@ -1,6 +1,6 @@
 """Orderings that a kernel has to ask for and that no result shows reliably, read off the sources:
-a wait that hands an accumulator in tensor memory over is followed by a tcgen05 fence before the
-next MMA, and the arrival that it waits for releases."""
+an accumulator in tensor memory is handed from its readers to the next MMA between two tcgen05
+fences, and a kernel that may start early makes no invariant loads."""
 import os
 import re
 
@@ -36,11 +36,16 @@ def test_issuer_fences_after_every_wait():
         assert rest.index("tcgen05.fence::after_thread_sync") < rest.index("mma_pair("), rest[:60]
 
 
-def test_accumulator_release_and_acquire_reach_the_cluster():
-    helpers = code("tcgen05.cuh")
-    assert "mbarrier.arrive.release.cluster" in function(helpers, "void arrive_remote(")
+def test_accumulator_is_handed_over_between_fences():
+    """Readers: wait::ld, fence::before_thread_sync, arrival at cluster scope; issuer: a wait at
+    cluster scope (and the fence of the test above)."""
+    oz, helpers = code("gemm_oz.cu"), code("tcgen05.cuh")
+    drain = function(oz, "auto drain = [&]")
+    order = [drain.index(x) for x in ("tcgen05.wait::ld", "tcgen05.fence::before_thread_sync", "__syncwarp()",
+                                      "arrive_remote(")]
+    assert order == sorted(order)
+    assert re.search(r"mbarrier\.arrive\.\w+\.cluster\.shared::cluster", function(helpers, "void arrive_remote("))
     assert "acquire.cluster" in function(helpers, "bool bar_test_cluster(")
-    oz = code("gemm_oz.cu")
     assert re.search(r"bar_poll_cluster\(&cfree\[", oz)
 
 
