@@ -78,7 +78,8 @@ DC_FN void setup(const G& g, const Merge& M, const double* q_last, const double*
   for (int i = g.tid; i < m; i += g.size) zm = fmax(zm, fabs(M.zs[i]));
   zm = g.max(zm);
   const double dm = fmax(fabs(M.ds[0]), fabs(M.ds[m - 1]));
-  const double tol = 8.0 * kEps * fmax(dm, zm);
+  // relative to D + rho z z^T (the eigenvalues carry the matrix's scale, z is a unit vector)
+  const double tol = 8.0 * kEps * fmax(dm, M.rho * zm);
   for (int r = g.tid; r < m; r += g.size) {
     const double z = M.zs[r];
     M.small[r] = !(M.rho * fabs(z) > tol);

@@ -1,0 +1,98 @@
+"""The direct eigensolver at every scale of the matrix: what it leaves out is small against the
+matrix it is given, not against one.
+
+Bounds as for matrices of norm about 1, relative to the norm: 4 n 2^-53 for divide and conquer
+alone (on the CPU), 40 n 2^-53 for a Rayleigh-Ritz step over the whole space (on the GPU)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import workloads as W
+from test_eigh import U, cl, dc, tridiagonals  # noqa: F401  (fixtures)
+
+
+def ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def solve(dc, d, e):
+    n = len(d)
+    D, Q = np.empty(n), np.empty((n, n), order="F")
+    d, e = np.ascontiguousarray(d), np.ascontiguousarray(np.concatenate([e, [0.0]]))
+    dc.dc_solve(n, ptr(d), ptr(e), ptr(D), ptr(Q))
+    return D, Q
+
+
+def check(name, d, e, D, Q, s):
+    """Against T / s, s a power of two that brings T to norm about 1."""
+    n = len(d)
+    d, e, D = d / s, e / s, D / s
+    T = np.diag(d) + np.diag(e, 1) + np.diag(e, -1)
+    norm = np.abs(T).sum(axis=1).max()
+    assert np.all(np.diff(D) >= 0), name
+    assert np.abs(T @ Q - Q * D).max() <= 4 * n * U * norm, name
+    assert np.abs(Q.T @ Q - np.eye(n)).max() <= 4 * n * U, name
+    assert np.abs(D - np.linalg.eigvalsh(T)).max() <= 4 * n * U * norm, name
+
+
+@pytest.mark.parametrize("n", [2, 3, 17, 33, 100, 257])
+@pytest.mark.parametrize("k", [-300, -60, -40, -27, -10, 30, 300])
+def test_divide_and_conquer_is_relative_to_the_matrix(dc, n, k):
+    s = 2.0 ** k
+    for name, d, e in tridiagonals(n):
+        check(name, s * d, s * e, *solve(dc, s * d, s * e), s)
+
+
+torch = pytest.importorskip("torch")
+
+
+def scaled_rayleigh_ritz(cl, complex_, n, k, prec):
+    """Eigenvalues and vectors of 2^k A by one Rayleigh-Ritz step over the whole space, and A's."""
+    lam = np.sort(np.random.default_rng(n).uniform(-1.0, 1.0, n))
+    A = W.known_spectrum_matrix(lam, 7, complex_).numpy()
+    s = 2.0 ** k
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(np.asarray(x).T)).cuda().mT
+    V = dev(W.start_block(n, n, 8, complex_))
+    h = cl.Handle(0)
+    try:
+        cfg = cl.config_default(prec=prec, opt_degree=0, deg_init=1, max_iter=1, qr_force=4, tol=1e-10 * s)
+        rc, ev, _, _, _ = cl.chase_solve(h, dev(s * A), V, n, 0, (s * lam[0], s * (lam[-1] + 20.0), s * 1000.0), cfg)
+    finally:
+        h.close()
+    assert rc == 0
+    return A, lam, ev / s, V.cpu().numpy()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("n,k", [(33, -40), (129, -27), (300, -40), (129, 30)])
+def test_whole_space_rayleigh_ritz_at_scale(cl, complex_, n, k):
+    A, lam, ev, Y = scaled_rayleigh_ritz(cl, complex_, n, k, cl.CHASE_FP64)
+    tol = 40 * n * U
+    assert np.abs(ev - lam).max() <= tol
+    assert np.abs(Y.conj().T @ Y - np.eye(n)).max() <= tol
+    assert np.abs(A @ Y - Y * ev).max() <= tol
+
+
+def lanczos(cl, A, V, steps, ell):
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(np.asarray(x).T)).cuda().mT
+    h = cl.Handle(0)
+    try:
+        return np.array(cl.chase_lanczos_bounds(h, dev(A), dev(V), steps, ell))
+    finally:
+        h.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("k", [-60, -100, 100])
+def test_lanczos_bounds_scale_with_the_matrix(cl, complex_, k):
+    n, steps, ell = 600, 25, 60
+    lam = W.spectrum_uniform(n, -1.0, 1.0, 5)
+    A = W.known_spectrum_matrix(lam, 5, complex_).numpy()
+    V = W.start_block(n, 4, 6, complex_)
+    one, got = lanczos(cl, A, V, steps, ell), lanczos(cl, 2.0 ** k * A, V, steps, ell) / 2.0 ** k
+    # a power of two changes no rounding; only which couplings are left out may depend on it
+    assert np.abs(got - one).max() <= 100 * steps * U
+    assert got[2] >= lam[-1]
