@@ -353,12 +353,14 @@ struct DcWork {
   int n;
   double* D[2];
   double *ds, *zs, *dl, *w, *mu, *zh, *lam, *rc, *rs;
+  double* es;        // off-diagonal entries of 2^ex T
   int *perm, *idx, *defl, *pos, *gat, *org, *rp, *rq, *dest, *cnt;
   unsigned char *small, *close, *type;
   double *Q[2], *U;  // n x n
   int* bad;          // T was not finite
+  int* ex;           // D holds the eigenvalues of 2^ex T (see dc::scale_of)
 };
-constexpr int kDcDoubles = 11, kDcInts = 13, kDcBytes = 3;
+constexpr int kDcDoubles = 12, kDcInts = 13, kDcBytes = 3;
 
 __host__ __device__ inline size_t dc_align(size_t x) { return (x + 255) & ~(size_t)255; }
 inline size_t dc_bytes(int n) {
@@ -369,7 +371,7 @@ __host__ __device__ inline DcWork dc_vectors(char* base, int n) {
   DcWork W{};
   W.n = n;
   double* f = (double*)base;
-  double** fs[] = {&W.D[0], &W.D[1], &W.ds, &W.zs, &W.dl, &W.w, &W.mu, &W.zh, &W.lam, &W.rc, &W.rs};
+  double** fs[] = {&W.D[0], &W.D[1], &W.ds, &W.zs, &W.dl, &W.w, &W.mu, &W.zh, &W.lam, &W.rc, &W.rs, &W.es};
   for (int i = 0; i < kDcDoubles; ++i) *fs[i] = f + (size_t)i * n;
   int* q = (int*)(f + (size_t)kDcDoubles * n);
   int** is[] = {&W.perm, &W.idx, &W.defl, &W.pos, &W.gat, &W.org, &W.rp, &W.rq, &W.dest};
@@ -388,6 +390,7 @@ inline DcWork dc_carve(char* base, int n) {
   W.U = (double*)p;
   p += dc_align((size_t)8 * n * n);
   W.bad = (int*)p;
+  W.ex = W.bad + 1;
   return W;
 }
 // The arrays of problem b (every array a uniform stride of `stride` bytes further on).
@@ -395,7 +398,7 @@ __device__ inline DcWork dc_at(DcWork W, size_t off) {
   auto mv = [&](auto*& p) { p = (std::remove_reference_t<decltype(p)>)((char*)p + off); };
   mv(W.D[0]); mv(W.D[1]); mv(W.ds); mv(W.zs); mv(W.dl); mv(W.w); mv(W.mu); mv(W.zh); mv(W.lam); mv(W.rc); mv(W.rs);
   mv(W.perm); mv(W.idx); mv(W.defl); mv(W.pos); mv(W.gat); mv(W.org); mv(W.rp); mv(W.rq); mv(W.dest); mv(W.cnt);
-  mv(W.small); mv(W.close); mv(W.type); mv(W.Q[0]); mv(W.Q[1]); mv(W.U); mv(W.bad);
+  mv(W.small); mv(W.close); mv(W.type); mv(W.Q[0]); mv(W.Q[1]); mv(W.U); mv(W.bad); mv(W.es); mv(W.ex);
   return W;
 }
 
@@ -498,7 +501,8 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
                                                       size_t stride) {
   dep_wait(false);
   __shared__ double sQ[LEAF * LEAF], sQn[LEAF * LEAF], sU[LEAF * LEAF];
-  __shared__ double s_red[8];
+  __shared__ double s_red[8], s_e[LEAF];
+  __shared__ long long s_max[8];
   __shared__ __align__(16) char s_vec[LEAF * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)];
   const DcWork W = dc_at(W0, stride * blockIdx.y);
   const double* d = d0 + (size_t)blockIdx.y * ld_de;
@@ -507,19 +511,31 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const DcWork V = dc_vectors(s_vec, LEAF);
   for (int u = tid; u < LEAF * LEAF; u += 256) sQ[u] = (u % LEAF == u / LEAF) ? 1.0 : 0.0;
+  // 2^ex T: its largest entry, by every leaf for itself
+  auto bits = [](double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; };
+  long long mx = 0;
+  for (int i = tid; i < n; i += 256) mx = max(mx, max(bits(d[i]), i + 1 < n ? bits(e[i]) : 0));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) s_max[warp] = mx;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) mx = max(mx, s_max[w]);
+  const int ex = dc::scale_of(__longlong_as_double(mx));
+  if (blockIdx.x == 0 && tid == 0) *W.ex = ex;
   for (int i = tid; i < m; i += 256) {
     const int r = s + i;
     // every off-diagonal is torn at some level
-    const double lo = r > 0 ? fabs(e[r - 1]) : 0.0, up = r + 1 < n ? fabs(e[r]) : 0.0;
-    V.D[0][i] = d[r] - lo - up;
-    if (!isfinite(d[r]) || !isfinite(up)) *W.bad = 1;
+    const double lo = r > 0 ? fabs(ldexp(e[r - 1], ex)) : 0.0, er = r + 1 < n ? ldexp(e[r], ex) : 0.0;
+    V.D[0][i] = ldexp(d[r], ex) - lo - fabs(er);
+    s_e[i] = er;
+    W.es[r] = er;
+    if (!isfinite(d[r]) || !isfinite(er)) *W.bad = 1;
   }
   __syncthreads();
   if (tid < 16) {  // single rows: at most one each side
     const long long i0 = ((long long)blockIdx.x << 5) + 2 * tid;
     const int a = dc_bound(n, i0, depth + 5) - s, b = dc_bound(n, i0 + 1, depth + 5) - s,
               c = dc_bound(n, i0 + 2, depth + 5) - s;
-    if (b > a && c > b) dc_pair(e[s + b - 1], V.D[0] + a, sQ + a + a * LEAF, LEAF);
+    if (b > a && c > b) dc_pair(s_e[b - 1], V.D[0] + a, sQ + a + a * LEAF, LEAF);
   }
   __syncthreads();
   for (int h = 3; h >= 0; --h) {
@@ -528,7 +544,7 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
     const int a = dc_bound(n, i0, depth + h + 1) - s, b = dc_bound(n, i0 + 1, depth + h + 1) - s,
               c = dc_bound(n, i0 + 2, depth + h + 1) - s;
     if (b > a && c > b) {  // (an empty half: nothing to merge)
-      const dc::Merge M = dc_merge(V, 0, a, b, c, e[s + b - 1]);
+      const dc::Merge M = dc_merge(V, 0, a, b, c, s_e[b - 1]);
       const int at = a + a * LEAF;
       if (h == 3)
         dc_merge_local(WarpGroup{lane, 32}, 0, 1, 8, M, V.D[0] + a, V.D[1] + a, sQ + at, sQn + at, sU + at, LEAF);
@@ -544,30 +560,28 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int n, int depth, const do
 }
 
 // Merge blockIdx.(y or z) of the level with 2^depth blocks below it; cur: input buffer.
-__device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, int q, const double* e, int* s) {
+__device__ inline dc::Merge dc_level_merge(const DcWork& W, int cur, int depth, int q, int* s) {
   const int a = dc_bound(W.n, 2 * q, depth), b = dc_bound(W.n, 2 * q + 1, depth), c = dc_bound(W.n, 2 * q + 2, depth);
   *s = a;
-  return dc_merge(W, cur, a, b, c, e[b - 1]);
+  return dc_merge(W, cur, a, b, c, W.es[b - 1]);
 }
 
-__global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                       const double* e0, int ld_de) {
+__global__ void __launch_bounds__(512) dc_setup_kernel(DcWork W0, size_t stride, int cur, int depth) {
   dep_wait(false);
   __shared__ double red[16];
   const DcWork W = dc_at(W0, stride * blockIdx.y);
   int s;
-  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.x, e0 + (size_t)blockIdx.y * ld_de, &s);
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.x, &s);
   const double* Qb = W.Q[cur] + s + (size_t)s * W.n;
   dc::setup(CtaGroup{(int)threadIdx.x, 512, red}, M, Qb + M.n1 - 1, Qb + M.n1 + (size_t)M.n1 * W.n, W.n);
 }
 
 // phase 0: roots, and the rotations of Q's rows; 1: corrected z; 2: U and the new order.
-__global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                       const double* e0, int ld_de, int phase) {
+__global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride, int cur, int depth, int phase) {
   dep_wait(false);
   const DcWork W = dc_at(W0, stride * blockIdx.z);
   int s;
-  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, e0 + (size_t)blockIdx.z * ld_de, &s);
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.y, &s);
   const Lanes L(32);
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5), nw = gridDim.x * 4;
   const int K = M.cnt[0];
@@ -585,12 +599,11 @@ __global__ void __launch_bounds__(128) dc_phase_kernel(DcWork W0, size_t stride,
 }
 
 // Q_new[:, dest] = Q[:, gathered] U (64 x 32 tiles, FP64), deflated columns copied.
-__global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth,
-                                                      const double* e0, int ld_de, int parts) {
+__global__ void __launch_bounds__(256) dc_gemm_kernel(DcWork W0, size_t stride, int cur, int depth, int parts) {
   dep_wait(false);
   const DcWork W = dc_at(W0, stride * (blockIdx.z / parts));
   int s;
-  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.z % parts, e0 + (size_t)(blockIdx.z / parts) * ld_de, &s);
+  const dc::Merge M = dc_level_merge(W, cur, depth, blockIdx.z % parts, &s);
   constexpr int BK = 16;
   __shared__ double As[BK][64], Bs[BK][33];
   const int m0 = blockIdx.y * 64, j0 = blockIdx.x * 32, m = M.m, n1 = M.n1, K = M.cnt[0], ld = W.n;
@@ -664,11 +677,11 @@ int stedc(cudaStream_t st, int n, int batch, const double* d, const double* e, i
   int nl = 1, c = 0;
   for (int h = depth; h > 0; --h) {
     const int parts = 1 << (h - 1), m = ceil_div(n, parts);  // rows of a merge, at most
-    launch_dep(st, dim3(parts, batch), 512, 0, dc_setup_kernel, W, stride, c, h, e, ld_de);
+    launch_dep(st, dim3(parts, batch), 512, 0, dc_setup_kernel, W, stride, c, h);
     for (int phase = 0; phase < 3; ++phase)
-      launch_dep(st, dim3(ceil_div(m, 4), parts, batch), 128, 0, dc_phase_kernel, W, stride, c, h, e, ld_de, phase);
+      launch_dep(st, dim3(ceil_div(m, 4), parts, batch), 128, 0, dc_phase_kernel, W, stride, c, h, phase);
     launch_dep(st, dim3(ceil_div(m, 32), ceil_div(m, 64), parts * batch), 256, 0, dc_gemm_kernel, W, stride, c, h,
-               e, ld_de, parts);
+               parts);
     nl += 5;
     c ^= 1;
   }
@@ -737,8 +750,8 @@ __device__ __forceinline__ z64 shfl_t(z64 v, int src) { return z64{shfl_t(v.x, s
 template <class T>
 __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ldh,
                                                        const T* Tb, const double* Z,
-                                                       const double* D, const int* bad, T* Wm, int ldw,
-                                                       double* dw) {
+                                                       const double* D, const int* bad, const int* ex, T* Wm,
+                                                       int ldw, double* dw) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -746,7 +759,7 @@ __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ld
   const bool nan_out = *bad != 0;
   T* z = (T*)bt_smem + (size_t)warp * l;
   for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(nan_out ? nan("") : Z[(size_t)i + (size_t)c * l]);
-  if (lane == 0) dw[c] = nan_out ? nan("") : D[c];
+  if (lane == 0) dw[c] = nan_out ? nan("") : ldexp(D[c], -*ex);
   __syncwarp();
   const int nb = nan_out ? 0 : (l - 1 + BTK - 1) / BTK;
   for (int b = nb - 1; b >= 0; --b) {
@@ -797,7 +810,7 @@ __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ld
 // (in_smem) or in place; dw = D (NaN if T was not finite).
 template <class T>
 __global__ void backtransform_kernel(int l, const T* H, int ldh, const T* tau,
-                                     const double* Z, const double* D, const int* bad,
+                                     const double* Z, const double* D, const int* bad, const int* ex,
                                      T* Wm, int ldw, double* dw, int in_smem) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
@@ -811,7 +824,7 @@ __global__ void backtransform_kernel(int l, const T* H, int ldh, const T* tau,
     return;
   }
   for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(Z[(size_t)i + (size_t)c * l]);
-  if (lane == 0) dw[c] = D[c];
+  if (lane == 0) dw[c] = ldexp(D[c], -*ex);
   __syncwarp();
   for (int j = l - 2; j >= 0; --j) {
     const T t = tau[j];
@@ -837,7 +850,7 @@ __global__ void dc_extract_kernel(DcWork W0, size_t stride, int cur, double* the
   const DcWork W = dc_at(W0, stride * blockIdx.x);
   for (int i = threadIdx.x; i < W.n; i += blockDim.x) {
     const double q = W.Q[cur][(size_t)i * W.n];
-    theta[(size_t)blockIdx.x * W.n + i] = *W.bad ? nan("") : W.D[cur][i];
+    theta[(size_t)blockIdx.x * W.n + i] = *W.bad ? nan("") : ldexp(W.D[cur][i], -*W.ex);
     weight[(size_t)blockIdx.x * W.n + i] = *W.bad ? nan("") : q * q;
   }
 }
@@ -931,12 +944,12 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
     launch_dep(st, ceil_div(l - 1, BTK), 256, 0, bt_factor_kernel<T>, l, H, ldh, tau, Tb);
     CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)bt_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)kSmemMax - 1024));
-    launch_dep(st, ceil_div(l, wpc), 32 * wpc, smem, bt_block_kernel<T>, l, H, ldh, Tb, D.Q[cur], D.D[cur], D.bad, W,
-               ldw, dw);
+    launch_dep(st, ceil_div(l, wpc), 32 * wpc, smem, bt_block_kernel<T>, l, H, ldh, Tb, D.Q[cur], D.D[cur], D.bad,
+               D.ex, W, ldw, dw);
     if (launches) ++*launches;
   } else {
     launch_dep(st, ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, backtransform_kernel<T>, l, H, ldh, tau, D.Q[cur],
-               D.D[cur], D.bad, W, ldw, dw, in_smem);
+               D.D[cur], D.bad, D.ex, W, ldw, dw, in_smem);
   }
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());

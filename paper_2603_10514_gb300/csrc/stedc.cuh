@@ -24,6 +24,15 @@ namespace dc {
 
 constexpr double kEps = 1.1102230246251565e-16;  // 2^-53
 
+// k with 2^k x in [0.5, 1) (0 for 0, infinity and NaN).  The steps below square and invert what they
+// are given, so a tridiagonal is first multiplied by 2^k of its largest entry, which rounds nothing.
+DC_FN int scale_of(double x) {
+  if (!(x > 0.0) || x - x != 0.0) return 0;
+  int e;
+  frexp(x, &e);
+  return -e;
+}
+
 // One merge: the eigensystems of two adjacent tridiagonal blocks (n1 and m - n1 rows) and the
 // coupling rho between them.  All arrays hold m entries.
 struct Merge {

@@ -4,12 +4,15 @@ matrix it is given, not against one.
 Bounds as for matrices of norm about 1, relative to the norm: 4 n 2^-53 for divide and conquer
 alone (on the CPU), 40 n 2^-53 for a Rayleigh-Ritz step over the whole space (on the GPU)."""
 import ctypes
+import os
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
 
 import workloads as W
-from test_eigh import U, cl, dc, tridiagonals  # noqa: F401  (fixtures)
+from test_eigh import CSRC, DRIVER, U, cl, dc, tridiagonals  # noqa: F401  (fixtures)
 
 
 def ptr(a):
@@ -42,6 +45,44 @@ def test_divide_and_conquer_is_relative_to_the_matrix(dc, n, k):
     s = 2.0 ** k
     for name, d, e in tridiagonals(n):
         check(name, s * d, s * e, *solve(dc, s * d, s * e), s)
+
+
+RANGE_DRIVER = DRIVER + r"""
+extern "C" void dc_solve_any(int n, const double* d, const double* e, double* D, double* Q) {
+  std::vector<double> a(d, d + n), b(e, e + n);
+  double x = 0;
+  for (int i = 0; i < n; ++i) x = std::max(x, std::max(std::fabs(a[i]), std::fabs(b[i])));
+  const int k = scale_of(x);
+  for (int i = 0; i < n; ++i) { a[i] = std::ldexp(a[i], k); b[i] = std::ldexp(b[i], k); }
+  dc_solve(n, a.data(), b.data(), D, Q);
+  for (int i = 0; i < n; ++i) D[i] = std::ldexp(D[i], -k);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def dc_range(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("g++ not available")
+    d = tmp_path_factory.mktemp("dcrange")
+    (d / "dc.cpp").write_text(RANGE_DRIVER)
+    so = str(d / "dc.so")
+    subprocess.run(["g++", "-O1", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, str(d / "dc.cpp"), "-o", so],
+                   check=True)
+    return ctypes.CDLL(so)
+
+
+@pytest.mark.parametrize("n", [1, 2, 17, 33, 100])
+@pytest.mark.parametrize("k", [-1000, -600, 0, 600, 1000])
+def test_divide_and_conquer_over_the_whole_range(dc_range, n, k):
+    """Scaled to its largest entry first, as the kernels do it: squares and reciprocals of the
+    entries stay in range."""
+    s = 2.0 ** k
+    for name, d, e in tridiagonals(n):
+        D, Q = np.empty(n), np.empty((n, n), order="F")
+        a, b = np.ascontiguousarray(s * d), np.ascontiguousarray(np.concatenate([s * e, [0.0]]))
+        dc_range.dc_solve_any(n, ptr(a), ptr(b), ptr(D), ptr(Q))
+        check(name, s * d, s * e, D, Q, s)
 
 
 torch = pytest.importorskip("torch")
@@ -86,7 +127,7 @@ def lanczos(cl, A, V, steps, ell):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("complex_", [False, True])
-@pytest.mark.parametrize("k", [-60, -100, 100])
+@pytest.mark.parametrize("k", [-60, -100, 100, -900, 900])
 def test_lanczos_bounds_scale_with_the_matrix(cl, complex_, k):
     n, steps, ell = 600, 25, 60
     lam = W.spectrum_uniform(n, -1.0, 1.0, 5)
