@@ -71,18 +71,20 @@ __device__ __forceinline__ double im_of(z64 a) { return a.y; }
 //   more on every SM, but no second wait on its owner -- and while one warp takes the reflector's
 //   square root and divisions (~35 dependent FP64 instructions), the others apply
 //   H -= v w^H + w v^H, w = x + alpha v, to the own columns.
+// All of it on 2^ex H, with its largest entry in [0.5, 1): the squares of the norms stay in range.
 // xb, cb: 2 l elements, part: 2 G doubles; scr: 3 l elements per CTA where they do not fit
-// shared memory (else null).
+// shared memory (else null); ex: one int, written.
 template <class T>
 __global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int in_smem, T* tau, double* d,
-                                                      double* e, T* xb, T* cb, double* part, T* scr, GridBar* gb,
-                                                      DevStatus* dst) {
+                                                      double* e, T* xb, T* cb, double* part, T* scr, int* ex,
+                                                      GridBar* gb, DevStatus* dst) {
   extern __shared__ __align__(16) unsigned char tri_smem[];
   const int G = gridDim.x, me = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = TNT / 32;
   __shared__ double sh[NW];
   __shared__ T sh_tau, sh_scale;
   __shared__ double sh_alpha;
+  __shared__ long long sh_max[NW];
   const int own = (l + G - 1) / G;                     // columns me, me + G, ...
   const int nc = me < l ? (l - 1 - me) / G + 1 : 0;
   T* sp = (T*)tri_smem;                                // 4 partial sums per own column
@@ -91,9 +93,23 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int 
   T *vs = vec, *xs = vec + l, *us = vec + 2 * (size_t)l;
   T* S = scr ? sq + 2 * own : vec + 3 * (size_t)l;
   auto column = [&](int k) -> T* { return in_smem ? S + (size_t)k * l : H + (size_t)(me + k * G) * ldh; };
-  if (in_smem)
-    for (int k = 0; k < nc; ++k)
-      for (int i = tid; i < l; i += TNT) S[(size_t)k * l + i] = H[(size_t)i + (size_t)(me + k * G) * ldh];
+  long long mx = 0;  // bits of the largest |re|, |im| of the own columns
+  auto bits = [](double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; };
+  for (int k = 0; k < nc; ++k)
+    for (int i = tid; i < l; i += TNT) {
+      const T h = H[(size_t)i + (size_t)(me + k * G) * ldh];
+      if (in_smem) S[(size_t)k * l + i] = h;
+      mx = max(mx, max(bits(Sc<T>::re(h)), bits(im_of(h))));
+    }
+  auto block_maxbits = [&](long long v) {
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if (lane == 0) sh_max[warp] = v;
+    __syncthreads();
+    for (int w = 0; w < NW; ++w) v = max(v, sh_max[w]);
+    return v;
+  };
+  mx = block_maxbits(mx);
 
   // Reflector j from u (rows j .. of the updated column j): its scalars, by one thread.
   auto scalars = [&](int j, const T* u) {
@@ -104,7 +120,7 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int 
     T t = Sc<T>::zero(), sc = Sc<T>::zero();
     double beta = ar;
     const double nn = ar * ar + ai * ai + x2;
-    if ((x2 != 0.0 || ai != 0.0) && !(nn < 1e-300)) {  // (below: nothing is left, and 1 / nn overflows)
+    if ((x2 != 0.0 || ai != 0.0) && !(nn < 1e-300)) {  // (below: nothing is left of a matrix of norm 1, and 1 / nn overflows)
       const double rn = rsqrt(nn);
       beta = -copysign(nn * rn, ar);
       const double ib = -copysign(rn, ar), dr = ar - beta, id = 1.0 / (dr * dr + ai * ai);
@@ -141,10 +157,31 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int 
 
   // reflector 0, by every CTA from the matrix (read before any column is overwritten: its owner
   // writes it after the first barrier's worth of work is published, see below)
+  for (int i = tid; i < l; i += TNT) us[i] = H[i];
+  unsigned bars = 0;
+  int par = 0;
+  if (G > 1) {
+    if (tid == 0) ((long long*)part)[me] = mx;
+    if (!grid_barrier(gb, G, bars)) {  // column 0 has been read everywhere
+      if (tid == 0) atomicOr(&dst->timeout, 16);
+      return;
+    }
+    for (int b = tid; b < G; b += TNT) mx = max(mx, __ldcg((const long long*)part + b));
+    mx = block_maxbits(mx);
+    par = 1;  // the first step writes the other half of `part`: this one may still be read
+  }
+  const int sx = dc::scale_of(__longlong_as_double(mx));
+  if (me == 0 && tid == 0) *ex = sx;
+  // (two factors: 2^sx alone may be out of range)
+  const double f0 = ldexp(1.0, sx / 2), f1 = ldexp(1.0, sx - sx / 2);
+  auto scaled = [&](T h) { return Sc<T>::scale(Sc<T>::scale(h, f0), f1); };
+  if (sx != 0)
+    for (int k = 0; k < nc; ++k)
+      for (int i = tid; i < l; i += TNT) column(k)[i] = scaled(column(k)[i]);
   {
     double s = 0.0;
     for (int i = tid; i < l; i += TNT) {
-      const T h = H[i];
+      const T h = scaled(us[i]);
       us[i] = h;
       if (i >= 2) s += Sc<T>::abs2(h);
     }
@@ -153,12 +190,6 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(int l, T* H, int ldh, int 
   __syncthreads();
   if (l == 1) {
     if (me == 0 && tid == 0) d[0] = Sc<T>::re(us[0]);
-    return;
-  }
-  unsigned bars = 0;
-  int par = 0;
-  if (G > 1 && !grid_barrier(gb, G, bars)) {  // column 0 has been read everywhere
-    if (tid == 0) atomicOr(&dst->timeout, 16);
     return;
   }
   if (tid == 0) scalars(0, us);
@@ -750,8 +781,8 @@ __device__ __forceinline__ z64 shfl_t(z64 v, int src) { return z64{shfl_t(v.x, s
 template <class T>
 __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ldh,
                                                        const T* Tb, const double* Z,
-                                                       const double* D, const int* bad, const int* ex, T* Wm,
-                                                       int ldw, double* dw) {
+                                                       const double* D, const int* bad, const int* ex, const int* ex0,
+                                                       T* Wm, int ldw, double* dw) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -759,7 +790,7 @@ __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ld
   const bool nan_out = *bad != 0;
   T* z = (T*)bt_smem + (size_t)warp * l;
   for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(nan_out ? nan("") : Z[(size_t)i + (size_t)c * l]);
-  if (lane == 0) dw[c] = nan_out ? nan("") : ldexp(D[c], -*ex);
+  if (lane == 0) dw[c] = nan_out ? nan("") : ldexp(D[c], -(*ex + *ex0));
   __syncwarp();
   const int nb = nan_out ? 0 : (l - 1 + BTK - 1) / BTK;
   for (int b = nb - 1; b >= 0; --b) {
@@ -811,7 +842,7 @@ __global__ void __launch_bounds__(128) bt_block_kernel(int l, const T* H, int ld
 template <class T>
 __global__ void backtransform_kernel(int l, const T* H, int ldh, const T* tau,
                                      const double* Z, const double* D, const int* bad, const int* ex,
-                                     T* Wm, int ldw, double* dw, int in_smem) {
+                                     const int* ex0, T* Wm, int ldw, double* dw, int in_smem) {
   dep_wait(false);
   extern __shared__ __align__(16) unsigned char bt_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -824,7 +855,7 @@ __global__ void backtransform_kernel(int l, const T* H, int ldh, const T* tau,
     return;
   }
   for (int i = lane; i < l; i += 32) z[i] = Sc<T>::from_re(Z[(size_t)i + (size_t)c * l]);
-  if (lane == 0) dw[c] = ldexp(D[c], -*ex);
+  if (lane == 0) dw[c] = ldexp(D[c], -(*ex + *ex0));
   __syncwarp();
   for (int j = l - 2; j >= 0; --j) {
     const T t = tau[j];
@@ -860,7 +891,7 @@ int tridiag_pass(int m, int batch) {
 }
 
 struct EighLayout {
-  size_t tau, d, e, xb, cb, part, scr, tb, dc, total;
+  size_t tau, d, e, xb, cb, part, scr, tb, ex, dc, total;
 };
 // Shared memory of the reduction: partial sums and factors of the own columns, three vectors.
 size_t tri_fixed_smem(int l, int own, size_t elem) { return elem * (6 * (size_t)own + 3 * (size_t)l); }
@@ -877,6 +908,7 @@ EighLayout eigh_layout(int l, size_t elem) {
   L.part = take(2 * 8 * kNumSMs);
   L.scr = take(tri_vec_smem(l, elem) ? 0 : elem * 3 * (size_t)l * kNumSMs);
   L.tb = take(sizeof(GridBar));
+  L.ex = take(sizeof(int));
   L.dc = take(dc_bytes(l));
   L.total = off;
   return L;
@@ -888,6 +920,7 @@ int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout&
   T *tau = (T*)(base + L.tau), *xb = (T*)(base + L.xb), *cb = (T*)(base + L.cb);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e), *part = (double*)(base + L.part);
   GridBar* gb = (GridBar*)(base + L.tb);
+  int* ex = (int*)(base + L.ex);
   // CTAs: one for every 1000 elements (complex: x 4), one alone below 3000, where a column's
   // FP64 work costs less than the grid barrier (measured: l = 30 real 0.142 ms on one CTA, 0.171
   // on four; l = 60 real 0.417 and 0.343; l = 230 complex 1.95 on 38, 1.73 on 76)
@@ -911,7 +944,8 @@ int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout&
                                       (int)kSmemMax - 1024));
   CHASE_CUDA_TRY(cudaMemsetAsync(gb, 0, sizeof(GridBar), st));
   void* args[] = {(void*)&l,  (void*)&H,  (void*)&ldh,  (void*)&in_smem, (void*)&tau, (void*)&d,  (void*)&e,
-                  (void*)&xb, (void*)&cb, (void*)&part, (void*)&scr,     (void*)&gb,  (void*)&dst};
+                  (void*)&xb, (void*)&cb, (void*)&part, (void*)&scr,     (void*)&ex,  (void*)&gb,
+                  (void*)&dst};
   CHASE_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)tridiag_kernel<T>, dim3(G), dim3(TNT), args, smem, st));
   if (launches) ++*launches;
   return 0;
@@ -930,6 +964,7 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   char* base = (char*)work;
   T* tau = (T*)(base + L.tau);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e);
+  const int* ex0 = (const int*)(base + L.ex);
   TRY_EIG(tridiag<T>(st, l, H, ldh, base, L, dst, ctas, launches));
   const DcWork D = dc_carve(base + L.dc, l);
   int cur = 0;
@@ -945,11 +980,11 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
     CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)bt_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)kSmemMax - 1024));
     launch_dep(st, ceil_div(l, wpc), 32 * wpc, smem, bt_block_kernel<T>, l, H, ldh, Tb, D.Q[cur], D.D[cur], D.bad,
-               D.ex, W, ldw, dw);
+               D.ex, ex0, W, ldw, dw);
     if (launches) ++*launches;
   } else {
     launch_dep(st, ceil_div(l, wpc), 32 * wpc, in_smem ? smem : 0, backtransform_kernel<T>, l, H, ldh, tau, D.Q[cur],
-               D.D[cur], D.bad, D.ex, W, ldw, dw, in_smem);
+               D.D[cur], D.bad, D.ex, ex0, W, ldw, dw, in_smem);
   }
   if (launches) ++*launches;
   CHASE_CUDA_TRY(cudaGetLastError());

@@ -116,6 +116,18 @@ def test_whole_space_rayleigh_ritz_at_scale(cl, complex_, n, k):
     assert np.abs(A @ Y - Y * ev).max() <= tol
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("n,k", [(1, -600), (2, 400), (33, -600), (129, -600), (129, 400), (300, -520), (601, -600)])
+def test_whole_space_rayleigh_ritz_over_the_range(cl, complex_, n, k):
+    """Squares of the entries leave the range of FP64 (n = 33 on one thread block, 601 on all)."""
+    A, lam, ev, Y = scaled_rayleigh_ritz(cl, complex_, n, k, cl.CHASE_FP64_EMU)
+    tol = 40 * max(n, 4) * U
+    assert np.abs(ev - lam).max() <= tol
+    assert np.abs(Y.conj().T @ Y - np.eye(n)).max() <= tol
+    assert np.abs(A @ Y - Y * ev).max() <= tol
+
+
 def lanczos(cl, A, V, steps, ell):
     dev = lambda x: torch.from_numpy(np.ascontiguousarray(np.asarray(x).T)).cuda().mT
     h = cl.Handle(0)
