@@ -32,6 +32,7 @@ constexpr int CB = 32;              // rows of a block
 constexpr int CT = 8;               // trailing tiles are 8 x 8
 constexpr int CNT = 256, CW = CNT / 32;
 constexpr int CLD = CB + 1;
+constexpr int kSmemMax = 227 * 1024;
 
 struct CholBar {
   GridBar bar;
@@ -223,7 +224,17 @@ __global__ void __launch_bounds__(CNT) chol_kernel(int n, T* G, int ldg, double 
   }
 }
 
-// Columns blockIdx.x and n - 1 - blockIdx.x of R^{-1} (n > CB).
+// Sum over four lanes, in their order.
+__device__ __forceinline__ double quad_sum(double a, int lane) {
+  double s = __shfl_sync(0xffffffffu, a, lane & ~3);
+#pragma unroll
+  for (int o = 1; o < 4; ++o) s += __shfl_sync(0xffffffffu, a, (lane & ~3) + o);
+  return s;
+}
+__device__ __forceinline__ z64 quad_sum(z64 a, int lane) { return z64{quad_sum(a.x, lane), quad_sum(a.y, lane)}; }
+
+// Columns blockIdx.x and n - 1 - blockIdx.x of R^{-1} (n > CB).  The column is all the shared memory
+// it takes: 227 KB hold 14528 complex rows.
 template <class T>
 __global__ void __launch_bounds__(128) trinv_kernel(int n, const T* R, int ldr,
                                                     const T* Mb, T* Rinv, int ldri,
@@ -231,9 +242,8 @@ __global__ void __launch_bounds__(128) trinv_kernel(int n, const T* R, int ldr,
   dep_wait();
   extern __shared__ __align__(16) unsigned char inv_smem[];
   T* x = (T*)inv_smem;
-  __shared__ T part[4][CB];
   if (dst->chol_info) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   for (int half = 0; half < 2; ++half) {
     const int j = half ? n - 1 - (int)blockIdx.x : (int)blockIdx.x;
     if (half && j <= (int)blockIdx.x) break;
@@ -253,17 +263,15 @@ __global__ void __launch_bounds__(128) trinv_kernel(int n, const T* R, int ldr,
         x[i] = a;
       }
       __syncthreads();
-      // block k - 1: x <- R_kk^{-1} x = M^H x, the sum over rows split over the four warps
+      // block k - 1: x <- R_kk^{-1} x = M^H x, four lanes to a row, each a quarter of its sum
       const T* M = Mb + (size_t)(k - 1) * CB * CB;
+      const int row = tid >> 2, part = tid & 3;
       T a = Sc<T>::zero();
 #pragma unroll
-      for (int p = 8 * warp; p < 8 * warp + 8; ++p) Sc<T>::fmac(a, M[p + lane * CB], x[off - CB + p]);
-      part[warp][lane] = a;
+      for (int p = 8 * part; p < 8 * part + 8; ++p) Sc<T>::fmac(a, M[p + row * CB], x[off - CB + p]);
+      a = quad_sum(a, lane);
       __syncthreads();
-      if (warp == 0) {
-        for (int w = 1; w < 4; ++w) a = Sc<T>::add(a, part[w][lane]);
-        x[off - CB + lane] = a;
-      }
+      if (part == 0) x[off - CB + row] = a;
       __syncthreads();
     }
     for (int i = tid; i < n; i += 128) Rinv[(size_t)i + (size_t)j * ldri] = i <= j ? x[i] : Sc<T>::zero();
@@ -294,8 +302,8 @@ int chol_inverse(cudaStream_t st, int n, T* G, int ldg, double shift_factor, T* 
   if (launches) ++*launches;
   if (n > CB) {
     const size_t xs = sizeof(T) * (size_t)ceil_div(n, CB) * CB;
-    if (xs > 48 * 1024)
-      CHASE_CUDA_TRY(cudaFuncSetAttribute(trinv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs));
+    // (always the same value: another thread may be about to launch with a longer column)
+    CHASE_CUDA_TRY(cudaFuncSetAttribute(trinv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
     launch_dep(st, ceil_div(n, 2), 128, xs, trinv_kernel<T>, n, G, ldg, Mb, Rinv, ldri, dst);
     if (launches) ++*launches;
   }
