@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <numeric>
 #include <vector>
 
@@ -114,10 +115,10 @@ __device__ __forceinline__ int4 lz_cut(z64 x, int e) {
 template <class T> struct LzInt { using type = int2; };
 template <> struct LzInt<z64> { using type = int4; };
 
-// Exponents of the columns of A (n x n), one warp each.
+// Exponents of the columns of A (n x n), one warp each, and the largest of them.
 template <class T>
 __global__ void __launch_bounds__(256) lz_colexp_kernel(int n, const T* A, int lda,
-                                                        int* ea) {
+                                                        int* ea, int* emax) {
   dep_wait();
   const int lane = threadIdx.x & 31, c = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (c >= n) return;
@@ -126,8 +127,15 @@ __global__ void __launch_bounds__(256) lz_colexp_kernel(int n, const T* A, int l
 #pragma unroll 8
   for (int i = lane; i < n; i += 32) m = max(m, lz_abs(col[i]));
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) ea[c] = lz_exp(m);
+  if (lane == 0) {
+    const int e = lz_exp(m);
+    ea[c] = e;
+    if (m > 0 && e < kLzBad) atomicMax(emax, e);
+  }
 }
+// The runs advance with 2^-em A, whose entries are below 1: at the ends of FP64's range its residuals
+// and their products would be subnormal or overflow.  emax starts far below any exponent.
+__host__ __device__ inline int lz_scale(int emax) { return emax < -kLzBad ? 0 : emax; }
 
 // Sums of products of high halves, low halves, and sums of halves.
 struct LzSum {
@@ -142,7 +150,7 @@ struct LzSum {
   }
 };
 
-// W[:, r] = A q_r for R runs: A is Hermitian, so entry c of the product is the dot product of
+// W[:, r] = 2^-em A q_r for R runs: A is Hermitian, so entry c of the product is the dot product of
 // A's column c with q_r -- one warp for KC columns, A read once for all runs in full lines; Qi, eq:
 // the q_r cut up.  A term of x is at most 2^56 (complex: two): the sums of a lane are taken out
 // after 120 (60) terms.  Bound by the wide multiply-adds.  Real n = 8000, 4 runs: FP64 465 us a
@@ -151,7 +159,7 @@ template <class T, int R, int KC>
 __global__ void __launch_bounds__(256) lz_product_kernel(int n, const T* A, int lda,
                                                          const int* ea,
                                                          const typename LzInt<T>::type* Qi,
-                                                         const int* eq, T* W) {
+                                                         const int* eq, const int* emax, T* W) {
   dep_wait();
   constexpr int NP = Sc<T>::cplx ? 2 : 1, NV = KC * R * NP;
   const int lane = threadIdx.x & 31, c0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * KC;
@@ -164,6 +172,7 @@ __global__ void __launch_bounds__(256) lz_product_kernel(int n, const T* A, int 
     col[k] = A + (size_t)c * lda;
     e[k] = ea[c];
   }
+  const int em = lz_scale(*emax);
   double sum[NV];
 #pragma unroll
   for (int u = 0; u < NV; ++u) sum[u] = 0.0;
@@ -210,28 +219,29 @@ __global__ void __launch_bounds__(256) lz_product_kernel(int n, const T* A, int 
       const int k = u / (R * NP), r = u / NP % R, x = e[k] + eq[r];
       if (c0 + k < n)
         ((double*)W)[((size_t)r * n + c0 + k) * NP + u % NP] =
-            x >= kLzBad / 2 ? nan("") : scalbn(sum[u], x - 2 * kLzBits);
+            x >= kLzBad / 2 ? nan("") : scalbn(sum[u], x - em - 2 * kLzBits);
     }
 }
 
 template <class T, int R>
 void lz_launch(cudaStream_t st, int n, const T* A, int lda, const int* ea, const typename LzInt<T>::type* Qi,
-               const int* eq, T* W) {
+               const int* eq, const int* emax, T* W) {
   constexpr int KC = Sc<T>::cplx ? 1 : 2;
-  launch_dep(st, ceil_div(n, 8 * KC), 256, 0, lz_product_kernel<T, R, KC>, n, A, lda, ea, Qi, eq, W);
+  launch_dep(st, ceil_div(n, 8 * KC), 256, 0, lz_product_kernel<T, R, KC>, n, A, lda, ea, Qi, eq, emax, W);
 }
 
 template <class T>
 int lz_product(cudaStream_t st, int n, int nruns, const T* A, int lda, const int* ea,
-               const typename LzInt<T>::type* Qi, const int* eq, T* W, int* nl) {
+               const typename LzInt<T>::type* Qi, const int* eq, const int* emax, T* W,
+               int* nl) {
   for (int r = 0; r < nruns; r += 4) {
     const auto* q = Qi + (size_t)r * n;
     T* w = W + (size_t)r * n;
     switch (std::min(4, nruns - r)) {
-      case 1: lz_launch<T, 1>(st, n, A, lda, ea, q, eq + r, w); break;
-      case 2: lz_launch<T, 2>(st, n, A, lda, ea, q, eq + r, w); break;
-      case 3: lz_launch<T, 3>(st, n, A, lda, ea, q, eq + r, w); break;
-      default: lz_launch<T, 4>(st, n, A, lda, ea, q, eq + r, w); break;
+      case 1: lz_launch<T, 1>(st, n, A, lda, ea, q, eq + r, emax, w); break;
+      case 2: lz_launch<T, 2>(st, n, A, lda, ea, q, eq + r, emax, w); break;
+      case 3: lz_launch<T, 3>(st, n, A, lda, ea, q, eq + r, emax, w); break;
+      default: lz_launch<T, 4>(st, n, A, lda, ea, q, eq + r, emax, w); break;
     }
     ++*nl;
   }
@@ -302,14 +312,14 @@ __global__ void __launch_bounds__(512) lz_normalize_kernel(int n, const T* W, T*
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) s += Sc<T>::abs2(Sc<T>::scale(w[i], scale));
   s = block_sum_t<double>(s, red);
-  const double b = scalbn(sqrt(s), ew);
-  if (threadIdx.x == 0) beta[r * m + j] = b;
+  const double b = sqrt(s);  // of w 2^-ew: 1 / |w| may be out of range
+  if (threadIdx.x == 0) beta[r * m + j] = scalbn(b, ew);
   const double inv = (b > 0.0) ? 1.0 / b : 0.0;
-  // the largest |q| is the largest |w| times inv (rounding keeps order)
-  const int e = lz_exp(lz_abs(__longlong_as_double(mx) * inv));
+  // the largest |q| is the largest |w| 2^-ew times inv (rounding keeps order)
+  const int e = lz_exp(lz_abs(__longlong_as_double(mx) * scale * inv));
   if (threadIdx.x == 0) eq[r] = e;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const T q = Sc<T>::scale(w[i], inv);
+    const T q = Sc<T>::scale(Sc<T>::scale(w[i], scale), inv);
     qn[(size_t)r * n + i] = q;
     qi[(size_t)r * n + i] = lz_cut<true>(q, e);
   }
@@ -335,19 +345,20 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   double* tw = (double*)(base + off); off += al(sizeof(double) * (size_t)nruns * m);
   using I = typename LzInt<T>::type;
   I* Qi = (I*)(base + off); off += al(sizeof(I) * pstride);
-  int* ea = (int*)(base + off); off += al(sizeof(int) * ((size_t)n + nruns));
-  int* eq = ea + n;
+  int* ea = (int*)(base + off); off += al(sizeof(int) * ((size_t)n + nruns + 1));
+  int *eq = ea + n, *emax = eq + nruns;
   if (off > work_bytes) return CHASE_ERR_OOM;
   int nl = 0;
+  CHASE_CUDA_TRY(cudaMemsetAsync(emax, 0x80, sizeof(int), st));
   // q_0 = v / ||v|| for every run
   TRY_LZ(copy_cols<T>(st, n, nruns, V0, ldv, W, n, &nl));
-  launch_dep(st, ceil_div(n, 8), 256, 0, lz_colexp_kernel<T>, n, A, lda, ea);
+  launch_dep(st, ceil_div(n, 8), 256, 0, lz_colexp_kernel<T>, n, A, lda, ea, emax);
   launch_dep(st, nruns, 512, 0, lz_normalize_kernel<T>, n, W, Qb, beta, m, 0, Qi, eq);  // beta[.,0] rewritten below
   nl += 2;
   const int blocks = (int)std::min<size_t>((pstride + 255) / 256, (size_t)kNumSMs * 16);
   for (int j = 0; j < m; ++j) {
     // W = A q_j (up to four runs per pass over A)
-    TRY_LZ(lz_product<T>(st, n, nruns, A, lda, ea, Qi, eq, W, &nl));
+    TRY_LZ(lz_product<T>(st, n, nruns, A, lda, ea, Qi, eq, emax, W, &nl));
     // coefficients against q_0..q_j: coef[., j] is alpha_j; subtracting all of them is the
     // three-term step plus full re-orthogonalisation (classical Gram-Schmidt, twice)
     for (int pass = 0; pass < 2; ++pass) {
@@ -366,7 +377,12 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   CHASE_CUDA_TRY(cudaMemcpyAsync(htau.data(), tw, sizeof(double) * (size_t)nruns * m, cudaMemcpyDeviceToHost, st));
   CHASE_CUDA_TRY(cudaMemcpyAsync(hbeta.data(), beta, sizeof(double) * (size_t)nruns * m,
                                  cudaMemcpyDeviceToHost, st));
+  int em = 0;
+  CHASE_CUDA_TRY(cudaMemcpyAsync(&em, emax, sizeof(int), cudaMemcpyDeviceToHost, st));
   CHASE_CUDA_TRY(cudaStreamSynchronize(st));
+  em = lz_scale(em);
+  for (double& t : hth) t = std::ldexp(t, em);
+  for (double& b : hbeta) b = std::ldexp(b, em);
   double bsup = -1e300, l1 = 1e300;
   for (int r = 0; r < nruns; ++r) {
     const double* t = hth.data() + (size_t)r * m;
@@ -393,7 +409,7 @@ size_t lanczos_work_bytes(size_t elem, int n, int nruns, int m) {
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t ps = (size_t)n * nruns;
   return al(elem * ps * (m + 1)) + al(elem * ps) + al(elem * (size_t)nruns * (m + 1)) +
-         4 * al(8 * (size_t)nruns * m) + al(elem * ps) + al(4 * ((size_t)n + nruns)) + tridiag_work_bytes(m, nruns);
+         4 * al(8 * (size_t)nruns * m) + al(elem * ps) + al(4 * ((size_t)n + nruns + 1)) + tridiag_work_bytes(m, nruns);
 }
 
 template int lanczos_bounds<double>(cudaStream_t, int, const double*, int, int, const double*, int,
