@@ -291,29 +291,67 @@ __global__ void lz_store_alpha_kernel(int nruns, const T* coef, int ldc, int j, 
   if (r < nruns) alpha[r * m + j] = Sc<T>::re(coef[(size_t)r * ldc + j]);
 }
 
-// beta_r = ||w_r||; q_{j+1}^r = w_r / beta_r (one CTA per run), and its integers and exponent.
+// A number in (-1, 1) from a counter.
+__device__ __forceinline__ double lz_random(uint32_t x) {
+  x ^= x >> 16; x *= 0x7FEB352Du;
+  x ^= x >> 15; x *= 0x846CA68Bu;
+  x ^= x >> 16;
+  return ((double)x + 0.5) * 0x1p-31 - 1.0;
+}
+
+// beta_r = ||w_r||; q_{j+1}^r = w_r / beta_r (one CTA per run), and its integers and exponent.  Where
+// nothing is left of w_r beside the terms that it was reduced by (np > 0 basis vectors at Qb), the
+// basis spans an invariant subspace and w_r has no direction of its own, least of all one orthogonal
+// to the basis: beta_r = 0 then, and the run goes on from a pseudo-random vector orthogonal to it.
 template <class T>
-__global__ void __launch_bounds__(512) lz_normalize_kernel(int n, const T* W, T* qn, double* beta,
-                                                            int m, int j, typename LzInt<T>::type* qi, int* eq) {
+__global__ void __launch_bounds__(512) lz_normalize_kernel(int n, T* W, T* qn, double* beta,
+                                                            int m, int j, typename LzInt<T>::type* qi, int* eq,
+                                                            const T* Qb, size_t pstride, int np, const double* alpha) {
   dep_wait();
   __shared__ double red[16];
   __shared__ long long redm[16];
   const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const T* w = W + (size_t)r * n;
-  long long mx = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) mx = max(mx, lz_abs(w[i]));
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) redm[warp] = mx;
-  __syncthreads();
-  for (int i = 0; i < (int)blockDim.x >> 5; ++i) mx = max(mx, redm[i]);
-  // squares of w 2^-ew neither overflow nor underflow
-  const int ew = lz_exp(mx) == kLzBad ? 0 : lz_exp(mx);
-  const double scale = scalbn(1.0, -ew);
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += Sc<T>::abs2(Sc<T>::scale(w[i], scale));
-  s = block_sum_t<double>(s, red);
-  const double b = sqrt(s);  // of w 2^-ew: 1 / |w| may be out of range
-  if (threadIdx.x == 0) beta[r * m + j] = scalbn(b, ew);
+  T* w = W + (size_t)r * n;
+  long long mx;
+  int ew;
+  double scale, b;  // b = ||w|| 2^-ew: 1 / ||w|| may be out of range
+  auto measure = [&]() {
+    mx = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) mx = max(mx, lz_abs(w[i]));
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    __syncthreads();
+    if (lane == 0) redm[warp] = mx;
+    __syncthreads();
+    for (int i = 0; i < (int)blockDim.x >> 5; ++i) mx = max(mx, redm[i]);
+    // squares of w 2^-ew neither overflow nor underflow
+    ew = lz_exp(mx) == kLzBad ? 0 : lz_exp(mx);
+    scale = scalbn(1.0, -ew);
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) s += Sc<T>::abs2(Sc<T>::scale(w[i], scale));
+    b = sqrt(block_sum_t<double>(s, red));
+  };
+  measure();
+  bool ended = false;
+  if (np > 0) {
+    const double left = fabs(alpha[r * m + j]) + (j > 0 ? fabs(beta[r * m + j - 1]) : 0.0);
+    ended = scalbn(b, ew) <= 0x1p-50 * left;
+  }
+  if (ended) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const uint32_t k = ((uint32_t)i * 64 + (uint32_t)r * 2) ^ ((uint32_t)j << 24);
+      if constexpr (Sc<T>::cplx) w[i] = z64{lz_random(k), lz_random(k + 1)};
+      else w[i] = lz_random(k);
+    }
+    for (int p = 0; p < 2 * np; ++p) {
+      const T* q = Qb + (size_t)(p % np) * pstride + (size_t)r * n;
+      T c = Sc<T>::zero();
+      for (int i = threadIdx.x; i < n; i += blockDim.x) Sc<T>::fmac(c, q[i], w[i]);
+      c = block_sum_t<T>(c, red);
+      for (int i = threadIdx.x; i < n; i += blockDim.x) w[i] = Sc<T>::sub(w[i], Sc<T>::mul(c, q[i]));
+    }
+    measure();
+  }
+  if (threadIdx.x == 0) beta[r * m + j] = ended ? 0.0 : scalbn(b, ew);
   const double inv = (b > 0.0) ? 1.0 / b : 0.0;
   // the largest |q| is the largest |w| 2^-ew times inv (rounding keeps order)
   const int e = lz_exp(lz_abs(__longlong_as_double(mx) * scale * inv));
@@ -353,7 +391,8 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
   // q_0 = v / ||v|| for every run
   TRY_LZ(copy_cols<T>(st, n, nruns, V0, ldv, W, n, &nl));
   launch_dep(st, ceil_div(n, 8), 256, 0, lz_colexp_kernel<T>, n, A, lda, ea, emax);
-  launch_dep(st, nruns, 512, 0, lz_normalize_kernel<T>, n, W, Qb, beta, m, 0, Qi, eq);  // beta[.,0] rewritten below
+  launch_dep(st, nruns, 512, 0, lz_normalize_kernel<T>, n, W, Qb, beta, m, 0, Qi, eq,
+             Qb, pstride, 0, alpha);  // beta[.,0] rewritten below
   nl += 2;
   const int blocks = (int)std::min<size_t>((pstride + 255) / 256, (size_t)kNumSMs * 16);
   for (int j = 0; j < m; ++j) {
@@ -367,7 +406,8 @@ int lanczos_bounds(cudaStream_t st, int n, const T* A, int lda, int nruns, const
       launch_dep(st, blocks, 256, 0, lz_sub_kernel<T>, n, nruns, Qb, pstride, W, coef, m + 1, j + 1);
       nl += (pass == 0) ? 3 : 2;
     }
-    launch_dep(st, nruns, 512, 0, lz_normalize_kernel<T>, n, W, Qb + (size_t)(j + 1) * pstride, beta, m, j, Qi, eq);
+    launch_dep(st, nruns, 512, 0, lz_normalize_kernel<T>, n, W, Qb + (size_t)(j + 1) * pstride, beta, m, j, Qi, eq,
+               Qb, pstride, j + 1, alpha);
     ++nl;
   }
   // Ritz values and weights of each run

@@ -1,6 +1,7 @@
-"""Lanczos runs whose residual vanishes beside a matrix near the lower end of FP64, where it would be
-a subnormal vector: its norm has no reciprocal in range and its inner products no digits.  c I has
-every Ritz value c; bound: the n roundings of the inner products."""
+"""Lanczos runs that end early.  A residual that vanishes beside a matrix near the lower end of FP64
+would be a subnormal vector: its norm has no reciprocal in range and its inner products no digits.
+c I has every Ritz value c; bound: the n roundings of the inner products.  From a start vector in
+an invariant subspace a run has to see the rest of the spectrum too."""
 import numpy as np
 import pytest
 
@@ -32,3 +33,29 @@ def test_multiple_of_the_identity(cl, complex_, c):
     finally:
         h.close()
     assert np.all(np.abs(got - c) <= 8 * n * 2.0 ** -53 * c)
+
+
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("rotated", [False, True])
+def test_start_in_an_invariant_subspace(cl, complex_, rotated):
+    """One run from the eigenvector of the eigenvalue 2 (exactly, or to rounding) of a matrix with
+    spectrum [2, 5], as many steps as there are: the Ritz values are eigenvalues (n steps on n = 24;
+    100 n roundings), beta ends small, and the bounds are those of the whole spectrum."""
+    n = 24
+    rng = np.random.default_rng(9)
+    lam = np.linspace(2.0, 5.0, n)
+    Q = np.eye(n)
+    if rotated:
+        Q = np.linalg.qr(rng.standard_normal((n, n)) + (1j * rng.standard_normal((n, n)) if complex_ else 0.0))[0]
+    A = (Q * lam) @ Q.conj().T
+    A = (0.5 * (A + A.conj().T)).astype(complex if complex_ else float)
+    v = Q[:, :1].astype(A.dtype)
+    h = cl.Handle(0)
+    try:
+        got = cl.chase_lanczos_bounds(h, cl.colmajor(torch.from_numpy(A).cuda()),
+                                      cl.colmajor(torch.from_numpy(v.copy()).cuda()), n - 1, n // 2)
+    finally:
+        h.close()
+    assert abs(got[0] - 2.0) <= 1e-2 and got[0] >= 2.0 - 100 * n * 2.0 ** -53
+    assert got[2] >= 5.0 - 100 * n * 2.0 ** -53
+    assert got[2] <= 5.0 + 3.0
