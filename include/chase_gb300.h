@@ -379,7 +379,8 @@ int chase_solve_batch(chase_handle h, int count, const chase_problem* problems,
 
 /*
  * chase_autotune_table -- the autotuner's picks so far (one text line per shape bucket:
- * shape, bucket, tile-width cap, K splits, measured seconds), NUL-terminated into buf (cap
+ * shape, bucket, tile-width cap, K splits, measured seconds, ring moduli or 0 for a real
+ * product; the two kinds are tuned apart), NUL-terminated into buf (cap
  * bytes; truncated if short).  *needed (may be NULL) receives the bytes the full table needs.
  * chase_autotune_clear -- forgets every pick.  The table is shared by the whole process.
  * No counterpart in the paper: the launch plans are this implementation's.

@@ -8,7 +8,8 @@
 // every plan gives bit-identical results, so the tuner times the candidates in place on the
 // caller's own data (each candidate overwrites the same output with the same values) the
 // first time a shape bucket is met, and keeps the fastest.  Buckets: the rows M and the
-// inner dimension K in quarter octaves (round(4 log2)), the columns N in steps of 32.  The
+// inner dimension K in quarter octaves (round(4 log2)), the columns N in steps of 32, real
+// and ring products (15 or 16 moduli, two plane sets, no K splits) apart.  The
 // table is process-wide (the plans are properties of the GPU and the shapes) and guarded
 // by a mutex (batch sessions call from several threads).
 #include <cuda_runtime.h>
@@ -39,29 +40,30 @@ std::mutex& table_mutex() {
   static std::mutex m;
   return m;
 }
-std::map<std::tuple<int, int, int>, Entry>& table() {
-  static std::map<std::tuple<int, int, int>, Entry> t;
+using Key = std::tuple<int, int, int, int>;
+std::map<Key, Entry>& table() {
+  static std::map<Key, Entry> t;
   return t;
 }
 
-std::tuple<int, int, int> key_of(int M, int N, int kp) {
+Key key_of(int M, int N, int kp, int ring) {
   return std::make_tuple((int)std::lround(4.0 * std::log2((double)std::max(M, 1))), (N + 31) / 32,
-                         (int)std::lround(4.0 * std::log2((double)std::max(kp, 1))));
+                         (int)std::lround(4.0 * std::log2((double)std::max(kp, 1))), ring);
 }
 
 }  // namespace
 
-bool oz_plan_lookup(int M, int N, int kp, OzPlan* plan) {
+bool oz_plan_lookup(int M, int N, int kp, int ring, OzPlan* plan) {
   std::lock_guard<std::mutex> g(table_mutex());
-  auto it = table().find(key_of(M, N, kp));
+  auto it = table().find(key_of(M, N, kp, ring));
   if (it == table().end()) return false;
   *plan = it->second.plan;
   return true;
 }
 
-void oz_plan_store(int M, int N, int kp, const OzPlan& plan, double seconds) {
+void oz_plan_store(int M, int N, int kp, int ring, const OzPlan& plan, double seconds) {
   std::lock_guard<std::mutex> g(table_mutex());
-  table()[key_of(M, N, kp)] = Entry{plan, seconds, M, N, kp};
+  table()[key_of(M, N, kp, ring)] = Entry{plan, seconds, M, N, kp};
 }
 
 int oz_plan_candidates(int N, OzPlan* out, int cap) {
@@ -94,9 +96,9 @@ int chase_autotune_table(char* buf, size_t cap, size_t* needed) {
     for (const auto& kv : chase::table()) {
       const chase::Entry& e = kv.second;
       snprintf(line, sizeof line,
-               "ozm M=%d N=%d K=%d bucket=(%d,%d,%d) tile_cap=%d splits=%d seconds=%.6e\n", e.shape_M,
+               "ozm M=%d N=%d K=%d bucket=(%d,%d,%d) tile_cap=%d splits=%d seconds=%.6e ring=%d\n", e.shape_M,
                e.shape_N, e.shape_K, std::get<0>(kv.first), std::get<1>(kv.first),
-               std::get<2>(kv.first), e.plan.bn_max, e.plan.splits, e.seconds);
+               std::get<2>(kv.first), e.plan.bn_max, e.plan.splits, e.seconds, std::get<3>(kv.first));
       s += line;
     }
   }

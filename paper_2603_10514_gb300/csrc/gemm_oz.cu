@@ -1474,7 +1474,7 @@ int oz_gemm(cudaStream_t st, int M, int kp, const void* Aplanes, const int* rowe
   if (N <= 0 || M <= 0) return 0;
   if (kp % MBK != 0 || kp > kOzMaxK) return CHASE_ERR_UNSUPPORTED;
   OzPlan plan;
-  const bool known = oz_plan_lookup(M, N, kp, &plan);
+  const bool known = oz_plan_lookup(M, N, kp, 0, &plan);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (tune && !known && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
       cs == cudaStreamCaptureStatusNone) {
@@ -1500,7 +1500,7 @@ int oz_gemm(cudaStream_t st, int M, int kp, const void* Aplanes, const int* rowe
         cudaEventElapsedTime(&ms, ev[i], ev[i + 1]);
         if (ms < tbest) { tbest = ms; best = i; }
       }
-      oz_plan_store(M, N, kp, cand[best], tbest * 1e-3);
+      oz_plan_store(M, N, kp, 0, cand[best], tbest * 1e-3);
       if (trials) *trials += nc;
       plan = cand[best];
     }
@@ -1630,7 +1630,7 @@ int tune_group_item(cudaStream_t st, const OzGroupItem& it, DevStatus* dst, int*
       cudaEventElapsedTime(&ms, ev[i], ev[i + 1]);
       if (ms < tbest) { tbest = ms; best = i; }
     }
-    oz_plan_store(it.M, it.N, it.kp, cand[best], tbest * 1e-3);
+    oz_plan_store(it.M, it.N, it.kp, it.ring ? ring_moduli(it.kp) : 0, cand[best], tbest * 1e-3);
     if (trials) *trials += nc;
   }
   for (int i = 0; i <= nc; ++i) cudaEventDestroy(ev[i]);
@@ -1669,12 +1669,13 @@ int oz_gemm_group(cudaStream_t st, int count, const OzGroupItem* items, DevStatu
     if (it.kp % MBK != 0 || it.kp > kOzSplitMaxK) return CHASE_ERR_UNSUPPORTED;  // K is not split here
     if (P.count + (it.ring ? 2 : 1) > kOzGroupMax || C.count + 1 > kOzGroupMax) TRY_OZ(flush());
     OzPlan plan;  // the autotuner's tile width for this shape, if it measured one
-    bool known = oz_plan_lookup(it.M, it.N, it.kp, &plan);
+    const int kind = it.ring ? ring_moduli(it.kp) : 0;
+    const bool known = oz_plan_lookup(it.M, it.N, it.kp, kind, &plan);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (tune && !known && count == 1 && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
         cs == cudaStreamCaptureStatusNone) {
       TRY_OZ(tune_group_item(st, it, dst, launches, trials));
-      oz_plan_lookup(it.M, it.N, it.kp, &plan);
+      oz_plan_lookup(it.M, it.N, it.kp, kind, &plan);
     }
     TRY_OZ(ozm_append(P, tiles, it, plan.bn_max));
     CrtItem& I = C.it[C.count++];

@@ -162,8 +162,9 @@ struct OzPlan {
   int splits = 0;
 };
 // The autotuner's table (autotune.cu): plans measured per shape bucket.
-bool oz_plan_lookup(int M, int N, int kp, OzPlan* plan);
-void oz_plan_store(int M, int N, int kp, const OzPlan& plan, double seconds);
+// ring: 0 for a real product, else the number of ring moduli.
+bool oz_plan_lookup(int M, int N, int kp, int ring, OzPlan* plan);
+void oz_plan_store(int M, int N, int kp, int ring, const OzPlan& plan, double seconds);
 int oz_plan_candidates(int N, OzPlan* out, int cap);
 // out64[:, col0 + c] = alpha * (A V)[:, col0 + c] + beta * X64 + gamma * Z64 for c < N.
 // A's planes are a_plane_rows * kp elements apart (0: M * kp).  resbuf: residues of the
