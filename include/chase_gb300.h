@@ -158,9 +158,9 @@ typedef struct {
   double t_rr_eig;         /* part of t_rr spent in the reduced problem's eigensolver */
   int jacobi_sweeps;       /* 0: the reduced eigensolver is direct (no Jacobi sweeps) */
   double t_filter_product; /* part of t_filter spent in the product kernels alone (CUDA events
-                              around each launch, around every eighth of emulated and BF16x3
-                              products below 2e10 operations; filters launched as graphs add
-                              nothing) */
+                              around each launch; of emulated and BF16x3 products below 2e10
+                              operations around one in eight, which stands for the eight;
+                              filters launched as graphs add nothing) */
   double t_graph_build;    /* graph_filter = 1: host seconds spent recording and instantiating
                               the filter graphs (inside t_filter) */
   int graph_launches;      /* graph_filter = 1: filter calls that ran as one graph launch */

@@ -25,6 +25,7 @@
 #include "../../include/chase_gb300.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "launch_sample.h"
 
 namespace chase {
 
@@ -40,7 +41,7 @@ using namespace chase;
 
 // CUDA-event time of selected launches on one stream (the filter's product kernels):
 // event pairs around each launch, summed once the stream has been synchronised.  Of short launches
-// (`few_us`) every eighth is timed and stands for eight: an event takes a few microseconds between
+// (`few_us`) one in eight is timed (launch_sample.h): an event takes a few microseconds between
 // two launches, and launch_dep's overlap with it (a filter step of n = 1000, 30 columns: 34 us
 // with two events in every step, 25 without).
 struct LaunchTimer {
@@ -48,20 +49,17 @@ struct LaunchTimer {
   size_t used = 0;
   bool enabled = true;  // off while a stream is being captured into a graph
   bool open = false;
-  std::vector<char> few;            // per pair: a short launch
-  size_t few_all = 0, few_timed = 0;
+  LaunchSample sample;
   void begin(cudaStream_t st, bool few_us = false) {
+    open = false;
     if (!enabled) return;
-    if (few_us && few_all++ % 8) return;
     while (ev.size() < used + 2) {
       cudaEvent_t e;
       if (cudaEventCreate(&e) != cudaSuccess) return;
       ev.push_back(e);
     }
+    if (!sample.next(few_us)) return;
     cudaEventRecord(ev[used], st);
-    few.resize(used / 2);
-    few.push_back(few_us);
-    few_timed += few_us;
     open = true;
   }
   void end(cudaStream_t st) {
@@ -71,13 +69,14 @@ struct LaunchTimer {
     open = false;
   }
   double collect() {  // seconds; call after the stream has been synchronised
-    double s = 0.0, f = 0.0;
-    for (size_t i = 0; i + 1 < used; i += 2) {
+    std::vector<double> t(used / 2, 0.0);
+    for (size_t i = 0; i < t.size(); ++i) {
       float ms = 0.f;
-      if (cudaEventElapsedTime(&ms, ev[i], ev[i + 1]) == cudaSuccess) (few[i / 2] ? f : s) += ms;
+      if (cudaEventElapsedTime(&ms, ev[2 * i], ev[2 * i + 1]) == cudaSuccess) t[i] = ms;
     }
-    if (few_timed) s += f * ((double)few_all / (double)few_timed);
-    used = few_all = few_timed = 0;
+    const double s = sample.total(t.data(), t.size());
+    sample.clear();
+    used = 0;
     return s * 1e-3;
   }
   // a product of fewer operations takes under ~100 us (the emulated one 60 us at 2e10)
