@@ -78,7 +78,6 @@ __device__ bool chol_block(int b, T* G, int ldg, int off, double shift, T* B, T*
     __syncwarp();
     if (lane > j) B[j * CLD + lane] = Sc<T>::scale(B[j * CLD + lane], r);
     else M[j * CLD + lane] = Sc<T>::scale(M[j * CLD + lane], r);
-    if (lane == j) B[j * CLD + j] = Sc<T>::from_re(d * r);
     if (lane == 0 && bad) {
       s_fail = 1;
       atomicCAS(&dst->chol_info, 0, off + j + 1);
@@ -102,7 +101,10 @@ __device__ bool chol_block(int b, T* G, int ldg, int off, double shift, T* B, T*
   }
   for (int t = tid; t < CB * CB; t += CNT) {
     const int i = t % CB, j = t / CB;
-    if (i <= j && j < b) G[(size_t)(off + i) + (size_t)(off + j) * ldg] = B[i * CLD + j];
+    // (the diagonal of B holds the pivots: their roots are taken here, off the chain)
+    const T r = B[i * CLD + j];
+    if (i <= j && j < b)
+      G[(size_t)(off + i) + (size_t)(off + j) * ldg] = i == j ? Sc<T>::from_re(sqrt(Sc<T>::re(r))) : r;
     Mb[t] = (i < b && j <= i) ? M[i * CLD + j] : Sc<T>::zero();  // column-major CB x CB
   }
   return true;
