@@ -915,7 +915,7 @@ EighLayout eigh_layout(int l, size_t elem) {
 }
 
 template <class T>
-int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout& L, DevStatus* dst, int ctas,
+int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout& L, DevStatus* dst,
             int* launches) {
   T *tau = (T*)(base + L.tau), *xb = (T*)(base + L.xb), *cb = (T*)(base + L.cb);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e), *part = (double*)(base + L.part);
@@ -926,7 +926,6 @@ int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout&
   // on four; l = 60 real 0.417 and 0.343; l = 230 complex 1.95 on 38, 1.73 on 76)
   const double work = (double)l * l * (Sc<T>::cplx ? 4.0 : 1.0);
   int G = work < 3000.0 ? 1 : (int)std::min<double>(kNumSMs, work / 1000.0);
-  if (ctas > 0) G = std::min(ctas, kNumSMs);
   const bool vec = tri_vec_smem(l, sizeof(T));
   if (!vec) G = kNumSMs;
   G = std::max(1, std::min(G, l));
@@ -957,7 +956,7 @@ size_t eigh_work_bytes(int l, size_t elem) { return eigh_layout(l, elem).total; 
 
 template <class T>
 int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work, size_t work_bytes,
-         DevStatus* dst, int* launches, int ctas) {
+         DevStatus* dst, int* launches) {
   if (l <= 0) return 0;
   const EighLayout L = eigh_layout(l, sizeof(T));
   if (L.total > work_bytes) return CHASE_ERR_OOM;
@@ -965,7 +964,7 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   T* tau = (T*)(base + L.tau);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e);
   const int* ex0 = (const int*)(base + L.ex);
-  TRY_EIG(tridiag<T>(st, l, H, ldh, base, L, dst, ctas, launches));
+  TRY_EIG(tridiag<T>(st, l, H, ldh, base, L, dst, launches));
   const DcWork D = dc_carve(base + L.dc, l);
   int cur = 0;
   TRY_EIG(stedc(st, l, 1, d, e, 0, D, 0, &cur, launches));
@@ -1010,7 +1009,7 @@ int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const d
   return 0;
 }
 
-template int eigh<double>(cudaStream_t, int, double*, int, double*, int, double*, void*, size_t, DevStatus*, int*, int);
-template int eigh<z64>(cudaStream_t, int, z64*, int, z64*, int, double*, void*, size_t, DevStatus*, int*, int);
+template int eigh<double>(cudaStream_t, int, double*, int, double*, int, double*, void*, size_t, DevStatus*, int*);
+template int eigh<z64>(cudaStream_t, int, z64*, int, z64*, int, double*, void*, size_t, DevStatus*, int*);
 
 }  // namespace chase

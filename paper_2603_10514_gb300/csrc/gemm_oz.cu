@@ -111,10 +111,6 @@ constexpr uint32_t big_mod_small(Big a, uint32_t p) {
   for (int i = 4; i >= 0; --i) r = ((r << 32) | a.w[i]) % p;
   return (uint32_t)r;
 }
-constexpr Big big_shr1(Big a) {
-  for (int i = 0; i < 5; ++i) a.w[i] = (a.w[i] >> 1) | (i < 4 ? (a.w[i + 1] << 31) : 0u);
-  return a;
-}
 constexpr uint32_t inv_mod(uint32_t a, uint32_t p) {  // a^{-1} mod p, gcd(a, p) = 1
   long long t = 0, nt = 1, r = p, nr = a % p;
   while (nr != 0) {
@@ -129,7 +125,6 @@ struct CrtTable {
   int p[kOzModuli];          // the moduli
   uint32_t C[kOzModuli][5];  // C_j = (P / p_j) ((P / p_j)^{-1} mod p_j) < P
   uint32_t P[5];
-  uint32_t Ph[5];            // P / 2
   float p96_over_P;          // 2^96 / P (rounded)
 };
 
@@ -148,11 +143,9 @@ constexpr CrtTable make_crt_table() {
     const Big Cj = big_mul_small(Mj, inv);
     for (int l = 0; l < 5; ++l) t.C[j][l] = Cj.w[l];
   }
-  const Big Ph = big_shr1(P);
   double pd = 0.0;
   for (int l = 4; l >= 0; --l) {
     t.P[l] = P.w[l];
-    t.Ph[l] = Ph.w[l];
     pd = pd * 4294967296.0 + (double)P.w[l];
   }
   t.p96_over_P = (float)(79228162514264337593543950336.0 / pd);  // 2^96 / P
@@ -231,7 +224,7 @@ __host__ __device__ constexpr uint32_t ring_root(int j) {
 template <int NM>
 struct RingTable {
   uint32_t Cre[NM][5], Cim[NM][5];
-  uint32_t P[5], Ph[5];
+  uint32_t P[5];
   float p96_over_P;
 };
 
@@ -253,11 +246,9 @@ constexpr RingTable<NM> make_ring_table() {
       t.Cim[j][l] = Cim.w[l];
     }
   }
-  const Big Ph = big_shr1(P);
   double pd = 0.0;
   for (int l = 4; l >= 0; --l) {
     t.P[l] = P.w[l];
-    t.Ph[l] = Ph.w[l];
     pd = pd * 4294967296.0 + (double)P.w[l];
   }
   t.p96_over_P = (float)(79228162514264337593543950336.0 / pd);
