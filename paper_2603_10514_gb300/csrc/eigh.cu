@@ -394,8 +394,9 @@ struct DcWork {
 constexpr int kDcDoubles = 12, kDcInts = 13, kDcBytes = 3;
 
 __host__ __device__ inline size_t dc_align(size_t x) { return (x + 255) & ~(size_t)255; }
-inline size_t dc_bytes(int n) {
-  return dc_align((size_t)n * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)) + 3 * dc_align((size_t)8 * n * n) + 256;
+// mats: n x n matrices among them (Q[0], or with Q[1] and U).
+inline size_t dc_bytes(int n, int mats) {
+  return dc_align((size_t)n * (8 * kDcDoubles + 4 * kDcInts + kDcBytes)) + mats * dc_align((size_t)8 * n * n) + 256;
 }
 // Carves the arrays of a problem of order n; with Q == nullptr-sized matrices left out (leaf).
 __host__ __device__ inline DcWork dc_vectors(char* base, int n) {
@@ -414,12 +415,19 @@ __host__ __device__ inline DcWork dc_vectors(char* base, int n) {
   W.type = c + 2 * (size_t)n;
   return W;
 }
-inline DcWork dc_carve(char* base, int n) {
+// Q1, U: n x n doubles each elsewhere, or both null.
+inline DcWork dc_carve(char* base, int n, double* Q1, double* U) {
   DcWork W = dc_vectors(base, n);
   char* p = base + dc_align((size_t)n * (8 * kDcDoubles + 4 * kDcInts + kDcBytes));
-  for (int i = 0; i < 2; ++i) { W.Q[i] = (double*)p; p += dc_align((size_t)8 * n * n); }
-  W.U = (double*)p;
-  p += dc_align((size_t)8 * n * n);
+  auto take = [&](double* given) {
+    if (given) return given;
+    double* q = (double*)p;
+    p += dc_align((size_t)8 * n * n);
+    return q;
+  };
+  W.Q[0] = take(nullptr);
+  W.Q[1] = take(Q1);
+  W.U = take(U);
   W.bad = (int*)p;
   W.ex = W.bad + 1;
   return W;
@@ -700,8 +708,11 @@ int dc_depth(int n) {
 int stedc(cudaStream_t st, int n, int batch, const double* d, const double* e, int ld_de, const DcWork& W,
           size_t stride, int* cur, int* launches) {
   for (int b = 0; b < batch; ++b) {
-    char* q = (char*)W.Q[0] + stride * b;  // Q[0], Q[1], U and the flag lie one after another
-    CHASE_CUDA_TRY(cudaMemsetAsync(q, 0, 3 * dc_align((size_t)8 * n * n) + sizeof(int), st));
+    // the flag lies behind Q[0], or behind Q[1] and U too
+    const size_t span = (char*)W.bad - (char*)W.Q[0];
+    CHASE_CUDA_TRY(cudaMemsetAsync((char*)W.Q[0] + stride * b, 0, span + sizeof(int), st));
+    if (span < 2 * dc_align((size_t)8 * n * n))
+      CHASE_CUDA_TRY(cudaMemsetAsync(W.Q[1], 0, (size_t)8 * n * n, st));
   }
   const int depth = dc_depth(n);
   launch_dep(st, dim3(1 << depth, batch), 256, 0, dc_leaf_kernel, n, depth, d, e, ld_de, W, stride);
@@ -887,7 +898,7 @@ __global__ void dc_extract_kernel(DcWork W0, size_t stride, int cur, double* the
 }
 // problems of one pass over the tridiagonals: as many as fit about 128 MB, at least one
 int tridiag_pass(int m, int batch) {
-  return (int)std::max<size_t>(1, std::min<size_t>(batch, ((size_t)128 << 20) / dc_align(dc_bytes(m))));
+  return (int)std::max<size_t>(1, std::min<size_t>(batch, ((size_t)128 << 20) / dc_align(dc_bytes(m, 3))));
 }
 
 struct EighLayout {
@@ -909,7 +920,7 @@ EighLayout eigh_layout(int l, size_t elem) {
   L.scr = take(tri_vec_smem(l, elem) ? 0 : elem * 3 * (size_t)l * kNumSMs);
   L.tb = take(sizeof(GridBar));
   L.ex = take(sizeof(int));
-  L.dc = take(dc_bytes(l));
+  L.dc = take(dc_bytes(l, 1));
   L.total = off;
   return L;
 }
@@ -955,17 +966,19 @@ int tridiag(cudaStream_t st, int l, T* H, int ldh, char* base, const EighLayout&
 size_t eigh_work_bytes(int l, size_t elem) { return eigh_layout(l, elem).total; }
 
 template <class T>
-int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work, size_t work_bytes,
+int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, T* spare, void* work, size_t work_bytes,
          DevStatus* dst, int* launches) {
   if (l <= 0) return 0;
   const EighLayout L = eigh_layout(l, sizeof(T));
   if (L.total > work_bytes) return CHASE_ERR_OOM;
+  if (ldw != l) return CHASE_ERR_UNSUPPORTED;
   char* base = (char*)work;
   T* tau = (T*)(base + L.tau);
   double *d = (double*)(base + L.d), *e = (double*)(base + L.e);
   const int* ex0 = (const int*)(base + L.ex);
   TRY_EIG(tridiag<T>(st, l, H, ldh, base, L, dst, launches));
-  const DcWork D = dc_carve(base + L.dc, l);
+  // (the eigenvectors' place holds U until they are formed)
+  const DcWork D = dc_carve(base + L.dc, l, (double*)spare, (double*)W);
   int cur = 0;
   TRY_EIG(stedc(st, l, 1, d, e, 0, D, 0, &cur, launches));
   const int wpc = (int)std::max<size_t>(1, std::min<size_t>(4, (kSmemMax - 1024) / (sizeof(T) * (size_t)l)));
@@ -974,7 +987,7 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)backtransform_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSmemMax - 1024));
   if (in_smem && l >= BT_MIN) {
-    T* Tb = (T*)D.U;  // free by now: l^2 doubles for 8 (l + 7) elements
+    T* Tb = (T*)D.Q[cur ^ 1];  // free by now: l^2 doubles for 8 (l + 7) elements
     launch_dep(st, ceil_div(l - 1, BTK), 256, 0, bt_factor_kernel<T>, l, H, ldh, tau, Tb);
     CHASE_CUDA_TRY(cudaFuncSetAttribute((const void*)bt_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)kSmemMax - 1024));
@@ -990,14 +1003,14 @@ int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void*
   return 0;
 }
 
-size_t tridiag_work_bytes(int m, int batch) { return dc_align(dc_bytes(m)) * tridiag_pass(m, batch); }
+size_t tridiag_work_bytes(int m, int batch) { return dc_align(dc_bytes(m, 3)) * tridiag_pass(m, batch); }
 
 int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const double* beta, double* theta,
                  double* weight, void* work, size_t work_bytes, int* launches) {
   if (m <= 0 || batch <= 0) return 0;
   if (tridiag_work_bytes(m, batch) > work_bytes) return CHASE_ERR_OOM;
-  const size_t stride = dc_align(dc_bytes(m));
-  const DcWork W = dc_carve((char*)work, m);
+  const size_t stride = dc_align(dc_bytes(m, 3));
+  const DcWork W = dc_carve((char*)work, m, nullptr, nullptr);
   for (int r = 0, nb = tridiag_pass(m, batch); r < batch; r += nb) {
     const int cnt = std::min(nb, batch - r);
     int cur = 0;
@@ -1009,7 +1022,7 @@ int tridiag_eigs(cudaStream_t st, int m, int batch, const double* alpha, const d
   return 0;
 }
 
-template int eigh<double>(cudaStream_t, int, double*, int, double*, int, double*, void*, size_t, DevStatus*, int*);
-template int eigh<z64>(cudaStream_t, int, z64*, int, z64*, int, double*, void*, size_t, DevStatus*, int*);
+template int eigh<double>(cudaStream_t, int, double*, int, double*, int, double*, double*, void*, size_t, DevStatus*, int*);
+template int eigh<z64>(cudaStream_t, int, z64*, int, z64*, int, double*, z64*, void*, size_t, DevStatus*, int*);
 
 }  // namespace chase

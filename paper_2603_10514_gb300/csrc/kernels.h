@@ -53,11 +53,11 @@ int hh_thin_identity(cudaStream_t st, int n, int l, T* X, int ldx, int* launches
 
 // ---- direct eigensolver (eigh.cu) -------------------------------------------
 // Eigenvalues (ascending, dw on the device) and eigenvectors W of the Hermitian H (l x l,
-// overwritten).  work: eigh_work_bytes(l, sizeof(T)).  A bounded wait that ran out sets
+// overwritten; ldw = l).  spare: l x l elements, overwritten; work: eigh_work_bytes(l, sizeof(T)).  A bounded wait that ran out sets
 // dst->timeout.
 size_t eigh_work_bytes(int l, size_t elem);
 template <class T>
-int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, void* work, size_t work_bytes,
+int eigh(cudaStream_t st, int l, T* H, int ldh, T* W, int ldw, double* dw, T* spare, void* work, size_t work_bytes,
          DevStatus* dst, int* launches);
 // Eigenvalues (ascending) and squared first eigenvector components of `batch` real symmetric
 // tridiagonals of order m: run r's diagonal at alpha + r m, off-diagonal at beta + r m; theta and

@@ -1177,7 +1177,7 @@ struct Solve final : SolveBase {
     cudaEventCreate(&j0);
     cudaEventCreate(&j1);
     cudaEventRecord(j0, st);
-    if (!rc) rc = eigh<T>(st, nu, H, nu, Wm, nu, dw, eigw, eigw_bytes, h->dstat, &h->launches);
+    if (!rc) rc = eigh<T>(st, nu, H, nu, Wm, nu, dw, G, eigw, eigw_bytes, h->dstat, &h->launches);
     cudaEventRecord(j1, st);
     // V <- Q2 W, AV = AQ W (into P)
     if (rc) {
