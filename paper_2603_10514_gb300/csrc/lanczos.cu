@@ -75,9 +75,11 @@ __device__ inline z64 block_sum_t<z64>(z64 v, double* red) {
 //   2^-56 / sqrt 3 sqrt(sum a^2 + sum b^2)            in fixed point, and about
 //   2^-53 sqrt(5.3 + 1700 / n) / 20.4 sum |a b|       in FP64 (chains of n / 32 terms, 5 more sums,
 //                                                       terms of either sign: less than for one sign);
-// every column of every step is checked for the first being the smaller, and summed in FP64 where it
-// is not: columns and vectors with large and small entries at different places.
+// every column of every step is checked for the first being the smaller.  Where it is not (sparse
+// columns, columns and vectors with large and small entries at different places) the column is summed
+// in FP64, for the rest of the call.
 constexpr int kLzBits = 55, kLzBad = 1 << 20;  // exponent of a column with NaN or infinity
+constexpr int kLzFp64 = -kLzBad;               // of one that is summed in FP64
 
 __device__ __forceinline__ long long lz_abs(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }
 __device__ __forceinline__ long long lz_abs(z64 a) { return max(lz_abs(a.x), lz_abs(a.y)); }
@@ -182,11 +184,12 @@ struct LzSum {
 // the q_r, cut up, their magnitudes, their exponents.  A term of x is at most 2^56 (complex: two): the
 // sums of a lane are taken out after 120 (60) terms.  Bound by the wide multiply-adds, the instructions
 // that cut A up and the loads of q from L2.  4 runs, 25 steps of n = 8000: real 12.8 ms in FP64 -> 7.7
-// (7.2 without the check, two columns to a warp), complex 22.2; two blocks per SM, since more columns
+// (7.2 without the check, two columns to a warp), complex 21.5; a sparse
+// real one, in FP64, 13.4.  Two blocks per SM, since more columns
 // at once spread the reads of A over more pages (three: 11 ms).
 template <class T, int R>
 __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, int lda,
-                                                            const int* ea, const T* Q,
+                                                            int* ea, const T* Q,
                                                             const typename LzInt<T>::type* Qi,
                                                             const float4* Qm, const int* eq,
                                                             const int* emax, T* W) {
@@ -253,7 +256,8 @@ __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, i
     }
   };
   constexpr int CHUNK = 32 * (Z ? 60 : 120), UNROLL = Z ? 2 : 8, ROWS = 32 * UNROLL;
-  for (int i0 = 0; i0 < n; i0 += CHUNK) {
+  bool exact = e != kLzFp64;
+  for (int i0 = 0; i0 < n && exact; i0 += CHUNK) {
 #pragma unroll
     for (int u = 0; u < NV; ++u) s[u] = LzSum{0, 0, 0};
     const int i1 = min(n, i0 + CHUNK);
@@ -271,34 +275,46 @@ __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, i
   }
   // sum a^2 + sum b^2 <= (2.4 + 780 / terms) (sum |a b|)^2; |q| = 1, so sum b^2 = 4^-eq
   const float a2 = warp_sumf(sa) * 0x1p-46f, lim = 2.4f + 780.0f / (float)(NP * n);
-  bool exact = true;
+  bool ok = true;
 #pragma unroll
   for (int u = 0; u < NV; ++u) {
     const int r = u / NP;
     const float2 v = sab[u % NP][r / 2];
     const float ab = warp_sumf(r % 2 ? v.y : v.x) * 0x1p-46f, b2 = exp2f(-2.0f * (float)max(eq[r], -50));
-    exact = exact && a2 + b2 <= lim * ab * ab;
+    ok = ok && a2 + b2 <= lim * ab * ab;
   }
-  exact = exact || a2 == 0.0f;  // (nothing beside the diagonal entry, or NaN)
+  exact = exact && (ok || a2 == 0.0f);  // (0: nothing beside the diagonal entry, or NaN)
   const double scale = scalbn(1.0, -em);
   if (!exact) {
+    if (lane == 0) ea[c] = kLzFp64;
 #pragma unroll
     for (int u = 0; u < NV; ++u) sum[u] = 0.0;
-#pragma unroll 2
-    for (int i = lane; i < n; i += 32) {
-      const T a = i == c ? Sc<T>::zero() : Sc<T>::scale(col[i], scale);
+    // (the scale after the sums, unless they might leave FP64's range: 1 FP64 instruction in 5)
+    const bool late = abs(em) < 400;
+    auto fp64 = [&](auto scaled) {
+#pragma unroll 4
+      for (int i = lane; i < n; i += 32) {
+        T a = i == c ? Sc<T>::zero() : col[i];
+        if (decltype(scaled)::value) a = Sc<T>::scale(a, scale);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const T q = Q[(size_t)r * n + i];
-        if constexpr (Z) {
-          z64 v{sum[2 * r], sum[2 * r + 1]};
-          Sc<T>::fmac(v, a, q);
-          sum[2 * r] = v.x;
-          sum[2 * r + 1] = v.y;
-        } else {
-          Sc<T>::fmac(sum[r], a, q);
+        for (int r = 0; r < R; ++r) {
+          const T q = Q[(size_t)r * n + i];
+          if constexpr (Z) {
+            z64 v{sum[2 * r], sum[2 * r + 1]};
+            Sc<T>::fmac(v, a, q);
+            sum[2 * r] = v.x;
+            sum[2 * r + 1] = v.y;
+          } else {
+            Sc<T>::fmac(sum[r], a, q);
+          }
         }
       }
+    };
+    if (late) fp64(std::false_type());
+    else fp64(std::true_type());
+    if (late) {
+#pragma unroll
+      for (int u = 0; u < NV; ++u) sum[u] *= scale;
     }
   }
   if constexpr (NV == 8) {  // lane 4 u gets sum u
@@ -313,7 +329,7 @@ __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, i
   for (int u = 0; u < NV; ++u)
     if (lane == u) {
       const int r = u / NP, x = e + eq[r];
-      double w = x >= kLzBad / 2 ? nan("") : exact ? scalbn(sum[u], x - em - 2 * kLzBits) : sum[u];
+      double w = !exact ? sum[u] : x >= kLzBad / 2 ? nan("") : scalbn(sum[u], x - em - 2 * kLzBits);
       const T a = Sc<T>::scale(col[c], scale), q = Q[(size_t)r * n + c];
       if constexpr (Z) w = u % 2 ? fma(a.x, q.y, fma(-a.y, q.x, w)) : fma(a.x, q.x, fma(a.y, q.y, w));
       else w = fma(a, q, w);
@@ -322,13 +338,13 @@ __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, i
 }
 
 template <class T, int R>
-void lz_launch(cudaStream_t st, int n, const T* A, int lda, const int* ea, const T* Q, const typename LzInt<T>::type* Qi,
+void lz_launch(cudaStream_t st, int n, const T* A, int lda, int* ea, const T* Q, const typename LzInt<T>::type* Qi,
                const float4* Qm, const int* eq, const int* emax, T* W) {
   launch_dep(st, ceil_div(n, 8), 256, 0, lz_product_kernel<T, R>, n, A, lda, ea, Q, Qi, Qm, eq, emax, W);
 }
 
 template <class T>
-int lz_product(cudaStream_t st, int n, int nruns, const T* A, int lda, const int* ea,
+int lz_product(cudaStream_t st, int n, int nruns, const T* A, int lda, int* ea,
                const T* Q, const typename LzInt<T>::type* Qi, const float4* Qm, const int* eq, const int* emax,
                T* W, int* nl) {
   for (int r = 0; r < nruns; r += 4) {

@@ -6,6 +6,8 @@ diagonal and sparse ones."""
 import numpy as np
 import pytest
 
+import oracle
+
 torch = pytest.importorskip("torch")
 
 pytestmark = pytest.mark.gpu
@@ -65,3 +67,23 @@ def test_one_step(cl, kind, n, scale, complex_):
         h.close()
     assert abs(l1 / scale - alpha) <= ea
     assert abs(bsup / scale - (alpha + beta)) <= ea + eb
+
+
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("kind", ["dominant", "diagonal", "sparse", "graded"])
+def test_bounds_of_several_steps(cl, kind, complex_):
+    """Columns that a first step sums in FP64 stay so in the next, and for further groups of runs;
+    against the oracle, tolerance as for dense matrices."""
+    n, nruns, steps, ell = 300, 6, 20, 30
+    rng = np.random.default_rng(5)
+    A, _ = problem(kind, n, complex_, rng)
+    A /= np.linalg.norm(A, 2)
+    V = rng.standard_normal((n, nruns)) + (1j * rng.standard_normal((n, nruns)) if complex_ else 0.0)
+    ref, _ = oracle.lanczos_bounds(A, V, steps, ell)
+    h = cl.Handle(0)
+    try:
+        got = cl.chase_lanczos_bounds(h, cl.colmajor(torch.from_numpy(A).cuda()),
+                                      cl.colmajor(torch.from_numpy(V).cuda()), steps, ell)
+    finally:
+        h.close()
+    np.testing.assert_allclose(got, ref, rtol=0, atol=2e-9)
