@@ -184,9 +184,8 @@ struct LzSum {
 // the q_r, cut up, their magnitudes, their exponents.  A term of x is at most 2^56 (complex: two): the
 // sums of a lane are taken out after 120 (60) terms.  Bound by the wide multiply-adds, the instructions
 // that cut A up and the loads of q from L2.  4 runs, 25 steps of n = 8000: real 12.8 ms in FP64 -> 7.7
-// (7.2 without the check, two columns to a warp), complex 21.5; a sparse
-// real one, in FP64, 13.4.  Two blocks per SM, since more columns
-// at once spread the reads of A over more pages (three: 11 ms).
+// (7.2 without the check, two columns to a warp), complex 21.5; a sparse real matrix, in FP64, 13.4.
+// Two blocks per SM, since more columns at once spread the reads of A over more pages (three: 11 ms).
 template <class T, int R>
 __global__ void __launch_bounds__(256, 2) lz_product_kernel(int n, const T* A, int lda,
                                                             int* ea, const T* Q,

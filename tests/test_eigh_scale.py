@@ -128,6 +128,35 @@ def test_whole_space_rayleigh_ritz_over_the_range(cl, complex_, n, k):
     assert np.abs(A @ Y - Y * ev).max() <= tol
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("complex_,n", [(True, 1500), (False, 2100)])
+@pytest.mark.parametrize("k", [0, -600])
+def test_columns_that_stay_in_global_memory(cl, complex_, n, k):
+    """Orders whose columns do not fit the shared memory of one wave of thread blocks: the matrix is
+    scaled where it lies."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    dt = torch.complex128 if complex_ else torch.float64
+    rand = lambda: torch.randn(n, n, generator=g, device="cuda", dtype=dt)
+    Q = torch.linalg.qr(rand())[0]
+    lam = torch.sort(torch.rand(n, generator=g, device="cuda", dtype=torch.float64) * 2 - 1)[0]
+    A = (Q * lam) @ Q.mH
+    A = 0.5 * (A + A.mH)
+    V = cl.colmajor(rand())
+    s = 2.0 ** k
+    h = cl.Handle(0)
+    try:
+        cfg = cl.config_default(prec=cl.CHASE_FP64_EMU, opt_degree=0, deg_init=1, max_iter=1, qr_force=4, tol=1e-10 * s)
+        rc, ev, _, _, _ = cl.chase_solve(h, cl.colmajor(s * A), V, n, 0, (-s, 21.0 * s, 1000.0 * s), cfg)
+    finally:
+        h.close()
+    assert rc == 0
+    ev, tol = torch.from_numpy(np.asarray(ev)).cuda() / s, 40 * n * U
+    assert float((ev - lam).abs().max()) <= tol
+    assert float((V.mH @ V - torch.eye(n, device="cuda", dtype=dt)).abs().max()) <= tol
+    assert float((A @ V - V * ev).abs().max()) <= tol
+
+
 def lanczos(cl, A, V, steps, ell):
     dev = lambda x: torch.from_numpy(np.ascontiguousarray(np.asarray(x).T)).cuda().mT
     h = cl.Handle(0)
