@@ -746,7 +746,6 @@ def main():
                         "shifted_cholqr2": st["n_shifted"], "householder": st["n_hhqr"]},
         "phase_s": {k: st[k] for k in ("t_filter", "t_qr", "t_rr", "t_rr_eig", "t_resid", "t_total",
                                         "t_filter_lowprec")},
-        "jacobi_sweeps": st["jacobi_sweeps"],
         "lowprec_iterations": st["n_lowprec_iters"],
         "iteration_log": [{"it": g["iteration"], "locked": g["locked_before"],
                            "variant": g["variant"], "log10_cond_est": g["log_cond_est"] / 2.302585092994046,

@@ -18,7 +18,7 @@
 // What binds is FP64 at 2 FMAs per clock per SM (a warp instruction takes 64 clocks of a
 // sub-partition) and, in A, the chain of pivots: blocks of 32 keep A's share on one SM short
 // (64 would take four times that: the FP64 work of a block grows with its cube), the rest is
-// spread over all SMs.  n = 600 complex: 4.8 -> 2.0 ms (1.59 factor, 0.40 inverse) against blocks
+// spread over all SMs.  n = 600 complex: 4.8 -> 2.0 ms (1.62 factor, 0.41 inverse) against blocks
 // of 64 in separate launches and an inverse by single columns; n = 30 real 57 -> 26 us.
 #include "../../include/chase_gb300.h"
 #include "common.cuh"

@@ -18,6 +18,8 @@
 // conquer, 2.05 back-transformation), l = 230 complex 31 -> 3.0, l = 600 real 80 -> 6.7, l = 30
 // real 2.0 -> 0.41.
 //
+// H and then T are multiplied by powers of two that bring their largest entries to [0.5, 1), the
+// eigenvalues back at the end, so squares and reciprocals stay in range at every scale.
 // Every wait is bounded; a CTA that waits too long raises an abort flag that the others see, and
 // the kernel sets DevStatus.timeout.  Sums are taken in fixed orders: results are reproducible.
 // A non-finite T gives NaN eigenvalues and vectors.
