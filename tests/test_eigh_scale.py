@@ -178,3 +178,27 @@ def test_lanczos_bounds_scale_with_the_matrix(cl, complex_, k):
     # a power of two changes no rounding; only which couplings are left out may depend on it
     assert np.abs(got - one).max() <= 100 * steps * U
     assert got[2] >= lam[-1]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["CHASE_FP64_EMU", "CHASE_FP64"])
+@pytest.mark.parametrize("complex_,k", [(False, 0), (False, -60), (True, -60), (True, 60)])
+def test_solve_that_is_given_no_bounds(cl, complex_, k, prec):
+    """A small or large matrix (2^-60: energies in joules) with a tolerance to match and its bounds
+    from Lanczos runs, as at scale 1."""
+    n, nev, nex = 400, 20, 8
+    lam = W.spectrum_uniform(n, -1.0, 1.0, 5)
+    A = W.known_spectrum_matrix(lam, 5, complex_).numpy()
+    s = 2.0 ** k
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(np.asarray(x).T)).cuda().mT
+    V = dev(W.start_block(n, nev + nex, 6, complex_))
+    h = cl.Handle(0)
+    try:
+        cfg = cl.config_default(prec=getattr(cl, prec), opt_degree=1, tol=1e-10 * s)
+        rc, ev, res, st, _ = cl.chase_solve(h, dev(s * A), V, nev, nex, None, cfg)
+    finally:
+        h.close()
+    assert rc == 0 and st["iterations"] < 15
+    assert np.abs(np.asarray(ev) / s - lam[:nev]).max() <= 1e-10
+    Y = V.cpu().numpy()[:, :nev]
+    assert np.linalg.norm(A @ Y - Y * (np.asarray(ev) / s), axis=0).max() <= 2e-10
