@@ -1722,6 +1722,14 @@ int qr_impl(chase_ctx* h, int n, int l, T* X, int ldx, double est, int force, ch
   return rc;
 }
 
+// Lanczos bounds as a filter can use them: a damped interval of some width.  A multiple of the identity
+// has none of its own beyond rounding, any will do.
+void usable_bounds(chase_bounds* b) {
+  const double unit = 0x1p-48 * std::max(std::fabs(b->lambda1), std::fabs(b->b_sup));
+  if (!(b->b_sup - b->lambda1 > unit)) b->b_sup = b->lambda1 + std::fabs(b->lambda1);
+  if (!(b->b_sup > b->lambda_ell)) b->lambda_ell = 0.5 * (b->lambda1 + b->b_sup);
+}
+
 int lanczos_entry(chase_ctx* h, chase_dtype dtype, int n, const void* dA, int lda, int nruns,
                   const void* dV0, int ldv, int steps, int ell, chase_bounds* out) {
   const size_t elem = (dtype == CHASE_R64) ? sizeof(double) : sizeof(z64);
@@ -1871,7 +1879,7 @@ int chase_solve(chase_handle h, chase_dtype dtype, int n, const void* dA, int ld
     const int nruns = std::min(4, l), steps = std::min(25, n - 1);
     int rc = lanczos_entry(h, dtype, n, dA, lda, nruns, dV, ldv, steps, l, &bd);
     if (rc) return rc;
-    if (!(bd.b_sup > bd.lambda_ell)) bd.lambda_ell = 0.5 * (bd.lambda1 + bd.b_sup);
+    usable_bounds(&bd);
   }
   if (dtype == CHASE_R64)
     return solve_impl<double>(h, n, (const double*)dA, lda, nev, nex, c, bd, (double*)dV, ldv,
@@ -2033,7 +2041,7 @@ int chase_batch_add(chase_batch b, chase_dtype dtype, int n, const void* dA, int
     const int nruns = std::min(4, l), steps = std::min(25, n - 1);
     const int rc = lanczos_entry(h, dtype, n, dA, lda, nruns, dV, ldv, steps, l, &bd);
     if (rc) return rc;
-    if (!(bd.b_sup > bd.lambda_ell)) bd.lambda_ell = 0.5 * (bd.lambda1 + bd.b_sup);
+    usable_bounds(&bd);
   }
   chase_batch_ctx::Item it{};
   const size_t wsb = (dtype == CHASE_R64) ? solve_bytes<double>(n, l, c.prec) : solve_bytes<z64>(n, l, c.prec);

@@ -59,3 +59,42 @@ def test_start_in_an_invariant_subspace(cl, complex_, rotated):
     assert abs(got[0] - 2.0) <= 1e-2 and got[0] >= 2.0 - 100 * n * 2.0 ** -53
     assert got[2] >= 5.0 - 100 * n * 2.0 ** -53
     assert got[2] <= 5.0 + 3.0
+
+
+@pytest.mark.parametrize("complex_", [False, True])
+@pytest.mark.parametrize("c", [1.0, -3.0, 1e-18])
+@pytest.mark.parametrize("prec", ["CHASE_FP64", "CHASE_FP64_EMU"])
+def test_solve_of_a_multiple_of_the_identity(cl, prec, c, complex_):
+    """No bounds given, and none to be found but c itself."""
+    n, nev, nex = 100, 6, 3
+    rng = np.random.default_rng(4)
+    V = rng.standard_normal((n, nev + nex)) + (1j * rng.standard_normal((n, nev + nex)) if complex_ else 0.0)
+    Vd = cl.colmajor(torch.from_numpy(V).cuda())
+    h = cl.Handle(0)
+    try:
+        cfg = cl.config_default(prec=getattr(cl, prec), opt_degree=1, tol=1e-10 * abs(c))
+        rc, ev, _, _, _ = cl.chase_solve(h, cl.colmajor(torch.from_numpy(c * np.eye(n, dtype=V.dtype)).cuda()), Vd,
+                                         nev, nex, None, cfg)
+    finally:
+        h.close()
+    assert rc == 0
+    np.testing.assert_allclose(ev, c, rtol=1e-12)
+    Y = Vd[:, :nev]
+    eye = torch.eye(nev, device="cuda", dtype=Y.dtype)
+    assert float((Y.mH @ Y - eye).abs().max()) <= 1e-12
+
+
+@pytest.mark.parametrize("n", [3, 4, 5, 6, 7, 8, 9, 10, 12, 16])
+@pytest.mark.parametrize("c", [1.0, -2.0])
+def test_solve_whose_bounds_coincide(cl, n, c):
+    """One run of few steps from a unit vector: every Ritz value may round to c itself, which leaves the
+    filter no interval."""
+    V = np.eye(n)[:, :1]
+    Vd = cl.colmajor(torch.from_numpy(V.copy()).cuda())
+    h = cl.Handle(0)
+    try:
+        cfg = cl.config_default(prec=cl.CHASE_FP64, opt_degree=1, tol=1e-10)
+        rc, ev, _, _, _ = cl.chase_solve(h, cl.colmajor(torch.from_numpy(c * np.eye(n)).cuda()), Vd, 1, 0, None, cfg)
+    finally:
+        h.close()
+    assert rc == 0 and abs(ev[0] - c) <= 1e-12
